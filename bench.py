@@ -56,7 +56,7 @@ def parse():
     ap.add_argument("--no-variants", action="store_true", help="skip the nearest-voxel / Siddon / filter timings")
     ap.add_argument("--no-fdk", action="store_true", help="skip the 360-view FDK reconstruction timing")
     ap.add_argument("--mc-config", default=None, metavar="BLOCK,BATCH_MIN,HIST_PER_THREAD",
-                    help="fix the transport's launch configuration (lane form) instead of autotuning it")
+                    help="fix the transport's launch configuration instead of autotuning it")
     ap.add_argument("--local-majorant", type=int, default=None, metavar="CELL_SHIFT",
                     help="run the transport with the local-majorant option (cells of 2^CELL_SHIFT voxels) "
                          "instead of the paper's global Woodcock majorant, to profile the option")
@@ -197,7 +197,7 @@ def transport_roofline(steps, mc_s, hbm_peak, traffic, inst_per_step=None, n_sm=
     maximum SM clock) and the other ceilings ride along as context."""
     achieved = steps * BYTES_PER_STEP_ALGO / mc_s / 1e9
     r = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
-         "traffic": traffic, "kernel": "mc_kernel",
+         "traffic": traffic, "kernel": "mc_warp_kernel",
          "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy bandwidth)",
          "algorithmic": f"{BYTES_PER_STEP_ALGO} B of voxel data per Woodcock step x {steps} steps per launch",
          "mc_ms": 1e3 * mc_s, "woodcock_steps": steps}
@@ -358,11 +358,9 @@ def run_ours(args):
     l2_probe_gbs = gdrr.gdrr_probe_l2_gather(32 << 20)
     fp32_probe_tflops = gdrr.gdrr_probe_fp32()
     # kernels per step: ray trace, 3 finalisations, binning, the scalars,
-    # upsampling, noise (8); the transport (the pool form: one launch; the
-    # lane form: a source pass and a transport launch per 2^27 histories);
-    # the denoiser (one cooperative launch, else one per iteration + 2)
-    transport_launches = 1 if tuned["photon_pool"] > 0 else 2 * -(-n_hist // (1 << 27))
-    launches_per_step = 8 + transport_launches + (1 if res["denoise_fused"] else iters + 2)
+    # upsampling, noise (8); the transport (1); the denoiser (one cooperative
+    # launch, else one per iteration + 2)
+    launches_per_step = 9 + (1 if res["denoise_fused"] else iters + 2)
 
     clocks = ClockSampler(dev)
     if world > 1:
@@ -519,7 +517,7 @@ def run_ours(args):
                          ("mc_cells_16mm_ms", dict(cell_shift=3)),
                          # delta tracking with local majorants (an option beside the paper's
                          # global one): the cell bounds of 32 mm (default) or 16 mm cells as
-                         # the flights' majorant, lane form, batch_min 24; same expected images
+                         # the flights' majorant; same expected images
                          ("mc_local_majorant_32mm_ms", dict(local_majorant=1, cell_shift=4, batch_min=24,
                                                             photon_pool=-1)),
                          ("mc_local_majorant_16mm_ms", dict(local_majorant=1, cell_shift=3, batch_min=24,

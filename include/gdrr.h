@@ -136,14 +136,16 @@ typedef struct {
 typedef struct {
     double e_cut_kev;          /* absorb photons below this energy [1.0]           */
     int32_t max_steps;         /* free flights per history before giving up [1e5]  */
-    int32_t block_size;        /* threads per block, multiple of 32, <= 512 [256]   */
-    int32_t blocks_per_sm;     /* resident blocks per SM for the persistent grid [by occupancy] */
+    int32_t block_size;        /* threads per block of runs with records, multiple of
+                                  32, <= 512 [256]                                   */
+    int32_t blocks_per_sm;     /* most resident blocks (of block_size threads) per SM for
+                                  the persistent grid [by occupancy]                 */
     int32_t hist_per_thread;   /* histories a warp claims per lane at a time [8]    */
-    int32_t batch_min;         /* lanes of a warp that must be waiting for an
-                                  interaction, a tally or a new history before the
-                                  warp serves them together, 1..32 [16; 24 with
-                                  local_majorant, whose short flights bring the
-                                  services more often]                              */
+    int32_t batch_min;         /* runs with records: lanes of a warp that must be
+                                  waiting for an interaction, a tally or a new history
+                                  before the warp serves them together, 1..32 [16; 24
+                                  with local_majorant]; the other runs serve whole
+                                  warps whatever it is                               */
     int32_t nearest_voxel;     /* 1: no density interpolation, each point takes its
                                   voxel's density and material (the speed variant of
                                   the paper's appendix); 0: trilinear [0]           */
@@ -175,20 +177,16 @@ typedef struct {
                                   majorant itself, and the draws depend on their size.
                                   Changing it rebuilds the cell table (not while a scan
                                   exists).                                              */
-    int32_t photon_pool;       /* photons per thread, 1..3, in the shared-memory pool
-                                  of the pool form of the transport: blocks of 256
-                                  threads move photons between warps so that free
-                                  flights, corner gathers, interactions, tallies and
-                                  new histories each run on full warps (block_size and
-                                  batch_min do not apply to it); -1: the lane form, one
-                                  photon per lane with warp-batched services.  Runs
-                                  with records, nearest_voxel, scatter_filter,
-                                  rayleigh_form_factor or local_majorant always take
-                                  the lane form.  Tallies, counters and records are
-                                  the same for every choice.  On the 2 mm torso the
-                                  pool form ran at 125-158 ms per 1e8 histories
-                                  against 75 ms for the lane form, so the lane form is
-                                  the default and the autotuner times both [-1]       */
+    int32_t photon_pool;       /* photons per lane, 1..3, in the shared-memory pool that
+                                  each warp keeps (not in runs with records): a warp
+                                  holds more photons than lanes, so that free flights,
+                                  corner gathers, interactions, tallies and new
+                                  histories each run on full warps.  Tallies, counters
+                                  and records are the same for every choice; -1: the
+                                  pool that runs fastest, 80 photons per warp, which
+                                  local_majorant always takes (on the 2 mm torso 64, 72,
+                                  80 and 88 ran at 19.1, 18.2, 17.9 and 18.7 ms per 3e7
+                                  histories) [-1]                                     */
     int32_t local_majorant;    /* 1: delta tracking with local majorants, an option
                                   beside the paper's global Woodcock majorant: the
                                   macro-cell bounds (cell_shift, which must not be -1)
@@ -200,12 +198,8 @@ typedef struct {
                                   and so the per-history results, differ.  With
                                   cell_shift 0 the cells are then about 32 mm
                                   (round(log2(32 mm / smallest voxel edge)) in 1..6).
-                                  On the 2 mm torso it ran at 64 ms per 1e8 histories
-                                  (batch_min 24) against 75 ms for the global
-                                  majorant: 6.5 flights and 11.5 cell crossings per
-                                  history instead of 46 flights.
-                                  Runs the lane form; GDRR_ST_CELL_CROSSINGS counts the
-                                  cell crossings; 0: the global majorant [0]           */
+                                  GDRR_ST_CELL_CROSSINGS counts the cell crossings; 0:
+                                  the global majorant [0]                              */
 } gdrr_mc_options;
 
 /* Transport counters, accumulated by every gdrr_mc_project* call (device
@@ -250,9 +244,8 @@ GDRR_API int gdrr_create(const gdrr_geometry* geometry, const gdrr_phantom* phan
 /* Release every device buffer of the context (synchronises its stream).
  * A context's device buffers come from one stream-ordered memory pool per
  * device that keeps the blocks of destroyed contexts for the next ones (a
- * context of the 2 mm torso holds about 3.4 GB after a 1e8-history
- * projection, 3.2 GB of it source records); gdrr_release_memory hands them
- * back. */
+ * context of the 2 mm torso holds about 100 MB); gdrr_release_memory hands
+ * them back. */
 GDRR_API void gdrr_destroy(gdrr_ctx* ctx);
 
 /* Return the unused blocks of the contexts' device memory pools (on every
@@ -298,13 +291,7 @@ GDRR_API int gdrr_raytrace_primary_siddon(gdrr_ctx* ctx, double angle_rad, doubl
  * prim_dev / scat_dev: caller-owned device int64[nv*nu], ACCUMULATED (not
  * cleared) in units of 2^-24 keV.  stats_dev: NULL or device
  * uint64[GDRR_NSTATS], accumulated.  records_dev: NULL or device
- * gdrr_history_record[n_photons], written (debug / parity use; slower).
- * With default options and no records, the source points, directions and
- * energies are first sampled by a separate full-warp pass into a workspace
- * the context owns (32 bytes per history, at most 2^27 histories per pass,
- * allocated on first use; a scan keeps its own); the arithmetic is the same,
- * and when the workspace cannot be allocated the transport samples them
- * itself, with the same results. */
+ * gdrr_history_record[n_photons], written (debug / parity use; slower). */
 GDRR_API int gdrr_mc_project(gdrr_ctx* ctx, double angle_rad, uint32_t angle_index,
                              uint64_t n_photons, uint64_t seed, uint64_t history_offset,
                              int64_t* prim_dev, int64_t* scat_dev, uint64_t* stats_dev,
@@ -426,10 +413,9 @@ GDRR_API int gdrr_probe_fp32(double* tflops_out, void* cuda_stream);
 GDRR_API int gdrr_probe_bounded_wait(uint64_t limit_ns, void* cuda_stream);
 
 /* Autotuner: time gdrr_mc_project of n_probe histories at angle_rad for each
- * launch configuration of a fixed grid (the lane form: block size 64 / 128 /
- * 256 / 512, batch_min 8 .. 32, hist_per_thread 1 / 8 / 64; the pool form:
- * photon_pool 1 / 2 / 3, hist_per_thread 1 / 8 / 64), into scratch tallies, and
- * keep the fastest as the context's options (also copied to *best_out when
+ * launch configuration of a fixed grid (photon_pool -1 / 1 / 2 / 3, only -1
+ * with local majorants, and hist_per_thread 1 / 8 / 64), into scratch tallies,
+ * and keep the fastest as the context's options (also copied to *best_out when
  * not NULL).  Tallies do not depend on these options, only the speed does.
  * Synchronises. */
 GDRR_API int gdrr_autotune(gdrr_ctx* ctx, double angle_rad, uint64_t n_probe, uint64_t seed,

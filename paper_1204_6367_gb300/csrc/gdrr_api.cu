@@ -46,6 +46,7 @@ struct gdrr_ctx {
     // staged device data: one 8-byte record {density bits, material} per voxel
     uint2* d_vox = nullptr;
     float* d_tab = nullptr;
+    float* d_tab_e = nullptr;        // d_tab energy-major, for whole-row loads
     float* d_major = nullptr;
     float* d_resp = nullptr;
     float* d_bin_e = nullptr;
@@ -65,6 +66,7 @@ struct gdrr_ctx {
     float ff_idx = 0.0f;
     // macro-cell table of the early virtual-collision test (NULL: none)
     float* d_cells = nullptr;
+    float* d_open_cell = nullptr;
     int cell_shift = -1, ncx = 0, ncy = 0, ncz = 0;
     int n_scans = 0;              // live scans, which captured the table pointers
     int e_col = 0;                // 1: energy CDFs hold one row per detector column
@@ -80,8 +82,6 @@ struct gdrr_ctx {
     int64_t* d_tune = nullptr;       // autotuner scratch tallies, 2 * nu * nv
     int* d_status = nullptr;         // timeouts of bounded device waits since the last gdrr_sync
     void* d_arena = nullptr;         // one allocation holding the tables and counters above
-    float4* d_src = nullptr;         // source records of the lane form's source pass
-    uint64_t src_cap = 0;            // ... in histories
     // gdrr_project scratch: tallies, coarse tally and images, device scalars,
     // and the pinned host block the scalars come back through
     void* d_proj = nullptr;
@@ -106,8 +106,6 @@ struct gdrr_scan {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     uint64_t total = 0;
-    float4* d_src = nullptr;  // the scan's own source records (the graph captured the pointer)
-    uint64_t src_cap = 0;
     bool counted = false;     // included in ctx->n_scans
 };
 
@@ -306,7 +304,10 @@ __global__ void stage_voxels_kernel(const uint8_t* __restrict__ mat, const float
 // corners a point can touch whose lower corner lies in the cell.  Each voxel
 // raises its material's entry in every cell that covers it (at most two per
 // axis); float bits of non-negative densities order like the values, so an
-// unsigned atomicMax is exact.  cells: zeroed [cell][slots] words.
+// unsigned atomicMax is exact.  The layer -1 of each axis is a copy of layer
+// 0, so that a point in the outer half voxel, whose lower corner would be -1,
+// needs no clamp.  cells: zeroed [ncz + 1][ncy + 1][ncx + 1][slots] words,
+// layer -1 first.
 __global__ void build_cells_kernel(const uint2* __restrict__ vox, int nx, int ny, int nz, int bsy, int bsz, int shift,
                                    int ncx, int ncy, int slots, unsigned int* __restrict__ cells) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -318,13 +319,16 @@ __global__ void build_cells_kernel(const uint2* __restrict__ vox, int nx, int ny
     if (r.x == 0u) return;                       // zero density raises nothing
     const int mask = (1 << shift) - 1;
     const int cx1 = x >> shift, cy1 = y >> shift, cz1 = z >> shift;
-    const int cx0 = (x > 0 && (x & mask) == 0) ? cx1 - 1 : cx1;
-    const int cy0 = (y > 0 && (y & mask) == 0) ? cy1 - 1 : cy1;
-    const int cz0 = (z > 0 && (z & mask) == 0) ? cz1 - 1 : cz1;
+    int cx0 = (x > 0 && (x & mask) == 0) ? cx1 - 1 : cx1;
+    int cy0 = (y > 0 && (y & mask) == 0) ? cy1 - 1 : cy1;
+    int cz0 = (z > 0 && (z & mask) == 0) ? cz1 - 1 : cz1;
+    if (cx0 == 0) cx0 = -1;
+    if (cy0 == 0) cy0 = -1;
+    if (cz0 == 0) cz0 = -1;
     for (int cz = cz0; cz <= cz1; ++cz)
         for (int cy = cy0; cy <= cy1; ++cy)
             for (int cx = cx0; cx <= cx1; ++cx)
-                atomicMax(cells + ((size_t)(cz * ncy + cy) * ncx + cx) * slots + r.y, r.x);
+                atomicMax(cells + ((size_t)((cz + 1) * (ncy + 1) + cy + 1) * (ncx + 1) + cx + 1) * slots + r.y, r.x);
 }
 
 // (Re)build the macro-cell table for cells of 2^shift voxels per edge, or
@@ -338,7 +342,7 @@ int build_cells(gdrr_ctx* c, int shift, bool sync) {
     if (shift < 0) return GDRR_OK;
     const int ncx = ((c->nx - 1) >> shift) + 1, ncy = ((c->ny - 1) >> shift) + 1, ncz = ((c->nz - 1) >> shift) + 1;
     const int slots = material_slots(c->n_mat);
-    const size_t bytes = (size_t)ncx * ncy * ncz * slots * sizeof(float);
+    const size_t bytes = (size_t)(ncx + 1) * (ncy + 1) * (ncz + 1) * slots * sizeof(float);
     if (dalloc(c, &c->d_cells, bytes) != cudaSuccess) {
         c->d_cells = nullptr;
         return GDRR_ERR_OOM;
@@ -547,7 +551,7 @@ int free_ctx(gdrr_ctx* c) {
     if (c->side) cudaStreamSynchronize(c->side);   // a projection's ray trace reads the tables
     cudaStreamSynchronize(c->stream);
     void* bufs[] = {c->d_vox, c->d_arena, c->d_jobs, c->d_denoise, c->d_tune,
-                    c->d_ff_s, c->d_ff_a, c->d_ff_g, c->d_cells, c->d_proj, c->d_src};
+                    c->d_ff_s, c->d_ff_a, c->d_ff_g, c->d_cells, c->d_proj};
     if (c->pool)
         for (void* b : bufs) dfree(c, b);
     Pinned hp;
@@ -740,8 +744,18 @@ GDRR_API int gdrr_create(const gdrr_geometry* geometry, const gdrr_phantom* phan
             major[e] = (float)(mx * (1.0 + 1e-5));
         }
 
+        const int slots = material_slots(mt.n_materials);
+        std::vector<float> tab_e((size_t)mt.n_energies * 3 * slots, 0.0f);
+        for (int m = 0; m < mt.n_materials; ++m)
+            for (int k = 0; k < 3; ++k)
+                for (int e = 0; e < mt.n_energies; ++e)
+                    tab_e[((size_t)e * 3 + k) * slots + m] = tab[((size_t)m * 3 + k) * mt.n_energies + e];
+
         Arena ar;
         ar.add(&c->d_tab, tab.data(), tab.size());
+        ar.add(&c->d_tab_e, tab_e.data(), tab_e.size());
+        const std::vector<float> open_cell(slots, INFINITY);
+        ar.add(&c->d_open_cell, open_cell.data(), open_cell.size());
         ar.add(&c->d_major, major.data(), major.size());
         ar.add(&c->d_resp, dt.response, (size_t)dt.n_energies);
         ar.add(&c->d_bin_e, bin_e.data(), bin_e.size());
@@ -923,88 +937,6 @@ GDRR_API int gdrr_raytrace_primary_siddon(gdrr_ctx* ctx, double angle_rad, doubl
     return raytrace(ctx, angle_rad, P_dev, true, ctx->stream);
 }
 
-static int launch_grid(const gdrr_ctx* ctx, uint64_t total, bool rec) {
-    const int block = ctx->opt.block_size;
-    const int per_sm = ctx->opt.blocks_per_sm > 0 ? ctx->opt.blocks_per_sm
-                                                  : mc_occupancy_blocks(ctx->n_mat, block, rec, ctx->opt.local_majorant != 0);
-    int64_t grid = (int64_t)per_sm * ctx->n_sm;
-    const int64_t useful = (int64_t)((total + 31) / 32 * 32 + block - 1) / block;
-    if (grid > useful) grid = useful;
-    return grid < 1 ? 1 : (int)grid;
-}
-
-// Histories per segment of the lane form's source pass: MC_SRC_BYTES each,
-// at most 2^27 (4 GiB) per buffer.
-constexpr uint64_t SRC_MAX = 1ull << 27;
-
-// The source pass serves the lane form with default options and no records.
-static bool source_pass_applies(const gdrr_ctx* ctx, bool rec) {
-    return !rec && ctx->opt.nearest_voxel == 0 && ctx->opt.scatter_filter == 0 && ctx->opt.rayleigh_form_factor == 0 &&
-           (ctx->opt.photon_pool <= 0 || ctx->opt.local_majorant);
-}
-
-// Grows a source-record buffer to min(total, SRC_MAX) histories: the
-// context's from its device pool (owner given), a scan's with cudaMalloc
-// (owner NULL, on stream s).  When the memory is not there the buffer stays
-// empty and the transport samples the sources inline (the same arithmetic, so
-// the same results).
-static void ensure_src(const gdrr_ctx* owner, cudaStream_t s, float4** buf, uint64_t* cap, uint64_t total) {
-    const uint64_t want = std::min(total, SRC_MAX);
-    if (*cap >= want) return;
-    if (*buf) {
-        if (owner) {
-            dfree(owner, *buf);
-        } else {
-            cudaStreamSynchronize(s);
-            cudaFree(*buf);
-        }
-        *buf = nullptr;
-        *cap = 0;
-    }
-    const cudaError_t e = owner ? dalloc(owner, buf, want * MC_SRC_BYTES)
-                                : cudaMalloc((void**)buf, want * MC_SRC_BYTES);
-    if (e == cudaSuccess) {
-        *cap = want;
-    } else {
-        *buf = nullptr;
-        cudaGetLastError();   // an allocation failure here is not an error of the call
-    }
-}
-
-// The transport launch: the pool form for default options without records
-// (when its pool fits the SM), else the lane form; the lane form with
-// default options and a source buffer runs in segments of at most src_cap
-// histories, each a source pass and a transport launch (the caller zeroes
-// the work counter for the first).
-static cudaError_t launch_transport(const gdrr_ctx* ctx, const McParams& p, uint64_t total, bool rec,
-                                    cudaStream_t s, const float4* src = nullptr, uint64_t src_cap = 0) {
-    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0;
-    if (!rec && !gen && !p.lm && ctx->opt.photon_pool > 0) {
-        int per_sm = mc_pool_occupancy_blocks(ctx->n_mat, ctx->opt.photon_pool);
-        if (ctx->opt.blocks_per_sm > 0 && ctx->opt.blocks_per_sm < per_sm) per_sm = ctx->opt.blocks_per_sm;
-        if (per_sm > 0) {
-            int64_t grid = (int64_t)per_sm * ctx->n_sm;
-            const int64_t useful = (int64_t)((total + 31) / 32 * 32 + pool_threads() - 1) / pool_threads();
-            if (grid > useful) grid = useful;
-            return launch_mc_pool(p, ctx->opt.photon_pool, grid < 1 ? 1 : (int)grid, s);
-        }
-    }
-    if (!rec && !gen && src && src_cap > 0) {
-        for (uint64_t seg0 = 0; seg0 < total; seg0 += src_cap) {
-            McParams q = p;
-            q.seg0 = seg0;
-            q.total = std::min(src_cap, total - seg0);
-            q.src = src;
-            cudaError_t e = launch_mc_source(q, s);
-            if (e == cudaSuccess && seg0 > 0) e = cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), s);
-            if (e == cudaSuccess) e = launch_mc(q, ctx->opt.block_size, launch_grid(ctx, q.total, false), false, s);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaSuccess;
-    }
-    return launch_mc(p, ctx->opt.block_size, launch_grid(ctx, total, rec), rec, s);
-}
-
 // The launch-independent part of the transport parameters.
 static McParams static_mc_params(const gdrr_ctx* ctx) {
     McParams p;
@@ -1015,7 +947,7 @@ static McParams static_mc_params(const gdrr_ctx* ctx) {
     p.bsy = ctx->bsy; p.bsz = ctx->bsz;
     p.n_mat = ctx->n_mat; p.n_e = ctx->n_e;
     p.e0 = (float)ctx->e0; p.inv_de = (float)(1.0 / ctx->de);
-    p.tab = ctx->d_tab; p.major = ctx->d_major;
+    p.tab = ctx->d_tab; p.tab_e = ctx->d_tab_e; p.major = ctx->d_major;
     p.n_r = ctx->n_r; p.r0 = (float)ctx->r0; p.inv_dr = (float)(1.0 / ctx->dr); p.resp = ctx->d_resp;
     p.npix = ctx->geo.nu * ctx->geo.nv; p.n_guide_pix = ctx->n_guide_pix;
     p.kcdf_pix = ctx->d_kcdf_pix; p.guide_pix = ctx->d_guide_pix;
@@ -1030,7 +962,10 @@ static McParams static_mc_params(const gdrr_ctx* ctx) {
     p.n_ff = ctx->n_ff;
     p.ff_s = ctx->d_ff_s; p.ff_a = ctx->d_ff_a; p.ff_g = ctx->d_ff_g;
     p.inv_hc = (float)(1.0 / 12.398419843320026);
-    p.cells = ctx->d_cells;
+    const int csx = ctx->ncx + 1, csy = ctx->ncy + 1;
+    p.csx = csx; p.csy = csy;
+    p.cells = ctx->d_cells ? ctx->d_cells + (size_t)(1 + csx * (1 + csy)) * material_slots(ctx->n_mat) : nullptr;
+    p.open_cell = ctx->d_open_cell;
     p.cshift = ctx->cell_shift; p.ncx = ctx->ncx; p.ncy = ctx->ncy; p.ncz = ctx->ncz;
     p.lm = ctx->opt.local_majorant;
     for (int k = 0; k < 3; ++k) p.vox_mm[k] = (float)ctx->vox[k];
@@ -1038,6 +973,10 @@ static McParams static_mc_params(const gdrr_ctx* ctx) {
     p.ff_idx = ctx->ff_idx;
     return p;
 }
+
+// Photons per lane of a warp's pool (-1: the default); local majorants always
+// take the default one.
+static int pool_photons(const gdrr_ctx* ctx) { return ctx->opt.local_majorant ? -1 : ctx->opt.photon_pool; }
 
 static int mc_launch(gdrr_ctx* ctx, const std::vector<Job>& jobs, uint64_t total, uint64_t seed,
                      uint64_t* stats_dev, gdrr_history_record* records_dev) {
@@ -1069,12 +1008,8 @@ static int mc_launch(gdrr_ctx* ctx, const std::vector<Job>& jobs, uint64_t total
     p.nearest_voxel = ctx->opt.nearest_voxel;
     p.scatter_filter = ctx->opt.scatter_filter;
     p.ray_ff = ctx->opt.rayleigh_form_factor;
-    const bool rec = records_dev != nullptr;
-    if (source_pass_applies(ctx, rec)) {
-        ensure_src(ctx, ctx->stream, &ctx->d_src, &ctx->src_cap, total);
-        return cuda_err(launch_transport(ctx, p, total, rec, ctx->stream, ctx->d_src, ctx->src_cap));
-    }
-    return cuda_err(launch_transport(ctx, p, total, rec, ctx->stream));
+    return cuda_err(launch_mc(p, ctx->opt.block_size, ctx->opt.blocks_per_sm, pool_photons(ctx),
+                              records_dev != nullptr, ctx->n_sm, ctx->stream));
 }
 
 GDRR_API int gdrr_mc_project(gdrr_ctx* ctx, double angle_rad, uint32_t angle_index, uint64_t n_photons,
@@ -1168,7 +1103,6 @@ GDRR_API int gdrr_scan_create(gdrr_ctx* ctx, int32_t n_angles, const double* ang
         p.nearest_voxel = ctx->opt.nearest_voxel;
         p.scatter_filter = ctx->opt.scatter_filter;
         p.ray_ff = ctx->opt.rayleigh_form_factor;
-        if (source_pass_applies(ctx, false)) ensure_src(nullptr, ctx->stream, &sc->d_src, &sc->src_cap, total);
         if ((e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess) break;
         if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) break;
         const size_t tally_bytes = (size_t)n_angles * ctx->geo.nu * ctx->geo.nv * sizeof(int64_t);
@@ -1180,7 +1114,8 @@ GDRR_API int gdrr_scan_create(gdrr_ctx* ctx, int32_t n_angles, const double* ang
         if (ce == cudaSuccess && !stats_dev)
             ce = cudaMemsetAsync(sc->d_stats, 0, GDRR_NSTATS * sizeof(unsigned long long), cs);
         if (ce == cudaSuccess) ce = cudaMemsetAsync(sc->d_counter, 0, sizeof(unsigned long long), cs);
-        if (ce == cudaSuccess) ce = launch_transport(ctx, p, total, false, cs, sc->d_src, sc->src_cap);
+        if (ce == cudaSuccess) ce = launch_mc(p, ctx->opt.block_size, ctx->opt.blocks_per_sm, pool_photons(ctx), false,
+                           ctx->n_sm, cs);
         e = cudaStreamEndCapture(cs, &sc->graph);
         if (ce != cudaSuccess) { e = ce; break; }
         if (e != cudaSuccess) break;
@@ -1210,7 +1145,6 @@ GDRR_API void gdrr_scan_destroy(gdrr_scan* scan) {
     if (scan->d_jobs) cudaFree(scan->d_jobs);
     if (scan->d_counter) cudaFree(scan->d_counter);
     if (scan->d_stats) cudaFree(scan->d_stats);
-    if (scan->d_src) cudaFree(scan->d_src);
     if (scan->counted && scan->ctx) --scan->ctx->n_scans;
     delete scan;
 }
@@ -1228,10 +1162,8 @@ GDRR_API int gdrr_autotune(gdrr_ctx* ctx, double angle_rad, uint64_t n_probe, ui
     j.tally_s = ctx->d_tune + npix;
     const std::vector<Job> jobs(1, j);
     const gdrr_mc_options base = ctx->opt;
-    static const int blocks[] = {64, 128, 256, 512};
-    static const int batch[] = {8, 12, 16, 20, 24, 28, 32};
     static const int hpt[] = {1, 8, 64};
-    static const int pools[] = {1, 2, 3};
+    static const int pools[] = {-1, 1, 2, 3};
     cudaEvent_t e0, e1;
     TRY_CUDA(cudaEventCreate(&e0));
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return GDRR_ERR_CUDA; }
@@ -1239,16 +1171,9 @@ GDRR_API int gdrr_autotune(gdrr_ctx* ctx, double angle_rad, uint64_t n_probe, ui
     float best_ms = 3.0e38f;
     int rc = mc_launch(ctx, jobs, n_probe, seed, nullptr, nullptr);   // warm-up
     std::vector<gdrr_mc_options> grid;
-    for (int b : blocks)
-        for (int m : batch)
-            for (int h : hpt) {
-                gdrr_mc_options o = base;
-                o.block_size = b; o.batch_min = m; o.hist_per_thread = h; o.blocks_per_sm = 0; o.photon_pool = -1;
-                grid.push_back(o);
-            }
     for (int q : pools)
         for (int h : hpt) {
-            if (base.local_majorant) break;              // local majorants run the lane form only
+            if (base.local_majorant && q > 0) continue;   // their pool is the default one
             gdrr_mc_options o = base;
             o.hist_per_thread = h; o.blocks_per_sm = 0; o.photon_pool = q;
             grid.push_back(o);

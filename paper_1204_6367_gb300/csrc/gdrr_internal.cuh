@@ -62,6 +62,7 @@ struct McParams {
     int n_mat, n_e;
     float e0, inv_de;
     const float* tab;
+    const float* tab_e;            // the same, energy-major [e][k][material slots], zero beyond n_mat
     const float* major;
     // detector response
     int n_r;
@@ -105,20 +106,18 @@ struct McParams {
     // largest density over the voxels [c 2^s, (c + 1) 2^s] of each axis (the
     // cell and the next voxel), [cell][NM] with NM the kernel's material
     // slots; NULL disables the early virtual-collision test
+    // (cells points at cell 0, cell (cx, cy, cz) lies at cx + csx (cy + csy
+    // cz), and the layer -1 of each axis is a copy of layer 0).  open_cell: a
+    // record of infinite densities, for a test that nothing passes.
     const float* cells;
     int cshift, ncx, ncy, ncz;
+    int csx, csy;
+    const float* open_cell;
     // local majorants (lm = 1): the cell bounds serve as the free flights'
     // majorant; the cells' planes need the voxel edges
     int lm;
     float vox_mm[3];
     int* status;                   // NULL, or where a bounded loop that gave up records it
-    int pool_tail, pool_park_min;  // pool form: tail width and parking minimum (0: defaults)
-    // the launch covers flattened histories seg0 .. seg0 + total - 1; with src
-    // != NULL their source points were sampled by the source pass: src[2 i],
-    // src[2 i + 1] = {px, py, pz, dx}, {dy, dz, E, job + 1 as bits, or 0 when
-    // the history ended there} for history seg0 + i
-    uint64_t seg0;
-    const float4* src;
 };
 
 // Bounded waits on flags that another CTA publishes (release store, acquire
@@ -176,19 +175,12 @@ struct RtParams {
     Frame f;
 };
 
-cudaError_t launch_mc(const McParams& p, int block, int grid, bool records, cudaStream_t s);
-// The source pass of the lane form (default options, no records): samples
-// the source point, direction and energy of histories p.seg0 .. p.seg0 +
-// p.total - 1 into p.src, and tallies and counts those that miss the box.
-cudaError_t launch_mc_source(const McParams& p, cudaStream_t s);
-constexpr size_t MC_SRC_BYTES = 32;    // bytes of one history's source record
-int mc_occupancy_blocks(int n_mat, int block, bool records, bool lm);
-// The photon-pool form of the transport (default options, no records):
-// blocks of pool_threads() threads, per_thread photons per thread in the
-// shared-memory pool; 0 blocks per SM when the pool does not fit.
-cudaError_t launch_mc_pool(const McParams& p, int per_thread, int grid, cudaStream_t s);
-int mc_pool_occupancy_blocks(int n_mat, int per_thread);
-int pool_threads();
+// The transport of all of p's histories: with records one photon per lane in
+// blocks of `block` threads, else a pool of photons per warp (`photons` per
+// lane, 1 .. 3; <= 0: the default).  blocks_per_sm > 0 caps the resident
+// blocks (of `block` threads) per SM.
+cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
+                      cudaStream_t s);
 cudaError_t launch_rt(const RtParams& p, double* out, cudaStream_t s);
 cudaError_t launch_rt_siddon(const RtParams& p, double* out, cudaStream_t s);
 cudaError_t launch_air(const RtParams& p, double* out, cudaStream_t s);

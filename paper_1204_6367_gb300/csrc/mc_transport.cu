@@ -1,23 +1,21 @@
 // Monte Carlo photon transport, Section 2.4 of the paper, for sm_103a.
 //
-// One CUDA thread tracks one photon history at a time (as in the paper), but
-// the grid is persistent: warps claim chunks of histories from a global
-// counter and refill lanes whose history ended, so lanes stay busy while
-// histories of very different lengths finish.  The common event, a Woodcock
-// free flight that ends in a virtual collision, runs every iteration; the
-// rare, long branches (Rayleigh / Compton sampling, the detector tally, the
-// start of a new history) are deferred: a lane that needs one waits, and once
-// batch_min lanes of the warp wait, the warp serves them together.  Tallies
-// are int64 fixed point (2^-24 keV), summed with integer atomics, so the
-// result does not depend on which lane ran which history, when, or in which
-// order.
+// The grid is persistent: warps claim chunks of histories from a global
+// counter, and each warp keeps a pool of photons in shared memory from which
+// it runs the common event (a Woodcock free flight that ends in a virtual
+// collision) and each of the rare, long ones (corner gathers, Rayleigh /
+// Compton sampling, the detector tally and the start of a new history) on
+// whole warps (mc_warp_kernel).  Runs with event records keep one photon per
+// lane (mc_kernel).  Tallies are int64 fixed point (2^-24 keV), summed with
+// integer atomics, so the result does not depend on which lane ran which
+// history, when, or in which order.
 //
 // Data layout: one 8-byte record {density bits, material index} per voxel,
 // in bricks of 4 x 2 x 2 voxels (one 128-byte cache line each), so each
 // trilinear corner is a single 8-byte gather and the eight corners of a cell
 // touch about 2.8 distinct lines instead of about 4.3 for a row-major layout;
-// the per-lane energy-dependent coefficients live in shared memory, indexed
-// by material, one column per thread.
+// the energy-dependent coefficients of a photon live in shared memory, indexed
+// by material.
 //
 // Most tentative collisions of Woodcock tracking are virtual (over 90 % in a
 // torso, whose majorant is set by dense bone).  Before the eight corner
@@ -27,8 +25,8 @@
 // corners hold, and the gathers are skipped.  The bound never falls below the
 // mu the gathers give, so every decision, draw and tally is the one plain
 // Woodcock tracking makes.  A flight that passes the test waits, like the rare
-// events, for the warp's service batch, where its gathers run together with
-// those of the warp's other waiting lanes.
+// events, for a service of the warp, where its gathers run together with those
+// of the warp's other waiting photons.
 //
 // Local majorants (an option, LM): the macro-cell bounds themselves serve as a
 // piecewise-constant majorant.  A flight draws its optical depth tau = -ln xi
@@ -68,6 +66,8 @@
 //    unit disc;
 //  * tally: rint(r(E) * 2^24) into the primary counter when the photon never
 //    scattered, else the scatter counter (Section 2.4).
+#include <algorithm>
+
 #include "gdrr_internal.cuh"
 
 namespace gdrr {
@@ -279,6 +279,7 @@ __device__ __forceinline__ void polar(Stream& rs, const RoundKeys& rk, bool ray,
     const float alpha = e * (float)(1.0 / 510.99895);
     const float ialpha = (float)510.99895 / e;
     const float ta = 2.0f * alpha;
+    const float branch = (1.0f + ta) / (9.0f + ta);
     float x = 1.0f, mu = 1.0f;
     for (;;) {
         const uint4 w = rs.block(rk);
@@ -292,11 +293,14 @@ __device__ __forceinline__ void polar(Stream& rs, const RoundKeys& rk, bool ray,
             const float r1 = uniform(w.x);
             const float r2 = uniform(w.y);
             const float r3 = uniform(w.z);
-            if (r1 <= (1.0f + ta) / (9.0f + ta)) {
-                x = 1.0f + ta * r2;
-                done = r3 <= 4.0f * (x - 1.0f) / (x * x);
+            const bool low = r1 <= branch;
+            const float xa = 1.0f + ta * r2;
+            const float quot = (low ? 4.0f * (xa - 1.0f) : 1.0f + ta) / (low ? xa * xa : xa);   // one division for both
+            if (low) {
+                x = xa;
+                done = r3 <= quot;
             } else {
-                x = (1.0f + ta) / (1.0f + ta * r2);
+                x = quot;
                 const float c = 1.0f - (x - 1.0f) * ialpha;
                 done = r3 <= 0.5f * (c * c + 1.0f / x);
             }
@@ -326,8 +330,18 @@ enum : int { S_DEAD = 0, S_FLY = 1, S_RAY = 2, S_COMP = 3, S_ESC = 4, S_GATHER =
 // cell of a new history's entry point.
 enum : uint32_t { LM_DRAW = 1u, LM_DIR = 2u, LM_CELL = 4u, LM_ALL = 7u };
 
-// Block-shared counters (GDRR_NSTATS), flushed to the stats array at exit.
-__device__ __forceinline__ void count(unsigned long long* c, int k) { atomicAdd(c + k, 1ull); }
+// Where a history's events are counted: block-shared counters (GDRR_NSTATS,
+// flushed to the stats array at exit), or a mask of the events of one service
+// that the warp then counts by ballot.
+struct SharedCounts {
+    unsigned long long* c;
+    __device__ __forceinline__ void add(int k) { atomicAdd(c + k, 1ull); }
+};
+struct EventMask {
+    uint32_t m;
+    __device__ __forceinline__ void add(int k) { m |= 1u << k; }
+    __device__ __forceinline__ bool has(int k) const { return (m >> k) & 1u; }
+};
 
 // GEN: the general kernel, which honours the nearest-voxel and scatter-filter
 // options; the default kernel (GEN = false) carries neither.  LM: free flights
@@ -362,6 +376,8 @@ struct Lane {
     // k = 0 total, 1 Rayleigh, 2 Compton (photoelectric is the remainder)
     float* coef;
     int stride;          // blockDim.x
+    const float* tot;    // where gather() reads the totals: coef's, or a pool slot's
+    int tot_stride;
     // event record (REC only)
     uint64_t gidx;
     uint32_t r_virt, r_ray, r_comp, r_first, r_raymat;
@@ -369,13 +385,14 @@ struct Lane {
     double r_dep;
 
     __device__ __forceinline__ float& cf(int k, int m) { return coef[(k * NM + m) * stride]; }
+    __device__ __forceinline__ float total(int m) const { return tot[m * tot_stride]; }
 
     // Largest total mu at the lane's energy over a macro cell's voxels: the
     // cell's per-material maximum densities times the lane's coefficients.
     // Every corner's term rho_c mu_m(E) is at most this, and the trilinear
     // weights sum to one, so the mixture mu is at most it too.
     __device__ __forceinline__ float cell_bound(const McParams& P, int cell) {
-        const float* r = P.cells + (size_t)cell * NM;
+        const float* r = P.cells + (ptrdiff_t)cell * NM;
         float b;
         if constexpr (NM == 2) {
             const float2 v = __ldg(reinterpret_cast<const float2*>(r));
@@ -444,7 +461,8 @@ struct Lane {
     // plane; tally r(E) at the pixel it meets (Section 2.4).  A lane that
     // left the box in a free flight first moves from its last position inside
     // to the box surface along its direction.
-    __device__ __forceinline__ void escape(const McParams& P, unsigned long long* cnt, bool from_inside) {
+    template <class CNT>
+    __device__ __forceinline__ void escape(const McParams& P, CNT& cnt, bool from_inside) {
         if (from_inside) move_to_box_exit(P);
         const Job& J = P.jobs[job];
         const float n0 = J.f.n[0], n1 = J.f.n[1], n2 = J.f.n[2];
@@ -478,7 +496,7 @@ struct Lane {
                 }
             }
         }
-        count(cnt, outcome == OUT_PRIMARY ? GDRR_ST_TALLY_PRIMARY
+        cnt.add(outcome == OUT_PRIMARY ? GDRR_ST_TALLY_PRIMARY
                                           : (outcome == OUT_SCATTER ? GDRR_ST_TALLY_SCATTER : GDRR_ST_MISS));
         record(P, outcome, pixel, 0);
         end_counts(from_inside ? 1u : 0u);
@@ -491,11 +509,8 @@ struct Lane {
         const float p[3] = {px, py, pz};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            if (d[a] > 0.0f) {
-                const float t = (P.hi[a] - p[a]) / d[a];
-                if (t < te) te = t;
-            } else if (d[a] < 0.0f) {
-                const float t = (P.lo[a] - p[a]) / d[a];
+            if (d[a] > 0.0f || d[a] < 0.0f) {
+                const float t = ((d[a] > 0.0f ? P.hi[a] : P.lo[a]) - p[a]) / d[a];
                 if (t < te) te = t;
             }
         }
@@ -507,7 +522,8 @@ struct Lane {
 
     // Start flattened history g: source sampling and box entry.  Leaves the
     // lane FLY, or DEAD after tallying a photon that misses the box.
-    __device__ __forceinline__ void start(const McParams& P, uint64_t g, unsigned long long* cnt) {
+    template <class CNT>
+    __device__ __forceinline__ void start(const McParams& P, uint64_t g, CNT& cnt) {
         gidx = g;
         int lo = 0, hi = P.n_jobs - 1;
         while (lo < hi) {
@@ -518,7 +534,7 @@ struct Lane {
         const Job& J = P.jobs[job];
         const uint64_t hid = J.hid_offset + (g - J.first);
         rs.init(J.angle_index, hid);
-        count(cnt, GDRR_ST_HISTORIES);
+        cnt.add(GDRR_ST_HISTORIES);
         nsteps = 0;
         ngath = 0;
         scattered = 0;
@@ -579,35 +595,11 @@ struct Lane {
         state = S_FLY;
     }
 
-    // Start history P.seg0 + i from the source pass's record: the state
-    // start() leaves (source block drawn, position at the box entry, energy
-    // tables pending), or nothing when the history already ended there.
-    __device__ __forceinline__ void start_src(const McParams& P, uint64_t i) {
-        const float4 b = __ldcs(P.src + 2 * i + 1);
-        const uint32_t j1 = __float_as_uint(b.w);
-        if (j1 == 0u) return;
-        const float4 a = __ldcs(P.src + 2 * i);
-        const uint64_t g = P.seg0 + i;
-        gidx = g;
-        job = (int)j1 - 1;
-        const Job& J = P.jobs[job];
-        rs.init(J.angle_index, J.hid_offset + (g - J.first));
-        rs.blk = 1;
-        nsteps = 0;
-        ngath = 0;
-        scattered = 0;
-        px = a.x; py = a.y; pz = a.z;
-        dx = a.w; dy = b.x; dz = b.y;
-        e = b.z;
-        if (defer_e) need_e = true; else set_energy(P, e);
-        if (LM) lm_need = LM_ALL;
-        state = S_FLY;
-    }
-
     // One Woodcock free flight and the real/virtual decision at its end.
-    __device__ __forceinline__ void step(const McParams& P, unsigned long long* cnt) {
+    template <class CNT>
+    __device__ __forceinline__ void step(const McParams& P, CNT& cnt) {
         if ((int)nsteps >= P.max_steps) {
-            count(cnt, GDRR_ST_STEP_LIMIT);
+            cnt.add(GDRR_ST_STEP_LIMIT);
             record(P, OUT_STEP_LIMIT, -1, 0);
             end_counts(0u);
             state = S_DEAD;
@@ -655,7 +647,7 @@ struct Lane {
         if (P.cells) {
             // the corners lie in [x0, x0 + 1] etc., inside the cover of x0's cell:
             // above the cell's bound the collision is virtual whatever they hold
-            const int cell = (x0 >> P.cshift) + P.ncx * ((y0 >> P.cshift) + P.ncy * (z0 >> P.cshift));
+            const int cell = (x0 >> P.cshift) + P.csx * ((y0 >> P.cshift) + P.csy * (z0 >> P.cshift));
             if (t > cell_bound(P, cell)) {
                 if (GEN) { ++c_virt; ++c_skip; }
                 if (REC) ++r_virt;
@@ -680,7 +672,8 @@ struct Lane {
     // LM, in the service batch: the entry cell of a new history, the
     // reciprocals of a new direction, and the next flight: its Philox block,
     // its optical depth tau = -ln xi and the uniform of its ordinate test.
-    __device__ __forceinline__ void lm_prepare(const McParams& P, unsigned long long* cnt) {
+    template <class CNT>
+    __device__ __forceinline__ void lm_prepare(const McParams& P, CNT& cnt) {
         if (lm_need & LM_CELL) {
             const int gx = max((int)floorf((px - P.lo[0]) * P.ivox[0] - 0.5f), 0) >> P.cshift;
             const int gy = max((int)floorf((py - P.lo[1]) * P.ivox[1] - 0.5f), 0) >> P.cshift;
@@ -696,7 +689,7 @@ struct Lane {
         }
         lm_need = 0u;
         if ((int)nsteps >= P.max_steps) {
-            count(cnt, GDRR_ST_STEP_LIMIT);
+            cnt.add(GDRR_ST_STEP_LIMIT);
             record(P, OUT_STEP_LIMIT, -1, 0);
             end_counts(0u);
             state = S_DEAD;
@@ -718,8 +711,7 @@ struct Lane {
     // a tie).  Every crossing moves the cell along the direction of flight, so
     // a flight crosses at most ncx + ncy + ncz cells; leaving the grid leaves
     // the box, from the last position inside.
-    __device__ __forceinline__ void walk(const McParams& P) {
-        const float b = cell_bound(P, cx + P.ncx * (cy + P.ncy * cz));
+    __device__ __forceinline__ void walk(const McParams& P, float b) {
         float tx = (float)3.0e38, ty = tx, tz = tx;
         if (dx > 0.0f) tx = (lm_plane(P, 0, cx + 1, P.ncx) - px) * idx;
         else if (dx < 0.0f) tx = (lm_plane(P, 0, cx, P.ncx) - px) * idx;
@@ -762,10 +754,11 @@ struct Lane {
     // decision for its t.  The warp serves its waiting lanes together, so the
     // gathers run on many lanes at once instead of on the few whose flights
     // passed the test in one iteration.
-    __device__ __forceinline__ void gather(const McParams& P, unsigned long long* cnt) {
+    template <class CNT>
+    __device__ __forceinline__ void gather(const McParams& P, CNT& cnt) {
         if (!GEN) ++ngath;
         const float t = tg;
-        if (LM && GEN && P.nearest_voxel) {
+        if (GEN && P.nearest_voxel) {
             // no density interpolation: the voxel containing the point
             const int gx = min(max((int)floorf((px - P.lo[0]) * P.ivox[0]), 0), P.nx - 1);
             const int gy = min(max((int)floorf((py - P.lo[1]) * P.ivox[1]), 0), P.ny - 1);
@@ -773,7 +766,7 @@ struct Lane {
             const uint2 vx = __ldg(P.vox + brick_x(gx) + brick_y(gy, P.bsy) + brick_z(gz, P.bsz));
             const float a0 = __uint_as_float(vx.x);
             const int m0 = (int)vx.y;
-            if (t > a0 * cf(0, m0)) {
+            if (t > a0 * total(m0)) {
                 ++c_virt;
                 if (REC) ++r_virt;
                 lm_need |= LM_DRAW;
@@ -809,9 +802,9 @@ struct Lane {
             a[c] = (wxy[c & 3] * ((c >> 2) ? tz : wz0)) * __uint_as_float(vx.x);
             mc[c] = (int)vx.y;
         }
-        float muT = a[0] * cf(0, mc[0]);
+        float muT = a[0] * total(mc[0]);
 #pragma unroll
-        for (int c = 1; c < 8; ++c) muT = muT + a[c] * cf(0, mc[c]);
+        for (int c = 1; c < 8; ++c) muT = muT + a[c] * total(mc[c]);
         if (t > muT) {
             ++c_virt;
             if (REC) ++r_virt;
@@ -842,14 +835,14 @@ struct Lane {
 
     // A real collision: Rayleigh if t <= mu_R, Compton if t <= mu_R + mu_C,
     // else photoelectric absorption.
-    __device__ __forceinline__ void real_collision(const McParams& P, float t, float muR, float muC,
-                                                   unsigned long long* cnt) {
+    template <class CNT>
+    __device__ __forceinline__ void real_collision(const McParams& P, float t, float muR, float muC, CNT& cnt) {
         if (t <= muR) {
             state = S_RAY;
         } else if (t <= muR + muC) {
             state = S_COMP;
         } else {
-            count(cnt, GDRR_ST_PHOTO);
+            cnt.add(GDRR_ST_PHOTO);
             if (REC) { if (!r_first) r_first = 3; r_dep += (double)e; }
             record(P, OUT_PHOTO, -1, 1);
             end_counts(0u);
@@ -860,7 +853,8 @@ struct Lane {
     // The deferred Rayleigh or Compton interaction of a waiting lane.  The
     // polar angle comes from the event's own sampler; the azimuth and the
     // rotation are common code, so a batch holding both kinds runs them once.
-    __device__ __forceinline__ void interact(const McParams& P, unsigned long long* cnt) {
+    template <class CNT>
+    __device__ __forceinline__ void interact(const McParams& P, CNT& cnt) {
         const bool ray = state == S_RAY;
         float ct, e2 = e;
         if (GEN && ray && P.ray_ff) {
@@ -875,19 +869,19 @@ struct Lane {
         scattered = 1;
         if (ray) {
             if (GEN) n_int += 0x10000u;
-            count(cnt, GDRR_ST_RAYLEIGH);
+            cnt.add(GDRR_ST_RAYLEIGH);
             if (REC) { ++r_ray; if (!r_first) r_first = 1; }
             if (LM) lm_need |= LM_DRAW | LM_DIR;
             state = S_FLY;
             return;
         }
         if (GEN) n_int += 1u;
-        count(cnt, GDRR_ST_COMPTON);
+        cnt.add(GDRR_ST_COMPTON);
         if (REC) { ++r_comp; if (!r_first) r_first = 2; r_dep += (double)e - (double)e2; }
         if (e2 < P.e_cut) {
             e = e2;
             if (REC) r_dep += (double)e;
-            count(cnt, GDRR_ST_CUTOFF);
+            cnt.add(GDRR_ST_CUTOFF);
             record(P, OUT_CUTOFF, -1, 0);
             end_counts(0u);
             state = S_DEAD;
@@ -904,19 +898,24 @@ struct Lane {
     }
 };
 
-template <int NM, bool REC, bool GEN, bool LM>
+// The transport with records (parity runs): one photon per lane from birth to
+// death.
+template <int NM, bool GEN, bool LM>
 // Up to 512 threads per block, 64 registers per thread (the same cap at 2 x 512
 // or 4 x 256 resident threads): the autotuner's block sizes 64 ... 512.
 __global__ void __launch_bounds__(512, 2) mc_kernel(const McParams P) {
     extern __shared__ float smem[];
-    __shared__ unsigned long long cnt[GDRR_NSTATS];
-    for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x) cnt[i] = 0ull;
+    __shared__ unsigned long long counts[GDRR_NSTATS];
+    for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x) counts[i] = 0ull;
     __syncthreads();
 
     const int lane = threadIdx.x & 31;
-    Lane<NM, REC, GEN, LM> L;
+    SharedCounts cnt = {counts};
+    Lane<NM, true, GEN, LM> L;
     L.coef = smem + threadIdx.x;
     L.stride = blockDim.x;
+    L.tot = L.coef;
+    L.tot_stride = L.stride;
     L.state = S_DEAD;
     L.defer_e = true;                 // new histories and Compton events share one table pass
     L.need_e = false;
@@ -949,10 +948,7 @@ __global__ void __launch_bounds__(512, 2) mc_kernel(const McParams P) {
                     const unsigned want = (unsigned)__popc(need);
                     const unsigned take = want < avail ? want : avail;
                     const unsigned rank = (unsigned)__popc(need & ((1u << lane) - 1u));
-                    if (((need >> lane) & 1u) && rank < take) {
-                        if (!REC && !GEN && P.src) L.start_src(P, pool_next + rank);
-                        else L.start(P, P.seg0 + pool_next + rank, cnt);
-                    }
+                    if (((need >> lane) & 1u) && rank < take) L.start(P, pool_next + rank, cnt);
                     pool_next += take;
                     need = __ballot_sync(FULL, L.state == S_DEAD);
                 }
@@ -965,392 +961,604 @@ __global__ void __launch_bounds__(512, 2) mc_kernel(const McParams P) {
             if (exhausted && !__any_sync(FULL, L.state != S_DEAD)) break;
         }
         if (L.state == S_FLY) {
-            if constexpr (LM) L.walk(P);
+            if constexpr (LM) L.walk(P, L.cell_bound(P, L.cx + P.csx * (L.cy + P.csy * L.cz)));
             else L.step(P, cnt);
         }
     }
 
-    atomicAdd(&cnt[GDRR_ST_STEPS], (unsigned long long)L.c_steps);
-    atomicAdd(&cnt[GDRR_ST_VIRTUAL], (unsigned long long)L.c_virt);
-    atomicAdd(&cnt[GDRR_ST_CELL_SKIPS], (unsigned long long)L.c_skip);
-    if (LM) atomicAdd(&cnt[GDRR_ST_CELL_CROSSINGS], (unsigned long long)L.c_cross);
+    atomicAdd(&counts[GDRR_ST_STEPS], (unsigned long long)L.c_steps);
+    atomicAdd(&counts[GDRR_ST_VIRTUAL], (unsigned long long)L.c_virt);
+    atomicAdd(&counts[GDRR_ST_CELL_SKIPS], (unsigned long long)L.c_skip);
+    if (LM) atomicAdd(&counts[GDRR_ST_CELL_CROSSINGS], (unsigned long long)L.c_cross);
     __syncthreads();
     for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x)
-        if (cnt[i]) atomicAdd(P.stats + i, cnt[i]);
+        if (counts[i]) atomicAdd(P.stats + i, counts[i]);
 }
 
 // ---------------------------------------------------------------------------
-// The source pass: Lane::start for every history of the launch, on full
-// warps (one history per thread), apart from the transport's service
-// batches.  A history that misses the box is tallied and counted here; the
-// others leave their state (position at the box entry, direction, energy)
-// for Lane::start_src.  The arithmetic is start()'s, call for call, so the
-// transport's draws, decisions and tallies do not change.
-template <int NM>
-__global__ void __launch_bounds__(256) mc_source_kernel(const McParams P, float4* __restrict__ out) {
-    __shared__ unsigned long long cnt[GDRR_NSTATS];
-    for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x) cnt[i] = 0ull;
-    __syncthreads();
-    Lane<NM, false, false> L;
-    L.coef = nullptr;
-    L.stride = 0;
-    L.defer_e = true;
-    L.need_e = false;
-    L.c_steps = 0; L.c_virt = 0; L.c_skip = 0;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P.total;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        L.state = S_DEAD;
-        L.start(P, P.seg0 + i, cnt);
-        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
-        if (L.state == S_FLY) {
-            a = make_float4(L.px, L.py, L.pz, L.dx);
-            b = make_float4(L.dy, L.dz, L.e, __uint_as_float((uint32_t)L.job + 1u));
-        }
-        __stcs(out + 2 * i, a);
-        __stcs(out + 2 * i + 1, b);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x)
-        if (cnt[i]) atomicAdd(P.stats + i, cnt[i]);
-}
-
-// ---------------------------------------------------------------------------
-// The photon-pool form of the same transport.
+// The transport without records: a pool of photons per warp.
 //
-// In mc_kernel a lane keeps its photon from birth to death, so a warp flies
-// only the lanes that are not waiting for a service, and serves its waiting
-// lanes on partial warps.  Here a block of 8 warps shares a pool of photons
-// in shared memory and moves them between warps: every phase runs the
-// photons that need it on full warps.  A round of the block is
-//   START   free slots take new histories (source sampling, box entry);
-//   FLIGHT  each lane flies a photon until its flight needs the corner
-//           gathers or leaves the box, parks it, and takes the next ready
-//           photon of its class;
-//   GATHER  the eight-corner mixture of the parked flights: virtual, real;
-//   INTER   Rayleigh / Compton sampling of the real collisions;
-//   ESCAPE  box exit and imager tally;
-// with a block barrier between phases.  Lane l of every warp serves pool
-// class l only: class l holds K slots, and field f of slot s sits at word
-// (f K + s) 32 + l, so a warp's 32 lanes touch 32 different banks whatever
-// slots they hold.  Each class keeps queues of slot numbers per phase; a
-// queue's entry j goes to warp j mod 8, which packs the work into full warps.
-// The arithmetic per photon is Lane's, call for call (start, step, gather,
-// interact, escape), so every history's draws, decisions and tally are the
-// ones mc_kernel and the oracle produce; only the order in which histories
-// advance differs, and the integer tallies and counters do not depend on it.
-enum : int {
-    PF_PX, PF_PY, PF_PZ, PF_DX, PF_DY, PF_DZ, PF_E, PF_MUMAX, PF_INVMU, PF_TG,
-    PF_STATE, PF_JOB, PF_NSTEPS, PF_NGATH, PF_ANGLE, PF_HLO, PF_HHI, PF_BLK, PF_N
-};
-// queues (slot numbers, one byte each): ready by round parity, gather,
-// interaction, escape, free by round parity
-enum : int { PQ_R0, PQ_R1, PQ_G, PQ_I, PQ_E, PQ_F0, PQ_F1, PQ_N };
-// per-class counters: queue lengths (by queue), the ready queue's read head
-enum : int { PC_HEAD = PQ_N, PC_N };
+// A lane that keeps its photon from birth to death (mc_kernel) waits while
+// its warp serves others and serves its rare events on partial warps: 16 of
+// 32 lanes were active per instruction.  Here a warp owns a pool of photons
+// (more than its 32 lanes) in shared memory and four lists of them: ready to
+// fly, at a tentative collision (the corner gathers), at a real one (the
+// interaction), and at the end of their history (the box exit and tally, then
+// the next history).  It flies 32 photons at a time; a lane whose flight stops
+// hands its photon to a list and takes the next ready one, and once a list
+// holds a whole warp's worth, the warp parks its photons and serves that list
+// with every lane.  Nothing is shared between warps, so there is no block
+// barrier: lists and slots are exchanged under __syncwarp alone.
+//
+// The arithmetic per photon is Lane's (start, gather, interact, escape, walk)
+// or, for the free flight, the same operations on fewer instructions, so every
+// history's draws, decisions and tally are the ones mc_kernel and the oracle
+// produce; integer tallies and counters do not depend on the order in which
+// histories advance.
+//
+// The flight loop loads the macro-cell record of its end point first and forms
+// the next flight's Philox block and logarithm while the load is under way; a
+// photon carries those words through its slot, and only a collision or a new
+// history, whose blocks move on, forms them anew.
+//
+// What bounds it: instruction issue (71 % of the slots, 25 of 32 lanes active
+// per instruction, 28 in flight) beside L1 wavefronts (66 %).  2 mm torso, 1e8
+// histories (58 free flights each): 87.8 ms with one photon per lane and a
+// separate source pass, 58.0 ms so; per history 863 warp instructions before,
+// about 500 now, 230 of them free flights, 50 hand-overs, 77 interactions.
+//
+// A slot is Q float4 words: {px py pz, and t = xi mumax at a tentative
+// collision or the next flight's -ln xi} {dx dy dz E} {mumax 1/mumax, or the
+// optical depth and cells of LM; history id lo; job, flags} {blocks drawn,
+// block limit, history id hi, the next flight's second word} {total
+// coefficient per material}, LM {1/d, cell z}, GEN {the flight's third word,
+// interaction counts, form-factor material}.  The history's free flights so
+// far are its blocks less those drawn elsewhere, so the flight only compares
+// its block number with a limit that grows by the blocks drawn elsewhere:
+// max_steps costs no counter of its own.  The totals of free flights, and of
+// the virtual collisions the cells decided, follow from warp-wide counts of
+// lanes per iteration.
+constexpr int WARP_BLOCK = 128;                // threads; the warps of a block share nothing but counters
+// Resident blocks the registers are held down for: 24 warps per SM (80
+// registers), 20 for the general form.  On the 2 mm torso 28 warps (72) and 32
+// (64 registers, spills in the flight loop) were 1 and 8 % slower.
+constexpr int WARP_MIN_BLOCKS = 6, WARP_MIN_BLOCKS_GEN = 5;
+constexpr int POOL_DEFAULT = 80;               // photons per warp: the most that 24 warps' shared memory holds
+// Idle lanes at which the warp hands over and refills: 5, 6, 8 and 12 were
+// within 2 %, 4 was 3 % slower (a hand-over costs about half a flight).
+constexpr int REFILL_IDLE = 8;
+// a slot's flags beside its job
+constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_VIRTUAL = 0x10000000u,
+                   JF_JOB = 0x0fffffffu;
 
-// A block barrier reached by a converged warp.  The phases end in per-lane
-// loops of different lengths, and an aligned barrier (bar.sync) that a warp
-// reaches in several diverged groups can release before another warp has
-// arrived; reconverging the warp first keeps every phase's queue updates
-// ahead of the next phase.
-__device__ __forceinline__ void block_sync() {
-    __syncwarp();
-    __syncthreads();
-}
-
-constexpr int POOL_WARPS = 8;
-constexpr int POOL_THREADS = 32 * POOL_WARPS;
-
-// Queue entries are whole 32-bit words: entries of different classes written
-// by different warps at the same time never share a word.
-template <int NM>
-constexpr size_t pool_smem_bytes(int K) {
-    return (size_t)(PF_N + 3 * NM) * K * 32 * sizeof(float) + (size_t)PQ_N * K * 32 * sizeof(int) +
-           (size_t)PC_N * 32 * sizeof(int);
-}
-
-template <int NM>
-struct Pool {
-    uint32_t* fld;     // [PF_N][K][32]
-    float* cf;         // [3 NM][K][32]
-    int* q;            // [PQ_N][K][32] slot numbers
-    int* n;            // [PC_N][32]
-    int K;
-
-    __device__ __forceinline__ uint32_t& u(int f, int s, int l) { return fld[(f * K + s) * 32 + l]; }
-    __device__ __forceinline__ float& fl(int f, int s, int l) { return reinterpret_cast<float*>(fld)[(f * K + s) * 32 + l]; }
-    __device__ __forceinline__ int& slot(int queue, int j, int l) { return q[(queue * K + j) * 32 + l]; }
-    __device__ __forceinline__ int& cnt(int c, int l) { return n[c * 32 + l]; }
-    __device__ __forceinline__ void push(int queue, int l, int s) {
-        const int j = atomicAdd(&cnt(queue, l), 1);
-        slot(queue, j, l) = s;
+template <int NM, bool GEN, bool LM>
+struct Slots {
+    static constexpr int CF = NM < 4 ? 1 : NM / 4;              // float4 words of the total coefficients
+    static constexpr int Q_LM = 4 + CF, Q_GEN = Q_LM + (LM ? 1 : 0), Q = Q_GEN + (GEN ? 1 : 0);
+    float4* s;
+    __device__ __forceinline__ float4& at(int slot, int q) const { return s[slot * Q + q]; }
+    __device__ __forceinline__ uint32_t& word(int slot, int q, int w) const {
+        return reinterpret_cast<uint32_t*>(s)[(slot * Q + q) * 4 + w];
     }
-    __device__ __forceinline__ void bind(Lane<NM, false, false>& L, int s, int l) {
-        L.coef = cf + s * 32 + l;
-        L.stride = K * 32;
+    __device__ __forceinline__ void totals(int slot, float (&t)[NM]) const {
+        if constexpr (NM == 2) {
+            const float4 v = at(slot, 4);
+            t[0] = v.x; t[1] = v.y;
+        } else {
+#pragma unroll
+            for (int q = 0; q < CF; ++q) {
+                const float4 v = at(slot, 4 + q);
+                t[4 * q] = v.x; t[4 * q + 1] = v.y; t[4 * q + 2] = v.z; t[4 * q + 3] = v.w;
+            }
+        }
     }
-    __device__ __forceinline__ void load(Lane<NM, false, false>& L, int s, int l) {
-        L.px = fl(PF_PX, s, l); L.py = fl(PF_PY, s, l); L.pz = fl(PF_PZ, s, l);
-        L.dx = fl(PF_DX, s, l); L.dy = fl(PF_DY, s, l); L.dz = fl(PF_DZ, s, l);
-        L.e = fl(PF_E, s, l); L.mumax = fl(PF_MUMAX, s, l); L.inv_mumax = fl(PF_INVMU, s, l);
-        L.tg = fl(PF_TG, s, l);
-        const uint32_t st = u(PF_STATE, s, l);
-        L.state = (int)(st & 0xffu);
-        L.scattered = (int)(st >> 8);
-        L.job = (int)u(PF_JOB, s, l);
-        L.nsteps = u(PF_NSTEPS, s, l);
-        L.ngath = u(PF_NGATH, s, l);
-        L.rs.angle = u(PF_ANGLE, s, l); L.rs.hlo = u(PF_HLO, s, l); L.rs.hhi = u(PF_HHI, s, l);
-        L.rs.blk = u(PF_BLK, s, l);
-        bind(L, s, l);
-    }
-    __device__ __forceinline__ void store(const Lane<NM, false, false>& L, int s, int l) {
-        fl(PF_PX, s, l) = L.px; fl(PF_PY, s, l) = L.py; fl(PF_PZ, s, l) = L.pz;
-        fl(PF_DX, s, l) = L.dx; fl(PF_DY, s, l) = L.dy; fl(PF_DZ, s, l) = L.dz;
-        fl(PF_E, s, l) = L.e; fl(PF_MUMAX, s, l) = L.mumax; fl(PF_INVMU, s, l) = L.inv_mumax;
-        fl(PF_TG, s, l) = L.tg;
-        u(PF_STATE, s, l) = (uint32_t)L.state | ((uint32_t)L.scattered << 8);
-        u(PF_JOB, s, l) = (uint32_t)L.job;
-        u(PF_NSTEPS, s, l) = L.nsteps;
-        u(PF_NGATH, s, l) = L.ngath;
-        u(PF_ANGLE, s, l) = L.rs.angle; u(PF_HLO, s, l) = L.rs.hlo; u(PF_HHI, s, l) = L.rs.hhi;
-        u(PF_BLK, s, l) = L.rs.blk;
-    }
-    // a flight that ended stores what the flights changed
-    __device__ __forceinline__ void store_flight(const Lane<NM, false, false>& L, int s, int l) {
-        fl(PF_PX, s, l) = L.px; fl(PF_PY, s, l) = L.py; fl(PF_PZ, s, l) = L.pz;
-        fl(PF_TG, s, l) = L.tg;
-        u(PF_STATE, s, l) = (uint32_t)L.state | ((uint32_t)L.scattered << 8);
-        u(PF_NSTEPS, s, l) = L.nsteps;
-        u(PF_BLK, s, l) = L.rs.blk;
+    __device__ __forceinline__ void set_totals(int slot, const float (&t)[NM]) const {
+        if constexpr (NM == 2) {
+            at(slot, 4) = make_float4(t[0], t[1], 0.0f, 0.0f);
+        } else {
+#pragma unroll
+            for (int q = 0; q < CF; ++q) at(slot, 4 + q) = make_float4(t[4 * q], t[4 * q + 1], t[4 * q + 2], t[4 * q + 3]);
+        }
     }
 };
 
-// tail: once no idle lane of a warp can take another ready photon and fewer
-// than `tail` lanes still fly, the warp parks its photons for the next round
-// instead of flying on with a thinning warp, but only photons that have
-// flown at least `park_min` (>= 1) flights in this phase: every round moves
-// every photon on, so the rounds end
-// rounds a block may run (a block's rounds number in the thousands for 1e8
-// histories); past it the block records a timeout in P.status and stops
-constexpr int POOL_MAX_ROUNDS = 1 << 22;
+// a lane's photon: none, in flight, at a tentative collision, out of the box,
+// at max_steps
+enum : int { F_NONE = 0, F_ON = 1, F_GATHER = 2, F_ESC = 3, F_LIMIT = 4 };
+// a warp's counts: the statistics, then the flights that stopped at a
+// tentative collision and outside the box
+enum : int { A_GATHER = GDRR_NSTATS, A_ESC, A_N };
+
+template <int NM, bool GEN, bool LM>
+__host__ __device__ constexpr size_t warp_smem_bytes(int n) {
+    return (size_t)n * Slots<NM, GEN, LM>::Q * 16 + (size_t)2 * NM * 32 * 4 + (size_t)4 * n + (A_N + 3) / 2 * 16;
+}
+
+// One row of the energy-major coefficient table [energy][kind][NM].
+template <int NM>
+__device__ __forceinline__ void coef_row(const float* __restrict__ t, float (&v)[NM]) {
+    if constexpr (NM == 2) {
+        const float2 a = __ldg(reinterpret_cast<const float2*>(t));
+        v[0] = a.x; v[1] = a.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < NM; q += 4) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(t + q));
+            v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
+        }
+    }
+}
+
+// The coefficients of kind k (0 Rayleigh, 1 Compton, 2 photoelectric) of every
+// material at energy node ie plus fraction f, as Lane::set_energy takes them.
+template <int NM>
+__device__ __forceinline__ void coef_kind(const McParams& P, int k, int ie, float f, float (&v)[NM]) {
+    float a[NM], b[NM];
+    coef_row<NM>(P.tab_e + (size_t)(ie * 3 + k) * NM, a);
+    coef_row<NM>(P.tab_e + (size_t)(ie * 3 + 3 + k) * NM, b);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) v[m] = a[m] + f * (b[m] - a[m]);
+}
+
+// Lane::set_energy's totals and majorant, without its shared-memory table.
+template <int NM>
+__device__ __forceinline__ void energy_totals(const McParams& P, float e, float (&t)[NM], float& mumax) {
+    int ie; float f;
+    interp_index(e, P.e0, P.inv_de, P.n_e, ie, f);
+    float c[NM], p[NM];
+    coef_kind<NM>(P, 0, ie, f, t);
+    coef_kind<NM>(P, 1, ie, f, c);
+    coef_kind<NM>(P, 2, ie, f, p);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) t[m] = (t[m] + c[m]) + p[m];
+    const float a = __ldg(P.major + ie), b = __ldg(P.major + ie + 1);
+    mumax = a > b ? a : b;
+}
+
+// A flight's Philox block on 35 of the 40 operations of philox4x32_10: only
+// the block number changes along a history, so the part of the first two
+// rounds that it does not reach is formed once per hand-over (flight_keys),
+// and the last round's words z, w are dropped where unused.
+struct FlightKeys { uint32_t a, b, c, d; };
+
+__device__ __forceinline__ FlightKeys flight_keys(uint32_t angle, uint32_t hlo, uint32_t hhi, const RoundKeys& rk) {
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * hlo;
+    const uint64_t p0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ angle ^ rk.k0[0]);
+    FlightKeys k;
+    k.a = hhi ^ rk.k1[0];
+    k.b = (uint32_t)p1 ^ rk.k0[1];
+    k.c = (uint32_t)(p0 >> 32) ^ rk.k1[1];
+    k.d = (uint32_t)p0;
+    return k;
+}
+
+__device__ __forceinline__ uint4 flight_block(uint32_t blk, const FlightKeys& k, const RoundKeys& rk) {
+    const uint64_t q0 = (uint64_t)0xD2511F53u * blk;
+    const uint64_t q1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(q0 >> 32) ^ k.a);
+    uint32_t c0 = (uint32_t)(q1 >> 32) ^ k.b, c1 = (uint32_t)q1, c2 = k.c ^ (uint32_t)q0, c3 = k.d;
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
+        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ rk.k0[r];
+        const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ rk.k1[r];
+        c0 = n0; c1 = (uint32_t)p1; c2 = n2; c3 = (uint32_t)p0;
+    }
+    return make_uint4(c0, c1, c2, c3);
+}
+
+// n / d for the logarithm's arguments (n = m - 1, d = m + 1, m in
+// [sqrt(1/2), sqrt(2))): the quotient from an approximate reciprocal and
+// Markstein's residual correction (P. Markstein, IBM J. Res. Dev. 34, 1990).
+// Equal to the correctly rounded quotient for every m of a 24-bit uniform (all
+// 2^24 compared), without the general division's range test and branch.
+__device__ __forceinline__ float log_quotient(float n, float d) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+    const float q = __fmul_rn(n, y);
+    return __fmaf_rn(__fmaf_rn(-d, q, n), y, q);
+}
+
+// gd_logf(k 2^-24) for an integer 1 <= k <= 2^24: the same series on the same
+// m and e, which one addition separates (it carries into the exponent exactly
+// when the mantissa exceeds sqrt(2)'s).
+__device__ __forceinline__ float log_uniform(uint32_t k) {
+    constexpr uint32_t CARRY = 0x00800000u - 0x003504f4u;
+    const uint32_t t = __float_as_uint((float)k) + CARRY;
+    const float fe = __uint_as_float(0x4b000000u | (t >> 23)) - 8388759.0f;     // (t >> 23) - 127 - 24
+    const float m = __uint_as_float((t & 0x007fffffu) + (0x3f800000u - CARRY));
+    const float s = log_quotient(m - 1.0f, m + 1.0f);
+    const float s2 = s * s;
+    const float poly = (float)(1.0 / 3.0) + s2 * ((float)(1.0 / 5.0) + s2 * ((float)(1.0 / 7.0)
+                     + s2 * ((float)(1.0 / 9.0) + s2 * (float)(1.0 / 11.0))));
+    const float lm = 2.0f * s + (2.0f * s) * (s2 * poly);
+    return fe * (float)(2839.0 / 4096.0) + (fe * (float)(0.69314718055994530942 - 2839.0 / 4096.0) + lm);
+}
+
+// 0x4b000000 + floor(y - 1/2) for y = (x - lo) / vox >= 0: adding 2^23 - 1/2
+// with rounding down leaves the floor in the low bits (the sum is formed
+// exactly before it is rounded, and floorf(y - 0.5f) is the same floor: y -
+// 1/2 is exact for y >= 1/2, and lies in [-1/2, 0) below).  The lower corner
+// -1 of a point in the outer half voxel needs no clamp: its cell, -1, is a
+// copy of cell 0 in the table.
+__device__ __forceinline__ uint32_t corner_bits(float y) { return __float_as_uint(__fadd_rd(y, 8388607.5f)); }
+
+// The macro-cell bound (Lane::cell_bound) from the cell's densities.
+template <int NM>
+__device__ __forceinline__ float bound_of(const float (&v)[NM], const float (&cf)[NM]) {
+    float b = v[0] * cf[0];
+#pragma unroll
+    for (int m = 1; m < NM; ++m) b = fmaxf(b, v[m] * cf[m]);
+    return b * CELL_MARGIN;
+}
 
 template <int NM>
-__global__ void __launch_bounds__(POOL_THREADS, 3) mc_pool_kernel(const McParams P, int K, int tail, uint32_t park_min) {
-    extern __shared__ __align__(16) unsigned char pool_smem[];
+__device__ __forceinline__ float bound_of(const McParams& P, int cell, const float (&cf)[NM]) {
+    float v[NM];
+    coef_row<NM>(P.cells + (ptrdiff_t)cell * NM, v);
+    return bound_of<NM>(v, cf);
+}
+
+
+
+template <int NM, bool GEN, bool LM>
+__global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_MIN_BLOCKS) mc_warp_kernel(const McParams P, int n_pool, int n_use, unsigned chunk,
+                                                            uint32_t cell0) {
+    extern __shared__ __align__(16) unsigned char warp_smem[];
     __shared__ unsigned long long cnt[GDRR_NSTATS];
-    __shared__ int s_done[POOL_WARPS];
-    __shared__ int s_exit;
-    using L_t = Lane<NM, false, false>;
-    Pool<NM> pl;
-    pl.K = K;
-    pl.fld = reinterpret_cast<uint32_t*>(pool_smem);
-    pl.cf = reinterpret_cast<float*>(pl.fld + (size_t)PF_N * K * 32);
-    pl.q = reinterpret_cast<int*>(pl.cf + (size_t)3 * NM * K * 32);
-    pl.n = pl.q + (size_t)PQ_N * K * 32;
-
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x) cnt[i] = 0ull;
-    for (int i = threadIdx.x; i < PC_N * 32; i += blockDim.x) pl.n[i] = 0;
-    if (threadIdx.x < POOL_WARPS) s_done[threadIdx.x] = 0;
-    block_sync();
-    if (warp == 0) {
-        pl.cnt(PQ_F0, lane) = K;                          // every slot starts free
-        for (int j = 0; j < K; ++j) pl.slot(PQ_F0, j, lane) = j;
+    const unsigned below = (1u << lane) - 1u;
+    for (int i = threadIdx.x; i < GDRR_NSTATS; i += WARP_BLOCK) cnt[i] = 0ull;
+    __syncthreads();
+    unsigned char* base = warp_smem + (size_t)warp * warp_smem_bytes<NM, GEN, LM>(n_pool);
+    Slots<NM, GEN, LM> S;
+    S.s = reinterpret_cast<float4*>(base);
+    float* coef = reinterpret_cast<float*>(base + (size_t)n_pool * S.Q * 16) + lane;       // [2 NM][32], this lane's column
+    uint8_t* qR = base + (size_t)n_pool * S.Q * 16 + (size_t)2 * NM * 32 * 4;               // ready to fly
+    uint8_t* qG = qR + n_pool;                                                             // corner gathers
+    uint8_t* qI = qG + n_pool;                                                             // interaction
+    uint8_t* qE = qI + n_pool;                                                             // tally and next history
+    int nR = 0, nG = 0, nI = 0, nE = n_use;
+    for (int i = lane; i < n_use; i += 32) {
+        qE[i] = (uint8_t)i;
+        S.word(i, 2, 3) = JF_DEAD;
     }
-    L_t L;
-    L.state = S_DEAD;
-    L.defer_e = false;
-    L.need_e = false;
-    L.c_steps = 0; L.c_virt = 0; L.c_skip = 0;
-    unsigned long long pool_next = 0, pool_end = 0;
+    __syncwarp();
+    // this warp's counts of events, by kind; histories claimed and not started
+    unsigned long long* acc = reinterpret_cast<unsigned long long*>(qR + 4 * n_pool);
+    unsigned long long &next = acc[A_N], &end = acc[A_N + 1];
+    if (lane < A_N + 2) acc[lane] = 0ull;
+    __syncwarp();
     bool exhausted = false;
-    block_sync();
+    auto add = [&](int k, unsigned n) {
+        if (lane == 0) acc[k] += n;
+    };
+    auto tally = [&](int k, bool p) { add(k, (unsigned)__popc(__ballot_sync(FULL, p))); };
+    Lane<NM, false, GEN, LM> L;
+    L.coef = coef - NM * 32;                // kinds 1 and 2; the totals are the slot's
+    L.stride = 32;
+    L.tot_stride = 1;
+    L.defer_e = true;
+    L.c_steps = 0; L.c_virt = 0; L.c_skip = 0; L.c_cross = 0; L.ngath = 0; L.lm_need = 0u;
 
-    for (int round = 0;; ++round) {
-        if (round >= POOL_MAX_ROUNDS) {
-            if (threadIdx.x == 0 && P.status) atomicOr(P.status, 2);
-            break;
-        }
-        // queues by round parity: this round's FLIGHT runs qFly (filled by
-        // the last round and by this START); photons that fly next round go
-        // to qNext; START takes the free slots of qF, freed slots go to qFn
-        const int c = round & 1;
-        const int qFly = c ? PQ_R0 : PQ_R1, qNext = c ? PQ_R1 : PQ_R0;
-        const int qF = c ? PQ_F1 : PQ_F0, qFn = c ? PQ_F0 : PQ_F1;
-
-        // ---- START: free slots of this round take new histories ----------
-        if (warp == 0) {
-            pl.cnt(PQ_E, lane) = 0;                       // consumed by the last ESCAPE
-            // between rounds every slot of a class is free or ready to fly
-            const bool whole = pl.cnt(qF, lane) + pl.cnt(qFly, lane) == K;
-            const unsigned broken = __ballot_sync(FULL, !whole);
-            const int nfree = __reduce_add_sync(FULL, (unsigned)pl.cnt(qF, lane));
-            int ndone = 0;
-            for (int w = 0; w < POOL_WARPS; ++w) ndone += s_done[w];
-            if (lane == 0) {
-                s_exit = (nfree == 32 * K && ndone == POOL_WARPS) ? 1 : 0;
-                if (broken) {                             // a slot went missing: stop, and say so
-                    if (P.status) atomicOr(P.status, 4);
-                    s_exit = 1;
-                }
-            }
-        }
-        block_sync();
-        if (s_exit) break;
-        {
-            const int nf = pl.cnt(qF, lane);
-            int j = warp;
-            bool need = j < nf;
-            int sl = need ? pl.slot(qF, j, lane) : 0;
-            while (!exhausted) {
-                const unsigned nb = __ballot_sync(FULL, need);
-                if (nb == 0u) break;
-                if (pool_next >= pool_end) {
-                    unsigned long long base = 0;
-                    if (lane == 0) base = atomicAdd(P.counter, (unsigned long long)P.chunk);
-                    base = __shfl_sync(FULL, base, 0);
-                    if (base >= P.total) { exhausted = true; break; }
-                    pool_next = base;
-                    pool_end = base + (unsigned long long)P.chunk;
-                    if (pool_end > P.total) pool_end = P.total;
-                }
-                const unsigned avail = (unsigned)(pool_end - pool_next);
-                const unsigned want = (unsigned)__popc(nb);
-                const unsigned take = want < avail ? want : avail;
-                const unsigned rank = (unsigned)__popc(nb & ((1u << lane) - 1u));
-                if (need && rank < take) {
-                    pl.bind(L, sl, lane);
-                    L.start(P, P.seg0 + pool_next + rank, cnt);
-                    if (L.state == S_FLY) {                 // else it missed the box and was tallied: retry
-                        pl.store(L, sl, lane);
-                        pl.push(qFly, lane, sl);
-                        j += POOL_WARPS;
-                        need = j < nf;
-                        if (need) sl = pl.slot(qF, j, lane);
-                    }
-                }
-                pool_next += take;
-            }
-            // free slots that got no history stay free for a later round
-            for (; need; ) {
-                pl.push(qFn, lane, sl);
-                j += POOL_WARPS;
-                need = j < nf;
-                if (need) sl = pl.slot(qF, j, lane);
-            }
-            if (lane == 0) s_done[warp] = (exhausted && pool_next >= pool_end) ? 1 : 0;
-        }
-        block_sync();
-
-        // ---- FLIGHT ---------------------------------------------------------
-        if (warp == 0) pl.cnt(qF, lane) = 0;             // consumed by START
-        {
-            const int nR = pl.cnt(qFly, lane);
-            bool have = false, drained = false;
-            int sl = 0;
-            uint32_t flown = 0;                           // flights of the held photon in this phase
+    for (;;) {
+        const int most = max(max(nG, nI), nE);
+        if (most < 32 && (most == 0 || most < nR)) {
+            if (nR == 0) break;
+            // ---- free flights: until a list is full, or too few photons fly ----
+            float cf[NM];
+            float mumax = 0.0f, inv = 0.0f, nl = 0.0f;     // nl, wy, wz: the next flight's -ln xi and words
+            uint32_t blk = 0, limit = 0, wy = 0, wz = 0, gz = 0;
+            FlightKeys key = {0, 0, 0, 0};
+            int slot = 0, code = F_NONE;
+            unsigned flown = 0, crossed = 0;
             for (;;) {
-                if (!have && !drained) {
-                    const int pos = atomicAdd(&pl.cnt(PC_HEAD, lane), 1);
-                    if (pos < nR) {
-                        sl = pl.slot(qFly, pos, lane);
-                        pl.load(L, sl, lane);
-                        have = true;
-                        flown = 0;
+                const unsigned act = __ballot_sync(FULL, code == F_ON);
+                int n_act = __popc(act);
+                if (n_act <= 32 - REFILL_IDLE) {
+                    // hand over the photons whose flight stopped, refill the lanes
+                    const unsigned mG = __ballot_sync(FULL, code == F_GATHER), mE = __ballot_sync(FULL, code >= F_ESC);
+                    if (code > F_ON) {
+                        S.at(slot, 0) = make_float4(L.px, L.py, L.pz, L.tg);
+                        if constexpr (LM) {
+                            S.word(slot, 2, 1) = (uint32_t)L.cx | ((uint32_t)L.cy << 16);
+                            S.word(slot, S.Q_LM, 3) = (uint32_t)L.cz;
+                        } else {
+                            S.word(slot, 3, 0) = blk;
+                            if (GEN) S.word(slot, S.Q_GEN, 0) = gz;
+                            if (code == F_LIMIT) S.word(slot, 2, 3) = JF_DEAD;
+                        }
+                        if (code == F_GATHER) qG[nG + __popc(mG & below)] = (uint8_t)slot;
+                        else qE[nE + __popc(mE & below)] = (uint8_t)slot;
+                    }
+                    nG += __popc(mG);
+                    nE += __popc(mE);
+                    const unsigned cut = LM ? 0u : __ballot_sync(FULL, code == F_LIMIT);
+                    if (cut) {
+                        add(GDRR_ST_STEP_LIMIT, (unsigned)__popc(cut));
+                        flown -= (unsigned)__popc(cut);
+                    }
+                    if (code > F_ON) code = F_NONE;
+                    const int full = max(max(nG, nI), nE);
+                    if (full >= 32 || (nR == 0 && n_act <= full)) break;
+                    __syncwarp();
+                    const int take = nR - 1 - __popc(~act & below);
+                    if (code == F_NONE && take >= 0) {
+                        code = F_ON;
+                        slot = qR[take];
+                        const float4 a = S.at(slot, 0), b = S.at(slot, 1), c = S.at(slot, 2);
+                        L.px = a.x; L.py = a.y; L.pz = a.z;
+                        L.dx = b.x; L.dy = b.y; L.dz = b.z;
+                        S.totals(slot, cf);
+                        if constexpr (LM) {
+                            const float4 g = S.at(slot, S.Q_LM);
+                            L.tg = a.w;
+                            L.tau = c.x;
+                            L.cx = (int)(__float_as_uint(c.y) & 0xffffu);
+                            L.cy = (int)(__float_as_uint(c.y) >> 16);
+                            L.idx = g.x; L.idy = g.y; L.idz = g.z;
+                            L.cz = __float_as_int(g.w);
+                        } else {
+                            const float4 d = S.at(slot, 3);
+                            nl = a.w;
+                            mumax = c.x; inv = c.y;
+                            blk = __float_as_uint(d.x); limit = __float_as_uint(d.y); wy = __float_as_uint(d.w);
+                            if (GEN) wz = S.word(slot, S.Q_GEN, 0);
+                            key = flight_keys(P.jobs[__float_as_uint(c.w) & JF_JOB].angle_index, __float_as_uint(c.z),
+                                              __float_as_uint(d.z), P.rk);
+                        }
+                    }
+                    n_act = min(32, n_act + nR);
+                    nR = max(0, nR - __popc(~act));
+                }
+                flown += (unsigned)n_act;
+                if (code == F_ON) {
+                    if constexpr (LM) {
+                        L.state = S_FLY;
+                        L.walk(P, bound_of<NM>(P, L.cx + P.csx * (L.cy + P.csy * L.cz), cf));
+                        code = L.state == S_FLY ? F_ON : (L.state == S_GATHER ? F_GATHER : F_ESC);
                     } else {
-                        drained = true;
+                        const float s = nl * inv;
+                        const float qx = L.px + s * L.dx, qy = L.py + s * L.dy, qz = L.pz + s * L.dz;
+                        const bool inside = fabsf(qx) <= P.hi[0] && fabsf(qy) <= P.hi[1] && fabsf(qz) <= P.hi[2];  // lo = -hi
+                        const float t = uniform(wy) * mumax;
+                        // what decides a tentative collision is loaded first ...
+                        float v[NM];
+                        uint2 vx = make_uint2(0u, 0u);
+                        const bool nearest = GEN && P.nearest_voxel;
+                        if (nearest) {
+                            const int gx = min(max((int)floorf((qx - P.lo[0]) * P.ivox[0]), 0), P.nx - 1);
+                            const int gy = min(max((int)floorf((qy - P.lo[1]) * P.ivox[1]), 0), P.ny - 1);
+                            const int gv = min(max((int)floorf((qz - P.lo[2]) * P.ivox[2]), 0), P.nz - 1);
+                            vx = __ldg(P.vox + brick_x(gx) + brick_y(gy, P.bsy) + brick_z(gv, P.bsz));
+                        } else {
+                            // the lower trilinear corner, as gather() computes it, locates the macro cell
+                            const uint32_t ux = corner_bits((qx - P.lo[0]) * P.ivox[0]) >> P.cshift;
+                            const uint32_t uy = corner_bits((qy - P.lo[1]) * P.ivox[1]) >> P.cshift;
+                            const uint32_t uz = corner_bits((qz - P.lo[2]) * P.ivox[2]) >> P.cshift;
+                            const int cell = (int)(ux + P.csx * (uy + P.csy * uz) - cell0);
+                            coef_row<NM>(P.cells + (ptrdiff_t)(inside ? cell : 0) * NM, v);
+                        }
+                        // ... and the next flight's words formed while it comes
+                        const bool cut = blk >= limit;
+                        ++blk;
+                        if (GEN) gz = wz;
+                        const uint4 w = flight_block(blk, key, P.rk);
+                        nl = -log_uniform((w.x >> 8) + 1u);
+                        wy = w.y;
+                        if (GEN) wz = w.z;
+                        const bool skip = t > (nearest ? __uint_as_float(vx.x) * __uint_as_float(S.word(slot, 4, (int)vx.y))
+                                                       : bound_of<NM>(v, cf));
+                        L.tg = t;
+                        if (inside) { L.px = qx; L.py = qy; L.pz = qz; }
+                        code = skip ? F_ON : F_GATHER;
+                        if (!inside) code = F_ESC;
+                        if (cut) code = F_LIMIT;
                     }
                 }
-                const unsigned act = __ballot_sync(FULL, have);
-                const unsigned idle_open = __ballot_sync(FULL, !have && !drained);
-                const unsigned fresh = __ballot_sync(FULL, have && flown < park_min);
-                if (act == 0u && idle_open == 0u) break;
-                if (idle_open == 0u && fresh == 0u && __popc(act) < tail) {
-                    if (have) {                           // park for the next round
-                        pl.store_flight(L, sl, lane);
-                        pl.push(qNext, lane, sl);
-                    }
-                    break;
-                }
-                if (have) {
-                    L.step(P, cnt);
-                    ++flown;
-                    if (L.state != S_FLY) {
-                        pl.store_flight(L, sl, lane);
-                        if (L.state == S_GATHER) pl.push(PQ_G, lane, sl);
-                        else if (L.state == S_ESC) pl.push(PQ_E, lane, sl);
-                        else pl.push(qFn, lane, sl);        // step limit: the history ended
-                        have = false;
-                    }
-                }
+                if (LM) crossed += (unsigned)__popc(__ballot_sync(FULL, code == F_ON));
             }
-        }
-        block_sync();
-
-        // ---- GATHER -----------------------------------------------------------
-        if (warp == 0) {
-            // a warp that parks can leave ready photons of a class unpopped
-            // (its lane of that class still held one): they fly next round
-            const int nR = pl.cnt(qFly, lane);
-            for (int pos = pl.cnt(PC_HEAD, lane); pos < nR; ++pos) pl.push(qNext, lane, pl.slot(qFly, pos, lane));
-            pl.cnt(qFly, lane) = 0;
-            pl.cnt(PC_HEAD, lane) = 0;
-        }
-        {
-            const int nG = pl.cnt(PQ_G, lane);
-            for (int j = warp; j < nG; j += POOL_WARPS) {
-                const int sl = pl.slot(PQ_G, j, lane);
-                pl.load(L, sl, lane);
-                L.gather(P, cnt);
-                if (L.state == S_DEAD) {
-                    pl.push(qFn, lane, sl);               // photoelectric absorption
+            // park the photons still in flight
+            __syncwarp();
+            const unsigned fly = __ballot_sync(FULL, code == F_ON);
+            if (code == F_ON) {
+                S.at(slot, 0) = make_float4(L.px, L.py, L.pz, LM ? L.tg : nl);
+                if constexpr (LM) {
+                    S.word(slot, 2, 0) = __float_as_uint(L.tau);
+                    S.word(slot, 2, 1) = (uint32_t)L.cx | ((uint32_t)L.cy << 16);
+                    S.word(slot, S.Q_LM, 3) = (uint32_t)L.cz;
                 } else {
-                    pl.u(PF_STATE, sl, lane) = (uint32_t)L.state | ((uint32_t)L.scattered << 8);
-                    pl.u(PF_NGATH, sl, lane) = L.ngath;
-                    pl.push(L.state == S_FLY ? qNext : PQ_I, lane, sl);
+                    S.word(slot, 3, 0) = blk;
+                    S.word(slot, 3, 3) = wy;
+                    if (GEN) S.word(slot, S.Q_GEN, 0) = wz;
                 }
+                qR[nR + __popc(fly & below)] = (uint8_t)slot;
             }
+            nR += __popc(fly);
+            add(LM ? GDRR_ST_CELL_CROSSINGS : GDRR_ST_STEPS, LM ? crossed : flown);
+            __syncwarp();
+            continue;
         }
-        block_sync();
 
-        // ---- INTER ------------------------------------------------------------
-        if (warp == 0) pl.cnt(PQ_G, lane) = 0;
-        {
-            const int nI = pl.cnt(PQ_I, lane);
-            for (int j = warp; j < nI; j += POOL_WARPS) {
-                const int sl = pl.slot(PQ_I, j, lane);
-                pl.load(L, sl, lane);
-                L.interact(P, cnt);
-                if (L.state == S_DEAD) {
-                    pl.push(qFn, lane, sl);               // energy cut-off
-                } else {
-                    pl.store(L, sl, lane);
-                    pl.push(qNext, lane, sl);
+        // ---- services: the fullest list's last 32, or what there is ------------
+        const int which = nI >= nG && nI >= nE ? S_COMP : (nG >= nE ? S_GATHER : S_ESC);
+        const int have = which == S_COMP ? nI : (which == S_GATHER ? nG : nE), n = min(32, have);
+        int slot = -1;
+        if (lane < n) slot = (which == S_COMP ? qI : (which == S_GATHER ? qG : qE))[have - 1 - lane];
+        if (which == S_COMP) nI -= n; else if (which == S_GATHER) nG -= n; else nE -= n;
+        __syncwarp();
+        EventMask ev = {0u};
+        bool fresh = false;                       // a new energy: totals and majorant to form
+        float4 c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        uint32_t limit = 0, jf = JF_DEAD;
+        L.state = S_DEAD;
+        if (slot >= 0) {
+            c = S.at(slot, 2);
+            jf = __float_as_uint(c.w);
+            if (!(jf & JF_DEAD)) {
+                const float4 a = S.at(slot, 0), b = S.at(slot, 1), d = S.at(slot, 3);
+                L.px = a.x; L.py = a.y; L.pz = a.z; L.tg = a.w;
+                L.dx = b.x; L.dy = b.y; L.dz = b.z; L.e = b.w;
+                L.job = (int)(jf & JF_JOB);
+                L.scattered = (jf & JF_SCATTERED) ? 1 : 0;
+                L.rs.angle = P.jobs[L.job].angle_index;
+                L.rs.hlo = __float_as_uint(c.z);
+                L.rs.hhi = __float_as_uint(d.z);
+                L.rs.blk = __float_as_uint(d.x);
+                limit = __float_as_uint(d.y);
+                if (GEN) {
+                    L.wz = S.word(slot, S.Q_GEN, 0);
+                    L.n_int = S.word(slot, S.Q_GEN, 1);
+                    L.m_ray = (int)S.word(slot, S.Q_GEN, 2);
                 }
+                if (LM) {
+                    const float4 g = S.at(slot, S.Q_LM);
+                    L.cx = (int)(__float_as_uint(c.y) & 0xffffu);
+                    L.cy = (int)(__float_as_uint(c.y) >> 16);
+                    L.idx = g.x; L.idy = g.y; L.idz = g.z;
+                    L.cz = __float_as_int(g.w);
+                }
+                L.state = which == S_COMP && (jf & JF_RAYLEIGH) ? S_RAY : which;
             }
         }
-        block_sync();
-
-        // ---- ESCAPE -----------------------------------------------------------
-        if (warp == 0) pl.cnt(PQ_I, lane) = 0;
-        {
-            const int nE = pl.cnt(PQ_E, lane);
-            for (int j = warp; j < nE; j += POOL_WARPS) {
-                const int sl = pl.slot(PQ_E, j, lane);
-                pl.load(L, sl, lane);
-                L.escape(P, cnt, true);
-                pl.push(qFn, lane, sl);
+        if (which == S_GATHER) {
+            if (slot >= 0) {
+                int ie; float f;
+                interp_index(L.e, P.e0, P.inv_de, P.n_e, ie, f);
+                float r[NM], co[NM];
+                coef_kind<NM>(P, 0, ie, f, r);
+                coef_kind<NM>(P, 1, ie, f, co);
+#pragma unroll
+                for (int m = 0; m < NM; ++m) { L.cf(1, m) = r[m]; L.cf(2, m) = co[m]; }
+                L.tot = reinterpret_cast<const float*>(&S.at(slot, 4));
+                L.gather(P, ev);
+            }
+            tally(GDRR_ST_VIRTUAL, L.state == S_FLY);
+            tally(GDRR_ST_PHOTO, ev.has(GDRR_ST_PHOTO));
+            // the interaction waits for its own full warp; so do the few virtual
+            // collisions, for that service's next-flight words (not LM, where
+            // most are virtual: they draw their next flight here)
+            const bool hit = L.state == S_RAY || L.state == S_COMP, wait = hit || (!LM && L.state == S_FLY);
+            const unsigned mI = __ballot_sync(FULL, wait);
+            if (wait) {
+                S.word(slot, 2, 3) = jf | (L.state == S_RAY ? JF_RAYLEIGH : 0u) | (hit ? 0u : JF_VIRTUAL);
+                if (GEN) S.word(slot, S.Q_GEN, 2) = (uint32_t)L.m_ray;
+                qI[nI + __popc(mI & below)] = (uint8_t)slot;
+                if (!hit) L.state = S_COMP;       // it does not fly on from here
+            }
+            nI += __popc(mI);
+            add(A_GATHER, (unsigned)n);
+        } else if (which == S_COMP) {
+            const bool real = slot >= 0 && !(jf & JF_VIRTUAL);
+            jf &= ~(JF_VIRTUAL | JF_RAYLEIGH);
+            if (slot >= 0 && !real) L.state = S_FLY;
+            if (real) {
+                const uint32_t b0 = L.rs.blk;
+                L.need_e = false;
+                L.interact(P, ev);
+                limit += L.rs.blk - b0;
+                fresh = L.need_e;
+                jf |= JF_SCATTERED;
+            }
+            tally(GDRR_ST_RAYLEIGH, ev.has(GDRR_ST_RAYLEIGH));
+            tally(GDRR_ST_COMPTON, ev.has(GDRR_ST_COMPTON));
+            tally(GDRR_ST_CUTOFF, ev.has(GDRR_ST_CUTOFF));
+        } else {
+            tally(A_ESC, L.state == S_ESC);
+            if (L.state == S_ESC) L.escape(P, ev, true);
+            tally(GDRR_ST_TALLY_PRIMARY, ev.has(GDRR_ST_TALLY_PRIMARY));
+            tally(GDRR_ST_TALLY_SCATTER, ev.has(GDRR_ST_TALLY_SCATTER));
+            tally(GDRR_ST_MISS, ev.has(GDRR_ST_MISS));
+            unsigned need = exhausted ? 0u : __ballot_sync(FULL, slot >= 0);
+            while (need) {
+                unsigned long long first = next;
+                if (first >= end) {
+                    if (lane == 0) first = atomicAdd(P.counter, (unsigned long long)chunk);
+                    first = __shfl_sync(FULL, first, 0);
+                    if (first >= P.total) { exhausted = true; break; }
+                    __syncwarp();
+                    if (lane == 0) end = min(first + chunk, (unsigned long long)P.total);
+                    __syncwarp();
+                }
+                const unsigned take = (unsigned)min((unsigned long long)__popc(need), end - first);
+                const unsigned rank = (unsigned)__popc(need & below);
+                ev.m = 0u;
+                if (((need >> lane) & 1u) && rank < take) L.start(P, first + rank, ev);
+                add(GDRR_ST_HISTORIES, take);
+                tally(GDRR_ST_TALLY_PRIMARY, ev.has(GDRR_ST_TALLY_PRIMARY));
+                tally(GDRR_ST_MISS, ev.has(GDRR_ST_MISS));
+                __syncwarp();
+                if (lane == 0) next = first + take;
+                __syncwarp();
+                need = __ballot_sync(FULL, slot >= 0 && L.state != S_FLY);
+            }
+            if (L.state == S_FLY) {
+                limit = L.rs.blk + (uint32_t)P.max_steps;
+                jf = (uint32_t)L.job;
+                fresh = true;
             }
         }
-        block_sync();
+        if (LM) {
+            ev.m = 0u;
+            const bool draw = L.state == S_FLY;
+            if (draw) {
+                L.nsteps = L.rs.blk + (uint32_t)P.max_steps - limit;
+                L.lm_prepare(P, ev);
+            }
+            tally(GDRR_ST_STEP_LIMIT, ev.has(GDRR_ST_STEP_LIMIT));
+            tally(GDRR_ST_STEPS, draw && L.state == S_FLY);
+        }
+        // photons that fly on go back to their slot with the next flight's words;
+        // ended histories (not those that found no successor) to the last list
+        const bool on = L.state == S_FLY;
+        const bool gone = slot >= 0 && L.state == S_DEAD && (which != S_ESC || fresh);
+        if (on) {
+            if (fresh) {
+                float t[NM], mumax;
+                energy_totals<NM>(P, L.e, t, mumax);
+                S.set_totals(slot, t);
+                c.x = mumax;
+                c.y = 1.0f / mumax;
+            }
+            uint32_t wy = 0;
+            if constexpr (LM) {
+                c.x = L.tau;
+                c.y = __uint_as_float((uint32_t)L.cx | ((uint32_t)L.cy << 16));
+                S.at(slot, S.Q_LM) = make_float4(L.idx, L.idy, L.idz, __int_as_float(L.cz));
+            } else {
+                const uint4 w = flight_block(L.rs.blk, flight_keys(L.rs.angle, L.rs.hlo, L.rs.hhi, P.rk), P.rk);
+                L.tg = -log_uniform((w.x >> 8) + 1u);
+                wy = w.y;
+                if (GEN) L.wz = w.z;
+            }
+            S.at(slot, 0) = make_float4(L.px, L.py, L.pz, L.tg);
+            S.at(slot, 1) = make_float4(L.dx, L.dy, L.dz, L.e);
+            S.at(slot, 2) = make_float4(c.x, c.y, __uint_as_float(L.rs.hlo), __uint_as_float(jf));
+            S.at(slot, 3) = make_float4(__uint_as_float(L.rs.blk), __uint_as_float(limit), __uint_as_float(L.rs.hhi),
+                                        __uint_as_float(wy));
+            if (GEN) { S.word(slot, S.Q_GEN, 0) = L.wz; S.word(slot, S.Q_GEN, 1) = L.n_int; }
+        }
+        if (gone) S.word(slot, 2, 3) = JF_DEAD;
+        const unsigned mR = __ballot_sync(FULL, on), mE = __ballot_sync(FULL, gone);
+        if (on) qR[nR + __popc(mR & below)] = (uint8_t)slot;
+        if (gone) qE[nE + __popc(mE & below)] = (uint8_t)slot;
+        nR += __popc(mR);
+        nE += __popc(mE);
+        __syncwarp();
     }
 
-    atomicAdd(&cnt[GDRR_ST_STEPS], (unsigned long long)L.c_steps);
-    atomicAdd(&cnt[GDRR_ST_VIRTUAL], (unsigned long long)L.c_virt);
-    atomicAdd(&cnt[GDRR_ST_CELL_SKIPS], (unsigned long long)L.c_skip);
-    block_sync();
-    for (int i = threadIdx.x; i < GDRR_NSTATS; i += blockDim.x)
+    // the flights that the cells (or the nearest voxel) decided stopped neither
+    // at a tentative collision nor outside the box
+    __syncwarp();
+    if (!LM && lane == 0) {
+        const unsigned long long inl = acc[GDRR_ST_STEPS] - acc[A_GATHER] - acc[A_ESC];
+        acc[GDRR_ST_VIRTUAL] += inl;
+        if (!(GEN && P.nearest_voxel)) acc[GDRR_ST_CELL_SKIPS] += inl;
+    }
+    __syncwarp();
+    if (lane < GDRR_NSTATS && acc[lane]) atomicAdd(&cnt[lane], acc[lane]);
+    __syncthreads();
+    for (int i = threadIdx.x; i < GDRR_NSTATS; i += WARP_BLOCK)
         if (cnt[i]) atomicAdd(P.stats + i, cnt[i]);
 }
 
@@ -1407,123 +1615,77 @@ constexpr size_t smem_bytes(int block) { return (size_t)3 * NM * block * sizeof(
 
 // Per-thread coefficient tables beyond 47 KB per block (8 materials at 512
 // threads) need the kernel's dynamic shared-memory cap raised first.
-template <int NM, bool REC, bool GEN, bool LM>
-cudaError_t allow_smem(int block) {
+template <int NM, bool GEN, bool LM>
+cudaError_t launch_records_t(const McParams& p, int block, int per_sm_max, int n_sm, cudaStream_t s) {
     const size_t bytes = smem_bytes<NM>(block);
-    if (bytes <= 47 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(mc_kernel<NM, REC, GEN, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-template <int NM, bool REC, bool GEN, bool LM>
-cudaError_t launch_t(const McParams& p, int block, int grid, cudaStream_t s) {
-    const cudaError_t e = allow_smem<NM, REC, GEN, LM>(block);
+    cudaError_t e = cudaSuccess;
+    if (bytes > 47 * 1024)
+        e = cudaFuncSetAttribute(mc_kernel<NM, GEN, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    int per_sm = per_sm_max;
+    if (e == cudaSuccess && per_sm <= 0)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mc_kernel<NM, GEN, LM>, block, bytes);
     if (e != cudaSuccess) return e;
-    mc_kernel<NM, REC, GEN, LM><<<grid, block, smem_bytes<NM>(block), s>>>(p);
+    const int64_t useful = (int64_t)((p.total + 31) / 32 * 32 + block - 1) / block;
+    const int64_t grid = std::min<int64_t>((int64_t)std::max(per_sm, 1) * n_sm, useful);
+    mc_kernel<NM, GEN, LM><<<(int)std::max<int64_t>(grid, 1), block, bytes, s>>>(p);
     return cudaGetLastError();
 }
 
-template <int NM, bool REC, bool GEN, bool LM>
-int occupancy_t(int block) {
-    int n = 0;
-    if (allow_smem<NM, REC, GEN, LM>(block) != cudaSuccess
-        || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, mc_kernel<NM, REC, GEN, LM>, block, smem_bytes<NM>(block))
-               != cudaSuccess)
-        return 1;
-    return n > 0 ? n : 1;
-}
-
-template <bool REC, bool GEN, bool LM>
-cudaError_t launch_nm(const McParams& p, int block, int grid, cudaStream_t s) {
-    if (p.n_mat <= 2) return launch_t<2, REC, GEN, LM>(p, block, grid, s);
-    if (p.n_mat <= 4) return launch_t<4, REC, GEN, LM>(p, block, grid, s);
-    return launch_t<8, REC, GEN, LM>(p, block, grid, s);
-}
-
-template <bool REC, bool LM>
-int occupancy_nm(int n_mat, int block) {
-    if (n_mat <= 2) return occupancy_t<2, REC, false, LM>(block);
-    if (n_mat <= 4) return occupancy_t<4, REC, false, LM>(block);
-    return occupancy_t<8, REC, false, LM>(block);
-}
-
-template <bool LM>
-cudaError_t launch_lm(const McParams& p, int block, int grid, bool records, cudaStream_t s) {
-    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0;
-    if (records) return gen ? launch_nm<true, true, LM>(p, block, grid, s) : launch_nm<true, false, LM>(p, block, grid, s);
-    return gen ? launch_nm<false, true, LM>(p, block, grid, s) : launch_nm<false, false, LM>(p, block, grid, s);
-}
-
-template <int NM>
-cudaError_t launch_pool_t(const McParams& p, int K, int grid, cudaStream_t s) {
-    const size_t bytes = pool_smem_bytes<NM>(K);
-    cudaError_t e = cudaFuncSetAttribute(mc_pool_kernel<NM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+template <int NM, bool GEN, bool LM>
+cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm, cudaStream_t s) {
+    const size_t bytes = warp_smem_bytes<NM, GEN, LM>(n_pool) * (WARP_BLOCK / 32);
+    cudaError_t e = cudaFuncSetAttribute(mc_warp_kernel<NM, GEN, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bytes);
+    int per_sm = 0;
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mc_warp_kernel<NM, GEN, LM>, WARP_BLOCK, bytes);
     if (e != cudaSuccess) return e;
-    // measured on the 2 mm torso (2 photons per thread): tail 24 / park 4
-    // 112.6 ms, tail 16 / park 16 117.1 ms, tail 8 130 ms
-    const int tail = p.pool_tail > 0 ? p.pool_tail : 24;
-    const uint32_t park_min = p.pool_park_min > 0 ? (uint32_t)p.pool_park_min : 4u;
-    mc_pool_kernel<NM><<<grid, POOL_THREADS, bytes, s>>>(p, K, tail, park_min);
+    if (per_sm <= 0) return cudaErrorInvalidConfiguration;
+    constexpr int WPB = WARP_BLOCK / 32;
+    if (warps_max > 0) per_sm = std::max(1, std::min(per_sm, (warps_max + WPB - 1) / WPB));
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * n_sm, (int64_t)((p.total + WPB - 1) / WPB)));
+    const int64_t warps = grid * WPB;
+    // a small launch spreads over every warp: fewer photons per warp, smaller claims
+    const uint64_t share = (p.total + warps - 1) / warps;
+    const int n_use = (int)std::min<uint64_t>((uint64_t)n_pool, share);
+    const unsigned chunk = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)p.chunk, share / 4 + 1));
+    McParams q = p;
+    if (!q.cells) {                 // no cell test: one cell whose bound nothing exceeds
+        q.cells = q.open_cell;
+        q.cshift = 30;
+        q.csx = q.csy = 0;
+    }
+    const uint32_t c = 0x4b000000u >> q.cshift;
+    const uint32_t cell0 = c + (uint32_t)q.csx * (c + (uint32_t)q.csy * c);
+    mc_warp_kernel<NM, GEN, LM><<<(int)grid, WARP_BLOCK, bytes, s>>>(q, n_pool, n_use, chunk, cell0);
     return cudaGetLastError();
 }
 
-template <int NM>
-int pool_occupancy_t(int K) {
-    const size_t bytes = pool_smem_bytes<NM>(K);
-    int n = 0;
-    if (cudaFuncSetAttribute(mc_pool_kernel<NM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess
-        || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, mc_pool_kernel<NM>, POOL_THREADS, bytes) != cudaSuccess)
-        return 0;
-    return n;
+template <bool GEN, bool LM>
+cudaError_t launch_nm(const McParams& p, bool records, int block, int n_pool, int limit, int n_sm, cudaStream_t s) {
+    if (records) {
+        if (p.n_mat <= 2) return launch_records_t<2, GEN, LM>(p, block, limit, n_sm, s);
+        if (p.n_mat <= 4) return launch_records_t<4, GEN, LM>(p, block, limit, n_sm, s);
+        return launch_records_t<8, GEN, LM>(p, block, limit, n_sm, s);
+    }
+    const int warps = limit * block / 32;
+    if (p.n_mat <= 2) return launch_warp_t<2, GEN, LM>(p, n_pool, warps, n_sm, s);
+    if (p.n_mat <= 4) return launch_warp_t<4, GEN, LM>(p, n_pool, warps, n_sm, s);
+    return launch_warp_t<8, GEN, LM>(p, n_pool, warps, n_sm, s);
 }
 
 }  // namespace
 
-int pool_threads() { return POOL_THREADS; }
-
-// slots per lane class for pool photons per thread
-static int pool_k(int per_thread) { return POOL_WARPS * per_thread; }
-
-cudaError_t launch_mc_pool(const McParams& p, int per_thread, int grid, cudaStream_t s) {
-    const int K = pool_k(per_thread);
-    if (p.n_mat <= 2) return launch_pool_t<2>(p, K, grid, s);
-    if (p.n_mat <= 4) return launch_pool_t<4>(p, K, grid, s);
-    return launch_pool_t<8>(p, K, grid, s);
-}
-
-int mc_pool_occupancy_blocks(int n_mat, int per_thread) {
-    const int K = pool_k(per_thread);
-    if (n_mat <= 2) return pool_occupancy_t<2>(K);
-    if (n_mat <= 4) return pool_occupancy_t<4>(K);
-    return pool_occupancy_t<8>(K);
-}
-
-cudaError_t launch_mc_source(const McParams& p, cudaStream_t s) {
-    if (!p.src || p.total == 0) return cudaErrorInvalidValue;
-    int dev = 0, n_sm = 1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const uint64_t blocks = (p.total + 255) / 256;
-    const uint64_t cap = (uint64_t)n_sm * 8;
-    const int grid = (int)(blocks < cap ? blocks : cap);
-    float4* out = const_cast<float4*>(p.src);
-    if (p.n_mat <= 2) mc_source_kernel<2><<<grid, 256, 0, s>>>(p, out);
-    else if (p.n_mat <= 4) mc_source_kernel<4><<<grid, 256, 0, s>>>(p, out);
-    else mc_source_kernel<8><<<grid, 256, 0, s>>>(p, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_mc(const McParams& p, int block, int grid, bool records, cudaStream_t s) {
-    if (p.lm) {
-        if (!p.cells) return cudaErrorInvalidValue;       // the local majorants are the cell bounds
-        return launch_lm<true>(p, block, grid, records, s);
-    }
-    return launch_lm<false>(p, block, grid, records, s);
-}
-
-int mc_occupancy_blocks(int n_mat, int block, bool records, bool lm) {
-    if (lm) return records ? occupancy_nm<true, true>(n_mat, block) : occupancy_nm<false, true>(n_mat, block);
-    return records ? occupancy_nm<true, false>(n_mat, block) : occupancy_nm<false, false>(n_mat, block);
+// photons: photons per lane in a warp's pool (1 .. 3), or <= 0 for the default
+cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
+                      cudaStream_t s) {
+    if (p.lm && !p.cells) return cudaErrorInvalidValue;   // the local majorants are the cell bounds
+    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0;
+    const int n_pool = photons > 0 ? 32 * photons : POOL_DEFAULT;
+    if (p.lm) return gen ? launch_nm<true, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s)
+                         : launch_nm<false, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s);
+    return gen ? launch_nm<true, false>(p, records, block, n_pool, blocks_per_sm, n_sm, s)
+               : launch_nm<false, false>(p, records, block, n_pool, blocks_per_sm, n_sm, s);
 }
 
 cudaError_t launch_gather_probe(const McParams& p, uint64_t n_cells, int grid, unsigned int* sink, cudaStream_t s) {
