@@ -357,6 +357,11 @@ GDRR_API int gdrr_air_scan(gdrr_ctx* ctx, double* I0_dev);
 GDRR_API int gdrr_line_integrals(const double* signal_dev, const double* air_dev, int64_t n, double floor_rel,
                                  float* out_dev, void* cuda_stream);
 
+/* The same for n_views images of n pixels [n_views][n] that share one air scan
+ * of n pixels (the views of a scan): out [n_views][n]. */
+GDRR_API int gdrr_line_integrals_views(const double* signal_dev, const double* air_dev, int64_t n_views, int64_t n,
+                                       double floor_rel, float* out_dev, void* cuda_stream);
+
 /* Geometry of an FDK reconstruction: the circular orbit of Section 2.1
  * (source at sad_mm from the isocentre, imager at sdd_mm from the source,
  * opposite it: theta = 0), the detector grid, and the output voxel grid of

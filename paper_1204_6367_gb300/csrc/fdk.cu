@@ -12,9 +12,9 @@
 //   * voxel-driven backprojection f(x) = sum_beta dbeta (SAD / depth)^2
 //     Qf(a(x), b(x)), depth = SAD + x.n, bilinear on the pixel-centre grid,
 //     zero outside the detector.
-// The filter is a short dense row convolution (nu^2 / 2 FMAs per row) done
-// in shared memory with register tiling; the backprojection gathers 4 detector samples per voxel
-// and view from L1 / L2 and keeps 8 voxels of a column in registers, so the
+// The filter is a dense row convolution (nu^2 / 2 FMAs per row) from shared
+// memory with register tiles; the backprojection gathers 4 detector samples per voxel
+// and view from L1 / L2 and keeps a few voxels of a column in registers, so the
 // per-view geometry (depth, u, weight) is computed once per column.
 #include <cmath>
 
@@ -26,8 +26,9 @@ namespace {
 constexpr int FILTER_BLOCK = 256;
 constexpr int FILTER_MAX_NU = 4096;
 constexpr int BP_MAX_ANGLES = 128;     // views per backprojection launch (kernel parameters)
-constexpr int BP_ZT = 8;               // voxels of a column per thread
-constexpr int BP_BX = 32, BP_BY = 8;
+constexpr int BP_ZT = 4;               // voxels of a column per thread
+constexpr int BP_BX = 32, BP_BY = 8;   // voxels of a block in x and y, by warps of 8 x 4
+constexpr int BP_WX = 8;
 
 struct FilterParams {
     int nu, nv;
@@ -36,83 +37,141 @@ struct FilterParams {
     float scale;            // 1 / (2 tau_u)
 };
 
-// Register tiling: a thread owns FJ outputs of one parity, n_j = n0 + 2j.
-// Only sources k of the other parity contribute (odd offsets), and as k
-// advances by 2 the offsets |n_j - k| all move by 2 in the same direction, so
-// the FJ coefficients in use form a window that slides by one slot per
-// source: one shared-memory load of q(k) and one of the entering coefficient
-// serve FJ FMAs.  Sources between n_0 and n_{FJ-1} are taken directly.
-constexpr int FJ = 4;
+// The convolution of one parity is a product with a Toeplitz matrix: outputs
+// n = 2a + par take sources k = 2b + 1 - par (odd offsets only) with the
+// coefficient T[a - b + nb], one signed table per parity.  A thread owns FO
+// outputs (consecutive a) of FR rows: as b advances by one, its FO
+// coefficients slide by one slot, so a step loads one coefficient and, two
+// sources at a time, the FR rows' samples, for FO x FR FMAs, packed in pairs
+// of rows (fma.rn.f32x2).  The rows sit in shared memory weighted, split by
+// parity and interleaved in pairs, zero beyond the row; the table is padded by one slot in FO so that
+// the lanes of a warp (FO slots apart) read different banks.
+//
+// Bound: FP32 FMA (nu^2 / 2 per row; 18.1 G for 360 views of 512 x 384: 0.49 ms
+// at 128 per SM and cycle) and the rows' weighting before it: 0.88 ms.  One row
+// per block and 4 outputs per thread took 2.6 ms at the full shared-memory
+// rate; 8 rows per thread (2 blocks per SM) 0.95 ms, 2 rows 0.85 ms.
+constexpr int FO = 8, FR = 4, FL = 16;
+constexpr int FILTER_TASKS = FILTER_BLOCK;      // thread tasks a block aims at
 
-__global__ void __launch_bounds__(FILTER_BLOCK) fdk_filter_kernel(const FilterParams p, const float* __restrict__ g,
-                                                                 float* __restrict__ out) {
-    extern __shared__ float sm[];
-    float* q = sm;                // weighted row [nu]
-    float* c = sm + p.nu;         // offset |d| -> kernel coefficient [nu + 2 FJ]
+struct FilterShape {
+    int nb;          // sources of a parity, rounded up to a multiple of FO
+    int oct;         // output groups of FO per parity
+    int stride;      // samples of a row and parity in shared memory
+    int tab;         // padded coefficients per parity
+    int rows;        // rows per block, a multiple of FR
+};
+
+__host__ __device__ inline int filter_pad(int i) { return i + i / FO; }
+
+inline FilterShape filter_shape(int nu) {
+    FilterShape f;
+    f.nb = ((nu + 1) / 2 + FO - 1) / FO * FO;
+    f.oct = f.nb / FO;
+    f.stride = f.nb + 4;
+    f.tab = (filter_pad(2 * f.nb + FO) + 3) / 4 * 4;
+    const int groups = FILTER_TASKS / (2 * f.oct);
+    f.rows = FR * (groups < 1 ? 1 : groups);
+    return f;
+}
+
+inline size_t filter_smem(const FilterShape& f) { return sizeof(float) * ((size_t)2 * f.rows * f.stride + 2 * f.tab); }
+
+__device__ __forceinline__ uint64_t twice(float v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
+__global__ void __launch_bounds__(FILTER_BLOCK, 3) fdk_filter_kernel(const FilterParams p, const FilterShape f,
+                                                                    int64_t n_rows, const float* __restrict__ g,
+                                                                    float* __restrict__ out) {
+    extern __shared__ __align__(16) float sm[];
     const int nu = p.nu;
-    const int row = blockIdx.x;
-    const size_t base = ((size_t)blockIdx.y * p.nv + row) * nu;
-    const float b = ((float)row + 0.5f - 0.5f * (float)p.nv) * p.mag_dv;
-    const float sad2b2 = p.sad * p.sad + b * b;
-    for (int k = threadIdx.x; k < nu; k += blockDim.x) {
-        const float a = ((float)k + 0.5f - 0.5f * (float)nu) * p.mag_du;
-        q[k] = g[base + k] * (p.sad / sqrtf(sad2b2 + a * a));
+    float* q = sm;                                            // [2][rows][stride]
+    float* tab = sm + (size_t)2 * f.rows * f.stride;          // [2][tab]
+    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
+    const int rows = (int)min((int64_t)f.rows, n_rows - r0);
+    // T[a - b + nb] of parity par: offset n - k = 2 (a - b) + 2 par - 1
+    for (int i = threadIdx.x; i < 2 * (2 * f.nb + FO); i += FILTER_BLOCK) {
+        const int par = i / (2 * f.nb + FO), j = i - par * (2 * f.nb + FO);
+        const float pd = 3.14159265358979f * (float)(2 * (j - f.nb) + 2 * par - 1);
+        tab[par * f.tab + filter_pad(j)] = -1.0f / (pd * pd);
     }
-    for (int k = threadIdx.x; k < nu + 2 * FJ; k += blockDim.x) {
-        float ck = 0.0f;
-        if (k == 0) {
-            ck = 0.25f;
-        } else if (k & 1) {
-            const float pd = 3.14159265358979f * (float)k;
-            ck = -1.0f / (pd * pd);
+    for (int r = threadIdx.x >> 5; r < f.rows; r += FILTER_BLOCK / 32) {
+        const float b = ((float)((r0 + r) % p.nv) + 0.5f - 0.5f * (float)p.nv) * p.mag_dv;
+        const float sad2b2 = p.sad * p.sad + b * b;
+        const float* gr = g + (r0 + r) * nu;
+        for (int k0 = threadIdx.x & 31; k0 < 2 * f.nb; k0 += 32 * FL) {
+            float v[FL];                                      // FL loads under way at a time
+#pragma unroll
+            for (int i = 0; i < FL; ++i) v[i] = (r < rows && k0 + 32 * i < nu) ? __ldcs(gr + k0 + 32 * i) : 0.0f;
+#pragma unroll
+            for (int i = 0; i < FL; ++i) {
+                const int k = k0 + 32 * i;
+                const float a = ((float)k + 0.5f - 0.5f * (float)nu) * p.mag_du;
+                if (k < 2 * f.nb)
+                    q[((size_t)((k & 1) * (f.rows / 2) + (r >> 1)) * f.stride + (k >> 1)) * 2 + (r & 1)] =
+                        v[i] * (p.sad / sqrtf(sad2b2 + a * a));
+            }
         }
-        c[k] = ck;
     }
     __syncthreads();
-    const int n_groups = 2 * ((nu + 2 * FJ - 1) / (2 * FJ));
-    for (int grp = threadIdx.x; grp < n_groups; grp += blockDim.x) {
-        const int par = grp & 1;
-        const int n0 = 2 * FJ * (grp >> 1) + par;
-        float acc[FJ], w[FJ];
+    const int tasks = (f.rows / FR) * 2 * f.oct;
+    for (int task = threadIdx.x; task < tasks; task += FILTER_BLOCK) {
+        const int o = task % f.oct, par = (task / f.oct) & 1, rg = task / (2 * f.oct);
+        const uint64_t* q2 = reinterpret_cast<const uint64_t*>(q);            // one sample of two rows
+        const uint64_t* own = q2 + (size_t)(par * (f.rows / 2) + rg * (FR / 2)) * f.stride + o * FO;
+        const uint64_t* src = q2 + (size_t)((1 - par) * (f.rows / 2) + rg * (FR / 2)) * f.stride;
+        uint64_t acc[FR / 2][FO];
 #pragma unroll
-        for (int j = 0; j < FJ; ++j) acc[j] = (n0 + 2 * j < nu) ? c[0] * q[n0 + 2 * j] : 0.0f;
-        // sources below n0: offsets n_j - k, shrinking by 2 per source
-        int k = 1 - par;
-        if (k < n0) {
+        for (int r = 0; r < FR / 2; ++r)
 #pragma unroll
-            for (int j = 0; j < FJ; ++j) w[j] = c[n0 - k + 2 * j];
-            for (; k < n0; k += 2) {
-                const float qk = q[k];
+            for (int j = 0; j < FO; ++j) acc[r][j] = fma2(twice(0.25f), own[r * f.stride + j], 0ull);
+        // w[(j - b) mod FO] holds T[o FO + j - b + nb], twice
+        const float* t = tab + par * f.tab + filter_pad(o * FO + f.nb);
+        uint64_t w[FO];
 #pragma unroll
-                for (int j = 0; j < FJ; ++j) acc[j] += w[j] * qk;
+        for (int j = 0; j < FO; ++j) w[j] = twice(t[j]);
+        for (int b0 = 0; b0 < f.nb; b0 += FO) {
+            t -= FO + 1;                                      // the padded slot of FO coefficients further down
 #pragma unroll
-                for (int j = FJ - 1; j > 0; --j) w[j] = w[j - 1];
-                w[0] = c[max(n0 - k - 2, 0)];
-            }
-        }
-        // sources between n_0 and n_{FJ-1}
-        for (k = n0 + 1; k < n0 + 2 * (FJ - 1) && k < nu; k += 2) {
-            const float qk = q[k];
+            for (int h = 0; h < FO; h += 2) {
+                ulonglong2 s[FR / 2];
 #pragma unroll
-            for (int j = 0; j < FJ; ++j) acc[j] += c[abs(n0 + 2 * j - k)] * qk;
-        }
-        // sources above n_{FJ-1}: offsets k - n_j, growing by 2 per source
-        k = n0 + 2 * FJ - 1;
-        if (k < nu) {
+                for (int r = 0; r < FR / 2; ++r) s[r] = *reinterpret_cast<const ulonglong2*>(src + r * f.stride + b0 + h);
 #pragma unroll
-            for (int j = 0; j < FJ; ++j) w[j] = c[k - n0 - 2 * j];
-            for (; k < nu; k += 2) {
-                const float qk = q[k];
+                for (int b = h; b < h + 2; ++b) {
 #pragma unroll
-                for (int j = 0; j < FJ; ++j) acc[j] += w[j] * qk;
+                    for (int r = 0; r < FR / 2; ++r)
 #pragma unroll
-                for (int j = FJ - 1; j > 0; --j) w[j] = w[j - 1];
-                w[0] = c[min(k + 2 - n0, nu + 2 * FJ - 1)];
+                        for (int j = 0; j < FO; ++j)
+                            acc[r][j] = fma2(b == h ? s[r].x : s[r].y, w[(j - b + FO) % FO], acc[r][j]);
+                    w[FO - 1 - b] = twice(t[FO - 1 - b]);     // enters as the next source's first coefficient
+                }
             }
         }
 #pragma unroll
-        for (int j = 0; j < FJ; ++j)
-            if (n0 + 2 * j < nu) out[base + n0 + 2 * j] = p.scale * acc[j];
+        for (int r = 0; r < FR / 2; ++r)
+#pragma unroll
+            for (int j = 0; j < FO; ++j) {
+                const int n = 2 * (o * FO + j) + par;
+                const float2 v = unpack2(acc[r][j]);
+                if (n < nu) {
+                    if (rg * FR + 2 * r < rows) out[(r0 + rg * FR + 2 * r) * nu + n] = p.scale * v.x;
+                    if (rg * FR + 2 * r + 1 < rows) out[(r0 + rg * FR + 2 * r + 1) * nu + n] = p.scale * v.y;
+                }
+            }
     }
 }
 
@@ -134,10 +193,22 @@ __device__ __forceinline__ float tap(const float* __restrict__ img, int nu, int 
     return (iu >= 0 && iu < nu && iv >= 0 && iv < nv) ? __ldg(img + (size_t)iv * nu + iu) : 0.0f;
 }
 
-__global__ void __launch_bounds__(BP_BX * BP_BY) fdk_backproject_kernel(const BpParams p, const float* __restrict__ q,
+// A warp covers 8 x 4 columns, so that its detector samples of one view span a
+// few cache lines whatever the gantry angle (a row of 32 columns spans 125
+// samples at 90 degrees).  A group of voxels that misses the detector is left
+// at once; one whose samples all lie inside takes them unchecked, its row
+// index by adding 2^23 rounded down; only one across an edge tests every tap.
+//
+// Bound: instruction issue (66 % of the slots) beside L1 (57 %).  3.0e9
+// voxel-views (360 views of 512 x 384, 256 x 256 x 128 voxels of 2 mm, more
+// than half of them beyond the detector): 4.4 ms with rows of 32 columns and
+// every tap tested, 2.4 ms so.  Groups of 4, 6 and 8 voxels ran alike, 2 and 16
+// slower; so did more resident blocks at fewer registers.
+__global__ void __launch_bounds__(BP_BX * BP_BY, 4) fdk_backproject_kernel(const BpParams p, const float* __restrict__ q,
                                                                        float* __restrict__ vol) {
-    const int ix = blockIdx.x * BP_BX + threadIdx.x;
-    const int iy = blockIdx.y * BP_BY + threadIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ix = blockIdx.x * BP_BX + (warp % (BP_BX / BP_WX)) * BP_WX + lane % BP_WX;
+    const int iy = blockIdx.y * BP_BY + (warp / (BP_BX / BP_WX)) * (32 / BP_WX) + lane / BP_WX;
     const int iz0 = blockIdx.z * BP_ZT;
     if (ix >= p.nx || iy >= p.ny) return;
     const float x = p.x0 + (float)ix * p.dx;
@@ -146,10 +217,13 @@ __global__ void __launch_bounds__(BP_BX * BP_BY) fdk_backproject_kernel(const Bp
 #pragma unroll
     for (int k = 0; k < BP_ZT; ++k) acc[k] = 0.0f;
     const size_t view = (size_t)p.nu * p.nv;
+    const float z_lo = p.z0 + (float)iz0 * p.dz, z_hi = p.z0 + (float)(iz0 + BP_ZT - 1) * p.dz;
     for (int i = 0; i < p.n_ang; ++i) {
         const float cph = p.cs[i].x, sph = p.cs[i].y;
         const float depth = p.sad + x * cph + y * sph;
-        const float inv = 1.0f / depth;
+        float inv;                                                // Newton's step on an approximate reciprocal
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(depth));
+        inv = inv + inv * (1.0f - depth * inv);
         const float fu = p.sad * (x * sph - y * cph) * inv * p.inv_tau_u + p.hu;
         const float fiu = floorf(fu);
         if (fiu < -1.0f || fiu > (float)(p.nu - 1)) continue;   // the column misses the detector
@@ -159,6 +233,25 @@ __global__ void __launch_bounds__(BP_BX * BP_BY) fdk_backproject_kernel(const Bp
         const float w2 = p.d_beta * (m * m);
         const float sv = m * p.inv_tau_v;                           // dv-index per mm of z
         const float* img = q + (size_t)(p.first_view + i) * view;
+        const float wu0 = 1.0f - wu;
+        const float v_lo = z_lo * sv + p.hv, v_hi = z_hi * sv + p.hv;
+        if (v_hi <= -1.0f || v_lo >= (float)p.nv) continue;        // its voxels miss the detector
+        if (iu >= 0 && iu < p.nu - 1 && v_lo >= 0.0f && v_hi < (float)(p.nv - 1)) {
+            // 0x4b000000 + iv is the bit pattern of 2^23 + iv
+            const uint32_t nu = (uint32_t)p.nu, first = (uint32_t)iu - 0x4b000000u * nu;
+#pragma unroll
+            for (int k = 0; k < BP_ZT; ++k) {
+                const float z = p.z0 + (float)(iz0 + k) * p.dz;
+                const float fv = z * sv + p.hv;
+                const float t = __fadd_rd(fv, 8388608.0f);           // 2^23 + floor(fv)
+                const float wv = fv - (t - 8388608.0f);
+                const uint32_t o = __float_as_uint(t) * nu + first;
+                const float *r0 = img + o, *r1 = img + (o + nu);
+                const float v00 = __ldg(r0), v10 = __ldg(r0 + 1), v01 = __ldg(r1), v11 = __ldg(r1 + 1);
+                acc[k] += w2 * ((1.0f - wv) * (wu0 * v00 + wu * v10) + wv * (wu0 * v01 + wu * v11));
+            }
+            continue;
+        }
 #pragma unroll
         for (int k = 0; k < BP_ZT; ++k) {
             const float z = p.z0 + (float)(iz0 + k) * p.dz;
@@ -169,8 +262,7 @@ __global__ void __launch_bounds__(BP_BX * BP_BY) fdk_backproject_kernel(const Bp
             const float wv = fv - fiv;
             const float v00 = tap(img, p.nu, p.nv, iu, iv), v10 = tap(img, p.nu, p.nv, iu + 1, iv);
             const float v01 = tap(img, p.nu, p.nv, iu, iv + 1), v11 = tap(img, p.nu, p.nv, iu + 1, iv + 1);
-            const float val = (1.0f - wv) * ((1.0f - wu) * v00 + wu * v10) + wv * ((1.0f - wu) * v01 + wu * v11);
-            acc[k] += w2 * val;
+            acc[k] += w2 * ((1.0f - wv) * (wu0 * v00 + wu * v10) + wv * (wu0 * v01 + wu * v11));
         }
     }
 #pragma unroll
@@ -183,13 +275,113 @@ __global__ void __launch_bounds__(BP_BX * BP_BY) fdk_backproject_kernel(const Bp
     }
 }
 
-__global__ void line_integral_kernel(const double* __restrict__ s, const double* __restrict__ a, int64_t n,
-                                     double floor_rel, float* __restrict__ out) {
+// Line integrals -ln(max(s, floor a) / a), rounded to FP32 from the FP64
+// inputs.  GB300 runs FP64 at 1/64 of the FP32 rate and the FP64 logarithm
+// bound the kernel (5.2 ms for 70.8 M pixels against 0.13 ms of memory
+// traffic), 0.41 ms as below: the value is formed in pairs of floats from the integer bits of
+// the operands: with r = s / a brought to [sqrt(1/2), sqrt(2)) by a power of
+// two, ln r = 2 atanh(t), t = (ms - ma) / (ms + ma) (difference and sum of the
+// 53-bit significands, quotient with its remainder), atanh by its Taylor
+// series to t^15, whose first correction t^2 / 3 is also carried as a pair.
+// The result's relative error is below 2^-36; where that leaves the rounding
+// to FP32 open (one pixel in about 2000), and for operands that are not
+// positive normal numbers, the FP64 logarithm decides, so what is written is
+// the FP32 rounding of the logarithm, as before.
+constexpr int LI_VIEWS = 8;       // pixels of consecutive views per thread: the air pixel's part is formed once
+
+struct Pair {
+    float h, l;
+};
+
+__device__ __forceinline__ Pair two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+
+// the significand of a positive normal double as a pair in [1, 2): its first
+// 24 bits, and the 29 below as an integer (units of 2^-52)
+struct Significand {
+    float h;
+    int l;
+};
+constexpr float TWO_M52 = (float)(1.0 / 4503599627370496.0);
+
+__device__ __forceinline__ Significand significand(uint64_t bits) {
+    return {__uint_as_float(0x3f800000u | ((uint32_t)(bits >> 29) & 0x007fffffu)), (int)((uint32_t)bits & 0x1fffffffu)};
+}
+
+__device__ __noinline__ float line_integral_64(double s, double a, double floor_rel) {
+    return (float)(-log(fmax(s, floor_rel * a) / a));
+}
+
+__device__ __forceinline__ float line_integral(double s, double a, double least, double floor_rel,
+                                               Significand ma) {
+    const int64_t sb = __double_as_longlong(s), lb = __double_as_longlong(least);
+    const int64_t vb = sb > lb ? sb : lb;                 // positive doubles order like their bits
+    const int64_t ab = __double_as_longlong(a);
+    const int ev = (int)(vb >> 52), ea = (int)(ab >> 52);
+    if ((unsigned)(ev - 1) >= 2046u || (unsigned)(ea - 1) >= 2046u || lb <= 0) return line_integral_64(s, a, floor_rel);
+    const Significand mv = significand((uint64_t)vb);
+    // the power of two that brings the ratio to [sqrt(1/2), sqrt(2))
+    int e = ev - ea;
+    float k = 1.0f;
+    if (mv.h > 1.41421354f * ma.h) { k = 2.0f; e += 1; }
+    else if (1.41421354f * mv.h < ma.h) { k = 0.5f; e -= 1; }
+    const float ah = k * ma.h, vl = (float)mv.l * TWO_M52, al = (float)ma.l * TWO_M52 * k;
+    // near 1 the difference is small: its low part exactly, as two floats
+    const int dl = mv.l - ma.l;
+    const float d1 = (float)dl, d2 = (float)(dl - (int)d1);
+    Pair d = two_sum(__fsub_rn(mv.h, ah), k == 1.0f ? d1 * TWO_M52 : __fsub_rn(vl, al));   // the first difference is exact
+    if (k == 1.0f) d.l = __fmaf_rn(d2, TWO_M52, d.l);
+    Pair w = two_sum(mv.h, ah);
+    w.l = __fadd_rn(w.l, __fadd_rn(vl, al));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(w.h));
+    const float th = __fmul_rn(d.h, y);
+    const float tl = __fmul_rn(__fadd_rn(__fmaf_rn(-th, w.h, d.h), __fmaf_rn(-th, w.l, d.l)), y);
+    const float uh = __fmul_rn(th, th);
+    const float ul = __fmaf_rn(2.0f * th, tl, __fmaf_rn(th, th, -uh));
+    float p = (float)(1.0 / 15.0);
+    p = __fmaf_rn(p, uh, (float)(1.0 / 13.0));
+    p = __fmaf_rn(p, uh, (float)(1.0 / 11.0));
+    p = __fmaf_rn(p, uh, (float)(1.0 / 9.0));
+    p = __fmaf_rn(p, uh, (float)(1.0 / 7.0));
+    p = __fmaf_rn(p, uh, (float)(1.0 / 5.0));
+    constexpr float C3H = (float)(1.0 / 3.0), C3L = (float)(1.0 / 3.0 - (double)C3H);
+    const float ch = __fmul_rn(uh, C3H);
+    const float cl = __fadd_rn(__fmaf_rn(uh, C3H, -ch), __fmaf_rn(uh, C3L, __fmaf_rn(ul, C3H, __fmul_rn(uh, __fmul_rn(uh, p)))));
+    // ln r = 2 (t + t c)
+    const float bh = __fmul_rn(th, ch);
+    const float bl = __fmaf_rn(th, ch, -bh);
+    Pair g = two_sum(th, bh);
+    g.l = __fadd_rn(g.l, __fadd_rn(__fadd_rn(tl, bl), __fmaf_rn(tl, ch, __fmul_rn(th, cl))));
+    // + e ln 2: e times the 12-bit head is exact
+    const float fe = (float)e;
+    constexpr double LN2 = 0.69314718055994530942;
+    constexpr float L1 = (float)(2839.0 / 4096.0), L2 = (float)(LN2 - 2839.0 / 4096.0);
+    constexpr float L3 = (float)(LN2 - 2839.0 / 4096.0 - (double)L2);
+    const float mh = __fmul_rn(fe, L2);
+    Pair q = two_sum(__fmul_rn(fe, L1), 2.0f * g.h);
+    const Pair m = two_sum(q.h, mh);
+    q.l = __fadd_rn(__fadd_rn(q.l, m.l), __fmaf_rn(2.0f, g.l, __fmaf_rn(fe, L3, __fmaf_rn(fe, L2, -mh))));
+    const Pair r = two_sum(m.h, q.l);
+    const float err = fabsf(r.h) * (float)(1.0 / 34359738368.0);             // 2^-35
+    if (__fadd_rn(r.h, __fadd_rn(r.l, err)) != r.h || __fadd_rn(r.h, __fsub_rn(r.l, err)) != r.h)
+        return line_integral_64(s, a, floor_rel);
+    return -r.h;
+}
+
+__global__ void __launch_bounds__(256) line_integral_kernel(const double* __restrict__ s, const double* __restrict__ a,
+                                                           int64_t n_views, int64_t n, double floor_rel,
+                                                           float* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double i0 = a[i];
-    const double v = fmax(s[i], floor_rel * i0);
-    out[i] = (float)(-log(v / i0));
+    const double i0 = a[i], least = floor_rel * i0;
+    const Significand ma = significand((uint64_t)__double_as_longlong(i0));
+    const int64_t v0 = (int64_t)blockIdx.y * LI_VIEWS;
+#pragma unroll
+    for (int k = 0; k < LI_VIEWS; ++k)
+        if (v0 + k < n_views) out[(v0 + k) * n + i] = line_integral(s[(v0 + k) * n + i], i0, least, floor_rel, ma);
 }
 
 bool geometry_valid(const gdrr_fdk_geometry* g) {
@@ -201,15 +393,23 @@ bool geometry_valid(const gdrr_fdk_geometry* g) {
 }  // namespace
 }  // namespace gdrr
 
+extern "C" GDRR_API int gdrr_line_integrals_views(const double* signal_dev, const double* air_dev, int64_t n_views,
+                                                  int64_t n, double floor_rel, float* out_dev, void* cuda_stream) {
+    if (n < 0 || n_views < 0 || (n > 0 && n_views > 0 && (!signal_dev || !air_dev || !out_dev)) || !(floor_rel > 0.0)
+        || !(floor_rel < 1.0))
+        return GDRR_ERR_INVALID_ARG;
+    if (n == 0 || n_views == 0) return GDRR_OK;
+    if (n_views > 65535 * (int64_t)gdrr::LI_VIEWS) return GDRR_ERR_UNSUPPORTED;
+    const int block = 256;
+    const dim3 grid((unsigned)((n + block - 1) / block), (unsigned)((n_views + gdrr::LI_VIEWS - 1) / gdrr::LI_VIEWS));
+    gdrr::line_integral_kernel<<<grid, block, 0, (cudaStream_t)cuda_stream>>>(signal_dev, air_dev, n_views, n, floor_rel,
+                                                                             out_dev);
+    return cudaGetLastError() == cudaSuccess ? GDRR_OK : GDRR_ERR_CUDA;
+}
+
 extern "C" GDRR_API int gdrr_line_integrals(const double* signal_dev, const double* air_dev, int64_t n,
                                             double floor_rel, float* out_dev, void* cuda_stream) {
-    if (n < 0 || (n > 0 && (!signal_dev || !air_dev || !out_dev)) || !(floor_rel > 0.0) || !(floor_rel < 1.0))
-        return GDRR_ERR_INVALID_ARG;
-    if (n == 0) return GDRR_OK;
-    const int block = 256;
-    gdrr::line_integral_kernel<<<(unsigned)((n + block - 1) / block), block, 0, (cudaStream_t)cuda_stream>>>(
-        signal_dev, air_dev, n, floor_rel, out_dev);
-    return cudaGetLastError() == cudaSuccess ? GDRR_OK : GDRR_ERR_CUDA;
+    return gdrr_line_integrals_views(signal_dev, air_dev, 1, n, floor_rel, out_dev, cuda_stream);
 }
 
 extern "C" GDRR_API int gdrr_fdk_filter(const gdrr_fdk_geometry* g, int32_t n_proj, const float* proj_dev,
@@ -225,9 +425,13 @@ extern "C" GDRR_API int gdrr_fdk_filter(const gdrr_fdk_geometry* g, int32_t n_pr
     p.mag_dv = (float)(g->dv_mm * mag);
     p.sad = (float)g->sad_mm;
     p.scale = (float)(0.5 / (g->du_mm * mag));
-    const dim3 grid((unsigned)g->nv, (unsigned)n_proj);
-    const size_t smem = sizeof(float) * (2 * (size_t)g->nu + 2 * gdrr::FJ);
-    gdrr::fdk_filter_kernel<<<grid, gdrr::FILTER_BLOCK, smem, (cudaStream_t)cuda_stream>>>(p, proj_dev, filtered_dev);
+    const gdrr::FilterShape f = gdrr::filter_shape(g->nu);
+    const size_t smem = gdrr::filter_smem(f);
+    if (cudaFuncSetAttribute(gdrr::fdk_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return GDRR_ERR_CUDA;
+    const int64_t n_rows = (int64_t)g->nv * n_proj;
+    gdrr::fdk_filter_kernel<<<(unsigned)((n_rows + f.rows - 1) / f.rows), gdrr::FILTER_BLOCK, smem,
+                              (cudaStream_t)cuda_stream>>>(p, f, n_rows, proj_dev, filtered_dev);
     return cudaGetLastError() == cudaSuccess ? GDRR_OK : GDRR_ERR_CUDA;
 }
 
@@ -258,7 +462,7 @@ extern "C" GDRR_API int gdrr_fdk_backproject(const gdrr_fdk_geometry* g, int32_t
     p.hu = (float)(0.5 * g->nu - 0.5);
     p.hv = (float)(0.5 * g->nv - 0.5);
     p.d_beta = (float)d_beta;
-    const dim3 block(gdrr::BP_BX, gdrr::BP_BY);
+    const int block = gdrr::BP_BX * gdrr::BP_BY;
     const dim3 grid((unsigned)((g->nx + gdrr::BP_BX - 1) / gdrr::BP_BX), (unsigned)((g->ny + gdrr::BP_BY - 1) / gdrr::BP_BY),
                     (unsigned)((g->nz + gdrr::BP_ZT - 1) / gdrr::BP_ZT));
     if (n_proj == 0 && !accumulate) {

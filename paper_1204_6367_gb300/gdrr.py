@@ -167,6 +167,7 @@ def lib():
             "gdrr_probe_l2_gather": [i64, vp, vp],
             "gdrr_probe_fp32": [vp, vp],
             "gdrr_line_integrals": [vp, vp, i64, dbl, vp, vp],
+            "gdrr_line_integrals_views": [vp, vp, i64, i64, dbl, vp, vp],
             "gdrr_fdk_filter": [vp, i32, vp, vp, vp],
             "gdrr_fdk_backproject": [vp, i32, vp, dbl, vp, vp, i32, vp],
             "gdrr_project": [vp, vp, vp, vp],
@@ -684,6 +685,20 @@ def gdrr_line_integrals(signal, air, floor_rel: float = 1e-6, out=None, stream=N
                                                             _dev_ptr(air, torch.float64, n, "air"), n,
                                                             float(floor_rel), _dev_ptr(out, torch.float32, n, "out"),
                                                             h))
+    return out
+
+
+def gdrr_line_integrals_views(signal, air, floor_rel: float = 1e-6, out=None, stream=None):
+    """The same for views signal [n_views, ...] that share one air scan air [...]."""
+    import torch
+    if out is None:
+        out = torch.empty(signal.shape, dtype=torch.float32, device="cuda")
+    h, _ = _stream_handle(stream)
+    n_views, n = signal.shape[0], air.numel()
+    _check("gdrr_line_integrals_views",
+           lib().gdrr_line_integrals_views(_dev_ptr(signal, torch.float64, n_views * n, "signal"),
+                                           _dev_ptr(air, torch.float64, None, "air"), n_views, n, float(floor_rel),
+                                           _dev_ptr(out, torch.float32, n_views * n, "out"), h))
     return out
 
 

@@ -58,7 +58,7 @@ def scan(ctx, n_views: int, components: str = "P", n_photons: int = 1_000_000, s
 def reconstruct(ctx, angles, signal, shape, voxel, floor_rel: float = 1e-6):
     """FDK volume [nz, ny, nx] FP32 (attenuation, 1/mm) of a scan's signals."""
     I0 = gdrr.gdrr_air_scan(ctx)
-    g = gdrr.gdrr_line_integrals(signal, I0.expand_as(signal).contiguous(), floor_rel)
+    g = gdrr.gdrr_line_integrals_views(signal, I0, floor_rel)
     p = ctx.prob
     geo = gdrr.fdk_geometry(p.sad, p.sdd, ctx.nu, ctx.nv, p.du, p.dv, shape, voxel)
     return gdrr.fdk(geo, g, angles)
