@@ -173,12 +173,12 @@ void dfree(const gdrr_ctx* c, void* p) {
 // kernel's counters, gdrr_project's scalars), kept for reuse: a page-locked
 // allocation costs far more than the copies it serves, and contexts come and
 // go.  take_pinned hands out the smallest free block that is large enough.
-struct Pinned {
-    void* p = nullptr;
-    size_t cap = 0;
-};
 std::mutex g_host_mutex;
 std::vector<Pinned> g_host_free;
+
+}  // namespace
+
+namespace gdrr {
 
 Pinned take_pinned(size_t bytes) {
     {
@@ -207,6 +207,10 @@ void give_pinned(Pinned b) {
     std::lock_guard<std::mutex> lock(g_host_mutex);
     g_host_free.push_back(b);
 }
+
+}  // namespace gdrr
+
+namespace {
 
 #define TRY_CUDA(x)                               \
     do {                                          \

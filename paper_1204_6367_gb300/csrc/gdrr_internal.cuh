@@ -181,6 +181,16 @@ struct RtParams {
 // blocks (of `block` threads) per SM.
 cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
                       cudaStream_t s);
+// Page-locked host blocks, kept on a free list of the process for reuse (p is
+// NULL when there is no memory); the device reads and writes them in place.
+// gdrr_release_memory frees the list.
+struct Pinned {
+    void* p = nullptr;
+    size_t cap = 0;
+};
+Pinned take_pinned(size_t bytes);
+void give_pinned(Pinned b);
+
 cudaError_t launch_rt(const RtParams& p, double* out, cudaStream_t s);
 cudaError_t launch_rt_siddon(const RtParams& p, double* out, cudaStream_t s);
 cudaError_t launch_air(const RtParams& p, double* out, cudaStream_t s);

@@ -784,8 +784,8 @@ def gdrr_gemm_bf16(a, b, splits: int = 1, out=None, stream=None):
     import torch
     M, K = a.shape
     N = b.shape[0]
-    if out is None:
-        out = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    if out is None:      # one split overwrites every element; more add into zeros
+        out = (torch.empty if splits == 1 else torch.zeros)((M, N), dtype=torch.float32, device="cuda")
     h, _ = _stream_handle(stream)
     _check("gdrr_gemm_bf16", lib().gdrr_gemm_bf16(_row_major_ptr(a, torch.bfloat16, "A"), a.stride(0),
                                                   _row_major_ptr(b, torch.bfloat16, "B"), b.stride(0),
