@@ -411,7 +411,7 @@ GDRR_API int gdrr_probe_l2_gather(int64_t working_set_bytes, double* gbs_out, vo
 GDRR_API int gdrr_probe_fp32(double* tflops_out, void* cuda_stream);
 
 /* Check of the bounded device-side wait (not part of the method): one CTA
- * waits, with the same bounded wait the denoiser's row bands use, for a flag
+ * waits, with a wait bounded by %globaltimer as the denoiser's are, for a flag
  * that nothing sets.  The wait gives up after limit_ns nanoseconds (1 ..
  * 2e9) and the call returns GDRR_ERR_TIMEOUT; GDRR_OK would mean the flag was
  * seen.  Allocates 16 bytes, runs on cuda_stream, synchronises. */

@@ -1229,9 +1229,10 @@ GDRR_API int gdrr_upsample(gdrr_ctx* ctx, const double* coarse_dev, int32_t cu, 
     return cuda_err(launch_upsample(coarse_dev, cu, cv, factor, fine_dev, ctx->stream));
 }
 
-// The context's denoiser scratch, grown to the larger of the two forms' needs.
+// The context's denoiser scratch, grown to what the image's form needs.
 static int denoise_scratch(gdrr_ctx* ctx, int nu, int nv) {
-    const size_t need = std::max(denoise_scratch_doubles(nu, nv) * sizeof(double), denoise_fused_scratch_bytes(nu, nv));
+    const size_t need = denoise_fused_fits(nu, nv) ? denoise_fused_scratch_bytes(nu, nv)
+                                                   : denoise_scratch_doubles(nu, nv) * sizeof(double);
     if (need > ctx->denoise_cap) {
         dfree(ctx, ctx->d_denoise);
         ctx->d_denoise = nullptr;

@@ -162,134 +162,183 @@ size_t denoise_scratch_doubles(int nu, int nv) { return 2 * (size_t)nu * nv; }
 // ---------------------------------------------------------------------------
 // The Eq. 5 iteration in one launch.
 //
-// Each CTA owns a band of whole image rows and keeps, per owned pixel, the
-// count-scale data S^ and the current iterate in registers.  Iterates travel
-// through two ping-pong images in global memory (L2-resident: 2 x 96 KB at
-// 128 x 96); after writing its rows of iterate k + 1 a CTA publishes k + 2 in
-// its flag, and before reading iterate k it waits until the CTAs of the rows
-// above and below have published k + 1.  That one wait also shows that those
-// neighbours have finished reading the buffer the CTA is about to overwrite
-// (they read it before publishing), so no grid-wide barrier is needed.  The
-// launch is cooperative, which guarantees that every CTA is resident, and
+// Each CTA owns a tile of the image and keeps, per owned pixel, the
+// count-scale data S^ and the current iterate in registers; inside the tile
+// iterates travel through shared memory.  A pixel on the tile's edge is also
+// published to global memory (L2) as two 8-byte words, each holding half of
+// the value and the iterate's number, and a pixel of the neighbouring tile
+// polls exactly the words it needs until both carry the number it waits for:
+// the data is its own flag, so one iteration costs one trip through L2 instead
+// of a barrier, a fence, a flag and then the data.  Two sets of words are
+// enough: a pixel publishes iterate k + 2 only after it has read iterate k + 1
+// of every pixel across the edge, and those were formed after their owners had
+// read its iterate k.  The part of an update that needs only the pixel itself
+// (the FP64 division above all) runs while the neighbours' words travel.
+//
+// The launch is cooperative, which guarantees that every CTA is resident, and
 // every wait is bounded (about a second of %globaltimer): on expiry the CTA
 // records a timeout in *status and stops.  The arithmetic per pixel is that
 // of denoise_step, in the same order, so both forms give the same result.
+//
+// Bound: FP64, 18 operations per pixel and iteration at 2 per SM and cycle
+// (0.4 us for a tile of 86 pixels), beside the trip through L2.  128 x 96, 300
+// iterations: 1.03 ms with row bands and neighbour flags, 0.49 ms so.
 namespace {
 
 constexpr int FUSED_MAX_PPT = 4;                    // owned pixels per thread
 constexpr unsigned long long WAIT_NS = 1000000000ull;
 
+// value and number of an iterate, as two self-numbered words
+__device__ __forceinline__ void publish(ulonglong2* p, double v, unsigned number) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const unsigned long long n = (unsigned long long)number << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(n | (bits & 0xffffffffull)),
+                 "l"(n | (bits >> 32)) : "memory");
+}
+
+__device__ __forceinline__ bool poll(const ulonglong2* p, unsigned number, double& v) {
+    unsigned long long lo, hi;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+    v = __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
+    return (unsigned)(lo >> 32) == number && (unsigned)(hi >> 32) == number;
+}
+
+// PPT: owned pixels per thread (1, 2 or FUSED_MAX_PPT)
+template <int PPT>
 __global__ void __launch_bounds__(1024) denoise_fused_kernel(
-    const double* __restrict__ s_hat, double* __restrict__ s_out, int nu, int nv, int rows_per_cta,
-    double count_scale_h, double beta_h, const double* __restrict__ scal, double omega, int iters,
-    double* buf0, double* buf1, unsigned* flags, int* status) {
-    __shared__ int s_abort;
-    const int b = blockIdx.x, G = gridDim.x;
-    const int r0 = b * rows_per_cta;
-    const int r1 = min(nv, r0 + rows_per_cta);
-    const int npx = (r1 - r0) * nu;
+    const double* __restrict__ s_hat, double* __restrict__ s_out, int nu, int nv, int tile_w, int tile_h, int tiles_x,
+    double count_scale_h, double beta_h, const double* __restrict__ scal, double omega, int iters, ulonglong2* words,
+    int* status) {
+    extern __shared__ double img[];                  // [2][tile_h tile_w]
+    const int x0 = (blockIdx.x % tiles_x) * tile_w, y0 = (blockIdx.x / tiles_x) * tile_h;
+    const int w = min(tile_w, nu - x0), h = min(tile_h, nv - y0), npx = w * h;
     const double count_scale = scal ? scal[0] : count_scale_h;
     const double beta = scal ? scal[1] : beta_h;
     const double inv_scale = 1.0 / count_scale, inv_beta = 1.0 / beta;
-    double sc[FUSED_MAX_PPT], cur[FUSED_MAX_PPT];
+    const double keep = 1.0 - omega, step = omega / 4.0;
+    const size_t n = (size_t)nu * nv;
+    double sc[PPT], cur[PPT];
+    // per pixel: where it lies, and which of its neighbours (right, down,
+    // left, up) are its own copy (bits 0-3) or across the tile's edge (4-7)
+    int at[PPT];
+    unsigned edge[PPT];
 #pragma unroll
-    for (int p = 0; p < FUSED_MAX_PPT; ++p) {
+    for (int p = 0; p < PPT; ++p) {
         const int i = threadIdx.x + p * blockDim.x;
         sc[p] = 0.0;
         cur[p] = DENOISE_EPS;
+        at[p] = 0;
+        edge[p] = 0u;
         if (i < npx) {
-            const int g = r0 * nu + i;
-            const double v = s_hat[g] * inv_scale;
+            const int lx = i % w, ly = i / w, x = x0 + lx, y = y0 + ly;
+            at[p] = y * nu + x;
+            if (lx == w - 1) edge[p] |= x == nu - 1 ? 0x01u : 0x10u;
+            if (ly == h - 1) edge[p] |= y == nv - 1 ? 0x02u : 0x20u;
+            if (lx == 0) edge[p] |= x == 0 ? 0x04u : 0x40u;
+            if (ly == 0) edge[p] |= y == 0 ? 0x08u : 0x80u;
+            const double v = s_hat[at[p]] * inv_scale;
             sc[p] = v;
             cur[p] = fmax(v, DENOISE_EPS);
-            buf0[g] = cur[p];
+            if (iters > 0 && (edge[p] & 0xf0u)) publish(words + at[p], cur[p], 1u);
+            img[i] = cur[p];
         }
     }
-    if (threadIdx.x == 0) s_abort = 0;
-    __syncwarp();                                 // converged warps at every block barrier
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        st_release_u32(flags + b, 1u);
-    }
+    int fail = 0;
     for (int k = 0; k < iters; ++k) {
-        if (threadIdx.x == 0) {
-            if (!wait_band_neighbours(flags, b, G, (unsigned)k + 1u, WAIT_NS)) {
-                atomicOr(status, 1);
-                s_abort = 1;
-            }
-            __threadfence();
-        }
-        __syncwarp();
-        __syncthreads();
-        if (s_abort) return;
-        const double* src = (k & 1) ? buf1 : buf0;
-        double* dst = (k & 1) ? buf0 : buf1;
+        // the pixel's own part, while the neighbours' words travel
+        double own[PPT], fid[PPT];
 #pragma unroll
-        for (int p = 0; p < FUSED_MAX_PPT; ++p) {
+        for (int p = 0; p < PPT; ++p) {
+            if (threadIdx.x + p * blockDim.x < npx) {
+                own[p] = keep * cur[p];
+                fid[p] = inv_beta * (1.0 - sc[p] / cur[p]);
+            }
+        }
+        __syncwarp();                                // converged warps at the block barrier
+        if (__syncthreads_or(fail)) return;
+        const double* src = img + (k & 1) * npx;
+        double* dst = img + ((k + 1) & 1) * npx;
+        const ulonglong2* in = words + (k & 1) * n;
+        ulonglong2* out = words + ((k + 1) & 1) * n;
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
             const int i = threadIdx.x + p * blockDim.x;
             if (i < npx) {
-                const int iv = r0 + i / nu, iu = i % nu;
-                const double c = cur[p];
-                const double right = __ldcg(src + iv * nu + min(iu + 1, nu - 1));
-                const double down = __ldcg(src + min(iv + 1, nv - 1) * nu + iu);
-                const double left = __ldcg(src + iv * nu + max(iu - 1, 0));
-                const double up = __ldcg(src + max(iv - 1, 0) * nu + iu);
-                const double sigma = ((right + down) + left) + up;
-                const double v = (1.0 - omega) * c + (omega / 4.0) * (sigma - inv_beta * (1.0 - sc[p] / c));
+                const unsigned e = edge[p], own_or_edge = e | (e >> 4);
+                double nb[4];
+                nb[0] = (own_or_edge & 1u) ? cur[p] : src[i + 1];
+                nb[1] = (own_or_edge & 2u) ? cur[p] : src[i + w];
+                nb[2] = (own_or_edge & 4u) ? cur[p] : src[i - 1];
+                nb[3] = (own_or_edge & 8u) ? cur[p] : src[i - w];
+                unsigned want = e >> 4;
+                if (want) {
+                    const ulonglong2* me = in + at[p];
+                    unsigned long long t0 = 0;
+                    for (unsigned tries = 0; want; ++tries) {
+                        if ((want & 1u) && poll(me + 1, (unsigned)k + 1u, nb[0])) want &= ~1u;
+                        if ((want & 2u) && poll(me + nu, (unsigned)k + 1u, nb[1])) want &= ~2u;
+                        if ((want & 4u) && poll(me - 1, (unsigned)k + 1u, nb[2])) want &= ~4u;
+                        if ((want & 8u) && poll(me - nu, (unsigned)k + 1u, nb[3])) want &= ~8u;
+                        if ((tries & 63u) == 63u) {
+                            if (t0 == 0) t0 = globaltimer_ns();
+                            if (globaltimer_ns() - t0 > WAIT_NS) {
+                                atomicOr(status, 1);
+                                fail = 1;
+                                break;
+                            }
+                        }
+                    }
+                }
+                const double sigma = ((nb[0] + nb[1]) + nb[2]) + nb[3];
+                const double v = own[p] + step * (sigma - fid[p]);
                 cur[p] = fmax(v, DENOISE_EPS);
-                dst[iv * nu + iu] = cur[p];
+                if (e & 0xf0u) publish(out + at[p], cur[p], (unsigned)k + 2u);
+                dst[i] = cur[p];
             }
-        }
-        __syncwarp();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            st_release_u32(flags + b, (unsigned)k + 2u);
         }
     }
 #pragma unroll
-    for (int p = 0; p < FUSED_MAX_PPT; ++p) {
-        const int i = threadIdx.x + p * blockDim.x;
-        if (i < npx) s_out[r0 * nu + i] = cur[p] * count_scale;
-    }
+    for (int p = 0; p < PPT; ++p)
+        if (threadIdx.x + p * blockDim.x < npx) s_out[at[p]] = cur[p] * count_scale;
 }
 
 struct FusedShape {
-    int rows, grid, block;
+    int tile_w, tile_h, tiles_x, grid, block;
 };
 
-// The band shape of the one-launch form on this device, or grid = 0 when the
-// image does not fit it (more owned pixels per thread than the registers
-// hold, or more bands than can be resident at once).
+// The tiles of the one-launch form on this device, or grid = 0 when the image
+// does not fit it (more owned pixels per thread than the registers hold): one
+// tile per SM, of the split into columns and rows whose tile has the fewest
+// warps of pixels (128 x 96 on 152 SMs: 144 tiles of 43 x 2).
 FusedShape fused_shape(int nu, int nv) {
-    FusedShape f{0, 0, 0};
-    int dev = 0, n_sm = 0, coop = 0, per_sm = 0;
+    FusedShape f{0, 0, 0, 0, 0};
+    int dev = 0, n_sm = 0, coop = 0;
     if (nu <= 0 || nv <= 0) return f;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, denoise_fused_kernel, 1024, 0) != cudaSuccess)
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess)
         return f;
-    if (!coop || n_sm <= 0 || per_sm <= 0) return f;
-    const int rows = (nv + n_sm - 1) / n_sm;
-    const int64_t band = (int64_t)rows * nu;
-    int block = (int)std::min<int64_t>(1024, (band + 31) / 32 * 32);
-    if ((band + block - 1) / block > FUSED_MAX_PPT) return f;
-    const int grid = (nv + rows - 1) / rows;
-    if (grid > n_sm * per_sm) return f;
-    f.rows = rows;
-    f.grid = grid;
-    f.block = block;
+    if (!coop || n_sm <= 0) return f;
+    int64_t best = 0;
+    for (int tx = 1; tx <= std::min(nu, n_sm); ++tx) {
+        const int rows = (nv + n_sm / tx - 1) / (n_sm / tx), w = (nu + tx - 1) / tx;
+        const int64_t warps = ((int64_t)rows * w + 31) / 32;
+        if (best && warps >= best) continue;
+        best = warps;
+        f.tile_w = w;
+        f.tile_h = rows;
+        f.tiles_x = (nu + w - 1) / w;
+        f.grid = f.tiles_x * ((nv + rows - 1) / rows);
+        f.block = (int)std::min<int64_t>(1024, warps * 32);
+    }
+    if (best * 32 > (int64_t)FUSED_MAX_PPT * 1024) f.grid = 0;
     return f;
 }
 
 }  // namespace
 
-// scratch of the one-launch form: two ping-pong images, then one flag per band
-size_t denoise_fused_scratch_bytes(int nu, int nv) {
-    return 2 * (size_t)nu * nv * sizeof(double) + (size_t)(nv + 1) * sizeof(unsigned);
-}
+// scratch of the one-launch form: two sets of the pixels' published words
+size_t denoise_fused_scratch_bytes(int nu, int nv) { return 2 * (size_t)nu * nv * sizeof(ulonglong2); }
 
 bool denoise_fused_fits(int nu, int nv) { return fused_shape(nu, nv).grid > 0; }
 
@@ -298,16 +347,22 @@ cudaError_t launch_denoise_fused(const double* s_hat, double* s_out, int nu, int
                                  int* status, cudaStream_t stream) {
     const FusedShape f = fused_shape(nu, nv);
     if (!f.grid) return cudaErrorInvalidConfiguration;
-    double* buf0 = static_cast<double*>(scratch);
-    double* buf1 = buf0 + (size_t)nu * nv;
-    unsigned* flags = reinterpret_cast<unsigned*>(buf1 + (size_t)nu * nv);
-    cudaError_t e = cudaMemsetAsync(flags, 0, (size_t)f.grid * sizeof(unsigned), stream);
+    ulonglong2* words = static_cast<ulonglong2*>(scratch);
+    cudaError_t e = cudaMemsetAsync(words, 0, denoise_fused_scratch_bytes(nu, nv), stream);   // no iterate's number
     if (e != cudaSuccess) return e;
-    int rows = f.rows;
-    void* args[] = {(void*)&s_hat, (void*)&s_out, (void*)&nu, (void*)&nv, (void*)&rows, (void*)&count_scale,
-                    (void*)&beta, (void*)&scal_dev, (void*)&omega, (void*)&iters, (void*)&buf0, (void*)&buf1,
-                    (void*)&flags, (void*)&status};
-    return cudaLaunchCooperativeKernel((const void*)denoise_fused_kernel, dim3(f.grid), dim3(f.block), args, 0,
+    int tile_w = f.tile_w, tile_h = f.tile_h, tiles_x = f.tiles_x;
+    const size_t smem = 2 * (size_t)tile_w * tile_h * sizeof(double);
+    const int ppt = (tile_w * tile_h + f.block - 1) / f.block;
+    const void* kernel = ppt <= 1 ? (const void*)denoise_fused_kernel<1>
+                       : ppt <= 2 ? (const void*)denoise_fused_kernel<2> : (const void*)denoise_fused_kernel<FUSED_MAX_PPT>;
+    if (smem > 48 * 1024) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    void* args[] = {(void*)&s_hat, (void*)&s_out, (void*)&nu, (void*)&nv, (void*)&tile_w, (void*)&tile_h,
+                    (void*)&tiles_x, (void*)&count_scale, (void*)&beta, (void*)&scal_dev, (void*)&omega, (void*)&iters,
+                    (void*)&words, (void*)&status};
+    return cudaLaunchCooperativeKernel(kernel, dim3(f.grid), dim3(f.block), args, smem,
                                        stream);
 }
 
