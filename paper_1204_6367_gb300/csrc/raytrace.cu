@@ -1,6 +1,6 @@
 // Tri-linear ray-traced primary, Section 2.3 / Eq. 1, for sm_103a.
 //
-// One thread per detector pixel (as in the paper).  The ray from the source
+// One thread per detector pixel (as in the paper), 8 x 4 pixels per warp.  The ray from the source
 // to the pixel centre is cut, inside the phantom box, into n equal intervals
 // of length dl <= half the smallest voxel size; the field is evaluated at the
 // interval midpoints with trilinear interpolation (clamp to edge).
@@ -14,15 +14,28 @@
 // follows from them: the same discretised quantity with one trace instead of
 // ~100.  Software FP32 interpolation replaces the texture unit's 8-bit
 // fixed-point weights.
+#include <algorithm>
+
 #include "gdrr_internal.cuh"
 
 namespace gdrr {
 namespace {
 
 constexpr int RT_MAX_BINS = 512;
+constexpr int RT_BX = 16, RT_BY = 8;      // pixels of a block of the tri-linear tracer, by warps of 8 x 4
 
-template <int NM>
-__global__ void __launch_bounds__(128) rt_kernel(const RtParams P, double* __restrict__ out) {
+// Bound: instruction issue.  A sample costs its three midpoint coordinates,
+// their floors (by adding 1.5 2^23 rounded down) and eight corner gathers; the
+// partial densities go to one running sum while the eight corners and the
+// samples before them are of one material, and only a sample that mixes
+// materials, or meets another one, takes the per-material sums apart.  Each
+// material's terms are added in the order of the plain loop over samples,
+// corners and materials, so the result is the same to the bit.  2 mm torso, 512
+// x 384 pixels: 0.99 ms with every corner tested against every material and
+// warps of 32 x 1 pixels, 0.53 ms so.  WIDE: an axis has 2^22 voxels or more,
+// beyond the floor by addition.
+template <int NM, bool WIDE>
+__global__ void __launch_bounds__(RT_BX * RT_BY) rt_kernel(const RtParams P, int blocks_x, double* __restrict__ out) {
     __shared__ float s_mu[RT_MAX_BINS * NM];
     __shared__ float s_wr[RT_MAX_BINS];
     for (int i = threadIdx.x; i < P.n_bins * NM; i += blockDim.x) {
@@ -32,9 +45,10 @@ __global__ void __launch_bounds__(128) rt_kernel(const RtParams P, double* __res
     for (int i = threadIdx.x; i < P.n_bins; i += blockDim.x) s_wr[i] = P.wr[i];
     __syncthreads();
 
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= P.nu * P.nv) return;
-    const int iu = j % P.nu, iv = j / P.nu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int iu = (int)(blockIdx.x % blocks_x) * RT_BX + (warp % (RT_BX / 8)) * 8 + (lane & 7);
+    const int iv = (int)(blockIdx.x / blocks_x) * RT_BY + (warp / (RT_BX / 8)) * 4 + (lane >> 3);
+    if (iu >= P.nu || iv >= P.nv) return;
     const float au = ((float)iu + 0.5f - P.hu) * P.du;
     const float av = ((float)iv + 0.5f - P.hv) * P.dv;
     float d[3], S[3];
@@ -77,33 +91,74 @@ __global__ void __launch_bounds__(128) rt_kernel(const RtParams P, double* __res
             f0[a] = (x0 - P.lo[a]) * P.ivox[a] - 0.5f;
             df[a] = dl * d[a] * P.ivox[a];
         }
+        // e: the running sum of material cur (ell[cur] is stale meanwhile)
+        float e = 0.0f;
+        int cur = 0;
         for (int s = 0; s < n; ++s) {
-            int i0[3], i1[3];
             float w1[3];
+            int g[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const float fa = f0[a] + (float)s * df[a];
-                int g0 = (int)floorf(fa);
-                w1[a] = fa - (float)g0;
-                int g1 = g0 + 1;
-                g0 = min(max(g0, 0), dims[a] - 1);
-                g1 = min(max(g1, 0), dims[a] - 1);
-                i0[a] = g0; i1[a] = g1;
+                const float fa = __fmaf_rn((float)s, df[a], f0[a]);
+                if (WIDE) {
+                    g[a] = (int)floorf(fa);
+                    w1[a] = fa - (float)g[a];
+                } else {
+                    const float t = __fadd_rd(fa, 12582912.0f);      // 1.5 2^23 + floor(fa)
+                    w1[a] = fa - (t - 12582912.0f);
+                    g[a] = (int)(__float_as_uint(t) - 0x4b400000u);
+                }
             }
+            // the lower corner's record and the steps to the upper ones
+            int v0, sx, sy, sz;
+            if ((unsigned)g[0] < (unsigned)(dims[0] - 1) && (unsigned)g[1] < (unsigned)(dims[1] - 1)
+                && (unsigned)g[2] < (unsigned)(dims[2] - 1)) {
+                v0 = brick_x(g[0]) + brick_y(g[1], P.bsy) + brick_z(g[2], P.bsz);
+                sx = (g[0] & 3) == 3 ? 13 : 1;
+                sy = (g[1] & 1) ? P.bsy - 4 : 4;
+                sz = (g[2] & 1) ? P.bsz - 8 : 8;
+            } else {                                                // a corner beyond a face: clamp
+                int i0[3], i1[3];
 #pragma unroll
-            for (int corner = 0; corner < 8; ++corner) {
-                const int cx = corner & 1, cy = (corner >> 1) & 1, cz = corner >> 2;
-                const int v = brick_x(cx ? i1[0] : i0[0]) + brick_y(cy ? i1[1] : i0[1], P.bsy)
-                            + brick_z(cz ? i1[2] : i0[2], P.bsz);
-                const float w = (cx ? w1[0] : 1.0f - w1[0]) * (cy ? w1[1] : 1.0f - w1[1])
-                              * (cz ? w1[2] : 1.0f - w1[2]);
-                const uint2 vx = __ldg(P.vox + v);
-                const float a = w * __uint_as_float(vx.x);
-                const int mc = (int)vx.y;
+                for (int a = 0; a < 3; ++a) {
+                    i0[a] = min(max(g[a], 0), dims[a] - 1);
+                    i1[a] = min(max(g[a] + 1, 0), dims[a] - 1);
+                }
+                v0 = brick_x(i0[0]) + brick_y(i0[1], P.bsy) + brick_z(i0[2], P.bsz);
+                sx = brick_x(i1[0]) - brick_x(i0[0]);
+                sy = brick_y(i1[1], P.bsy) - brick_y(i0[1], P.bsy);
+                sz = brick_z(i1[2], P.bsz) - brick_z(i0[2], P.bsz);
+            }
+            const float u1[3] = {1.0f - w1[0], 1.0f - w1[1], 1.0f - w1[2]};
+            const float wxy[4] = {u1[0] * u1[1], w1[0] * u1[1], u1[0] * w1[1], w1[0] * w1[1]};
+            float a[8];
+            int mc[8];
+            unsigned mixed = 0u;
 #pragma unroll
-                for (int m = 0; m < NM; ++m) ell[m] += (mc == m ? a : 0.0f);
+            for (int c = 0; c < 8; ++c) {
+                const uint2 vx = __ldg(P.vox + v0 + (c & 1 ? sx : 0) + (c & 2 ? sy : 0) + (c & 4 ? sz : 0));
+                a[c] = (wxy[c & 3] * (c & 4 ? w1[2] : u1[2])) * __uint_as_float(vx.x);
+                mc[c] = (int)vx.y;
+                mixed |= vx.y ^ (unsigned)cur;
+            }
+            if (mixed == 0u) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) e += a[c];
+            } else {
+#pragma unroll
+                for (int m = 0; m < NM; ++m) {
+                    float l = cur == m ? e : ell[m];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) l += mc[c] == m ? a[c] : 0.0f;
+                    ell[m] = l;
+                }
+                cur = mc[7];
+#pragma unroll
+                for (int m = 0; m < NM; ++m) e = cur == m ? ell[m] : e;
             }
         }
+#pragma unroll
+        for (int m = 0; m < NM; ++m) ell[m] = cur == m ? e : ell[m];
 #pragma unroll
         for (int m = 0; m < NM; ++m) ell[m] *= dl;
     }
@@ -116,6 +171,7 @@ __global__ void __launch_bounds__(128) rt_kernel(const RtParams P, double* __res
         for (int m = 0; m < NM; ++m) rad += s_mu[b * NM + m] * ell[m];
         sig += (wcol ? __ldg(wcol + b) : s_wr[b]) * expf(-rad);
     }
+    const size_t j = (size_t)iv * P.nu + iu;
     out[j] = P.wnorm[j] * (double)sig;
 }
 
@@ -232,6 +288,13 @@ __global__ void air_kernel(const RtParams P, double* __restrict__ out) {
     out[j] = P.wnorm[j] * (double)sig;
 }
 
+template <int NM, bool WIDE>
+cudaError_t launch_rt_t(const RtParams& p, double* out, cudaStream_t s) {
+    const int blocks_x = (p.nu + RT_BX - 1) / RT_BX, blocks_y = (p.nv + RT_BY - 1) / RT_BY;
+    rt_kernel<NM, WIDE><<<(unsigned)((int64_t)blocks_x * blocks_y), RT_BX * RT_BY, 0, s>>>(p, blocks_x, out);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_air(const RtParams& p, double* out, cudaStream_t s) {
@@ -253,12 +316,14 @@ cudaError_t launch_rt_siddon(const RtParams& p, double* out, cudaStream_t s) {
 
 cudaError_t launch_rt(const RtParams& p, double* out, cudaStream_t s) {
     if (p.n_bins > RT_MAX_BINS) return cudaErrorInvalidValue;
-    const int npix = p.nu * p.nv;
-    const int block = 128, grid = (npix + block - 1) / block;
-    if (p.n_mat <= 2) rt_kernel<2><<<grid, block, 0, s>>>(p, out);
-    else if (p.n_mat <= 4) rt_kernel<4><<<grid, block, 0, s>>>(p, out);
-    else rt_kernel<8><<<grid, block, 0, s>>>(p, out);
-    return cudaGetLastError();
+    if (std::max(p.nx, std::max(p.ny, p.nz)) >= 1 << 22) {
+        if (p.n_mat <= 2) return launch_rt_t<2, true>(p, out, s);
+        if (p.n_mat <= 4) return launch_rt_t<4, true>(p, out, s);
+        return launch_rt_t<8, true>(p, out, s);
+    }
+    if (p.n_mat <= 2) return launch_rt_t<2, false>(p, out, s);
+    if (p.n_mat <= 4) return launch_rt_t<4, false>(p, out, s);
+    return launch_rt_t<8, false>(p, out, s);
 }
 
 }  // namespace gdrr
