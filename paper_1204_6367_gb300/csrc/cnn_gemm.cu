@@ -614,8 +614,23 @@ __global__ void __launch_bounds__(PERSIST_THREADS) gemm_persistent_kernel(
 // applies bias and activation and stores BF16 (optionally upsampled into the
 // next level's concatenated input, optionally with the fused 1 x 1 head) or
 // FP32.
+//
+// A CTA's tile is MT such 128-pixel subtiles, one below the other, with an
+// accumulator each: a stage then holds the MT Hb + 2 input rows that all of
+// them read and one copy of the weight slices, instead of Hb + 2 rows and the
+// weights per subtile.  The K order of every accumulator is the same for each
+// MT, so the results are too.  The epilogue reads 32 columns from TMEM while it
+// packs the 32 before, and a warp's 32 pixels leave by TMA from shared memory
+// (one copy per upsampled position).
+//
+// Bounds: copies from L2 (75 bytes per ns and SM), MMA issue of narrow outputs
+// (37 ns per 128 x 32 x 16, 44 at 64, 60 at 128 columns) and, for little work per
+// pixel, the epilogue.  64 images of 96 x 128, base 32: the five layers of the
+// forward pass took 52, 34, 69, 100 and 166 us with one subtile and an epilogue
+// that stored each lane's pixel 16 columns at a time; 23, 17, 41, 58 and 86 so.
 constexpr int CONV_BK = 32;
 constexpr int CONV_MAX_STAGES = 8;
+constexpr int CONV_MAX_WIDE = 512;     // output columns whose bias the epilogue keeps in shared memory
 
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
     uint64_t d = 0;
@@ -644,6 +659,73 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// The accumulator's next 32 columns of the warp's 32 rows (one row per lane),
+// valid after tmem_wait_load.
+__device__ __forceinline__ void tmem_load32(uint32_t (&r)[32], uint32_t addr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_load() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// What epi_store makes of 32 columns: bias, activation, BF16; and its part of
+// the fused head, the columns in order.
+__device__ __forceinline__ void epi_pack32(const uint32_t (&v)[32], const float* bias, int relu, uint4 (&o)[4]) {
+    uint32_t w[16];
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+        float lo = __uint_as_float(v[i]) + bias[i], hi = __uint_as_float(v[i + 1]) + bias[i + 1];
+        if (relu) { lo = fmaxf(lo, 0.0f); hi = fmaxf(hi, 0.0f); }
+        const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+        w[i / 2] = *reinterpret_cast<const uint32_t*>(&p);
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) o[h] = make_uint4(w[4 * h], w[4 * h + 1], w[4 * h + 2], w[4 * h + 3]);
+}
+
+__device__ __forceinline__ float epi_head32(const uint4 (&o)[4], const float* w, float head) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        const uint32_t u[4] = {o[h].x, o[h].y, o[h].z, o[h].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            head += w[8 * h + 2 * k] * __uint_as_float(u[k] << 16);
+            head += w[8 * h + 2 * k + 1] * __uint_as_float(u[k] & 0xffff0000u);
+        }
+    }
+    return head;
+}
+
+__device__ __forceinline__ void st_shared(uint32_t addr, uint4 v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, uint32_t src, int c, int dx, int x, int dy, int y) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];"
+        :: "l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c), "r"(dx), "r"(x), "r"(dy), "r"(y)
+        : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// until at most PENDING of this thread's store groups still read shared memory
+template <int PENDING>
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" :: "n"(PENDING) : "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 struct ConvGeo {
     int H, W;          // grid of the input and the output
     int Wb;            // tile width: min(W, 128); the tile has 128 / Wb rows
@@ -651,14 +733,21 @@ struct ConvGeo {
     int c32;           // C / 32
     int n_kb;          // stages per tile: 3 * c32
     int stages;        // ring depth (<= CONV_MAX_STAGES)
-    uint32_t a_bytes;  // A part of a stage: (128 + 2 Wb) rows of 64 bytes
+    uint32_t a_bytes;  // A part of a stage: (128 MT + 2 Wb) rows of 64 bytes
 };
 
-template <int BN>
+// TMEM columns of MT accumulators of BN columns, and of two sets of them where
+// they fit (one tile's epilogue then runs under the next tile's MMAs)
+template <int BN, int MT>
+__host__ __device__ constexpr int conv_bufs() { return 2 * BN * MT <= 512 ? 2 : 1; }
+__host__ __device__ constexpr int tmem_columns(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512; }
+
+template <int BN, int MT>
 __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
-        const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW, const ConvGeo g, int M,
-        int N, const ConvEpi epi, int* err) {
+        const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
+        const __grid_constant__ CUtensorMap mapY, const ConvGeo g, int M, int N, const ConvEpi epi, int wide, int* err) {
     constexpr uint32_t B_TAP = BN * CONV_BK * 2, B_BYTES = 3 * B_TAP;
+    constexpr int BUFS = conv_bufs<BN, MT>(), COLS = tmem_columns(BUFS * MT * BN);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[CONV_MAX_STAGES], empty_bar[CONV_MAX_STAGES], tfull[2], tempty[2];
     __shared__ uint32_t tmem_base;
@@ -668,12 +757,27 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
     const int stages = g.stages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_n = (N + BN - 1) / BN;
-    const int n_tiles = (M / GEMM_BM) * tiles_n;
+    const int n_tiles = (M / (GEMM_BM * MT)) * tiles_n;
+    const int tiles_x = g.W / g.Wb, sub_step = g.W > g.Wb ? g.W : GEMM_BM;   // pixels from a subtile to the next
+    // pixel tile p: its image, first row and column, first pixel
+    auto place = [&](int p, int& b, int& y0, int& x0) {
+        const int rows = MT * (GEMM_BM / g.Wb), per_image = (g.H / rows) * tiles_x;
+        b = p / per_image;
+        const int r = p - b * per_image;
+        y0 = (r / tiles_x) * rows;
+        x0 = (r % tiles_x) * g.Wb;
+    };
     const uint32_t row_bytes = (uint32_t)g.Wb * (CONV_BK * 2);     // one input row of the tile in shared memory
+    __shared__ float s_bias[CONV_MAX_WIDE], s_head[CONV_MAX_WIDE];
+    if (wide == 1)
+        for (int i = threadIdx.x; i < N; i += PERSIST_THREADS) {
+            s_bias[i] = epi.bias ? epi.bias[i] : 0.0f;
+            s_head[i] = epi.head_out ? __bfloat162float(epi.head_w[i]) : 0.0f;
+        }
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_addr(&tmem_base)), "r"((uint32_t)(2 * BN)) : "memory");
+                     :: "r"(smem_addr(&tmem_base)), "r"((uint32_t)COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 32) {
@@ -702,13 +806,12 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
     // pixel tile's input in L2)
     if (warp == 0 && lane == 0) {
         // producer: the ring's stage counter runs across tiles
-        const int hw = g.H * g.W;
         int it = 0, s = 0;
         uint32_t ph = 0;                                   // parity of the pass over the ring
         for (int t = blockIdx.x; t < n_tiles && !*(volatile int*)&s_fail; t += gridDim.x) {
-            const int m0 = (t / tiles_n) * GEMM_BM, n0 = (t % tiles_n) * BN;
-            const int b = m0 / hw, r = m0 - b * hw;
-            const int y0 = r / g.W, x0 = r - y0 * g.W;
+            int b, y0, x0;
+            place(t / tiles_n, b, y0, x0);
+            const int n0 = (t % tiles_n) * BN;
             for (int kb = 0; kb < g.n_kb; ++kb, ++it) {
                 if (it >= stages && !mbar_wait(smem_addr(&empty_bar[s]), ph ^ 1u)) {
                     atomicExch(&s_fail, 1);
@@ -729,93 +832,168 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
             const int jt = it - 1 - j;                     // one of the last `last` stages issued
             mbar_wait(smem_addr(&full_bar[jt % stages]), (uint32_t)((jt / stages) & 1));
         }
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
+    } else if (warp == 1) {
+        // MMA issuer: the whole warp walks the loop, so that the descriptors stay
+        // warp-uniform, and one elected lane issues
         constexpr uint32_t idesc = instr_desc(GEMM_BM, BN);
+        const bool leader = elect_one();
+        const uint32_t row16 = row_bytes >> 4;             // descriptor addresses count 16 bytes
         int local = 0, s = 0;
         uint32_t ph = 0;
         for (int t = blockIdx.x; t < n_tiles && !*(volatile int*)&s_fail; t += gridDim.x, ++local) {
-            const int a = local & 1;
-            if (!mbar_wait(smem_addr(&tempty[a]), (uint32_t)(((local >> 1) & 1) ^ 1))) {
-                atomicExch(&s_fail, 1);
+            const int a = local % BUFS;
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_addr(&tempty[a]), (uint32_t)(((local / BUFS) & 1) ^ 1)))) {
+                if (leader) atomicExch(&s_fail, 1);
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t acc_tmem = tmem + (uint32_t)(a * BN);
+            const uint32_t acc_tmem = tmem + (uint32_t)(a * MT * BN);
             for (int kb = 0; kb < g.n_kb; ++kb) {
-                if (!mbar_wait(smem_addr(&full_bar[s]), ph)) {
-                    atomicExch(&s_fail, 1);
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_addr(&full_bar[s]), ph))) {
+                    if (leader) atomicExch(&s_fail, 1);
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t sa = ring + (uint32_t)s * stage_bytes;
+                const uint64_t ad0 = smem_desc_sw64(sa), bd0 = smem_desc_sw64(sa + g.a_bytes);
+                if (leader) {
 #pragma unroll
-                for (int ky = 0; ky < 3; ++ky) {
+                    for (int ky = 0; ky < 3; ++ky) {
 #pragma unroll
-                    for (int kk = 0; kk < CONV_BK / 16; ++kk) {
-                        // K16 step inside the 64-byte swizzle atom: advance the start by 32 bytes
-                        const uint64_t ad = smem_desc_sw64(sa + ky * row_bytes + kk * 32);
-                        const uint64_t bd = smem_desc_sw64(sa + g.a_bytes + ky * B_TAP + kk * 32);
-                        const uint32_t acc = (kb > 0 || ky > 0 || kk > 0) ? 1u : 0u;
-                        asm volatile(
-                            "{\n\t.reg .pred p;\n\t"
-                            "setp.ne.b32 p, %4, 0;\n\t"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                            :: "r"(acc_tmem), "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                            : "memory");
+                        for (int kk = 0; kk < CONV_BK / 16; ++kk) {
+                            // K16 step inside the 64-byte swizzle atom: advance the start by 32 bytes
+                            const uint64_t ad = ad0 + (uint64_t)(ky * row16 + kk * 2);
+                            const uint64_t bd = bd0 + (uint64_t)(ky * (B_TAP >> 4) + kk * 2);
+                            const uint32_t acc = (kb > 0 || ky > 0 || kk > 0) ? 1u : 0u;
+#pragma unroll
+                            for (int j = 0; j < MT; ++j) {
+                                // subtile j's rows follow subtile j - 1's 128
+                                asm volatile(
+                                    "{\n\t.reg .pred p;\n\t"
+                                    "setp.ne.b32 p, %4, 0;\n\t"
+                                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                    :: "r"(acc_tmem + (uint32_t)(j * BN)), "l"(ad + (uint64_t)(j * (GEMM_BM * CONV_BK * 2 >> 4))),
+                                       "l"(bd), "r"(idesc), "r"(acc)
+                                    : "memory");
+                            }
+                        }
                     }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                 :: "r"(smem_addr(&empty_bar[s])) : "memory");
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(smem_addr(&empty_bar[s])) : "memory");
+                __syncwarp();
                 if (++s == stages) { s = 0; ph ^= 1u; }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_addr(&tfull[a])) : "memory");
+            if (leader)
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             :: "r"(smem_addr(&tfull[a])) : "memory");
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // epilogue
         const int q = warp & 3;                               // TMEM lane quarter of this warp
+        const uint32_t stage_out = ring + (uint32_t)stages * stage_bytes + (uint32_t)q * 8192u;
         int local = 0;
+        unsigned n_out = 0;
         for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++local) {
-            const int m0 = (t / tiles_n) * GEMM_BM, n0 = (t % tiles_n) * BN;
-            const int a = local & 1;
-            const bool got = mbar_wait(smem_addr(&tfull[a]), (uint32_t)((local >> 1) & 1));
+            int b, y0, x0;
+            place(t / tiles_n, b, y0, x0);
+            const int n0 = (t % tiles_n) * BN;
+            const int a = local % BUFS;
+            const bool got = mbar_wait(smem_addr(&tfull[a]), (uint32_t)((local / BUFS) & 1));
             const bool good = __all_sync(0xffffffffu, got) && !*(volatile int*)&s_fail;
             if (!good) {
                 if (lane == 0) atomicExch(&s_fail, 1);
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int64_t row = (int64_t)m0 + q * 32 + lane;
-            float head = 0.0f;
+            const int64_t first = ((int64_t)b * g.H + y0) * g.W + x0;
 #pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 16) {
-                uint32_t r[16];
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN + c0);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                    "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                      "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                      "=r"(r[14]), "=r"(r[15])
-                    : "r"(taddr)
-                    : "memory");
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const int col = n0 + c0;
-                if (row < M && col < N) {
-                    float v[16];
+            for (int j = 0; j < MT; ++j) {
+                const int64_t row = first + (int64_t)j * sub_step + q * 32 + lane;
+                const uint32_t lane_tmem = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((a * MT + j) * BN);
+                if (wide != 0) {
+                    // 32 columns at a time, the next ones read from TMEM while these
+                    // are staged; the warp's 32 pixels leave by TMA
+                    const int cols = min(BN, N - n0), wpx = q * 32;
+                    const int sx = x0 + wpx % g.Wb, sy = b * g.H + y0 + j * (GEMM_BM / g.Wb) + wpx / g.Wb;
+                    float head = 0.0f;
+                    uint32_t r[2][32];
+                    tmem_load32(r[0], lane_tmem);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-                    epi_store(epi, row, col, min(16, N - col), v, epi.head_out ? &head : nullptr);
+                    for (int c0 = 0; c0 < BN; c0 += 32) {
+                        if (c0 >= cols) break;
+                        tmem_wait_load();
+                        if (c0 + 32 < cols) tmem_load32(r[(c0 / 32 + 1) & 1], lane_tmem + (uint32_t)(c0 + 32));
+                        const uint32_t (&v)[32] = r[(c0 / 32) & 1];
+                        if (wide == 1) {
+                            // four 2 KB buffers of 64-byte rows (64-byte swizzle)
+                            const uint32_t to = stage_out + (n_out++ & 3u) * 2048u;
+                            if (lane == 0) bulk_wait_read<3>();
+                            __syncwarp();
+                            uint4 o[4];
+                            epi_pack32(v, s_bias + n0 + c0, epi.relu, o);
+                            if (epi.head_out) head = epi_head32(o, s_head + c0, head);
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) st_shared(to + lane * 64 + ((h ^ ((lane >> 1) & 3)) << 4), o[h]);
+                            fence_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                for (int i = 0; i < epi.up; ++i)
+                                    for (int k = 0; k < epi.up; ++k) tma_store_5d(&mapY, to, n0 + c0, k, sx, i, sy);
+                                bulk_commit();
+                            }
+                        } else {
+                            // two 4 KB buffers of 128-byte rows (128-byte swizzle)
+                            const uint32_t to = stage_out + (n_out++ & 1u) * 4096u;
+                            if (lane == 0) bulk_wait_read<1>();
+                            __syncwarp();
+#pragma unroll
+                            for (int h = 0; h < 8; ++h)
+                                st_shared(to + lane * 128 + ((h ^ (lane & 7)) << 4),
+                                          make_uint4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]));
+                            fence_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                tma_store_5d(&mapY, to, n0 + c0, 0, sx, 0, sy);
+                                bulk_commit();
+                            }
+                        }
+                    }
+                    if (epi.head_out) epi_head(epi, row, head);
+                    continue;
                 }
+                float head = 0.0f;
+#pragma unroll 1
+                for (int c0 = 0; c0 < BN; c0 += 16) {
+                    uint32_t r[16];
+                    const uint32_t taddr = lane_tmem + (uint32_t)c0;
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+                          "=r"(r[14]), "=r"(r[15])
+                        : "r"(taddr)
+                        : "memory");
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const int col = n0 + c0;
+                    if (row < M && col < N) {
+                        float v[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+                        epi_store(epi, row, col, min(16, N - col), v, epi.head_out ? &head : nullptr);
+                    }
+                }
+                if (epi.head_out && row < M) epi_head(epi, row, head);
             }
-            if (epi.head_out && row < M) epi_head(epi, row, head);
             // this warp's TMEM reads are done: release the accumulator
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_addr(&tempty[a])) : "memory");
         }
+        if (lane == 0) bulk_wait_all();                       // the stores are done before the block leaves
     }
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -823,7 +1001,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
     if (threadIdx.x == 0 && *(volatile int*)&s_fail) atomicExch(err, 1);
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     :: "r"(tmem), "r"((uint32_t)(2 * BN)) : "memory");
+                     :: "r"(tmem), "r"((uint32_t)COLS) : "memory");
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -854,24 +1032,75 @@ bool make_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int b
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
-cudaError_t launch_conv_t(const CUtensorMap& mX, const CUtensorMap& mW, ConvGeo g, int M, int N, const ConvEpi& epi,
-                          int* err, cudaStream_t s) {
-    // the deepest ring that fits 216 KB of shared memory
-    const uint32_t stage = g.a_bytes + 3u * BN * CONV_BK * 2;
-    g.stages = (int)std::min<uint32_t>(CONV_MAX_STAGES, (216u * 1024u) / stage);
+// Shared-memory bytes of a stage and the ring's depth (184 KB at most, beside
+// the epilogue's 32 KB of staged output: a store waits behind the loads that
+// the TMA unit has queued, so several are under way).
+constexpr uint32_t CONV_RING = 184u * 1024u, CONV_OUT = 32u * 1024u;
+uint32_t conv_a_bytes(int Wb, int mt) { return (uint32_t)(GEMM_BM * mt + 2 * Wb) * (CONV_BK * 2); }
+int conv_stages(int Wb, int BN, int mt) {
+    return (int)std::min<uint32_t>(CONV_MAX_STAGES, CONV_RING / (conv_a_bytes(Wb, mt) + 3u * BN * CONV_BK * 2));
+}
+
+// Subtiles per tile: of the counts that divide an image's rows and whose
+// accumulators fit TMEM, the one with the least estimated time, in cycles: the
+// passes of n_sm tiles, each its stages' longer one of copies (39 bytes per SM
+// and cycle) and MMAs (60 + 0.45 N cycles), but no less than its epilogue (900
+// cycles per 32 columns and subtile), which adds to it where a second set of
+// accumulators does not fit to hide it.  The four rates reproduce the measured
+// times of every layer of the estimator at batches 16 and 64 for one to four
+// subtiles to 15 %.
+int conv_subtiles(int M, int H, int Wb, int tiles_n, int BN, int n_kb, int n_sm) {
+    int best = 1;
+    double least = 0.0;
+    for (int mt = 1; mt <= 4; ++mt) {
+        const int rows = mt * (GEMM_BM / Wb);
+        if (mt > 1 && (Wb < 8 || H % rows || mt * BN > 512 || conv_stages(Wb, BN, mt) < 2)) continue;
+        const int64_t tiles = (int64_t)(M / (GEMM_BM * mt)) * tiles_n;
+        const double work = n_kb * std::max((conv_a_bytes(Wb, mt) + 3.0 * BN * CONV_BK * 2) / 39.0, mt * 6.0 * (60.0 + 0.45 * BN));
+        const double out = mt * (BN / 32) * 900.0;
+        const double t = (double)((tiles + n_sm - 1) / n_sm) * (2 * mt * BN <= 512 ? std::max(work, out) : work + out);
+        if (mt == 1 || t < least) {
+            least = t;
+            best = mt;
+        }
+    }
+    return best;
+}
+
+// The convolution's tensor maps: input, weights, output (with wide != 0: 1
+// BF16, 2 FP32 without bias, 32 columns at a time; 0: stored column by column
+// by epi_store).
+struct ConvMaps {
+    CUtensorMap x, w, y;
+    int wide;
+};
+
+template <int BN, int MT>
+cudaError_t launch_conv_t(const ConvMaps& m, ConvGeo g, int M, int N, const ConvEpi& epi, int n_sm, int* err,
+                          cudaStream_t s) {
+    g.a_bytes = conv_a_bytes(g.Wb, MT);
+    g.stages = conv_stages(g.Wb, BN, MT);
     if (g.stages < 2) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)g.stages * stage + 1024;
-    cudaError_t e = cudaFuncSetAttribute(conv_implicit_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = (size_t)g.stages * (g.a_bytes + 3u * BN * CONV_BK * 2) + CONV_OUT + 1024;
+    cudaError_t e = cudaFuncSetAttribute(conv_implicit_kernel<BN, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, n_sm = 1;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int64_t n_tiles = (int64_t)(M / GEMM_BM) * ((N + BN - 1) / BN);
+    const int64_t n_tiles = (int64_t)(M / (GEMM_BM * MT)) * ((N + BN - 1) / BN);
     const int grid = (int)std::min<int64_t>(n_tiles, n_sm);
-    conv_implicit_kernel<BN><<<grid, PERSIST_THREADS, smem, s>>>(mX, mW, g, M, N, epi, err);
+    conv_implicit_kernel<BN, MT><<<grid, PERSIST_THREADS, smem, s>>>(m.x, m.w, m.y, g, M, N, epi, m.wide, err);
     return cudaGetLastError();
+}
+
+template <int BN>
+cudaError_t launch_conv_bn(int mt, const ConvMaps& m, const ConvGeo& g, int M, int N, const ConvEpi& epi, int n_sm,
+                           int* err, cudaStream_t s) {
+    switch (mt) {
+        case 1: return launch_conv_t<BN, 1>(m, g, M, N, epi, n_sm, err, s);
+        case 2: return launch_conv_t<BN, 2>(m, g, M, N, epi, n_sm, err, s);
+        case 3: if constexpr (BN <= 128) return launch_conv_t<BN, 3>(m, g, M, N, epi, n_sm, err, s); break;
+        case 4: if constexpr (BN <= 128) return launch_conv_t<BN, 4>(m, g, M, N, epi, n_sm, err, s); break;
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int BN, int STAGES>
@@ -933,7 +1162,7 @@ cudaError_t launch_gemm_t(const __nv_bfloat16* A, int lda, const __nv_bfloat16* 
 }  // namespace
 
 // The implicit-GEMM convolution: tensor maps of the NHWC input (box 32
-// channels x Wb pixels x (128 / Wb + 2) rows, 64-byte swizzle, zero fill
+// channels x Wb pixels x (MT 128 / Wb + 2) rows, 64-byte swizzle, zero fill
 // outside) and of the ky-major weights [ky][N][kx C + c] (box 32 x BN x 3),
 // then the persistent kernel with the narrowest output tile that covers N
 // (N > 256: column tiles of 128 or 256).
@@ -944,29 +1173,63 @@ cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
     if (!fn) return cudaErrorNotSupported;
     const int wb = a.W >= GEMM_BM ? GEMM_BM : a.W, hb = GEMM_BM / wb;
-    CUtensorMap mX, mW;
+    const int64_t M = (int64_t)a.B * a.H * a.W;
+    if (M % GEMM_BM || M > INT32_MAX) return cudaErrorInvalidValue;
+    const int BN = a.N <= 32 ? 32 : a.N <= 64 ? 64 : a.N <= 128 ? 128 : a.N <= 256 ? 256 : (a.N % 128 == 0 ? 128 : 256);
+    if (a.epi.head_out && (a.N > BN || !a.epi.y16)) return cudaErrorInvalidValue;
+    int dev = 0, n_sm = 1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int mt = conv_subtiles((int)M, a.H, wb, (a.N + BN - 1) / BN, BN, 3 * (a.C / CONV_BK), n_sm);
+    ConvMaps m;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
         const cuuint64_t px = (cuuint64_t)a.ldx * 2;
         const cuuint64_t strides[3] = {px, px * a.W, px * a.W * a.H};
-        const cuuint32_t box[4] = {(cuuint32_t)CONV_BK, (cuuint32_t)wb, (cuuint32_t)(hb + 2), 1};
+        const cuuint32_t box[4] = {(cuuint32_t)CONV_BK, (cuuint32_t)wb, (cuuint32_t)(mt * hb + 2), 1};
         const cuuint32_t elem[4] = {1, 1, 1, 1};
-        if (fn(&mX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(a.x), dims, strides, box, elem,
+        if (fn(&m.x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(a.x), dims, strides, box, elem,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    const int BN = a.N <= 32 ? 32 : a.N <= 64 ? 64 : a.N <= 128 ? 128 : a.N <= 256 ? 256 : (a.N % 128 == 0 ? 128 : 256);
-    if (a.epi.head_out && (a.N > BN || !a.epi.y16)) return cudaErrorInvalidValue;
     {
         // w3[ky][n][kx C + c]
         const cuuint64_t dims[3] = {(cuuint64_t)(3 * a.C), (cuuint64_t)a.N, 3};
         const cuuint64_t strides[2] = {(cuuint64_t)(3 * a.C) * 2, (cuuint64_t)a.N * (3 * a.C) * 2};
         const cuuint32_t box[3] = {(cuuint32_t)CONV_BK, (cuuint32_t)BN, 3};
         const cuuint32_t elem[3] = {1, 1, 1};
-        if (fn(&mW, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(a.w3), dims, strides, box, elem,
+        if (fn(&m.w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(a.w3), dims, strides, box, elem,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    m.wide = 0;
+    m.y = m.x;
+    const ConvEpi& epi = a.epi;
+    if (a.N % 32 == 0 && a.N <= CONV_MAX_WIDE && wb >= 8) {      // (below, a ring stage is not a multiple of 1024 bytes)
+        if (epi.y16 && !epi.yf && epi.ldy % 8 == 0 && epi.off % 8 == 0 && (reinterpret_cast<uintptr_t>(epi.y16) & 15u) == 0)
+            m.wide = 1;
+        else if (epi.yf && !epi.y16 && !epi.bias && !epi.head_out && epi.ldf % 4 == 0
+                 && (reinterpret_cast<uintptr_t>(epi.yf) & 15u) == 0)
+            m.wide = 2;
+    }
+    if (m.wide) {
+        // columns; the copies of an upsampled pixel along x; x; their rows; rows
+        // of all images.  Box: 32 columns of a warp's 32 pixels.
+        const bool half = m.wide == 1;
+        const cuuint64_t up = half ? (cuuint64_t)epi.up : 1u;
+        const cuuint64_t px = half ? (cuuint64_t)epi.ldy * 2 : (cuuint64_t)epi.ldf * 4, line = px * up * (cuuint64_t)a.W;
+        const cuuint64_t dims[5] = {(cuuint64_t)a.N, up, (cuuint64_t)a.W, up, (cuuint64_t)a.B * a.H};
+        const cuuint64_t strides[4] = {px, px * up, line, line * up};
+        const cuuint32_t bw = (cuuint32_t)std::min(wb, 32);
+        const cuuint32_t box[5] = {32, 1, bw, 1, 32 / bw};
+        const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
+        void* base = half ? static_cast<void*>(epi.y16 + epi.off) : static_cast<void*>(epi.yf);
+        if (fn(&m.y, half ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, base, dims, strides, box,
+               elem, CU_TENSOR_MAP_INTERLEAVE_NONE, half ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
     ConvGeo g;
@@ -977,14 +1240,12 @@ cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s) {
     g.c32 = a.C / CONV_BK;
     g.n_kb = 3 * g.c32;
     g.stages = 0;
-    g.a_bytes = (uint32_t)(wb * (hb + 2)) * (CONV_BK * 2);
-    const int64_t M = (int64_t)a.B * a.H * a.W;
-    if (M % GEMM_BM || M > INT32_MAX) return cudaErrorInvalidValue;
+    g.a_bytes = 0;
     switch (BN) {
-        case 32: return launch_conv_t<32>(mX, mW, g, (int)M, a.N, a.epi, err, s);
-        case 64: return launch_conv_t<64>(mX, mW, g, (int)M, a.N, a.epi, err, s);
-        case 128: return launch_conv_t<128>(mX, mW, g, (int)M, a.N, a.epi, err, s);
-        default: return launch_conv_t<256>(mX, mW, g, (int)M, a.N, a.epi, err, s);
+        case 32: return launch_conv_bn<32>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
+        case 64: return launch_conv_bn<64>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
+        case 128: return launch_conv_bn<128>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
+        default: return launch_conv_bn<256>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
     }
 }
 
