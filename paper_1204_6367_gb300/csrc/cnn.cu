@@ -51,6 +51,7 @@ cudaError_t launch_gemm_bf16(const void* A, int lda, const void* B, int ldb, flo
 namespace {
 
 typedef __nv_bfloat16 bf16;
+
 constexpr int TB = 256;
 inline int nblk(int64_t n) { return (int)((n + TB - 1) / TB); }
 inline int pad64(int64_t n) { return (int)((n + 63) / 64 * 64); }
@@ -72,17 +73,6 @@ __device__ __forceinline__ int64_t view_pixel(const View& v, int64_t p, int H, i
     const int y = r / W, x = r - y * W;
     const int s = v.up;
     return (b * H * s + (int64_t)y * s) * ((int64_t)W * s) + (int64_t)x * s;
-}
-
-// x[b][2][H][W] (FP32 NCHW) -> BF16 NHWC [b][H][W][2]
-__global__ void to_nhwc2_kernel(const float* __restrict__ x, int64_t P, int HW, bf16* __restrict__ y) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const int64_t b = p / HW, r = p % HW;
-    __nv_bfloat162 v;
-    v.x = __float2bfloat16_rn(x[(b * 2) * HW + r]);
-    v.y = __float2bfloat16_rn(x[(b * 2 + 1) * HW + r]);
-    reinterpret_cast<__nv_bfloat162*>(y)[p] = v;
 }
 
 // Column matrix rows: cols[p][k] (row K9p), k = tap C + c (tap = ky ks +
@@ -197,54 +187,118 @@ __global__ void im2col_t_any_kernel(const View X, int C, int B, int H, int W, in
     out[i] = v;
 }
 
-// A 3 x 3 convolution of an input with few channels (CI <= 4), computed
-// directly: one thread per output pixel loads its 9 CI input values once and
-// accumulates 16 output channels at a time in FP32 over k = tap CI + c in
-// order, with the weights w[co][k] (row ldw) from shared memory transposed
-// to [k][co] (16-byte loads of four channels).
-template <int CI>
-__global__ void __launch_bounds__(128) conv_small_kernel(const View X, int B, int H, int W,
-                                                         const bf16* __restrict__ w, int ldw, int N,
-                                                         const ConvEpi epi) {
-    constexpr int K = 9 * CI;
-    __shared__ __align__(16) float sw[K * 64];
-    const int Np = (N + 15) / 16 * 16;
-    for (int i = threadIdx.x; i < K * Np; i += blockDim.x) {
-        const int k = i / Np, co = i - k * Np;
-        sw[i] = co < N ? __bfloat162float(w[co * ldw + k]) : 0.0f;
+// The network's first layer with what stands beside it: the FP32 input [b][2][H][W]
+// rounded to BF16 (and kept as x16 [b][H][W][2] for the backward pass), its 3 x 3
+// convolution into N channels (bias, ReLU, BF16, at y, pixel pitch ldy), and
+// the 2 x 2 average of that output (yp [b][H/2][W/2][N]).  One thread per 2 x 2
+// block of pixels: a weight read from shared memory serves four pixels, and the
+// average needs no second pass over the output.  The outputs are staged per
+// warp and leave with neighbouring lanes on a pixel's neighbouring channels
+// (stored by the thread that made them, 16 bytes per lane and pixel, they took
+// half of the time).  Each output adds its 18 products in FP32 over k = 2 tap +
+// channel in order, two channels per instruction (fma.rn.f32x2).  H and W even,
+// N a multiple of 8, at most 64.
+//
+// Bound: the latency of few resident warps (12 us of FMAs); 64 images of 96 x
+// 128, 32 channels: 86 us as three kernels with a pixel per thread, 39 us so.
+constexpr int FIRST_WARPS = 4;
+inline size_t first_layer_smem(int N) { return 18 * 64 * 4 + 64 * 4 + (size_t)FIRST_WARPS * 160 * (2 * N + 16); }
+
+__global__ void __launch_bounds__(32 * FIRST_WARPS) first_layer_kernel(const float* __restrict__ x, int B, int H, int W,
+                                                                       const bf16* __restrict__ w, int ldw,
+                                                                       const float* __restrict__ bias, int N,
+                                                                       bf16* __restrict__ x16, bf16* __restrict__ y,
+                                                                       int ldy, bf16* __restrict__ yp) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    float* sw = reinterpret_cast<float*>(sm);                  // [18][N]
+    float* sb = sw + 18 * 64;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pitch = 2 * N + 16, octs = N / 8;
+    uint8_t* out = sm + 18 * 64 * 4 + 64 * 4 + warp * 160 * pitch;   // rows: 4 x 32 pixels, then 32 averages
+    for (int i = threadIdx.x; i < 18 * N; i += blockDim.x) {
+        const int k = i / N, co = i - k * N;
+        sw[i] = __bfloat162float(w[co * ldw + k]);
     }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) sb[i] = bias[i];
     __syncthreads();
-    const int64_t P = (int64_t)B * H * W;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const int HW = H * W;
-    const int b = (int)(p / HW), r = (int)(p - (int64_t)b * HW), y = r / W, x = r - y * W;
-    float xin[K];
+    const int h2 = H / 2, w2 = W / 2;
+    const int64_t n = (int64_t)B * h2 * w2, first = ((int64_t)blockIdx.x * FIRST_WARPS + warp) * 32;
+    const int64_t i = min(first + lane, n - 1);                // the lanes beyond the last block repeat it
+    const int b = (int)(i / (h2 * w2)), r = (int)(i - (int64_t)b * h2 * w2), y0 = r / w2 * 2, x0 = r % w2 * 2;
+    // the 4 x 4 window, all loads under way at once: clamped, then zeroed outside
+    float in[4][4][2];
+    const float* xb = x + (int64_t)b * 2 * H * W;
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-        const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-        const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
-        const bf16* src = X.p + (((int64_t)b * H + yy) * W + xx) * X.ld + X.off;
+    for (int dy = 0; dy < 4; ++dy)
 #pragma unroll
-        for (int c = 0; c < CI; ++c) xin[tap * CI + c] = in ? __bfloat162float(src[c]) : 0.0f;
+        for (int dx = 0; dx < 4; ++dx) {
+            const int o = min(max(y0 + dy - 1, 0), H - 1) * W + min(max(x0 + dx - 1, 0), W - 1);
+            in[dy][dx][0] = __ldg(xb + o);
+            in[dy][dx][1] = __ldg(xb + (int64_t)H * W + o);
+        }
+#pragma unroll
+    for (int dy = 0; dy < 4; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 4; ++dx) {
+            const bool ok = (unsigned)(y0 + dy - 1) < (unsigned)H && (unsigned)(x0 + dx - 1) < (unsigned)W;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) in[dy][dx][c] = ok ? __bfloat162float(__float2bfloat16_rn(in[dy][dx][c])) : 0.0f;
+        }
+    const int p0 = (b * H + y0) * W + x0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        __nv_bfloat162 v;
+        v.x = __float2bfloat16_rn(in[1 + (q >> 1)][1 + (q & 1)][0]);
+        v.y = __float2bfloat16_rn(in[1 + (q >> 1)][1 + (q & 1)][1]);
+        reinterpret_cast<__nv_bfloat162*>(x16)[p0 + (q >> 1) * W + (q & 1)] = v;
     }
-    for (int c0 = 0; c0 < N; c0 += 16) {
-        float acc[16];
+    for (int c0 = 0; c0 < N; c0 += 8) {
+        uint64_t acc[4][4];                                    // pixel, pair of channels
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = 0.0f;
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const float4* wk = reinterpret_cast<const float4*>(sw + k * Np + c0);
+            for (int j = 0; j < 4; ++j) acc[q][j] = 0ull;
+#pragma unroll
+        for (int k = 0; k < 18; ++k) {
+            const ulonglong2* wk = reinterpret_cast<const ulonglong2*>(sw + k * N + c0);
+            const ulonglong2 wa = wk[0], wb = wk[1];
+            const int ky = k / 6, kx = k / 2 % 3, c = k & 1;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float4 w4 = wk[q];
-                acc[4 * q] += xin[k] * w4.x;
-                acc[4 * q + 1] += xin[k] * w4.y;
-                acc[4 * q + 2] += xin[k] * w4.z;
-                acc[4 * q + 3] += xin[k] * w4.w;
+                const uint64_t v = twice(in[(q >> 1) + ky][(q & 1) + kx][c]);
+                acc[q][0] = fma2(v, wa.x, acc[q][0]);
+                acc[q][1] = fma2(v, wa.y, acc[q][1]);
+                acc[q][2] = fma2(v, wb.x, acc[q][2]);
+                acc[q][3] = fma2(v, wb.y, acc[q][3]);
             }
         }
-        epi_store(epi, p, c0, min(16, N - c0), acc);
+        float f[4][8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 t = unpack2(acc[q][j]);
+                f[q][2 * j] = __bfloat162float(__float2bfloat16_rn(fmaxf(t.x + sb[c0 + 2 * j], 0.0f)));
+                f[q][2 * j + 1] = __bfloat162float(__float2bfloat16_rn(fmaxf(t.y + sb[c0 + 2 * j + 1], 0.0f)));
+            }
+        __align__(16) bf16 o[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[j] = __float2bfloat16_rn(f[q][j]);
+            *reinterpret_cast<uint4*>(out + (q * 32 + lane) * pitch + 2 * c0) = *reinterpret_cast<const uint4*>(o);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) o[j] = __float2bfloat16_rn(0.25f * ((f[0][j] + f[1][j]) + (f[2][j] + f[3][j])));
+        *reinterpret_cast<uint4*>(out + (128 + lane) * pitch + 2 * c0) = *reinterpret_cast<const uint4*>(o);
+    }
+    __syncwarp();
+    for (int e = lane; e < 160 * octs; e += 32) {              // 160 octs is a multiple of 32: whole warps
+        const int row = e / octs, ch = e - row * octs, l = row & 31, q = row >> 5;
+        const int p = __shfl_sync(0xffffffffu, p0, l);
+        const uint4 v = *reinterpret_cast<const uint4*>(out + row * pitch + 16 * ch);
+        if (first + l >= n) continue;
+        bf16* to = q < 4 ? y + (int64_t)(p + (q >> 1) * W + (q & 1)) * ldy : yp + (first + l) * N;
+        *reinterpret_cast<uint4*>(to + 8 * ch) = v;
     }
 }
 
@@ -662,8 +716,7 @@ ConvEpi epi_f32(float* y, int ld, int H, int W) {
 
 // One convolution on the grid H x W of the plain NHWC input X (C channels)
 // into N output columns through epi: the implicit GEMM (ky-major weights w3)
-// where the grid tiles, a direct kernel for inputs of at most 4 channels,
-// else a column matrix (row K9p), the column-path GEMM with w (row ldw, K =
+// where the grid tiles, else a column matrix (row K9p), the column-path GEMM with w (row ldw, K =
 // (tap, c)) into n->gemm and the elementwise epilogue.
 cudaError_t conv_product(gdrr_cnn* n, const View& X, int C, int B, int H, int W, int ks, const bf16* w, int ldw,
                          const bf16* w3, int N, const ConvEpi& epi) {
@@ -675,16 +728,6 @@ cudaError_t conv_product(gdrr_cnn* n, const View& X, int C, int B, int H, int W,
         a.w3 = w3; a.N = N;
         a.epi = epi;
         return launch_conv_implicit(a, n->err, n->stream);
-    }
-    if (ks == 3 && C <= 4 && N <= 64) {
-        const unsigned g = (unsigned)((P + 127) / 128);
-        switch (C) {
-            case 1: conv_small_kernel<1><<<g, 128, 0, n->stream>>>(X, B, H, W, w, ldw, N, epi); break;
-            case 2: conv_small_kernel<2><<<g, 128, 0, n->stream>>>(X, B, H, W, w, ldw, N, epi); break;
-            case 3: conv_small_kernel<3><<<g, 128, 0, n->stream>>>(X, B, H, W, w, ldw, N, epi); break;
-            default: conv_small_kernel<4><<<g, 128, 0, n->stream>>>(X, B, H, W, w, ldw, N, epi); break;
-        }
-        return cudaGetLastError();
     }
     const int K9p = pad64((int64_t)ks * ks * C);
     im2col_nhwc_kernel<<<nblk(P * (K9p / 8)), TB, 0, n->stream>>>(X, C, B, H, W, ks, K9p, n->cols);
@@ -902,11 +945,14 @@ GDRR_API int gdrr_cnn_forward(gdrr_cnn* n, int32_t batch, const float* in_dev, f
     };
     const float* P = n->params;
     do {
-        to_nhwc2_kernel<<<nblk(s1), TB, 0, st>>>(in_dev, s1, H * W, n->x16);
-        if ((e = cudaGetLastError())) break;
         // encoder: e1 -> cat1[2c..3c), e2 -> cat2[4c..6c), e3 -> cat3[8c..12c), e4 -> cat3[0..8c) upsampled
-        if ((e = conv(0, plain(n->x16, 2), epi_bf16(P + L[0].b_off, 1, n->cat1, 3 * c, 2 * c, 1, H, W)))) break;
-        if ((e = pool(plain(n->cat1, 3 * c, 2 * c), c, H, W, n->p1))) break;
+        if ((e = cudaFuncSetAttribute(first_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)first_layer_smem(c))))
+            break;
+        first_layer_kernel<<<(unsigned)((s1 / 4 + 32 * FIRST_WARPS - 1) / (32 * FIRST_WARPS)), 32 * FIRST_WARPS,
+                             first_layer_smem(c), st>>>(
+            in_dev, B, H, W, L[0].w16, L[0].K9p, P + L[0].b_off, c, n->x16, n->cat1 + 2 * c, 3 * c, n->p1);
+        if ((e = cudaGetLastError())) break;
         if ((e = conv(1, plain(n->p1, c), epi_bf16(P + L[1].b_off, 1, n->cat2, 6 * c, 4 * c, 1, H / 2, W / 2)))) break;
         if ((e = pool(plain(n->cat2, 6 * c, 4 * c), 2 * c, H / 2, W / 2, n->p2))) break;
         if ((e = conv(2, plain(n->p2, 2 * c), epi_bf16(P + L[2].b_off, 1, n->cat3, 12 * c, 8 * c, 1, H / 4, W / 4))))

@@ -77,22 +77,6 @@ inline FilterShape filter_shape(int nu) {
 
 inline size_t filter_smem(const FilterShape& f) { return sizeof(float) * ((size_t)2 * f.rows * f.stride + 2 * f.tab); }
 
-__device__ __forceinline__ uint64_t twice(float v) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
-    return r;
-}
-
 __global__ void __launch_bounds__(FILTER_BLOCK, 3) fdk_filter_kernel(const FilterParams p, const FilterShape f,
                                                                     int64_t n_rows, const float* __restrict__ g,
                                                                     float* __restrict__ out) {

@@ -181,6 +181,23 @@ struct RtParams {
 // blocks (of `block` threads) per SM.
 cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
                       cudaStream_t s);
+// Packed FP32 pairs: each half is its own IEEE-rounded FMA.
+__device__ __forceinline__ uint64_t twice(float v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
 // Page-locked host blocks, kept on a free list of the process for reuse (p is
 // NULL when there is no memory); the device reads and writes them in place.
 // gdrr_release_memory frees the list.
