@@ -169,6 +169,7 @@ struct BpParams {
     float d_beta;
     int n_ang;
     int accumulate;          // 1: add to the volume, 0: overwrite it
+    int unchecked;           // 1: a view's rows and samples can be counted by the unchecked taps
     float2 cs[BP_MAX_ANGLES];   // (cos phi, sin phi) of each view
     int first_view;          // index of cs[0] in the filtered stack
 };
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(BP_BX * BP_BY, 4) fdk_backproject_kernel(const
         const float wu0 = 1.0f - wu;
         const float v_lo = z_lo * sv + p.hv, v_hi = z_hi * sv + p.hv;
         if (v_hi <= -1.0f || v_lo >= (float)p.nv) continue;        // its voxels miss the detector
-        if (iu >= 0 && iu < p.nu - 1 && v_lo >= 0.0f && v_hi < (float)(p.nv - 1)) {
+        if (p.unchecked && iu >= 0 && iu < p.nu - 1 && v_lo >= 0.0f && v_hi < (float)(p.nv - 1)) {
             // 0x4b000000 + iv is the bit pattern of 2^23 + iv
             const uint32_t nu = (uint32_t)p.nu, first = (uint32_t)iu - 0x4b000000u * nu;
 #pragma unroll
@@ -446,6 +447,7 @@ extern "C" GDRR_API int gdrr_fdk_backproject(const gdrr_fdk_geometry* g, int32_t
     p.hu = (float)(0.5 * g->nu - 0.5);
     p.hv = (float)(0.5 * g->nv - 0.5);
     p.d_beta = (float)d_beta;
+    p.unchecked = g->nv < (1 << 22) && (int64_t)g->nu * g->nv < ((int64_t)1 << 31) ? 1 : 0;
     const int block = gdrr::BP_BX * gdrr::BP_BY;
     const dim3 grid((unsigned)((g->nx + gdrr::BP_BX - 1) / gdrr::BP_BX), (unsigned)((g->ny + gdrr::BP_BY - 1) / gdrr::BP_BY),
                     (unsigned)((g->nz + gdrr::BP_ZT - 1) / gdrr::BP_ZT));
