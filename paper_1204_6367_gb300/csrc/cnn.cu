@@ -348,8 +348,8 @@ inline int act_tile(int co) { return co >= 256 ? 16 : (co >= 128 ? 32 : 64); }
 
 // dZ = dY * (Y > 0) (or dY when relu == 0) for a block of pt pixels (a
 // multiple of 16, at most 64) and all Co channels: BF16 NHWC dz16[p][c] (the
-// data gradient's convolution input), BF16 channel-major dz_cp[c][p] (row
-// ldp; the weight gradient's operand, zero for P <= p < ldp) through a
+// gradients' operand), where dz_cp != NULL BF16 channel-major dz_cp[c][p] (row
+// ldp; the column form's operand, zero for P <= p < ldp) through a
 // shared-memory transpose, and the block's FP32 bias-gradient part
 // part[block][c] (its pt pixels added in order).
 __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__ dy, const View Y, int H, int W,
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__
                 const float gg = (relu && !(yv[u] > 0.0f)) ? 0.0f : g[u];
                 if (p0 + px < P) dz16[p0 * Co + i] = __float2bfloat16_rn(gg);
                 sf[px * (Co + 1) + c] = gg;
-                sb[c * sp + px] = __float2bfloat16_rn(gg);
+                if (dz_cp) sb[c * sp + px] = __float2bfloat16_rn(gg);
             }
         }
     }
@@ -400,6 +400,7 @@ __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__
         for (int px = 0; px < pt; ++px) s += sf[px * (Co + 1) + c];
         part[(int64_t)blockIdx.x * Co + c] = s;
     }
+    if (!dz_cp) return;
     const int segs = pt / 8;
     for (int i = threadIdx.x; i < Co * segs; i += blockDim.x) {
         const int c = i / segs, seg = i - c * segs;
@@ -594,6 +595,19 @@ __global__ void unpad_kernel(const float* __restrict__ GT, int Co, int Ci, int k
     dw[i] = GT[((int64_t)tap * Ci + ci) * Co + co];
 }
 
+// dW[co][ci][tap] from the implicit form's partial products p[z][(tap, ci)][co],
+// added in the order z = 0, 1, ...
+__global__ void wgrad_sum_kernel(const float* __restrict__ p, int n_splits, int Co, int Ci, float* __restrict__ dw) {
+    const int64_t n = (int64_t)9 * Ci * Co;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float s = 0.0f;
+#pragma unroll 8
+    for (int z = 0; z < n_splits; ++z) s += p[(int64_t)z * n + i];
+    const int r = (int)(i / Co), co = (int)(i - (int64_t)r * Co), tap = r / Ci, ci = r - tap * Ci;
+    dw[((int64_t)co * Ci + ci) * 9 + tap] = s;
+}
+
 // out[i] = sum over z of p[z * stride + i], in the order z = 0, 1, ...
 __global__ void splits_sum_kernel(const float* __restrict__ p, int n_splits, int64_t stride, float* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -741,25 +755,12 @@ cudaError_t conv_product(gdrr_cnn* n, const View& X, int C, int B, int H, int W,
     return cudaGetLastError();
 }
 
-// Backward of one 3 x 3 convolution L on the grid H x W: dy (FP32 [P][co],
-// gradient of the layer output), Y (view of its BF16 output, for the ReLU
-// mask), X (its plain NHWC input, ci channels).  Writes the parameter
-// gradients and, when dx != NULL, dx (FP32 [P][ci]).
-cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const float* dy, const View& Y, const View& X,
-                          float* dx) {
+// The weight gradient through a transposed column matrix (layers the implicit
+// form does not take): dW[co][k] = sum_p dZ[p][co] cols[p][k].
+cudaError_t wgrad_columns(gdrr_cnn* n, const Conv& L, int B, const View& X) {
     const int64_t P = (int64_t)B * L.H * L.W;
     const int Pp = pad64(P);
     cudaStream_t st = n->stream;
-    const int pt = act_tile(L.co);
-    const int n_blk = (int)((P + pt - 1) / pt);
-    const size_t smem = (size_t)pt * (L.co + 1) * 4 + (size_t)L.co * (pt + 8) * 2;
-    CK(cudaFuncSetAttribute(act_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    act_back_kernel<<<n_blk, TB, smem, st>>>(dy, Y, L.H, L.W, P, L.co, L.relu, pt, n->dz16, n->dz_cp, Pp,
-                                             n->partials);
-    CK(cudaGetLastError());
-    parts_sum_kernel<<<L.co, 256, 0, st>>>(n->partials, n_blk, L.co, n->grads + L.b_off);
-    CK(cudaGetLastError());
-    // weight gradient: dW[co][k] = sum_p dZ[p][co] cols[p][k]
     if (L.ci % 32 == 0 && L.ks == 3 && X.up == 1 && X.ld % 8 == 0 && X.off % 8 == 0) {
         im2col_t_kernel<<<dim3((unsigned)(Pp / CT_PIX), (unsigned)(L.ci / 32)), TB, 0, st>>>(X, L.ci, B, L.H, L.W, Pp,
                                                                                             n->cols);
@@ -784,6 +785,40 @@ cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const float* dy, co
     }
     unpad_kernel<<<nblk((int64_t)L.co * L.K9), TB, 0, st>>>(n->gemm, L.co, L.ci, L.ks * L.ks, n->grads + L.w_off);
     CK(cudaGetLastError());
+    return cudaSuccess;
+}
+
+// Backward of one 3 x 3 convolution L on the grid H x W: dy (FP32 [P][co],
+// gradient of the layer output), Y (view of its BF16 output, for the ReLU
+// mask), X (its plain NHWC input, ci channels).  Writes the parameter
+// gradients and, when dx != NULL, dx (FP32 [P][ci]).
+cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const float* dy, const View& Y, const View& X,
+                          float* dx) {
+    const int64_t P = (int64_t)B * L.H * L.W;
+    const int Pp = pad64(P);
+    cudaStream_t st = n->stream;
+    const int pt = act_tile(L.co);
+    const int n_blk = (int)((P + pt - 1) / pt);
+    // the implicit weight gradient reads dZ as the data gradient does; the column
+    // form needs it channel-major too
+    const bool implicit = L.ks == 3 && X.up == 1 && X.ld % 8 == 0 && X.off % 8 == 0 && conv_wgrad_ok(L.ci, L.co, L.H, L.W);
+    const size_t smem = (size_t)pt * (L.co + 1) * 4 + (implicit ? 0 : (size_t)L.co * (pt + 8) * 2);
+    CK(cudaFuncSetAttribute(act_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    act_back_kernel<<<n_blk, TB, smem, st>>>(dy, Y, L.H, L.W, P, L.co, L.relu, pt, n->dz16,
+                                             implicit ? nullptr : n->dz_cp, Pp,
+                                             n->partials);
+    CK(cudaGetLastError());
+    parts_sum_kernel<<<L.co, 256, 0, st>>>(n->partials, n_blk, L.co, n->grads + L.b_off);
+    CK(cudaGetLastError());
+    if (implicit) {
+        int used = 1;
+        CK(launch_conv_wgrad(X.p + X.off, L.ci, X.ld, B, L.H, L.W, n->dz16, L.co, wgrad_splits(P), n->partials, &used,
+                             n->err, st));
+        wgrad_sum_kernel<<<nblk((int64_t)L.co * L.K9), TB, 0, st>>>(n->partials, used, L.co, L.ci, n->grads + L.w_off);
+        CK(cudaGetLastError());
+    } else {
+        CK(wgrad_columns(n, L, B, X));
+    }
     if (dx) {
         // data gradient: the convolution of dZ with the flipped weights
         CK(conv_product(n, plain(n->dz16, L.co), L.co, B, L.H, L.W, L.ks, L.wf16, L.K9dp, L.wf3, L.ci,

@@ -124,4 +124,14 @@ inline bool conv_implicit_ok(int C, int H, int W) {
 
 cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s);
 
+// The implicit weight gradient applies when both channel counts are multiples
+// of 32 and 16 pixels or more fit a row (or 64 consecutive pixels are whole
+// rows of one image).
+inline bool conv_wgrad_ok(int C, int N, int H, int W) {
+    if (C % 32 || C <= 0 || N % 32 || N <= 0 || W <= 0 || H <= 0) return false;
+    return W % 16 == 0 || (W == 8 && H % 8 == 0);
+}
+cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int C, int ldx, int B, int H, int W, const __nv_bfloat16* dz, int N,
+                              int splits, float* part, int* used, int* err, cudaStream_t s);
+
 }  // namespace gdrr

@@ -30,6 +30,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <numeric>
 
 #include "cnn_epi.cuh"
 #include "gdrr_internal.cuh"
@@ -1004,6 +1005,202 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
                      :: "r"(tmem), "r"((uint32_t)COLS) : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// Implicit weight gradient of a 3 x 3 convolution: dW^T[(tap, ci)][co] = the sum
+// over pixels of x[p + tap][ci] dZ[p][co], straight from the NHWC tensors.
+// Pixels are the product's K: a stage holds 64 pixels of dZ and of x shifted by
+// the tap, in slabs of 32 channels (64 pixels x 64 bytes, 64-byte swizzle, zero
+// fill outside the image), and the tensor core reads both operands MN-major, so
+// nothing is transposed and no column matrix is written.  A block takes one ky,
+// up to 12 of the 3 C / 32 slabs (kx, 32 input channels) as M tiles of four
+// slabs, NB output channels and one range of pixels; its accumulators stay in
+// TMEM for the whole range and leave as one FP32 partial product, which an
+// ordered pass adds to the others.  The ranges are the column form's, and both
+// take their pixels in order, 16 at a time: the sums are the same to the bit.
+//
+// Bound: about 600 clocks a stage of issuing its copies and products, then the
+// copies from L2 (each input pixel is read once per tap).  Against the column
+// form (a 9 C x P matrix written, read, and its product summed and reordered),
+// batch 16 on 96 x 128 pixels: 96 -> 32 channels 217 us -> 45, 192 -> 64 at half
+// the grid 125 -> 42, 384 -> 128 at a quarter 74 -> 36 (partial sums included).
+constexpr int WG_PIX = 64, WG_SLABS = 12;
+constexpr uint32_t WG_SLAB = WG_PIX * CONV_BK * 2;
+
+// 64-byte-swizzled MN-major operand: atoms of 32 channels x 8 pixels; the next
+// 32 channels a slab further, the next 8 pixels 512 bytes further.
+__device__ __forceinline__ uint64_t smem_desc_sw64_mn(uint32_t addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(WG_SLAB >> 4) << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
+struct WgradGeo {
+    int H, W;
+    int c32, slabs;        // C / 32, 3 C / 32
+    int groups, group;     // slab groups, and the slabs of one (at most WG_SLABS)
+    int a_slabs;           // slabs a stage has room for (a multiple of 4)
+    int box, boxes;        // pixels of one copy, copies of a slab's 64 pixels
+    uint32_t box_bytes;
+    int tiles, per_split;  // 64-pixel tiles, and those of one split
+    int stages;
+};
+
+template <int NB>
+__global__ void __launch_bounds__(PERSIST_THREADS) conv_wgrad_kernel(const __grid_constant__ CUtensorMap mapX,
+                                                                    const __grid_constant__ CUtensorMap mapZ,
+                                                                    const WgradGeo g, float* __restrict__ part, int N,
+                                                                    int* err) {
+    constexpr int COLS = tmem_columns(WG_SLABS / 4 * NB), Z_SLABS = NB / 32;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[CONV_MAX_STAGES], empty_bar[CONV_MAX_STAGES], done_bar;
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_fail;
+    const uint32_t ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
+    const uint32_t a_bytes = (uint32_t)g.a_slabs * WG_SLAB, stage_bytes = a_bytes + Z_SLABS * WG_SLAB;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ky = blockIdx.y % 3, group = blockIdx.y / 3 % g.groups, n0 = (int)(blockIdx.y / (3 * g.groups)) * NB;
+    const int s0 = group * g.group, ns = min(g.group, g.slabs - s0), m_tiles = (ns + 3) / 4;
+    const int t0 = blockIdx.x * g.per_split, t1 = min(g.tiles, t0 + g.per_split);
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_addr(&tmem_base)), "r"((uint32_t)COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int s = 0; s < g.stages; ++s) {
+            mbar_init(smem_addr(&full_bar[s]), 1);
+            mbar_init(smem_addr(&empty_bar[s]), 1);
+        }
+        mbar_init(smem_addr(&done_bar), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_fail = 0;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_base;
+
+    if (warp == 0) {
+        // producer: coordinates by stepping (a division a copy costs more than the
+        // copy), on the whole warp so that they stay in uniform registers
+        const bool leader = elect_one();
+        const int px0 = t0 * WG_PIX, step_y = WG_PIX / g.W, step_x = WG_PIX % g.W, kx0 = s0 / g.c32 - 1;
+        const int ch0 = s0 % g.c32 * CONV_BK, C = g.c32 * CONV_BK;
+        int b = px0 / (g.H * g.W), y = px0 / g.W % g.H, x = px0 % g.W;
+        int it = 0, s = 0;
+        uint32_t ph = 0;
+        for (int t = t0; t < t1; ++t, ++it) {
+            if (it >= g.stages && !__all_sync(0xffffffffu, mbar_wait(smem_addr(&empty_bar[s]), ph ^ 1u))) {
+                if (leader) atomicExch(&s_fail, 1);
+                break;
+            }
+            const uint32_t sa = ring + (uint32_t)s * stage_bytes, fb = smem_addr(&full_bar[s]);
+            if (leader) {
+                mbar_expect_tx(fb, (uint32_t)(ns + Z_SLABS) * WG_SLAB);
+#pragma unroll
+                for (int i = 0; i < Z_SLABS; ++i)
+                    tma_load_2d(sa + a_bytes + (uint32_t)i * WG_SLAB, &mapZ, n0 + i * CONV_BK, t * WG_PIX, fb);
+            }
+            uint32_t to = sa;
+            int bx = x, by = y, bb = b;
+            for (int o = 0; o < g.boxes; ++o, to += g.box_bytes) {
+                int kx = kx0, ch = ch0;
+                for (int i = 0; i < ns; ++i) {
+                    if (leader) tma_load_4d(to + (uint32_t)i * WG_SLAB, &mapX, ch, bx + kx, by + ky - 1, bb, fb);
+                    ch += CONV_BK;
+                    if (ch == C) { ch = 0; ++kx; }
+                }
+                bx += g.box;
+                if (bx >= g.W) { bx = 0; if (++by == g.H) { by = 0; ++bb; } }
+            }
+            x += step_x;
+            y += step_y;
+            if (x >= g.W) { x -= g.W; ++y; }
+            while (y >= g.H) { y -= g.H; ++b; }
+            if (++s == g.stages) { s = 0; ph ^= 1u; }
+        }
+        // the ring's last loads land before the CTA can leave (bounded)
+        const int last = min(it, g.stages);
+        for (int j = 0; j < last; ++j) {
+            const int jt = it - 1 - j;
+            mbar_wait(smem_addr(&full_bar[jt % g.stages]), (uint32_t)((jt / g.stages) & 1));
+        }
+    } else if (warp == 1) {
+        // MMA issuer: both operands MN-major (bits 15 and 16)
+        constexpr uint32_t idesc = instr_desc(GEMM_BM, NB) | (1u << 15) | (1u << 16);
+        const bool leader = elect_one();
+        int s = 0;
+        uint32_t ph = 0;
+        for (int t = t0; t < t1; ++t) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_addr(&full_bar[s]), ph))) {
+                if (leader) atomicExch(&s_fail, 1);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t sa = ring + (uint32_t)s * stage_bytes;
+            const uint64_t ad0 = smem_desc_sw64_mn(sa), bd0 = smem_desc_sw64_mn(sa + a_bytes);
+            if (leader) {
+#pragma unroll
+                for (int kk = 0; kk < WG_PIX / 16; ++kk) {
+                    // K16 step: 16 pixels of 64 bytes
+                    const uint32_t acc = (t > t0 || kk > 0) ? 1u : 0u;
+                    for (int m = 0; m < m_tiles; ++m)
+                        asm volatile(
+                            "{\n\t.reg .pred p;\n\t"
+                            "setp.ne.b32 p, %4, 0;\n\t"
+                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                            :: "r"(tmem + (uint32_t)(m * NB)), "l"(ad0 + (uint64_t)((m * 4 * WG_SLAB + kk * 1024) >> 4)),
+                               "l"(bd0 + (uint64_t)(kk * 1024 >> 4)), "r"(idesc), "r"(acc)
+                            : "memory");
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             :: "r"(smem_addr(&empty_bar[s])) : "memory");
+            }
+            __syncwarp();
+            if (++s == g.stages) { s = 0; ph ^= 1u; }
+        }
+        if (leader)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                         :: "r"(smem_addr(&done_bar)) : "memory");
+        __syncwarp();
+    } else if (warp >= 2) {
+        // the partial product, once the last MMA is done
+        const int q = warp & 3;
+        const bool got = mbar_wait(smem_addr(&done_bar), 0u);
+        if (__all_sync(0xffffffffu, got) && !*(volatile int*)&s_fail) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int m = 0; m < m_tiles; ++m) {
+                const int slab = 4 * m + q;               // this warp's quarter of the M tile
+                if (slab >= ns) break;
+                const int64_t row = ((int64_t)blockIdx.x * 3 + ky) * g.slabs * 32 + (s0 + slab) * 32 + lane;
+                float* to = part + row * N + n0;
+                uint32_t r[32];
+#pragma unroll
+                for (int c0 = 0; c0 < NB; c0 += 32) {
+                    tmem_load32(r, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(m * NB + c0));
+                    tmem_wait_load();
+#pragma unroll
+                    for (int h = 0; h < 32; h += 4)
+                        *reinterpret_cast<uint4*>(to + c0 + h) = make_uint4(r[h], r[h + 1], r[h + 2], r[h + 3]);
+                }
+            }
+        } else if (lane == 0) {
+            atomicExch(&s_fail, 1);
+        }
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && *(volatile int*)&s_fail) atomicExch(err, 1);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)COLS) : "memory");
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static std::once_flag once;
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -1246,6 +1443,102 @@ cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s) {
         case 64: return launch_conv_bn<64>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
         case 128: return launch_conv_bn<128>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
         default: return launch_conv_bn<256>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
+    }
+}
+
+// Slabs and output channels of a weight-gradient block: those with the least
+// of waves x the longest of a stage's copies (38 bytes a clock and SM), its MMAs
+// (60 + 0.45 NB clocks each) and its issue (600 clocks).  The pixel ranges are given (they fix the order of the
+// sums), so a narrow layer fills the chip by smaller blocks.
+struct WgradSplit {
+    int group, nb;
+};
+static WgradSplit wgrad_plan(int C, int N, int splits, int per_split) {
+    const int slabs = 3 * C / CONV_BK;
+    WgradSplit best{1, 32};
+    double least = 1e300;
+    for (int nb = 32; nb <= 128; nb += 32) {
+        if (N % nb) continue;
+        for (int gs = 1; gs <= std::min(WG_SLABS, slabs); ++gs) {
+            const int64_t blocks = (int64_t)splits * 3 * ((slabs + gs - 1) / gs) * (N / nb);
+            const double copies = (gs + nb / 32) * WG_SLAB / 38.0, mma = 4.0 * ((gs + 3) / 4) * (60.0 + 0.45 * nb);
+            const double t = (double)((blocks + 151) / 152) * (3000.0 + per_split * std::max({copies, mma, 600.0}));
+            if (t < least) {
+                least = t;
+                best = {gs, nb};
+            }
+        }
+    }
+    return best;
+}
+
+// Partial products [splits][(tap, ci)][co] of x (NHWC, C channels, pixel pitch
+// ldx) and dz ([P][N]) on the grid B x H x W (conv_wgrad_ok).
+// Split z takes the 64-pixel tiles [z per, (z + 1) per) of the *used splits.
+cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int C, int ldx, int B, int H, int W, const __nv_bfloat16* dz, int N,
+                              int splits, float* part, int* used, int* err, cudaStream_t s) {
+    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+    if (!fn) return cudaErrorNotSupported;
+    const int64_t P = (int64_t)B * H * W;
+    if (!conv_wgrad_ok(C, N, H, W) || P > INT32_MAX || ldx % 8 || ldx < C ||
+        ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dz)) & 15u) != 0)
+        return cudaErrorInvalidValue;
+    WgradGeo g;
+    g.tiles = (int)((P + WG_PIX - 1) / WG_PIX);
+    g.per_split = (g.tiles + std::max(1, std::min(splits, g.tiles)) - 1) / std::max(1, std::min(splits, g.tiles));
+    *used = splits = (g.tiles + g.per_split - 1) / g.per_split;
+    const WgradSplit plan = wgrad_plan(C, N, splits, g.per_split);
+    const int nb = plan.nb;
+    // a copy: as many pixels as divide both a row and a stage, and whole rows
+    // where a stage is whole rows of one image
+    const int rows = WG_PIX % W == 0 && H % (WG_PIX / W) == 0 ? WG_PIX / W : 1, wk = std::gcd(W, WG_PIX);
+    g.box = wk * rows;
+    g.boxes = WG_PIX / g.box;
+    g.box_bytes = (uint32_t)g.box * CONV_BK * 2;
+    CUtensorMap mX, mZ;
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+        const cuuint64_t px = (cuuint64_t)ldx * 2;
+        const cuuint64_t strides[3] = {px, px * W, px * W * H};
+        const cuuint32_t box[4] = {(cuuint32_t)CONV_BK, (cuuint32_t)wk, (cuuint32_t)rows, 1};
+        const cuuint32_t elem[4] = {1, 1, 1, 1};
+        if (fn(&mX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(x), dims, strides, box, elem,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)P};
+        const cuuint64_t strides[1] = {(cuuint64_t)N * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)CONV_BK, (cuuint32_t)WG_PIX};
+        const cuuint32_t elem[2] = {1, 1};
+        if (fn(&mZ, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(dz), dims, strides, box, elem,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    g.H = H;
+    g.W = W;
+    g.c32 = C / CONV_BK;
+    g.slabs = 3 * g.c32;
+    g.group = plan.group;
+    g.groups = (g.slabs + g.group - 1) / g.group;
+    g.a_slabs = (g.group + 3) / 4 * 4;
+    const uint32_t stage = (uint32_t)(g.a_slabs + nb / 32) * WG_SLAB;
+    g.stages = (int)std::min<uint32_t>(CONV_MAX_STAGES, 216u * 1024u / stage);
+    const size_t smem = (size_t)g.stages * stage + 1024;
+    const dim3 grid((unsigned)splits, (unsigned)(3 * g.groups * (N / nb)));
+    auto launch = [&](auto kernel) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, PERSIST_THREADS, smem, s>>>(mX, mZ, g, part, N, err);
+        return cudaGetLastError();
+    };
+    switch (nb) {
+        case 32: return launch(conv_wgrad_kernel<32>);
+        case 64: return launch(conv_wgrad_kernel<64>);
+        case 96: return launch(conv_wgrad_kernel<96>);
+        default: return launch(conv_wgrad_kernel<128>);
     }
 }
 
