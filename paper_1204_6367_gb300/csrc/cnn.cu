@@ -348,8 +348,8 @@ inline int act_tile(int co) { return co >= 256 ? 16 : (co >= 128 ? 32 : 64); }
 
 // dZ = dY * (Y > 0) (or dY when relu == 0) for a block of pt pixels (a
 // multiple of 16, at most 64) and all Co channels: BF16 NHWC dz16[p][c] (the
-// gradients' operand), where dz_cp != NULL BF16 channel-major dz_cp[c][p] (row
-// ldp; the column form's operand, zero for P <= p < ldp) through a
+// data gradient's operand), BF16 channel-major dz_cp[c][p] (row ldp; the column
+// form's weight-gradient operand, zero for P <= p < ldp) through a
 // shared-memory transpose, and the block's FP32 bias-gradient part
 // part[block][c] (its pt pixels added in order).
 __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__ dy, const View Y, int H, int W,
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__
                 const float gg = (relu && !(yv[u] > 0.0f)) ? 0.0f : g[u];
                 if (p0 + px < P) dz16[p0 * Co + i] = __float2bfloat16_rn(gg);
                 sf[px * (Co + 1) + c] = gg;
-                if (dz_cp) sb[c * sp + px] = __float2bfloat16_rn(gg);
+                sb[c * sp + px] = __float2bfloat16_rn(gg);
             }
         }
     }
@@ -400,13 +400,124 @@ __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__
         for (int px = 0; px < pt; ++px) s += sf[px * (Co + 1) + c];
         part[(int64_t)blockIdx.x * Co + c] = s;
     }
-    if (!dz_cp) return;
     const int segs = pt / 8;
     for (int i = threadIdx.x; i < Co * segs; i += blockDim.x) {
         const int c = i / segs, seg = i - c * segs;
         if (p0 + seg * 8 < ldp)
             *reinterpret_cast<uint4*>(dz_cp + (int64_t)c * ldp + p0 + seg * 8) =
                 *reinterpret_cast<const uint4*>(sb + c * sp + seg * 8);
+    }
+}
+
+// A layer's output gradient, on its grid H x W, from the gradients it reaches:
+// g itself (row pitch Co); the sum over the 2 x 2 block of an upsampled decoder
+// input's gradient (order (0,0), (0,1), (1,0), (1,1)); or a skip's part plus a
+// quarter of the pooled gradient dp (row pitch Co, grid H/2 x W/2).  g has row
+// pitch ld and starts at channel off.
+enum { GRAD_PLAIN, GRAD_PLACE, GRAD_POOL };
+struct GradSrc {
+    int mode;
+    const float* g;
+    int ld, off;
+    const float* dp;
+    float* buf;            // room for the gradient itself (column form)
+};
+constexpr int ACT_PIX = 128;   // at most this many pixels per block of act_back4_kernel
+
+// dZ = dY * (Y > 0) (or dY when relu == 0) with dY read as SRC says: BF16 NHWC
+// dz16[p][c], and per tile of pt pixels the FP32 bias-gradient part part[tile][c]
+// (its pixels added in order).  A block takes `tiles` tiles (at most ACT_PIX
+// pixels); four channels per thread, Co a multiple of 4.
+//
+// Bound: memory.  The gradient of an upsampled or pooled tensor is formed here
+// and not written out first, and the values are read 16 bytes a lane: six layers
+// of a training step (16 images of 96 x 128) took 153 us as a pass that forms
+// the gradient and a scalar one, 67 us so.
+template <int SRC>
+__global__ void __launch_bounds__(256) act_back4_kernel(const GradSrc G, const View Y, int H, int W, int64_t P, int Co,
+                                                        int relu, int pt, int tiles, bf16* __restrict__ dz16,
+                                                        float* __restrict__ part) {
+    extern __shared__ __align__(16) float sz[];                        // [tiles pt][Co + 4]
+    __shared__ int64_t ybase[ACT_PIX], gbase[ACT_PIX], pbase[ACT_PIX];
+    const int np = tiles * pt, c4 = Co / 4, pitch = Co + 4, n = np * c4;
+    const int64_t p0 = (int64_t)blockIdx.x * np;
+    const int W2 = 2 * W;
+    if ((int)threadIdx.x < np) {
+        const int64_t p = p0 + threadIdx.x;
+        if (p < P) {
+            ybase[threadIdx.x] = view_pixel(Y, p, H, W) * Y.ld + Y.off;
+            const View up{nullptr, 0, 0, SRC == GRAD_PLACE ? 2 : 1};
+            gbase[threadIdx.x] = (SRC == GRAD_PLACE ? view_pixel(up, p, H, W) : p) * G.ld + G.off;
+            if (SRC == GRAD_POOL) {
+                const int64_t b = p / ((int64_t)H * W);
+                const int r = (int)(p - b * H * W), y = r / W, x = r - y * W;
+                pbase[threadIdx.x] = ((b * (H / 2) + y / 2) * (W / 2) + x / 2) * Co;
+            }
+        }
+    }
+    __syncthreads();
+    constexpr int U = SRC == GRAD_PLACE ? 2 : 4;                       // values in flight per thread
+    for (int base = threadIdx.x; base < n; base += U * 256) {
+        float4 g[U], e[U][SRC == GRAD_PLACE ? 3 : 1];
+        uint2 yv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = base + u * 256, px = i / c4, c = 4 * (i - px * c4);
+            g[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            yv[u] = make_uint2(0u, 0u);
+            if (i < n && p0 + px < P) {
+                const float* d = G.g + gbase[px] + c;
+                g[u] = *reinterpret_cast<const float4*>(d);
+                if (SRC == GRAD_PLACE) {
+                    e[u][0] = *reinterpret_cast<const float4*>(d + G.ld);
+                    e[u][1] = *reinterpret_cast<const float4*>(d + (int64_t)W2 * G.ld);
+                    e[u][2] = *reinterpret_cast<const float4*>(d + (int64_t)W2 * G.ld + G.ld);
+                } else if (SRC == GRAD_POOL) {
+                    e[u][0] = *reinterpret_cast<const float4*>(G.dp + pbase[px] + c);
+                }
+                if (relu) yv[u] = *reinterpret_cast<const uint2*>(Y.p + ybase[px] + c);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = base + u * 256, px = i / c4, c = 4 * (i - px * c4);
+            if (i >= n) break;
+            float v[4] = {g[u].x, g[u].y, g[u].z, g[u].w};
+            if (p0 + px < P) {
+                if (SRC == GRAD_PLACE) {
+                    const float a1[4] = {e[u][0].x, e[u][0].y, e[u][0].z, e[u][0].w};
+                    const float a2[4] = {e[u][1].x, e[u][1].y, e[u][1].z, e[u][1].w};
+                    const float a3[4] = {e[u][2].x, e[u][2].y, e[u][2].z, e[u][2].w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[j] = ((0.0f + v[j]) + a1[j] + a2[j]) + a3[j];
+                } else if (SRC == GRAD_POOL) {
+                    v[0] += 0.25f * e[u][0].x;
+                    v[1] += 0.25f * e[u][0].y;
+                    v[2] += 0.25f * e[u][0].z;
+                    v[3] += 0.25f * e[u][0].w;
+                }
+                if (relu) {
+                    const bf16* yb = reinterpret_cast<const bf16*>(&yv[u]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[j] = __bfloat162float(yb[j]) > 0.0f ? v[j] : 0.0f;
+                }
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+                *reinterpret_cast<uint2*>(dz16 + (p0 + px) * Co + c) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
+            *reinterpret_cast<float4*>(sz + px * pitch + c) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+    }
+    __syncthreads();
+    const int64_t n_part = (P + pt - 1) / pt;
+    for (int i = threadIdx.x; i < tiles * Co; i += 256) {
+        const int t = i / Co, c = i - t * Co;
+        if ((int64_t)blockIdx.x * tiles + t >= n_part) break;
+        const float* z = sz + t * pt * pitch + c;
+        float s = 0.0f;
+#pragma unroll 8
+        for (int px = 0; px < pt; ++px) s += z[px * pitch];
+        part[((int64_t)blockIdx.x * tiles + t) * Co + c] = s;
     }
 }
 
@@ -788,11 +899,11 @@ cudaError_t wgrad_columns(gdrr_cnn* n, const Conv& L, int B, const View& X) {
     return cudaSuccess;
 }
 
-// Backward of one 3 x 3 convolution L on the grid H x W: dy (FP32 [P][co],
-// gradient of the layer output), Y (view of its BF16 output, for the ReLU
-// mask), X (its plain NHWC input, ci channels).  Writes the parameter
-// gradients and, when dx != NULL, dx (FP32 [P][ci]).
-cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const float* dy, const View& Y, const View& X,
+// Backward of one 3 x 3 convolution L on its grid: dy (gradient of the layer
+// output), Y (view of its BF16 output, for the ReLU mask), X (its plain NHWC
+// input, ci channels).  Writes the parameter gradients and, when dx != NULL, dx
+// (FP32 [P][ci]).
+cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const GradSrc& dy, const View& Y, const View& X,
                           float* dx) {
     const int64_t P = (int64_t)B * L.H * L.W;
     const int Pp = pad64(P);
@@ -802,11 +913,29 @@ cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const float* dy, co
     // the implicit weight gradient reads dZ as the data gradient does; the column
     // form needs it channel-major too
     const bool implicit = L.ks == 3 && X.up == 1 && X.ld % 8 == 0 && X.off % 8 == 0 && conv_wgrad_ok(L.ci, L.co, L.H, L.W);
-    const size_t smem = (size_t)pt * (L.co + 1) * 4 + (implicit ? 0 : (size_t)L.co * (pt + 8) * 2);
-    CK(cudaFuncSetAttribute(act_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    act_back_kernel<<<n_blk, TB, smem, st>>>(dy, Y, L.H, L.W, P, L.co, L.relu, pt, n->dz16,
-                                             implicit ? nullptr : n->dz_cp, Pp,
-                                             n->partials);
+    if (implicit) {
+        const int tiles = std::max(1, std::min(ACT_PIX / pt, 4096 / (pt * L.co)));
+        const size_t smem = (size_t)tiles * pt * (L.co + 4) * 4;
+        auto act = dy.mode == GRAD_PLACE ? act_back4_kernel<GRAD_PLACE>
+                   : dy.mode == GRAD_POOL ? act_back4_kernel<GRAD_POOL> : act_back4_kernel<GRAD_PLAIN>;
+        CK(cudaFuncSetAttribute(act, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        act<<<(n_blk + tiles - 1) / tiles, 256, smem, st>>>(dy, Y, L.H, L.W, P, L.co, L.relu, pt, tiles, n->dz16,
+                                                            n->partials);
+    } else {
+        const float* g = dy.g;
+        if (dy.mode != GRAD_PLAIN) {
+            g = dy.buf;
+            if (dy.mode == GRAD_PLACE)
+                place_back_kernel<<<nblk(P * L.co / 4), TB, 0, st>>>(dy.g, dy.ld, B, L.co, L.H, L.W, dy.buf);
+            else
+                pool_back_kernel<<<nblk(P * L.co / 4), TB, 0, st>>>(dy.g, dy.ld, dy.off, dy.dp, B, L.co, L.H, L.W, dy.buf);
+            CK(cudaGetLastError());
+        }
+        const size_t smem = (size_t)pt * (L.co + 1) * 4 + (size_t)L.co * (pt + 8) * 2;
+        CK(cudaFuncSetAttribute(act_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        act_back_kernel<<<n_blk, TB, smem, st>>>(g, Y, L.H, L.W, P, L.co, L.relu, pt, n->dz16, n->dz_cp, Pp,
+                                                 n->partials);
+    }
     CK(cudaGetLastError());
     parts_sum_kernel<<<L.co, 256, 0, st>>>(n->partials, n_blk, L.co, n->grads + L.b_off);
     CK(cudaGetLastError());
@@ -1044,25 +1173,29 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
         }
         // decoder: each input gradient g_cat splits into the upsampled part
         // (summed over 2 x 2 blocks) and the skip's part
-        if ((e = conv_backward(n, L[6], B, n->g_d1, plain(n->d1, c), plain(n->cat1, 3 * c), n->g_cat1))) break;
-        place_back_kernel<<<nblk(2 * c * s1 / 16), TB, 0, st>>>(n->g_cat1, 3 * c, B, 2 * c, H / 2, W / 2, n->g_d2);
-        if ((e = conv_backward(n, L[5], B, n->g_d2, View{n->cat1, 3 * c, 0, 2}, plain(n->cat2, 6 * c), n->g_cat2)))
+        auto grad = [](float* g, int ld) { return GradSrc{GRAD_PLAIN, g, ld, 0, nullptr, g}; };
+        auto place = [](float* dcat, int ld, float* buf) { return GradSrc{GRAD_PLACE, dcat, ld, 0, nullptr, buf}; };
+        auto pool = [](float* dcat, int ld, int off, float* dp, float* buf) { return GradSrc{GRAD_POOL, dcat, ld, off, dp, buf}; };
+        if ((e = conv_backward(n, L[6], B, grad(n->g_d1, c), plain(n->d1, c), plain(n->cat1, 3 * c), n->g_cat1))) break;
+        if ((e = conv_backward(n, L[5], B, place(n->g_cat1, 3 * c, n->g_d2), View{n->cat1, 3 * c, 0, 2},
+                               plain(n->cat2, 6 * c), n->g_cat2)))
             break;
-        place_back_kernel<<<nblk(4 * c * s1 / 64), TB, 0, st>>>(n->g_cat2, 6 * c, B, 4 * c, H / 4, W / 4, n->g_d3);
-        if ((e = conv_backward(n, L[4], B, n->g_d3, View{n->cat2, 6 * c, 0, 2}, plain(n->cat3, 12 * c), n->g_cat3)))
+        if ((e = conv_backward(n, L[4], B, place(n->g_cat2, 6 * c, n->g_d3), View{n->cat2, 6 * c, 0, 2},
+                               plain(n->cat3, 12 * c), n->g_cat3)))
             break;
-        place_back_kernel<<<nblk(8 * c * s1 / 256), TB, 0, st>>>(n->g_cat3, 12 * c, B, 8 * c, H / 8, W / 8, n->g_e4);
         // encoder: an output's gradient is its skip's part plus its pool's
-        if ((e = conv_backward(n, L[3], B, n->g_e4, View{n->cat3, 12 * c, 0, 2}, plain(n->p3, 4 * c), n->g_p3))) break;
-        pool_back_kernel<<<nblk(4 * c * s1 / 64), TB, 0, st>>>(n->g_cat3, 12 * c, 8 * c, n->g_p3, B, 4 * c, H / 4,
-                                                              W / 4, n->g_e3);
-        if ((e = conv_backward(n, L[2], B, n->g_e3, plain(n->cat3, 12 * c, 8 * c), plain(n->p2, 2 * c), n->g_p2)))
+        if ((e = conv_backward(n, L[3], B, place(n->g_cat3, 12 * c, n->g_e4), View{n->cat3, 12 * c, 0, 2},
+                               plain(n->p3, 4 * c), n->g_p3)))
             break;
-        pool_back_kernel<<<nblk(2 * c * s1 / 16), TB, 0, st>>>(n->g_cat2, 6 * c, 4 * c, n->g_p2, B, 2 * c, H / 2, W / 2,
-                                                             n->g_e2);
-        if ((e = conv_backward(n, L[1], B, n->g_e2, plain(n->cat2, 6 * c, 4 * c), plain(n->p1, c), n->g_p1))) break;
-        pool_back_kernel<<<nblk(c * s1 / 4), TB, 0, st>>>(n->g_cat1, 3 * c, 2 * c, n->g_p1, B, c, H, W, n->g_e1);
-        if ((e = conv_backward(n, L[0], B, n->g_e1, plain(n->cat1, 3 * c, 2 * c), plain(n->x16, 2), nullptr))) break;
+        if ((e = conv_backward(n, L[2], B, pool(n->g_cat3, 12 * c, 8 * c, n->g_p3, n->g_e3),
+                               plain(n->cat3, 12 * c, 8 * c), plain(n->p2, 2 * c), n->g_p2)))
+            break;
+        if ((e = conv_backward(n, L[1], B, pool(n->g_cat2, 6 * c, 4 * c, n->g_p2, n->g_e2),
+                               plain(n->cat2, 6 * c, 4 * c), plain(n->p1, c), n->g_p1)))
+            break;
+        if ((e = conv_backward(n, L[0], B, pool(n->g_cat1, 3 * c, 2 * c, n->g_p1, n->g_e1),
+                               plain(n->cat1, 3 * c, 2 * c), plain(n->x16, 2), nullptr)))
+            break;
         int bad = 0;
         if ((e = cudaMemcpyAsync(&bad, n->err, sizeof(int), cudaMemcpyDeviceToHost, st))) break;
         if ((e = cudaStreamSynchronize(st))) break;
