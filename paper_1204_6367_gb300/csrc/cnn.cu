@@ -521,22 +521,63 @@ __global__ void __launch_bounds__(256) act_back4_kernel(const GradSrc G, const V
     }
 }
 
-// out[c] = the sum over k of part[k][c] in a fixed order: one block per
-// channel, thread t adds parts t, t + 256, ... in turn, then a fixed tree
-// over the threads.
-__global__ void __launch_bounds__(256) parts_sum_kernel(const float* __restrict__ part, int n_part, int Co,
-                                                        float* __restrict__ out) {
-    __shared__ float red[256];
-    const int c = blockIdx.x;
+// The sums that end a backward pass.  A job adds parts[k][c] over k for co
+// channels (ci == 0) in a fixed order: one block per channel, thread t adds
+// parts t, t + 256, ... in turn, then a fixed tree over the threads.  Or (ci >
+// 0) an implicit weight gradient's partial products parts[z][(tap, ci)][co] in
+// the order z = 0, 1, ... into dw[co][ci][tap]: one block per input channel and
+// 32 output channels, whose 9 x 32 sums are exchanged so that they are written
+// as runs of taps.
+//
+// Bound: latency; one launch for all layers.  15 launches of 3 to 9 us (79 us a
+// training step of 16 images) became one of 19 us.
+struct SumJob {
+    const float* part;
+    float* out;
+    int n_part, co, ci, block0;
+};
+struct SumJobs {
+    SumJob job[16];
+    int n;
+    void add(const float* part, float* out, int n_part, int co, int ci) {
+        job[n] = SumJob{part, out, n_part, co, ci, blocks};
+        ++n;
+        blocks += ci ? ci * (co / 32) : co;
+    }
+    int blocks;
+};
+constexpr int SUM_THREADS = 9 * 32;
+
+__global__ void __launch_bounds__(SUM_THREADS) grad_sums_kernel(const SumJobs J) {
+    __shared__ float red[32 * 9];
+    int j = 0;
+    while (j + 1 < J.n && (int)blockIdx.x >= J.job[j + 1].block0) ++j;
+    const SumJob& d = J.job[j];
+    const int r = blockIdx.x - d.block0, t = threadIdx.x;
     float s = 0.0f;
-    for (int k = threadIdx.x; k < n_part; k += 256) s += part[(int64_t)k * Co + c];
-    red[threadIdx.x] = s;
+    if (d.ci) {
+        const int c0 = r / d.ci * 32, i = r % d.ci, tap = t >> 5, lane = t & 31;
+        const float* p = d.part + ((int64_t)tap * d.ci + i) * d.co + c0 + lane;
+        const int64_t step = (int64_t)9 * d.ci * d.co;
+#pragma unroll 8
+        for (int z = 0; z < d.n_part; ++z) s += p[z * step];
+        red[lane * 9 + tap] = s;
+        __syncthreads();
+        const int co = t / 9;
+        d.out[((int64_t)(c0 + co) * d.ci + i) * 9 + (t - co * 9)] = red[t];
+        return;
+    }
+    if (t < 256) {
+#pragma unroll 4
+        for (int k = t; k < d.n_part; k += 256) s += d.part[(int64_t)k * d.co + r];
+        red[t] = s;
+    }
     __syncthreads();
     for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        if (t < o) red[t] += red[t + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[c] = red[0];
+    if (t == 0) d.out[r] = red[0];
 }
 
 // Gradient of the upsampled part of a decoder input: g[b][y][x][c] = the sum
@@ -652,46 +693,51 @@ __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, 
     w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-// BF16 copies of a conv's weights w[co][ci][tap] (tap = ky ks + kx) in the
-// products' K order: w16[co][tap Ci + ci] (row K9p) for the column path's
-// forward, and wf16[ci][tap Co + co] = w[co][ci][kk - 1 - tap] (row K9dp),
-// the weights with the taps flipped for the data gradient (a convolution of
-// dZ: dX(y, x) = sum over co, ky, kx of dZ(y + ky - h, x + kx - h)
-// w[co][ci][ks - 1 - ky][ks - 1 - kx]); zero beyond the K extent.  For 3 x 3
-// layers also the implicit GEMM's ky-major copies w3[ky][co][kx Ci + ci] and
-// wf3[ky][ci][kx Co + co] (flipped).
-__global__ void weight_copies_kernel(const float* __restrict__ w, int Co, int Ci, int kk, int K9p, int K9dp,
-                                     bf16* __restrict__ w16, bf16* __restrict__ wf16, bf16* __restrict__ w3,
-                                     bf16* __restrict__ wf3) {
-    const int K9 = Ci * kk;
-    const int64_t n1 = (int64_t)Co * K9p, n2 = (int64_t)Ci * K9dp;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n1) {
-        const int co = (int)(i / K9p), k = (int)(i % K9p);
-        float v = 0.0f;
-        if (k < K9) {
-            const int tap = k / Ci, ci = k - tap * Ci;
-            v = w[(int64_t)co * K9 + (int64_t)ci * kk + tap];
+// BF16 copies of the convolutions' weights w[co][ci][tap] (tap = ky ks + kx) in
+// the products' K order, each where its product runs: w16[co][tap Ci + ci] (row
+// K9p) for the column path's forward, and wf16[ci][tap Co + co] =
+// w[co][ci][kk - 1 - tap] (row K9dp), the weights with the taps flipped for the
+// data gradient (a convolution of dZ: dX(y, x) = sum over co, ky, kx of
+// dZ(y + ky - h, x + kx - h) w[co][ci][ks - 1 - ky][ks - 1 - kx]); the rows'
+// ends beyond the K extent stay zero.  For the implicit GEMM w3[ky][co][kx Ci +
+// ci] and wf3[ky][ci][kx Co + co] (flipped).
+//
+// Bound: latency; one launch for all layers.  A thread reads the taps of one
+// (co, ci) and writes them to rows that its neighbours continue: first with ci
+// fastest (w16, w3), then with co fastest (wf16, wf3).  Eight launches of every
+// copy took 41 us, one of the copies in use takes 10 us.
+struct CopyJob {
+    const float* w;
+    int co, ci, kk, K9p, K9dp, block0;
+    bf16 *w16, *wf16, *w3, *wf3;
+};
+struct CopyJobs {
+    CopyJob job[8];
+    int n;
+};
+
+__global__ void weight_copies_kernel(const CopyJobs J) {
+    int j = 0;
+    while (j + 1 < J.n && (int)blockIdx.x >= J.job[j + 1].block0) ++j;
+    const CopyJob& d = J.job[j];
+    const int n = d.co * d.ci;
+    int i = (blockIdx.x - d.block0) * blockDim.x + threadIdx.x;
+    const bool flip = i >= n;
+    if (flip) i -= n;
+    if (i >= n || (flip ? !d.wf16 && !d.wf3 : !d.w16 && !d.w3)) return;
+    const int co = flip ? i % d.co : i / d.ci, ci = flip ? i / d.co : i % d.ci;
+    const float* w = d.w + ((int64_t)co * d.ci + ci) * d.kk;
+#pragma unroll 9
+    for (int tap = 0; tap < d.kk; ++tap) {
+        const bf16 v = __float2bfloat16_rn(w[tap]);
+        const int t = flip ? d.kk - 1 - tap : tap, ky = t / 3, kx = t - 3 * ky;
+        if (!flip) {
+            if (d.w16) d.w16[(int64_t)co * d.K9p + t * d.ci + ci] = v;
+            if (d.w3) d.w3[((int64_t)ky * d.co + co) * 3 * d.ci + kx * d.ci + ci] = v;
+        } else {
+            if (d.wf16) d.wf16[(int64_t)ci * d.K9dp + t * d.co + co] = v;
+            if (d.wf3) d.wf3[((int64_t)ky * d.ci + ci) * 3 * d.co + kx * d.co + co] = v;
         }
-        w16[i] = __float2bfloat16_rn(v);
-    }
-    if (i < n2) {
-        const int ci = (int)(i / K9dp), k = (int)(i % K9dp);
-        float v = 0.0f;
-        if (k < Co * kk) {
-            const int tap = k / Co, co = k - tap * Co;
-            v = w[(int64_t)co * K9 + (int64_t)ci * kk + (kk - 1 - tap)];
-        }
-        wf16[i] = __float2bfloat16_rn(v);
-    }
-    if (w3 && i < (int64_t)Co * K9) {
-        // w3[ky][co][kx Ci + ci] and wf3[ky][ci][kx Co + co], ky, kx < 3
-        const int ky = (int)(i / ((int64_t)Co * 3 * Ci));
-        const int r = (int)(i - (int64_t)ky * Co * 3 * Ci);
-        const int co = r / (3 * Ci), q = r - co * 3 * Ci, kx = q / Ci, ci = q - kx * Ci;
-        w3[i] = __float2bfloat16_rn(w[(int64_t)co * K9 + (int64_t)ci * kk + ky * 3 + kx]);
-        const int ci2 = r / (3 * Co), q2 = r - ci2 * 3 * Co, kx2 = q2 / Co, co2 = q2 - kx2 * Co;
-        wf3[i] = __float2bfloat16_rn(w[(int64_t)co2 * K9 + (int64_t)ci2 * kk + (8 - (ky * 3 + kx2))]);
     }
 }
 
@@ -704,19 +750,6 @@ __global__ void unpad_kernel(const float* __restrict__ GT, int Co, int Ci, int k
     const int co = (int)(i / ((int64_t)Ci * kk));
     const int r = (int)(i - (int64_t)co * Ci * kk), ci = r / kk, tap = r - ci * kk;
     dw[i] = GT[((int64_t)tap * Ci + ci) * Co + co];
-}
-
-// dW[co][ci][tap] from the implicit form's partial products p[z][(tap, ci)][co],
-// added in the order z = 0, 1, ...
-__global__ void wgrad_sum_kernel(const float* __restrict__ p, int n_splits, int Co, int Ci, float* __restrict__ dw) {
-    const int64_t n = (int64_t)9 * Ci * Co;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.0f;
-#pragma unroll 8
-    for (int z = 0; z < n_splits; ++z) s += p[(int64_t)z * n + i];
-    const int r = (int)(i / Co), co = (int)(i - (int64_t)r * Co), tap = r / Ci, ci = r - tap * Ci;
-    dw[((int64_t)co * Ci + ci) * 9 + tap] = s;
 }
 
 // out[i] = sum over z of p[z * stride + i], in the order z = 0, 1, ...
@@ -733,10 +766,14 @@ struct Conv {
     int K9, K9p, K9dp;     // ci ks^2, padded to 64; co ks^2 padded to 64 (data gradient)
     // parameters (FP32 master), gradients, Adam moments; offsets into the flat arrays
     int64_t w_off, b_off;
-    bf16* w16 = nullptr;   // [co][K9p], K = (tap, ci)
-    bf16* wf16 = nullptr;  // [ci][K9dp], K = (tap, co), taps flipped
-    bf16* w3 = nullptr;    // 3 x 3 layers: [ky][co][kx ci + c], the implicit GEMM's weights
-    bf16* wf3 = nullptr;   // 3 x 3 layers: [ky][ci][kx co + c], flipped
+    // weights in BF16, those that the layer's products use
+    bf16* w16 = nullptr;   // [co][K9p], K = (tap, ci): column form, first and last layer
+    bf16* wf16 = nullptr;  // [ci][K9dp], K = (tap, co), taps flipped: column form
+    bf16* w3 = nullptr;    // [ky][co][kx ci + c]: implicit GEMM
+    bf16* wf3 = nullptr;   // [ky][ci][kx co + c], flipped
+    bool implicit_dw = false;   // the weight gradient's form
+    float* dw_part = nullptr;   // its partial products
+    float* db_part = nullptr;   // the bias gradient's parts
 };
 
 // K splits of a weight-gradient product over P pixels (a function of P alone,
@@ -772,7 +809,7 @@ struct gdrr_cnn {
     // workspaces
     bf16* cols = nullptr;      // column matrix, either layout
     float* gemm = nullptr;     // column-path GEMM output
-    float* partials = nullptr; // per-split partial products of the weight gradients; bias-gradient parts
+    float* partials = nullptr; // per-split partial products of a column-form weight gradient
     bf16* dz16 = nullptr;      // dZ, NHWC
     bf16* dz_cp = nullptr;     // dZ, channel-major
     double* dloss = nullptr;
@@ -816,13 +853,15 @@ int err_code(cudaError_t e) {
     } while (0)
 
 cudaError_t refresh_weights(gdrr_cnn* n) {
-    for (Conv& L : n->conv) {
-        const int64_t cnt = std::max({(int64_t)L.co * L.K9p, (int64_t)L.ci * L.K9dp, (int64_t)L.co * L.K9});
-        weight_copies_kernel<<<nblk(cnt), TB, 0, n->stream>>>(n->params + L.w_off, L.co, L.ci, L.ks * L.ks, L.K9p,
-                                                              L.K9dp, L.w16, L.wf16, L.w3, L.wf3);
-        CK(cudaGetLastError());
+    CopyJobs J;
+    J.n = 0;
+    int blocks = 0;
+    for (const Conv& L : n->conv) {
+        J.job[J.n++] = CopyJob{n->params + L.w_off, L.co, L.ci, L.ks * L.ks, L.K9p, L.K9dp, blocks, L.w16, L.wf16, L.w3, L.wf3};
+        blocks += nblk((int64_t)2 * L.co * L.ci);
     }
-    return cudaSuccess;
+    weight_copies_kernel<<<blocks, TB, 0, n->stream>>>(J);
+    return cudaGetLastError();
 }
 
 ConvEpi epi_bf16(const float* bias, int relu, bf16* y, int ldy, int off, int up, int H, int W) {
@@ -841,12 +880,13 @@ ConvEpi epi_f32(float* y, int ld, int H, int W) {
 
 // One convolution on the grid H x W of the plain NHWC input X (C channels)
 // into N output columns through epi: the implicit GEMM (ky-major weights w3)
-// where the grid tiles, else a column matrix (row K9p), the column-path GEMM with w (row ldw, K =
-// (tap, c)) into n->gemm and the elementwise epilogue.
+// where there are such weights (the grid tiles), else a column matrix (row K9p),
+// the column-path GEMM with w (row ldw, K = (tap, c)) into n->gemm and the
+// elementwise epilogue.
 cudaError_t conv_product(gdrr_cnn* n, const View& X, int C, int B, int H, int W, int ks, const bf16* w, int ldw,
                          const bf16* w3, int N, const ConvEpi& epi) {
     const int64_t P = (int64_t)B * H * W;
-    if (ks == 3 && w3 && X.up == 1 && conv_implicit_ok(C, H, W) && X.ld % 8 == 0 && X.off % 8 == 0) {
+    if (w3) {
         ConvArgs a;
         a.x = X.p + X.off; a.C = C; a.ldx = X.ld;
         a.B = B; a.H = H; a.W = W;
@@ -901,10 +941,10 @@ cudaError_t wgrad_columns(gdrr_cnn* n, const Conv& L, int B, const View& X) {
 
 // Backward of one 3 x 3 convolution L on its grid: dy (gradient of the layer
 // output), Y (view of its BF16 output, for the ReLU mask), X (its plain NHWC
-// input, ci channels).  Writes the parameter gradients and, when dx != NULL, dx
-// (FP32 [P][ci]).
-cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const GradSrc& dy, const View& Y, const View& X,
-                          float* dx) {
+// input, ci channels).  Writes the parameter gradients, those that sums of parts
+// end with as jobs, and, when dx != NULL, dx (FP32 [P][ci]).
+cudaError_t conv_backward(gdrr_cnn* n, SumJobs& sums, const Conv& L, int B, const GradSrc& dy, const View& Y,
+                          const View& X, float* dx) {
     const int64_t P = (int64_t)B * L.H * L.W;
     const int Pp = pad64(P);
     cudaStream_t st = n->stream;
@@ -912,15 +952,14 @@ cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const GradSrc& dy, 
     const int n_blk = (int)((P + pt - 1) / pt);
     // the implicit weight gradient reads dZ as the data gradient does; the column
     // form needs it channel-major too
-    const bool implicit = L.ks == 3 && X.up == 1 && X.ld % 8 == 0 && X.off % 8 == 0 && conv_wgrad_ok(L.ci, L.co, L.H, L.W);
-    if (implicit) {
+    if (L.implicit_dw) {
         const int tiles = std::max(1, std::min(ACT_PIX / pt, 4096 / (pt * L.co)));
         const size_t smem = (size_t)tiles * pt * (L.co + 4) * 4;
         auto act = dy.mode == GRAD_PLACE ? act_back4_kernel<GRAD_PLACE>
                    : dy.mode == GRAD_POOL ? act_back4_kernel<GRAD_POOL> : act_back4_kernel<GRAD_PLAIN>;
         CK(cudaFuncSetAttribute(act, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         act<<<(n_blk + tiles - 1) / tiles, 256, smem, st>>>(dy, Y, L.H, L.W, P, L.co, L.relu, pt, tiles, n->dz16,
-                                                            n->partials);
+                                                            L.db_part);
     } else {
         const float* g = dy.g;
         if (dy.mode != GRAD_PLAIN) {
@@ -934,17 +973,15 @@ cudaError_t conv_backward(gdrr_cnn* n, const Conv& L, int B, const GradSrc& dy, 
         const size_t smem = (size_t)pt * (L.co + 1) * 4 + (size_t)L.co * (pt + 8) * 2;
         CK(cudaFuncSetAttribute(act_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         act_back_kernel<<<n_blk, TB, smem, st>>>(g, Y, L.H, L.W, P, L.co, L.relu, pt, n->dz16, n->dz_cp, Pp,
-                                                 n->partials);
+                                                 L.db_part);
     }
     CK(cudaGetLastError());
-    parts_sum_kernel<<<L.co, 256, 0, st>>>(n->partials, n_blk, L.co, n->grads + L.b_off);
-    CK(cudaGetLastError());
-    if (implicit) {
+    sums.add(L.db_part, n->grads + L.b_off, n_blk, L.co, 0);
+    if (L.implicit_dw) {
         int used = 1;
-        CK(launch_conv_wgrad(X.p + X.off, L.ci, X.ld, B, L.H, L.W, n->dz16, L.co, wgrad_splits(P), n->partials, &used,
+        CK(launch_conv_wgrad(X.p + X.off, L.ci, X.ld, B, L.H, L.W, n->dz16, L.co, wgrad_splits(P), L.dw_part, &used,
                              n->err, st));
-        wgrad_sum_kernel<<<nblk((int64_t)L.co * L.K9), TB, 0, st>>>(n->partials, used, L.co, L.ci, n->grads + L.w_off);
-        CK(cudaGetLastError());
+        sums.add(L.dw_part, n->grads + L.w_off, used, L.co, L.ci);
     } else {
         CK(wgrad_columns(n, L, B, X));
     }
@@ -999,8 +1036,7 @@ GDRR_API int gdrr_cnn_create(int32_t max_batch, int32_t height, int32_t width, i
         max_cols = std::max({max_cols, Pp * L.K9p, P * L.K9dp});
         max_gemm = std::max({max_gemm, P * L.ci, (int64_t)L.co * L.K9p, P * L.co});
         max_dz = std::max({max_dz, P * L.co, (int64_t)L.co * Pp});
-        max_part = std::max({max_part, (int64_t)wgrad_splits(P) * L.co * L.K9p, (Pp / act_tile(L.co) + 1) * L.co,
-                             (Pp / 256 + 1) * (L.ci + 1)});
+        max_part = std::max(max_part, (int64_t)wgrad_splits(P) * L.co * L.K9p);
     }
     cudaError_t e = cudaSuccess;
     do {
@@ -1009,8 +1045,18 @@ GDRR_API int gdrr_cnn_create(int32_t max_batch, int32_t height, int32_t width, i
             break;
         bool bad = false;
         for (Conv& L : n->conv) {
-            if (dalloc(n, &L.w16, (size_t)L.co * L.K9p) || dalloc(n, &L.wf16, (size_t)L.ci * L.K9dp)) bad = true;
-            if (L.ks == 3 && (dalloc(n, &L.w3, (size_t)L.co * L.K9) || dalloc(n, &L.wf3, (size_t)L.co * L.K9))) bad = true;
+            const int64_t P = B * L.H * L.W;
+            const bool first = &L == &n->conv.front(), last = L.ks == 1;
+            const bool fwd = !last && conv_implicit_ok(L.ci, L.H, L.W), back = conv_implicit_ok(L.co, L.H, L.W);
+            L.implicit_dw = !last && conv_wgrad_ok(L.ci, L.co, L.H, L.W);
+            const int64_t k16 = (int64_t)L.co * L.K9p, kf16 = (int64_t)L.ci * L.K9dp, k3 = (int64_t)L.co * L.K9;
+            if (fwd ? dalloc(n, &L.w3, k3) : (dalloc(n, &L.w16, k16) || cudaMemset(L.w16, 0, k16 * sizeof(bf16)))) bad = true;
+            if (!first && !last &&
+                (back ? dalloc(n, &L.wf3, k3) : (dalloc(n, &L.wf16, kf16) || cudaMemset(L.wf16, 0, kf16 * sizeof(bf16)))))
+                bad = true;
+            // the last layer's: parts of its weights, then of its bias, per 256 pixels
+            if (dalloc(n, &L.db_part, last ? (P + 255) / 256 * (L.ci + 1) : (P / act_tile(L.co) + 1) * L.co)) bad = true;
+            if (L.implicit_dw && dalloc(n, &L.dw_part, wgrad_splits(P) * k3)) bad = true;
         }
         if (bad) { e = cudaErrorMemoryAllocation; break; }
         const int64_t s1 = B * HW, s2 = s1 / 4, s3 = s1 / 16, s4 = s1 / 64;
@@ -1161,14 +1207,16 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
         if ((e = cudaMemsetAsync(n->dloss, 0, sizeof(double), st))) break;
         mse_kernel<<<nblk(s1), TB, 0, st>>>(n->out, target_dev, s1, n->g_out, n->dloss);
         if ((e = cudaMemcpyAsync(&loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, st))) break;
+        SumJobs sums;
+        sums.n = sums.blocks = 0;
         // the 1 x 1 output layer
         {
             const int nb = (int)((s1 + 255) / 256);
-            float* pw = n->partials;
-            float* pb = n->partials + (int64_t)nb * c;
+            float* pw = L[7].db_part;
+            float* pb = pw + (int64_t)nb * c;
             head_back_kernel<<<nb, 256, 0, st>>>(n->g_out, n->d1, c, L[7].w16, s1, n->g_d1, pw, pb);
-            parts_sum_kernel<<<c, 256, 0, st>>>(pw, nb, c, n->grads + L[7].w_off);
-            parts_sum_kernel<<<1, 256, 0, st>>>(pb, nb, 1, n->grads + L[7].b_off);
+            sums.add(pw, n->grads + L[7].w_off, nb, c, 0);
+            sums.add(pb, n->grads + L[7].b_off, nb, 1, 0);
             if ((e = cudaGetLastError())) break;
         }
         // decoder: each input gradient g_cat splits into the upsampled part
@@ -1176,26 +1224,28 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
         auto grad = [](float* g, int ld) { return GradSrc{GRAD_PLAIN, g, ld, 0, nullptr, g}; };
         auto place = [](float* dcat, int ld, float* buf) { return GradSrc{GRAD_PLACE, dcat, ld, 0, nullptr, buf}; };
         auto pool = [](float* dcat, int ld, int off, float* dp, float* buf) { return GradSrc{GRAD_POOL, dcat, ld, off, dp, buf}; };
-        if ((e = conv_backward(n, L[6], B, grad(n->g_d1, c), plain(n->d1, c), plain(n->cat1, 3 * c), n->g_cat1))) break;
-        if ((e = conv_backward(n, L[5], B, place(n->g_cat1, 3 * c, n->g_d2), View{n->cat1, 3 * c, 0, 2},
+        if ((e = conv_backward(n, sums, L[6], B, grad(n->g_d1, c), plain(n->d1, c), plain(n->cat1, 3 * c), n->g_cat1))) break;
+        if ((e = conv_backward(n, sums, L[5], B, place(n->g_cat1, 3 * c, n->g_d2), View{n->cat1, 3 * c, 0, 2},
                                plain(n->cat2, 6 * c), n->g_cat2)))
             break;
-        if ((e = conv_backward(n, L[4], B, place(n->g_cat2, 6 * c, n->g_d3), View{n->cat2, 6 * c, 0, 2},
+        if ((e = conv_backward(n, sums, L[4], B, place(n->g_cat2, 6 * c, n->g_d3), View{n->cat2, 6 * c, 0, 2},
                                plain(n->cat3, 12 * c), n->g_cat3)))
             break;
         // encoder: an output's gradient is its skip's part plus its pool's
-        if ((e = conv_backward(n, L[3], B, place(n->g_cat3, 12 * c, n->g_e4), View{n->cat3, 12 * c, 0, 2},
+        if ((e = conv_backward(n, sums, L[3], B, place(n->g_cat3, 12 * c, n->g_e4), View{n->cat3, 12 * c, 0, 2},
                                plain(n->p3, 4 * c), n->g_p3)))
             break;
-        if ((e = conv_backward(n, L[2], B, pool(n->g_cat3, 12 * c, 8 * c, n->g_p3, n->g_e3),
+        if ((e = conv_backward(n, sums, L[2], B, pool(n->g_cat3, 12 * c, 8 * c, n->g_p3, n->g_e3),
                                plain(n->cat3, 12 * c, 8 * c), plain(n->p2, 2 * c), n->g_p2)))
             break;
-        if ((e = conv_backward(n, L[1], B, pool(n->g_cat2, 6 * c, 4 * c, n->g_p2, n->g_e2),
+        if ((e = conv_backward(n, sums, L[1], B, pool(n->g_cat2, 6 * c, 4 * c, n->g_p2, n->g_e2),
                                plain(n->cat2, 6 * c, 4 * c), plain(n->p1, c), n->g_p1)))
             break;
-        if ((e = conv_backward(n, L[0], B, pool(n->g_cat1, 3 * c, 2 * c, n->g_p1, n->g_e1),
+        if ((e = conv_backward(n, sums, L[0], B, pool(n->g_cat1, 3 * c, 2 * c, n->g_p1, n->g_e1),
                                plain(n->cat1, 3 * c, 2 * c), plain(n->x16, 2), nullptr)))
             break;
+        grad_sums_kernel<<<sums.blocks, SUM_THREADS, 0, st>>>(sums);
+        if ((e = cudaGetLastError())) break;
         int bad = 0;
         if ((e = cudaMemcpyAsync(&bad, n->err, sizeof(int), cudaMemcpyDeviceToHost, st))) break;
         if ((e = cudaStreamSynchronize(st))) break;
