@@ -131,7 +131,8 @@ inline bool conv_wgrad_ok(int C, int N, int H, int W) {
     if (C % 32 || C <= 0 || N % 32 || N <= 0 || W <= 0 || H <= 0) return false;
     return W % 16 == 0 || (W == 8 && H % 8 == 0);
 }
-cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int C, int ldx, int B, int H, int W, const __nv_bfloat16* dz, int N,
-                              int splits, float* part, int* used, int* err, cudaStream_t s);
+// ks 3: the convolution's; ks 1: the product of each pixel's own C values.
+cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int ks, int C, int ldx, int B, int H, int W,
+                              const __nv_bfloat16* dz, int N, int splits, float* part, int* used, int* err, cudaStream_t s);
 
 }  // namespace gdrr

@@ -1040,7 +1040,8 @@ __device__ __forceinline__ uint64_t smem_desc_sw64_mn(uint32_t addr) {
 
 struct WgradGeo {
     int H, W;
-    int c32, slabs;        // C / 32, 3 C / 32
+    int ks;                // 3, or 1: a product of the pixels' own values
+    int c32, slabs;        // C / 32, ks C / 32
     int groups, group;     // slab groups, and the slabs of one (at most WG_SLABS)
     int a_slabs;           // slabs a stage has room for (a multiple of 4)
     int box, boxes;        // pixels of one copy, copies of a slab's 64 pixels
@@ -1062,7 +1063,8 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_wgrad_kernel(const __gri
     const uint32_t ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_bytes = (uint32_t)g.a_slabs * WG_SLAB, stage_bytes = a_bytes + Z_SLABS * WG_SLAB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ky = blockIdx.y % 3, group = blockIdx.y / 3 % g.groups, n0 = (int)(blockIdx.y / (3 * g.groups)) * NB;
+    const int ky = blockIdx.y % g.ks, group = blockIdx.y / g.ks % g.groups;
+    const int n0 = (int)(blockIdx.y / (g.ks * g.groups)) * NB;
     const int s0 = group * g.group, ns = min(g.group, g.slabs - s0), m_tiles = (ns + 3) / 4;
     const int t0 = blockIdx.x * g.per_split, t1 = min(g.tiles, t0 + g.per_split);
 
@@ -1089,7 +1091,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_wgrad_kernel(const __gri
         // producer: coordinates by stepping (a division a copy costs more than the
         // copy), on the whole warp so that they stay in uniform registers
         const bool leader = elect_one();
-        const int px0 = t0 * WG_PIX, step_y = WG_PIX / g.W, step_x = WG_PIX % g.W, kx0 = s0 / g.c32 - 1;
+        const int px0 = t0 * WG_PIX, step_y = WG_PIX / g.W, step_x = WG_PIX % g.W, kx0 = s0 / g.c32 - g.ks / 2;
         const int ch0 = s0 % g.c32 * CONV_BK, C = g.c32 * CONV_BK;
         int b = px0 / (g.H * g.W), y = px0 / g.W % g.H, x = px0 % g.W;
         int it = 0, s = 0;
@@ -1111,7 +1113,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_wgrad_kernel(const __gri
             for (int o = 0; o < g.boxes; ++o, to += g.box_bytes) {
                 int kx = kx0, ch = ch0;
                 for (int i = 0; i < ns; ++i) {
-                    if (leader) tma_load_4d(to + (uint32_t)i * WG_SLAB, &mapX, ch, bx + kx, by + ky - 1, bb, fb);
+                    if (leader) tma_load_4d(to + (uint32_t)i * WG_SLAB, &mapX, ch, bx + kx, by + ky - g.ks / 2, bb, fb);
                     ch += CONV_BK;
                     if (ch == C) { ch = 0; ++kx; }
                 }
@@ -1177,7 +1179,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_wgrad_kernel(const __gri
             for (int m = 0; m < m_tiles; ++m) {
                 const int slab = 4 * m + q;               // this warp's quarter of the M tile
                 if (slab >= ns) break;
-                const int64_t row = ((int64_t)blockIdx.x * 3 + ky) * g.slabs * 32 + (s0 + slab) * 32 + lane;
+                const int64_t row = ((int64_t)blockIdx.x * g.ks + ky) * g.slabs * 32 + (s0 + slab) * 32 + lane;
                 float* to = part + row * N + n0;
                 uint32_t r[32];
 #pragma unroll
@@ -1448,19 +1450,20 @@ cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s) {
 
 // Slabs and output channels of a weight-gradient block: those with the least
 // of waves x the longest of a stage's copies (38 bytes a clock and SM), its MMAs
-// (60 + 0.45 NB clocks each) and its issue (600 clocks).  The pixel ranges are given (they fix the order of the
-// sums), so a narrow layer fills the chip by smaller blocks.
+// (60 + 0.45 NB clocks each) and its issue (600 clocks).  The pixel ranges are
+// given (they fix the order of the sums), so a narrow layer fills the chip by
+// smaller blocks.
 struct WgradSplit {
     int group, nb;
 };
-static WgradSplit wgrad_plan(int C, int N, int splits, int per_split) {
-    const int slabs = 3 * C / CONV_BK;
+static WgradSplit wgrad_plan(int ks, int C, int N, int splits, int per_split) {
+    const int slabs = ks * C / CONV_BK;
     WgradSplit best{1, 32};
     double least = 1e300;
     for (int nb = 32; nb <= 128; nb += 32) {
         if (N % nb) continue;
         for (int gs = 1; gs <= std::min(WG_SLABS, slabs); ++gs) {
-            const int64_t blocks = (int64_t)splits * 3 * ((slabs + gs - 1) / gs) * (N / nb);
+            const int64_t blocks = (int64_t)splits * ks * ((slabs + gs - 1) / gs) * (N / nb);
             const double copies = (gs + nb / 32) * WG_SLAB / 38.0, mma = 4.0 * ((gs + 3) / 4) * (60.0 + 0.45 * nb);
             const double t = (double)((blocks + 151) / 152) * (3000.0 + per_split * std::max({copies, mma, 600.0}));
             if (t < least) {
@@ -1473,10 +1476,10 @@ static WgradSplit wgrad_plan(int C, int N, int splits, int per_split) {
 }
 
 // Partial products [splits][(tap, ci)][co] of x (NHWC, C channels, pixel pitch
-// ldx) and dz ([P][N]) on the grid B x H x W (conv_wgrad_ok).
-// Split z takes the 64-pixel tiles [z per, (z + 1) per) of the *used splits.
-cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int C, int ldx, int B, int H, int W, const __nv_bfloat16* dz, int N,
-                              int splits, float* part, int* used, int* err, cudaStream_t s) {
+// ldx) and dz ([P][N]) on the grid B x H x W (conv_wgrad_ok); with ks = 1 of
+// each pixel's own C values (one tap).  Split z takes the 64-pixel tiles [z per, (z + 1) per) of the *used splits.
+cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int ks, int C, int ldx, int B, int H, int W,
+                              const __nv_bfloat16* dz, int N, int splits, float* part, int* used, int* err, cudaStream_t s) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
     if (!fn) return cudaErrorNotSupported;
     const int64_t P = (int64_t)B * H * W;
@@ -1487,7 +1490,7 @@ cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int C, int ldx, int B, int
     g.tiles = (int)((P + WG_PIX - 1) / WG_PIX);
     g.per_split = (g.tiles + std::max(1, std::min(splits, g.tiles)) - 1) / std::max(1, std::min(splits, g.tiles));
     *used = splits = (g.tiles + g.per_split - 1) / g.per_split;
-    const WgradSplit plan = wgrad_plan(C, N, splits, g.per_split);
+    const WgradSplit plan = wgrad_plan(ks, C, N, splits, g.per_split);
     const int nb = plan.nb;
     // a copy: as many pixels as divide both a row and a stage, and whole rows
     // where a stage is whole rows of one image
@@ -1520,14 +1523,15 @@ cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int C, int ldx, int B, int
     g.H = H;
     g.W = W;
     g.c32 = C / CONV_BK;
-    g.slabs = 3 * g.c32;
+    g.ks = ks;
+    g.slabs = ks * g.c32;
     g.group = plan.group;
     g.groups = (g.slabs + g.group - 1) / g.group;
     g.a_slabs = (g.group + 3) / 4 * 4;
     const uint32_t stage = (uint32_t)(g.a_slabs + nb / 32) * WG_SLAB;
     g.stages = (int)std::min<uint32_t>(CONV_MAX_STAGES, 216u * 1024u / stage);
     const size_t smem = (size_t)g.stages * stage + 1024;
-    const dim3 grid((unsigned)splits, (unsigned)(3 * g.groups * (N / nb)));
+    const dim3 grid((unsigned)splits, (unsigned)(ks * g.groups * (N / nb)));
     auto launch = [&](auto kernel) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
