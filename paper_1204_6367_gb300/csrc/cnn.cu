@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(256) act_back_kernel(const float* __restrict__
 // input's gradient (order (0,0), (0,1), (1,0), (1,1)); or a skip's part plus a
 // quarter of the pooled gradient dp (row pitch Co, grid H/2 x W/2).  g has row
 // pitch ld and starts at channel off.
-enum { GRAD_PLAIN, GRAD_PLACE, GRAD_POOL };
+enum { GRAD_PLAIN, GRAD_PLACE, GRAD_POOL, GRAD_DONE };   // DONE: dZ and its bias parts are there
 struct GradSrc {
     int mode;
     const float* g;
@@ -679,6 +679,82 @@ __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict_
     float s = e * e;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(loss, (double)s / (double)n);
+}
+
+// Loss, output layer and dZ of the layer before it for a block of 256 pixels (C a
+// multiple of 8, its bias parts over 64 pixels): g = dL/dout of the mean square,
+// gr = BF16(g), dz16[p][c] = BF16(gr w[c]) where d1 > 0, the layer's bias parts
+// (sums of gr w[c]), and the output layer's parts of the weight gradient (sums
+// of gr d1[p][c]) and of the bias gradient (sums of g), each over its pixels in
+// order.
+//
+// Bound: latency (a load of d1, then a chain of 256 additions a block).  As three
+// kernels, with the gradient of d1 written in FP32 and read back, 57 us at 16
+// images of 96 x 128; so 14 us.
+__global__ void __launch_bounds__(256) head_grad_kernel(const float* __restrict__ out, const float* __restrict__ target,
+                                                        const bf16* __restrict__ d1, int C, const bf16* __restrict__ w,
+                                                        int64_t P, double* __restrict__ loss, bf16* __restrict__ dz16,
+                                                        float* __restrict__ part_db, float* __restrict__ part_w,
+                                                        float* __restrict__ part_b) {
+    extern __shared__ __align__(16) bf16 tile[];                       // [256][C]
+    __shared__ float sg[256], sgr[256];
+    __shared__ double red[8];
+    const int t = threadIdx.x;
+    const int64_t p0 = (int64_t)blockIdx.x * 256;
+    const int np = (int)min((int64_t)256, P - p0);
+    float e = 0.0f, g = 0.0f;
+    if (t < np) {
+        e = out[p0 + t] - target[p0 + t];
+        g = 2.0f * e / (float)P;
+    }
+    sg[t] = g;
+    sgr[t] = __bfloat162float(__float2bfloat16_rn(g));
+    float s2 = e * e;
+    for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    if ((t & 31) == 0) red[t >> 5] = (double)s2 / (double)P;
+    __syncthreads();
+    if (t == 0) {
+        double s = 0.0;
+        for (int i = 0; i < 8; ++i) s += red[i];
+        if (s != 0.0) atomicAdd(loss, s);
+    }
+    const int c8 = C / 8;
+#pragma unroll 4
+    for (int i = t; i < np * c8; i += 256) {
+        const int px = i / c8, c = 8 * (i - px * c8);
+        const uint4 dv = *reinterpret_cast<const uint4*>(d1 + p0 * C + 8 * (int64_t)i);
+        const uint4 wv = *reinterpret_cast<const uint4*>(w + c);
+        const bf16 *d = reinterpret_cast<const bf16*>(&dv), *ww = reinterpret_cast<const bf16*>(&wv);
+        __align__(16) bf16 o[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float gw = __fmul_rn(sgr[px], __bfloat162float(ww[j]));
+            o[j] = __float2bfloat16_rn(__bfloat162float(d[j]) > 0.0f ? gw : 0.0f);
+        }
+        *reinterpret_cast<uint4*>(dz16 + p0 * C + 8 * (int64_t)i) = *reinterpret_cast<const uint4*>(o);
+        *reinterpret_cast<uint4*>(tile + 8 * i) = dv;
+    }
+    __syncthreads();
+    for (int i = t; i <= 5 * C; i += 256) {
+        float s = 0.0f;
+        if (i < C) {
+#pragma unroll 16
+            for (int px = 0; px < np; ++px) s = __fmaf_rn(sgr[px], __bfloat162float(tile[px * C + i]), s);
+            part_w[(int64_t)blockIdx.x * C + i] = s;
+        } else if (i < 5 * C) {
+            const int q = i / C - 1, c = i - (q + 1) * C, end = min(64, np - 64 * q);
+            const float wc = __bfloat162float(w[c]);
+            if (end <= 0) continue;
+#pragma unroll 16
+            for (int px = 64 * q; px < 64 * q + end; ++px)
+                s += __bfloat162float(tile[px * C + c]) > 0.0f ? __fmul_rn(sgr[px], wc) : 0.0f;
+            part_db[((int64_t)blockIdx.x * 4 + q) * C + c] = s;
+        } else {
+#pragma unroll 16
+            for (int px = 0; px < np; ++px) s += sg[px];
+            part_b[blockIdx.x] = s;
+        }
+    }
 }
 
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
@@ -970,7 +1046,9 @@ cudaError_t conv_backward(gdrr_cnn* n, SumJobs& sums, const Conv& L, int B, cons
     const int n_blk = (int)((P + pt - 1) / pt);
     // the implicit weight gradient reads dZ as the data gradient does; the column
     // form needs it channel-major too
-    if (L.implicit_dw) {
+    if (dy.mode == GRAD_DONE) {
+        // written by head_grad_kernel
+    } else if (L.implicit_dw) {
         const int tiles = std::max(1, std::min(ACT_PIX / pt, 4096 / (pt * L.co)));
         const size_t smem = (size_t)tiles * pt * (L.co + 4) * 4;
         auto act = dy.mode == GRAD_PLACE ? act_back4_kernel<GRAD_PLACE>
@@ -1231,16 +1309,23 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
     double loss = 0.0;
     do {
         if ((e = cudaMemsetAsync(n->dloss, 0, sizeof(double), st))) break;
-        mse_kernel<<<nblk(s1), TB, 0, st>>>(n->out, target_dev, s1, n->g_out, n->dloss);
-        if ((e = cudaMemcpyAsync(&loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, st))) break;
         SumJobs sums;
         sums.n = sums.blocks = 0;
-        // the 1 x 1 output layer
+        // loss and the 1 x 1 output layer; the last 3 x 3 layer's dZ with them where
+        // its weight gradient does not need it channel-major
+        const bool fused_head = L[6].implicit_dw && act_tile(c) == 64;
         {
             const int nb = (int)((s1 + 255) / 256);
             float* pw = L[7].db_part;
             float* pb = pw + (int64_t)nb * c;
-            head_back_kernel<<<nb, 256, 0, st>>>(n->g_out, n->d1, c, L[7].w16, s1, n->g_d1, pw, pb);
+            if (fused_head) {
+                const size_t smem = (size_t)256 * c * sizeof(bf16);
+                head_grad_kernel<<<nb, 256, smem, st>>>(n->out, target_dev, n->d1, c, L[7].w16, s1, n->dloss, n->dz16,
+                                                        L[6].db_part, pw, pb);
+            } else {
+                mse_kernel<<<nblk(s1), TB, 0, st>>>(n->out, target_dev, s1, n->g_out, n->dloss);
+                head_back_kernel<<<nb, 256, 0, st>>>(n->g_out, n->d1, c, L[7].w16, s1, n->g_d1, pw, pb);
+            }
             sums.add(pw, n->grads + L[7].w_off, nb, 1, c, 0);
             sums.add(pb, n->grads + L[7].b_off, nb, 1, 1, 0);
             if ((e = cudaGetLastError())) break;
@@ -1250,7 +1335,8 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
         auto grad = [](float* g, int ld) { return GradSrc{GRAD_PLAIN, g, ld, 0, nullptr, g}; };
         auto place = [](float* dcat, int ld, float* buf) { return GradSrc{GRAD_PLACE, dcat, ld, 0, nullptr, buf}; };
         auto pool = [](float* dcat, int ld, int off, float* dp, float* buf) { return GradSrc{GRAD_POOL, dcat, ld, off, dp, buf}; };
-        if ((e = conv_backward(n, sums, L[6], B, grad(n->g_d1, c), plain(n->d1, c), plain(n->cat1, 3 * c), n->g_cat1))) break;
+        if ((e = conv_backward(n, sums, L[6], B, fused_head ? GradSrc{GRAD_DONE, nullptr, 0, 0, nullptr, nullptr} : grad(n->g_d1, c),
+                               plain(n->d1, c), plain(n->cat1, 3 * c), n->g_cat1))) break;
         if ((e = conv_backward(n, sums, L[5], B, place(n->g_cat1, 3 * c, n->g_d2), View{n->cat1, 3 * c, 0, 2},
                                plain(n->cat2, 6 * c), n->g_cat2)))
             break;
@@ -1273,6 +1359,7 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
         grad_sums_kernel<<<sums.blocks, SUM_THREADS, 0, st>>>(sums);
         if ((e = cudaGetLastError())) break;
         int bad = 0;
+        if ((e = cudaMemcpyAsync(&loss, n->dloss, sizeof(double), cudaMemcpyDeviceToHost, st))) break;
         if ((e = cudaMemcpyAsync(&bad, n->err, sizeof(int), cudaMemcpyDeviceToHost, st))) break;
         if ((e = cudaStreamSynchronize(st))) break;
         if (bad) return GDRR_ERR_TIMEOUT;
