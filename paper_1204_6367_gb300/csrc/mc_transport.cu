@@ -1009,9 +1009,9 @@ __global__ void __launch_bounds__(512, 2) mc_kernel(const McParams P) {
 //
 // A slot is Q float4 words: {px py pz, and t = xi mumax at a tentative
 // collision or the next flight's -ln xi} {dx dy dz E} {mumax 1/mumax, or the
-// optical depth and cells of LM; history id lo; job, flags} {blocks drawn,
-// block limit, history id hi, the next flight's second word} {total
-// coefficient per material}, LM {1/d, cell z}, GEN {the flight's third word,
+// optical depth and cell x of LM; history id lo; job, flags} {blocks drawn,
+// block limit, history id hi, the next flight's second word or LM's cell y}
+// {total coefficient per material}, LM {1/d, cell z}, GEN {the flight's third word,
 // interaction counts, form-factor material}.  The history's free flights so
 // far are its blocks less those drawn elsewhere, so the flight only compares
 // its block number with a limit that grows by the blocks drawn elsewhere:
@@ -1261,7 +1261,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                     if (code > F_ON) {
                         S.at(slot, 0) = make_float4(L.px, L.py, L.pz, L.tg);
                         if constexpr (LM) {
-                            S.word(slot, 2, 1) = (uint32_t)L.cx | ((uint32_t)L.cy << 16);
+                            S.word(slot, 2, 1) = (uint32_t)L.cx;
+                            S.word(slot, 3, 3) = (uint32_t)L.cy;
                             S.word(slot, S.Q_LM, 3) = (uint32_t)L.cz;
                         } else {
                             S.word(slot, 3, 0) = blk;
@@ -1294,8 +1295,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                             const float4 g = S.at(slot, S.Q_LM);
                             L.tg = a.w;
                             L.tau = c.x;
-                            L.cx = (int)(__float_as_uint(c.y) & 0xffffu);
-                            L.cy = (int)(__float_as_uint(c.y) >> 16);
+                            L.cx = __float_as_int(c.y);
+                            L.cy = (int)S.word(slot, 3, 3);
                             L.idx = g.x; L.idy = g.y; L.idz = g.z;
                             L.cz = __float_as_int(g.w);
                         } else {
@@ -1365,7 +1366,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                 S.at(slot, 0) = make_float4(L.px, L.py, L.pz, LM ? L.tg : nl);
                 if constexpr (LM) {
                     S.word(slot, 2, 0) = __float_as_uint(L.tau);
-                    S.word(slot, 2, 1) = (uint32_t)L.cx | ((uint32_t)L.cy << 16);
+                    S.word(slot, 2, 1) = (uint32_t)L.cx;
+                    S.word(slot, 3, 3) = (uint32_t)L.cy;
                     S.word(slot, S.Q_LM, 3) = (uint32_t)L.cz;
                 } else {
                     S.word(slot, 3, 0) = blk;
@@ -1413,8 +1415,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                 }
                 if (LM) {
                     const float4 g = S.at(slot, S.Q_LM);
-                    L.cx = (int)(__float_as_uint(c.y) & 0xffffu);
-                    L.cy = (int)(__float_as_uint(c.y) >> 16);
+                    L.cx = __float_as_int(c.y);
+                    L.cy = __float_as_int(d.w);
                     L.idx = g.x; L.idy = g.y; L.idz = g.z;
                     L.cz = __float_as_int(g.w);
                 }
@@ -1523,7 +1525,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
             uint32_t wy = 0;
             if constexpr (LM) {
                 c.x = L.tau;
-                c.y = __uint_as_float((uint32_t)L.cx | ((uint32_t)L.cy << 16));
+                c.y = __int_as_float(L.cx);
+                wy = (uint32_t)L.cy;
                 S.at(slot, S.Q_LM) = make_float4(L.idx, L.idy, L.idz, __int_as_float(L.cz));
             } else {
                 const uint4 w = flight_block(L.rs.blk, flight_keys(L.rs.angle, L.rs.hlo, L.rs.hhi, P.rk), P.rk);
@@ -1650,7 +1653,9 @@ cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm
     const int n_use = (int)std::min<uint64_t>((uint64_t)n_pool, share);
     const unsigned chunk = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)p.chunk, share / 4 + 1));
     McParams q = p;
-    if (!q.cells) {                 // no cell test: one cell whose bound nothing exceeds
+    // no cell test (or an axis whose corners corner_bits cannot count): one cell
+    // whose bound nothing exceeds
+    if (!q.cells || (!LM && std::max(q.nx, std::max(q.ny, q.nz)) >= 1 << 22)) {
         q.cells = q.open_cell;
         q.cshift = 30;
         q.csx = q.csy = 0;
