@@ -974,19 +974,20 @@ ConvEpi epi_f32(float* y, int ld, int H, int W) {
 
 // One convolution on the grid H x W of the plain NHWC input X (C channels)
 // into N output columns through epi: the implicit GEMM (ky-major weights w3)
-// where there are such weights (the grid tiles), else a column matrix (row K9p),
-// the column-path GEMM with w (row ldw, K = (tap, c)) into n->gemm and the
-// elementwise epilogue.
+// where there are such weights (the grid tiles), else the tap-ordered one with w
+// (row ldw, K = (tap, c)), else (channel counts that it does not take) a column
+// matrix (row K9p), the column-path GEMM with w into n->gemm and the elementwise
+// epilogue.
 cudaError_t conv_product(gdrr_cnn* n, const View& X, int C, int B, int H, int W, int ks, const bf16* w, int ldw,
                          const bf16* w3, int N, const ConvEpi& epi) {
     const int64_t P = (int64_t)B * H * W;
-    if (w3) {
+    if (w3 || (ks == 3 && conv_tap_ok(C, N))) {
         ConvArgs a;
         a.x = X.p + X.off; a.C = C; a.ldx = X.ld;
         a.B = B; a.H = H; a.W = W;
         a.w3 = w3; a.N = N;
         a.epi = epi;
-        return launch_conv_implicit(a, n->err, n->stream);
+        return w3 ? launch_conv_implicit(a, n->err, n->stream) : launch_conv_tap(a, w, ldw, n->err, n->stream);
     }
     const int K9p = pad64((int64_t)ks * ks * C);
     im2col_nhwc_kernel<<<nblk(P * (K9p / 8)), TB, 0, n->stream>>>(X, C, B, H, W, ks, K9p, n->cols);

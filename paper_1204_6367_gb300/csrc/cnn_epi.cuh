@@ -124,6 +124,11 @@ inline bool conv_implicit_ok(int C, int H, int W) {
 
 cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s);
 
+// Any other grid, with weights w[N][ldw], K = (tap, c) (a.w3 is not read): channel
+// counts that are multiples of 32; BF16 output with bias, or FP32 without.
+inline bool conv_tap_ok(int C, int N) { return C > 0 && C % 32 == 0 && N > 0 && N % 32 == 0; }
+cudaError_t launch_conv_tap(const ConvArgs& a, const __nv_bfloat16* w, int ldw, int* err, cudaStream_t s);
+
 // The implicit weight gradient applies when both channel counts are multiples
 // of 32 and 16 pixels or more fit a row (or 64 consecutive pixels are whole
 // rows of one image).

@@ -631,6 +631,9 @@ __global__ void __launch_bounds__(PERSIST_THREADS) gemm_persistent_kernel(
 // that stored each lane's pixel 16 columns at a time; 23, 17, 41, 58 and 86 so.
 constexpr int CONV_BK = 32;
 constexpr int CONV_MAX_STAGES = 8;
+// 184 KB at most, beside the epilogue's 32 KB of staged output (a store waits
+// behind the loads that the TMA unit has queued, so several are under way).
+constexpr uint32_t CONV_RING = 184u * 1024u, CONV_OUT = 32u * 1024u;
 constexpr int CONV_MAX_WIDE = 512;     // output columns whose bias the epilogue keeps in shared memory
 
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
@@ -1006,6 +1009,244 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
 }
 
 // ---------------------------------------------------------------------------
+// Implicit 3 x 3 convolution on any grid.  A tile is a box of wb x hb x bb pixels
+// (columns, rows, images; at most 128) whose input, shifted by a tap, is one
+// 4-D copy per 32 channels with zeros outside the image; K runs over (tap,
+// channel) with the weights as the column form stores them, so the sums are that
+// form's to the bit.  A stage holds `units` such steps of 32.  The box leaves as it
+// came, by one copy per 32 columns (and upsampled position) that the tensor map
+// clips at the grid's edges.
+//
+// Bound: about 400 clocks a stage of issue, then MMAs of which the box fills wb hb
+// bb of 128 rows.  Against a column matrix (9 C values per pixel written and read,
+// an FP32 product and an elementwise pass): 128 -> 256 channels on 64 grids of 12 x
+// 16, 47 us -> 20; the forward pass of 32 images of 72 x 96, 679 us -> 241, of one
+// image of 40 x 56, 181 -> 108.
+struct TapGeo {
+    int W, H, B;
+    int wb, hb, bb;        // the tile's box
+    int tx, ty;            // tiles across and down an image (group)
+    int tiles_n, n_tiles;
+    int C, n_units;        // 9 C / 32
+    int units, stages;     // steps of a stage
+    int up, fp32;
+};
+struct TapMaps {
+    CUtensorMap x, w, y[4];
+};
+
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c, int x, int y, int b) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+        :: "l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c), "r"(x), "r"(y), "r"(b)
+        : "memory");
+}
+// the four epilogue warps: a barrier, and one that says whether all of them are well
+__device__ __forceinline__ void epi_barrier() { asm volatile("barrier.cta.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ bool epi_all(bool ok) {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, 1, 128, p;\n\t"
+                 "selp.u32 %0, 1, 0, q;\n\t}" : "=r"(r) : "r"((uint32_t)ok) : "memory");
+    return r != 0;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(PERSIST_THREADS) conv_tap_kernel(const __grid_constant__ TapMaps maps, const TapGeo g,
+                                                                   int N, const float* __restrict__ bias, int relu,
+                                                                   int* err) {
+    constexpr uint32_t A_BYTES = GEMM_BM * CONV_BK * 2, UNIT = A_BYTES + BN * CONV_BK * 2;
+    constexpr int COLS = tmem_columns(2 * BN);
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[CONV_MAX_STAGES], empty_bar[CONV_MAX_STAGES], tfull[2], tempty[2];
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_fail;
+    __shared__ float s_bias[CONV_MAX_WIDE];
+    const uint32_t ring = (smem_addr(smem_raw) + 1023u) & ~1023u, stage_bytes = (uint32_t)g.units * UNIT;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto place = [&](int t, int& x0, int& y0, int& b0, int& n0) {
+        n0 = t % g.tiles_n * BN;
+        int p = t / g.tiles_n;
+        x0 = p % g.tx * g.wb;
+        p /= g.tx;
+        y0 = p % g.ty * g.hb;
+        b0 = p / g.ty * g.bb;
+    };
+    if (bias)
+        for (int i = threadIdx.x; i < N; i += PERSIST_THREADS) s_bias[i] = bias[i];
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_addr(&tmem_base)), "r"((uint32_t)COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int s = 0; s < g.stages; ++s) {
+            mbar_init(smem_addr(&full_bar[s]), 1);
+            mbar_init(smem_addr(&empty_bar[s]), 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(smem_addr(&tfull[a]), 1);
+            mbar_init(smem_addr(&tempty[a]), 4);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_fail = 0;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_base;
+
+    if (warp == 0) {
+        // producer
+        const bool leader = elect_one();
+        const uint32_t a_tx = (uint32_t)(g.wb * g.hb * g.bb) * (CONV_BK * 2);
+        int it = 0, s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
+            int x0, y0, b0, n0;
+            place(t, x0, y0, b0, n0);
+            int ch = 0, kx = -1, ky = -1;
+            for (int u = 0; u < g.n_units; ++it) {
+                if (it >= g.stages && !__all_sync(0xffffffffu, mbar_wait(smem_addr(&empty_bar[s]), ph ^ 1u))) {
+                    if (leader) atomicExch(&s_fail, 1);
+                    ok = false;
+                    break;
+                }
+                uint32_t sa = ring + (uint32_t)s * stage_bytes;
+                const uint32_t fb = smem_addr(&full_bar[s]);
+                const int end = min(g.n_units, u + g.units);
+                if (leader) mbar_expect_tx(fb, (uint32_t)(end - u) * (a_tx + BN * CONV_BK * 2));
+                for (; u < end; ++u, sa += UNIT) {
+                    if (leader) {
+                        tma_load_4d(sa, &maps.x, ch, x0 + kx, y0 + ky, b0, fb);
+                        tma_load_2d(sa + A_BYTES, &maps.w, u * CONV_BK, n0, fb);
+                    }
+                    ch += CONV_BK;
+                    if (ch == g.C) {
+                        ch = 0;
+                        if (++kx == 2) { kx = -1; ++ky; }
+                    }
+                }
+                if (++s == g.stages) { s = 0; ph ^= 1u; }
+            }
+        }
+        // the ring's last loads land before the CTA can leave (bounded)
+        const int last = min(it, g.stages);
+        for (int j = 0; j < last; ++j) {
+            const int jt = it - 1 - j;
+            mbar_wait(smem_addr(&full_bar[jt % g.stages]), (uint32_t)((jt / g.stages) & 1));
+        }
+    } else if (warp == 1) {
+        // MMA issuer
+        constexpr uint32_t idesc = instr_desc(GEMM_BM, BN);
+        const bool leader = elect_one();
+        int local = 0, s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++local) {
+            const int a = local & 1;
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&tempty[a]), (uint32_t)(((local >> 1) & 1) ^ 1)));
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t acc_tmem = tmem + (uint32_t)(a * BN);
+            for (int u = 0; u < g.n_units && ok;) {
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&full_bar[s]), ph));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                uint32_t sa = ring + (uint32_t)s * stage_bytes;
+                const int end = min(g.n_units, u + g.units);
+                for (; u < end; ++u, sa += UNIT) {
+                    const uint64_t ad = smem_desc_sw64(sa), bd = smem_desc_sw64(sa + A_BYTES);
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < CONV_BK / 16; ++kk)
+                            asm volatile(
+                                "{\n\t.reg .pred p;\n\t"
+                                "setp.ne.b32 p, %4, 0;\n\t"
+                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                :: "r"(acc_tmem), "l"(ad + (uint64_t)(kk * 2)), "l"(bd + (uint64_t)(kk * 2)), "r"(idesc),
+                                   "r"((u > 0 || kk > 0) ? 1u : 0u)
+                                : "memory");
+                    }
+                }
+                if (leader)
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                 :: "r"(smem_addr(&empty_bar[s])) : "memory");
+                __syncwarp();
+                if (++s == g.stages) { s = 0; ph ^= 1u; }
+            }
+            if (!ok && leader) atomicExch(&s_fail, 1);
+            if (leader)
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             :: "r"(smem_addr(&tfull[a])) : "memory");
+            __syncwarp();
+        }
+    } else {
+        // epilogue: rows of a box are staged as they will leave
+        const int q = warp & 3, row = q * 32 + lane;
+        const uint32_t out = ring + (uint32_t)g.stages * stage_bytes;
+        const bool store = warp == 2 && lane == 0;
+        int local = 0;
+        unsigned n_out = 0;
+        for (int t = blockIdx.x; t < g.n_tiles; t += gridDim.x, ++local) {
+            int x0, y0, b0, n0;
+            place(t, x0, y0, b0, n0);
+            const int a = local & 1;
+            const bool got = mbar_wait(smem_addr(&tfull[a]), (uint32_t)((local >> 1) & 1));
+            if (!epi_all(got && !*(volatile int*)&s_fail)) {
+                if (store) atomicExch(&s_fail, 1);
+                break;
+            }
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t lane_tmem = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN);
+            const int cols = min(BN, N - n0);
+            uint32_t r[2][32];
+            tmem_load32(r[0], lane_tmem);
+#pragma unroll
+            for (int c0 = 0; c0 < BN; c0 += 32) {
+                if (c0 >= cols) break;
+                tmem_wait_load();
+                if (c0 + 32 < cols) tmem_load32(r[(c0 / 32 + 1) & 1], lane_tmem + (uint32_t)(c0 + 32));
+                const uint32_t (&v)[32] = r[(c0 / 32) & 1];
+                const uint32_t to = out + (n_out++ & 1u) * (CONV_OUT / 2);
+                if (store) bulk_wait_read<1>();
+                epi_barrier();
+                if (!g.fp32) {
+                    uint4 o[4];
+                    epi_pack32(v, s_bias + n0 + c0, relu, o);
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) st_shared(to + row * 64 + ((h ^ ((row >> 1) & 3)) << 4), o[h]);
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 8; ++h)
+                        st_shared(to + row * 128 + ((h ^ (row & 7)) << 4),
+                                  make_uint4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]));
+                }
+                fence_async_smem();
+                epi_barrier();
+                if (store) {
+                    for (int i = 0; i < g.up * g.up; ++i) tma_store_4d(&maps.y[i], to, n0 + c0, x0, y0, b0);
+                    bulk_commit();
+                }
+                __syncwarp();
+            }
+            // this warp's TMEM reads are done: release the accumulator
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_addr(&tempty[a])) : "memory");
+        }
+        if (store) bulk_wait_all();
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && *(volatile int*)&s_fail) atomicExch(err, 1);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)COLS) : "memory");
+}
+
+// ---------------------------------------------------------------------------
 // Implicit weight gradient of a 3 x 3 convolution: dW^T[(tap, ci)][co] = the sum
 // over pixels of x[p + tap][ci] dZ[p][co], straight from the NHWC tensors.
 // Pixels are the product's K: a stage holds 64 pixels of dZ and of x shifted by
@@ -1231,10 +1472,7 @@ bool make_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int b
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Shared-memory bytes of a stage and the ring's depth (184 KB at most, beside
-// the epilogue's 32 KB of staged output: a store waits behind the loads that
-// the TMA unit has queued, so several are under way).
-constexpr uint32_t CONV_RING = 184u * 1024u, CONV_OUT = 32u * 1024u;
+// Shared-memory bytes of a stage and the ring's depth.
 uint32_t conv_a_bytes(int Wb, int mt) { return (uint32_t)(GEMM_BM * mt + 2 * Wb) * (CONV_BK * 2); }
 int conv_stages(int Wb, int BN, int mt) {
     return (int)std::min<uint32_t>(CONV_MAX_STAGES, CONV_RING / (conv_a_bytes(Wb, mt) + 3u * BN * CONV_BK * 2));
@@ -1445,6 +1683,96 @@ cudaError_t launch_conv_implicit(const ConvArgs& a, int* err, cudaStream_t s) {
         case 64: return launch_conv_bn<64>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
         case 128: return launch_conv_bn<128>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
         default: return launch_conv_bn<256>(mt, m, g, (int)M, a.N, a.epi, n_sm, err, s);
+    }
+}
+
+// The tap-ordered convolution (conv_tap_ok) with weights w[N][ldw], K = (tap, c).
+// Its box: whole rows where one fits 128 pixels, as many rows (images) as fill
+// them; the widest column tile of 128, 96, 64 and 32 that divides N, halved in
+// steps while the tiles are fewer than the SMs.
+cudaError_t launch_conv_tap(const ConvArgs& a, const __nv_bfloat16* w, int ldw, int* err, cudaStream_t s) {
+    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+    if (!fn) return cudaErrorNotSupported;
+    const ConvEpi& epi = a.epi;
+    const bool half = epi.y16 && !epi.yf;
+    if (!conv_tap_ok(a.C, a.N) || (int64_t)a.B * a.H * a.W > INT32_MAX || a.ldx % 8 || a.ldx < a.C || ldw % 8 ||
+        epi.head_out || (half ? epi.ldy % 8 || epi.off % 8 || !epi.bias || a.N > CONV_MAX_WIDE
+                              : !epi.yf || epi.y16 || epi.bias || epi.ldf % 4) ||
+        ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(epi.y16) |
+          reinterpret_cast<uintptr_t>(epi.yf)) & 15u) != 0)
+        return cudaErrorInvalidValue;
+    int dev = 0, n_sm = 1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    TapGeo g;
+    g.W = a.W;
+    g.H = a.H;
+    g.B = a.B;
+    g.tx = (a.W + GEMM_BM - 1) / GEMM_BM;
+    g.wb = (a.W + g.tx - 1) / g.tx;
+    g.hb = std::min(a.H, GEMM_BM / g.wb);
+    g.ty = (a.H + g.hb - 1) / g.hb;
+    g.hb = (a.H + g.ty - 1) / g.ty;
+    g.bb = g.ty == 1 && g.tx == 1 ? std::min(a.B, GEMM_BM / (g.wb * g.hb)) : 1;
+    const int pixel_tiles = g.tx * g.ty * ((a.B + g.bb - 1) / g.bb);
+    int BN = a.N % 128 == 0 ? 128 : a.N % 96 == 0 ? 96 : a.N % 64 == 0 ? 64 : 32;
+    while (BN > 32 && a.N % (BN / 2) == 0 && BN % 64 == 0 && (int64_t)pixel_tiles * (a.N / BN) < n_sm) BN /= 2;
+    g.tiles_n = a.N / BN;
+    g.n_tiles = pixel_tiles * g.tiles_n;
+    g.C = a.C;
+    g.n_units = 9 * (a.C / CONV_BK);
+    g.units = BN <= 64 ? 4 : 3;
+    const uint32_t stage = (uint32_t)g.units * (GEMM_BM + BN) * CONV_BK * 2;
+    g.stages = (int)std::min<uint32_t>(CONV_MAX_STAGES, CONV_RING / stage);
+    g.up = half ? epi.up : 1;
+    g.fp32 = half ? 0 : 1;
+    TapMaps m;
+    const cuuint32_t elem[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)CONV_BK, (cuuint32_t)g.wb, (cuuint32_t)g.hb, (cuuint32_t)g.bb};
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
+        const cuuint64_t px = (cuuint64_t)a.ldx * 2;
+        const cuuint64_t strides[3] = {px, px * a.W, px * a.W * a.H};
+        if (fn(&m.x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(a.x), dims, strides, box, elem,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)9 * a.C, (cuuint64_t)a.N};
+        const cuuint64_t strides[1] = {(cuuint64_t)ldw * 2};
+        const cuuint32_t wbox[2] = {(cuuint32_t)CONV_BK, (cuuint32_t)BN};
+        if (fn(&m.w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(w), dims, strides, wbox, elem,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    for (int i = 0; i < 4; ++i) {
+        const int k = i < g.up * g.up ? i : 0;             // (the unused ones are copies)
+        const cuuint64_t size = half ? 2 : 4, px = (cuuint64_t)(half ? epi.ldy : epi.ldf) * size;
+        const cuuint64_t line = px * a.W * g.up;           // a row of the output grid
+        const cuuint64_t dims[4] = {(cuuint64_t)a.N, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
+        const cuuint64_t strides[3] = {px * g.up, line * g.up, line * g.up * a.H};
+        uint8_t* base = half ? reinterpret_cast<uint8_t*>(epi.y16 + epi.off) : reinterpret_cast<uint8_t*>(epi.yf);
+        base += (k / g.up) * line + (k % g.up) * px;
+        if (fn(&m.y[i], half ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box,
+               elem, CU_TENSOR_MAP_INTERLEAVE_NONE, half ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    const size_t smem = (size_t)g.stages * stage + CONV_OUT + 1024;
+    auto launch = [&](auto kernel) {
+        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (r != cudaSuccess) return r;
+        kernel<<<std::min(g.n_tiles, n_sm), PERSIST_THREADS, smem, s>>>(m, g, a.N, half ? epi.bias : nullptr, epi.relu, err);
+        return cudaGetLastError();
+    };
+    switch (BN) {
+        case 32: return launch(conv_tap_kernel<32>);
+        case 64: return launch(conv_tap_kernel<64>);
+        case 96: return launch(conv_tap_kernel<96>);
+        default: return launch(conv_tap_kernel<128>);
     }
 }
 

@@ -29,7 +29,7 @@ def _rel(a, b):
 
 @pytest.mark.parametrize("c, H, W, B", [(8, 8, 8, 1), (24, 16, 24, 2), (32, 64, 64, 1), (32, 40, 128, 2), (48, 32, 32, 1),
                                         (64, 32, 64, 1), (32, 16, 256, 1), (16, 32, 128, 3), (32, 8, 128, 1), (32, 24, 48, 2),
-                                        (32, 24, 40, 3)])
+                                        (32, 24, 40, 3), (32, 8, 136, 2)])
 def test_forward_and_gradients(gd, c, H, W, B):
     rng = np.random.default_rng(c * H + W)
     flat = ocnn.init_params(c, c + H).astype(np.float32)
