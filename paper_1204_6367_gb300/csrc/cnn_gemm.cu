@@ -29,6 +29,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <numeric>
 
@@ -1009,6 +1010,243 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
 }
 
 // ---------------------------------------------------------------------------
+// Paired form for wide outputs: two CTAs of a cluster share a tile of 256 x 256.
+// Each copies its 128 rows of A and 128 of the columns of B; one instruction of
+// the even CTA multiplies both halves (cta_group::2), so a CTA copies and reads
+// half the columns that it multiplies by.  Its 128 rows of the accumulator lie in
+// its own TMEM, twice, and leave 32 columns at a time by TMA under the next tile's
+// MMAs.  The roles are the persistent form's; the even CTA's "full" barriers count
+// both CTAs' copies, its commits reach both CTAs' "empty" and accumulator barriers,
+// and both epilogues release an accumulator to it.
+//
+// Bound: the tensor cores (8192^3 at 0.94 of the measured cuBLAS rate).  One CTA a
+// tile of 128 x 256, whose instruction takes 175 clocks where the peak's rate is
+// 128, and lanes that store their rows: 8192^3 in 0.69 ms, 0.60 so; a call at 8192
+// x 8192 x 512 156 us -> 126, x 64, where the epilogue bound it, 140 -> 86.
+constexpr int PAIR_BN = 256, PAIR_STAGES = 6;
+constexpr uint32_t PAIR_HALF = 128 * GEMM_BK * 2;                    // a CTA's part of an operand's stage
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// the even CTA's copy of a shared-memory address
+__device__ __forceinline__ uint32_t even_cta(uint32_t addr) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+        "[%4];"
+        :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 :: "r"(bar), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
+                 :: "l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PERSIST_THREADS) gemm_pair_kernel(
+        const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+        const __grid_constant__ CUtensorMap mapC, int M, int N, int K, int k_split, int n_splits, int* err) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[PAIR_STAGES], empty_bar[PAIR_STAGES], tfull[2], tempty[2];
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_fail;
+    const uint32_t ring = (smem_addr(smem_raw) + 1023u) & ~1023u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int tiles_m = (M + 255) / 256, tiles_n = (N + PAIR_BN - 1) / PAIR_BN;
+    const int per_split = tiles_m * tiles_n, n_tiles = per_split * n_splits;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_addr(&tmem_base)), "r"((uint32_t)(2 * PAIR_BN)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int s = 0; s < PAIR_STAGES; ++s) {
+            mbar_init(smem_addr(&full_bar[s]), 1);
+            mbar_init(smem_addr(&empty_bar[s]), 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(smem_addr(&tfull[a]), 1);
+            mbar_init(smem_addr(&tempty[a]), 8);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_fail = 0;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_barrier();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_base;
+
+    // tile t -> (m0, n0, k range): grouped order within a split
+    auto tile_coords = [&](int t, int& m0, int& n0, int& split, int& k_begin, int& n_iter) {
+        split = t / per_split;
+        const int r = t % per_split, group = GROUP_M / 2;
+        const int per_group = group * tiles_n;
+        const int grp = r / per_group, in_grp = r % per_group;
+        const int first_m = grp * group;
+        const int size_m = min(group, tiles_m - first_m);
+        m0 = (first_m + in_grp % size_m) * 256 + (int)rank * 128;
+        n0 = (in_grp / size_m) * PAIR_BN;
+        k_begin = split * k_split;
+        n_iter = (min(K, k_begin + k_split) - k_begin) / GEMM_BK;
+    };
+
+    if (warp == 0) {
+        // producer: the ring's stage counter runs across tiles
+        const bool leader = elect_one();
+        int it = 0, s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = pair; t < n_tiles && ok; t += n_pairs) {
+            int m0, n0, split, kb, n_iter;
+            tile_coords(t, m0, n0, split, kb, n_iter);
+            for (int i = 0; i < n_iter; ++i, ++it) {
+                if (it >= PAIR_STAGES && !__all_sync(0xffffffffu, mbar_wait(smem_addr(&empty_bar[s]), ph ^ 1u))) {
+                    if (leader) atomicExch(&s_fail, 1);
+                    ok = false;
+                    break;
+                }
+                const uint32_t sa = ring + (uint32_t)s * (2 * PAIR_HALF);
+                const uint32_t fb = even_cta(smem_addr(&full_bar[s]));
+                if (leader) {
+                    if (rank == 0) mbar_expect_tx(smem_addr(&full_bar[s]), 4 * PAIR_HALF);
+                    tma_load_2d_pair(sa, &mapA, kb + i * GEMM_BK, m0, fb);
+                    tma_load_2d_pair(sa + PAIR_HALF, &mapB, kb + i * GEMM_BK, n0 + (int)rank * 128, fb);
+                }
+                __syncwarp();
+                if (++s == PAIR_STAGES) { s = 0; ph ^= 1u; }
+            }
+        }
+        // the ring's last loads, both CTAs', land before the CTAs can leave (bounded)
+        if (rank == 0) {
+            const int last = min(it, PAIR_STAGES);
+            for (int j = 0; j < last; ++j) {
+                const int jt = it - 1 - j;
+                mbar_wait(smem_addr(&full_bar[jt % PAIR_STAGES]), (uint32_t)((jt / PAIR_STAGES) & 1));
+            }
+        }
+    } else if (warp == 1) {
+        if (rank == 0) {
+            // MMA issuer of both CTAs
+            constexpr uint32_t idesc = instr_desc(256, PAIR_BN);
+            const bool leader = elect_one();
+            int local = 0, s = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int t = pair; t < n_tiles && ok; t += n_pairs, ++local) {
+                int m0, n0, split, kb, n_iter;
+                tile_coords(t, m0, n0, split, kb, n_iter);
+                const int a = local & 1;
+                // the accumulator is free once both epilogues released its previous tile
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&tempty[a]), (uint32_t)(((local >> 1) & 1) ^ 1)));
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t acc_tmem = tmem + (uint32_t)(a * PAIR_BN);
+                for (int i = 0; i < n_iter && ok; ++i) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&full_bar[s]), ph));
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t sa = ring + (uint32_t)s * (2 * PAIR_HALF);
+                    const uint64_t ad = smem_desc_sw128(sa), bd = smem_desc_sw128(sa + PAIR_HALF);
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < GEMM_BK / 16; ++kk)
+                            asm volatile(
+                                "{\n\t.reg .pred p;\n\t"
+                                "setp.ne.b32 p, %4, 0;\n\t"
+                                "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                :: "r"(acc_tmem), "l"(ad + (uint64_t)(kk * 2)), "l"(bd + (uint64_t)(kk * 2)), "r"(idesc),
+                                   "r"((i > 0 || kk > 0) ? 1u : 0u)
+                                : "memory");
+                        commit_pair(smem_addr(&empty_bar[s]));
+                    }
+                    __syncwarp();
+                    if (++s == PAIR_STAGES) { s = 0; ph ^= 1u; }
+                }
+                if (!ok && leader) atomicExch(&s_fail, 1);
+                if (leader) commit_pair(smem_addr(&tfull[a]));
+                __syncwarp();
+            }
+        }
+    } else {
+        // epilogue: this CTA's 128 rows, 32 columns at a time (two 4 KB buffers of
+        // 128-byte rows a warp, 128-byte swizzle)
+        const int q = warp & 3;
+        const uint32_t stage_out = ring + PAIR_STAGES * 2 * PAIR_HALF + (uint32_t)q * 8192u;
+        int local = 0;
+        unsigned n_out = 0;
+        for (int t = pair; t < n_tiles; t += n_pairs, ++local) {
+            int m0, n0, split, kb, n_iter;
+            tile_coords(t, m0, n0, split, kb, n_iter);
+            const int a = local & 1;
+            const bool got = mbar_wait(smem_addr(&tfull[a]), (uint32_t)((local >> 1) & 1));
+            if (!__all_sync(0xffffffffu, got && !*(volatile int*)&s_fail)) {
+                if (lane == 0) atomicExch(&s_fail, 1);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t lane_tmem = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * PAIR_BN);
+            const int row0 = m0 + q * 32, cols = min(PAIR_BN, N - n0);
+            uint32_t r[2][32];
+            tmem_load32(r[0], lane_tmem);
+#pragma unroll
+            for (int c0 = 0; c0 < PAIR_BN; c0 += 32) {
+                if (c0 >= cols) break;
+                tmem_wait_load();
+                if (c0 + 32 < cols) tmem_load32(r[(c0 / 32 + 1) & 1], lane_tmem + (uint32_t)(c0 + 32));
+                const uint32_t (&v)[32] = r[(c0 / 32) & 1];
+                const uint32_t to = stage_out + (n_out++ & 1u) * 4096u;
+                if (lane == 0) bulk_wait_read<1>();
+                __syncwarp();
+#pragma unroll
+                for (int h = 0; h < 8; ++h)
+                    st_shared(to + lane * 128 + ((h ^ (lane & 7)) << 4),
+                              make_uint4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]));
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0 && row0 < M) {
+                    tma_store_3d(&mapC, to, n0 + c0, row0, split);
+                    bulk_commit();
+                }
+                __syncwarp();
+            }
+            // this warp's TMEM reads are done: release the accumulator to the even CTA
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];"
+                             :: "r"(even_cta(smem_addr(&tempty[a]))) : "memory");
+        }
+        if (lane == 0) bulk_wait_all();
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && *(volatile int*)&s_fail) atomicExch(err, 1);
+    __syncwarp();
+    cluster_barrier();                    // neither CTA leaves or frees TMEM while the other may still reach it
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"
+                     :: "r"(tmem), "r"((uint32_t)(2 * PAIR_BN)) : "memory");
+    cluster_barrier();
+}
+
+// ---------------------------------------------------------------------------
 // Implicit 3 x 3 convolution on any grid.  A tile is a box of wb x hb x bb pixels
 // (columns, rows, images; at most 128) whose input, shifted by a tap, is one
 // 4-D copy per 32 channels with zeros outside the image; K runs over (tap,
@@ -1583,6 +1821,54 @@ cudaError_t launch_persistent_t(const __nv_bfloat16* A, int lda, const __nv_bflo
     return cudaGetLastError();
 }
 
+// The paired form, for outputs that TMA can store (16-byte rows, no adding splits).
+cudaError_t launch_pair(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, float* C, int ldc, int M, int N,
+                        int K, int splits, int64_t partial_stride, int* err, cudaStream_t s) {
+    const int k_slices = K / GEMM_BK;
+    splits = max(1, min(splits, k_slices));
+    const int per = (k_slices + splits - 1) / splits;
+    splits = (k_slices + per - 1) / per;
+    CUtensorMap mA, mB, mC;
+    if (!make_map(&mA, A, M, K, lda, 128) || !make_map(&mB, B, N, K, ldb, 128)) return cudaErrorInvalidValue;
+    {
+        const cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)splits};
+        const cuuint64_t strides[2] = {(cuuint64_t)ldc * 4, (cuuint64_t)(splits > 1 ? partial_stride : (int64_t)ldc * M) * 4};
+        const cuuint32_t box[3] = {32, 32, 1};
+        const cuuint32_t elem[3] = {1, 1, 1};
+        if (encode_fn()(&mC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, C, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    const size_t smem = (size_t)PAIR_STAGES * 2 * PAIR_HALF + CONV_OUT + 1024;
+    cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    // as many pairs as are resident at once (an odd SM of a cluster group stays idle)
+    static std::atomic<int> resident[64];
+    int dev = 0, pairs = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if (dev < 64) pairs = resident[dev].load(std::memory_order_relaxed);
+    if (pairs == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2);
+        cfg.blockDim = dim3(PERSIST_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if ((e = cudaOccupancyMaxActiveClusters(&pairs, gemm_pair_kernel, &cfg)) != cudaSuccess) return e;
+        if (pairs <= 0) return cudaErrorInvalidConfiguration;
+        if (dev < 64) resident[dev].store(pairs, std::memory_order_relaxed);
+    }
+    const int64_t n_tiles = (int64_t)((M + 255) / 256) * ((N + PAIR_BN - 1) / PAIR_BN) * splits;
+    const int grid = 2 * (int)std::min<int64_t>(n_tiles, pairs);
+    gemm_pair_kernel<<<grid, PERSIST_THREADS, smem, s>>>(mA, mB, mC, M, N, K, per * GEMM_BK, splits, err);
+    return cudaGetLastError();
+}
+
 template <int BN>
 cudaError_t launch_gemm_t(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, float* C, int ldc,
                           int M, int N, int K, int splits, int64_t partial_stride, int* err, cudaStream_t s) {
@@ -1894,9 +2180,11 @@ cudaError_t launch_gemm_bf16(const void* A, int lda, const void* B, int ldb, flo
         *splits_used = (k_slices + per - 1) / per;
     }
     if (N < 32) return launch_gemm_t<32>(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
-    // measured at 8192^3 (fraction of the BF16 peak): persistent 256-wide tiles
-    // with two TMEM accumulators 0.78; per-tile CTAs, two per SM, 256 x 2
-    // stages 0.74 and 128 x 3 stages 0.67 (persistent 128-wide: 0.52).
+    // measured at 8192^3 (fraction of the BF16 peak): pairs of CTAs on 256 x 256
+    // 0.94; one CTA a tile, persistent and 256 wide with two TMEM accumulators
+    // 0.78, which takes what the pairs' TMA stores cannot (rows of C that are not
+    // multiples of 16 bytes, splits that add up in place) and a single row of
+    // tiles; per-tile CTAs, two per SM, 256 x 2 stages 0.74 and 128 x 3 0.67.
     // Narrow outputs (the 32- and 64-channel convolutions: tall A streams
     // from memory, little work per tile) take the persistent form with a deep
     // operand ring.
@@ -1905,6 +2193,9 @@ cudaError_t launch_gemm_bf16(const void* A, int lda, const void* B, int ldb, flo
             return launch_persistent_t<32, 8>(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
         if (N <= 64)
             return launch_persistent_t<64, 6>(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
+        if (N >= 256 && M > 128 && ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0 &&
+            (splits == 1 || (partial_stride > 0 && partial_stride % 4 == 0)))
+            return launch_pair(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
         if (N >= 256)
             return launch_persistent_t<256, 4>(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
         return launch_tma_t<128, 3>(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
