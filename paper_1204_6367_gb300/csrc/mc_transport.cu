@@ -151,6 +151,34 @@ __device__ __forceinline__ float gd_logf(float x) {
     return fe * (float)(2839.0 / 4096.0) + (fe * (float)(0.69314718055994530942 - 2839.0 / 4096.0) + lm);
 }
 
+// n / d for the logarithm's arguments (n = m - 1, d = m + 1, m in
+// [sqrt(1/2), sqrt(2))): the quotient from an approximate reciprocal and
+// Markstein's residual correction (P. Markstein, IBM J. Res. Dev. 34, 1990).
+// Equal to the correctly rounded quotient for every m of a 24-bit uniform (all
+// 2^24 compared), without the general division's range test and branch.
+__device__ __forceinline__ float log_quotient(float n, float d) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+    const float q = __fmul_rn(n, y);
+    return __fmaf_rn(__fmaf_rn(-d, q, n), y, q);
+}
+
+// gd_logf(k 2^-24) for an integer 1 <= k <= 2^24: the same series on the same
+// m and e, which one addition separates (it carries into the exponent exactly
+// when the mantissa exceeds sqrt(2)'s).
+__device__ __forceinline__ float log_uniform(uint32_t k) {
+    constexpr uint32_t CARRY = 0x00800000u - 0x003504f4u;
+    const uint32_t t = __float_as_uint((float)k) + CARRY;
+    const float fe = __uint_as_float(0x4b000000u | (t >> 23)) - 8388759.0f;     // (t >> 23) - 127 - 24
+    const float m = __uint_as_float((t & 0x007fffffu) + (0x3f800000u - CARRY));
+    const float s = log_quotient(m - 1.0f, m + 1.0f);
+    const float s2 = s * s;
+    const float poly = (float)(1.0 / 3.0) + s2 * ((float)(1.0 / 5.0) + s2 * ((float)(1.0 / 7.0)
+                     + s2 * ((float)(1.0 / 9.0) + s2 * (float)(1.0 / 11.0))));
+    const float lm = 2.0f * s + (2.0f * s) * (s2 * poly);
+    return fe * (float)(2839.0 / 4096.0) + (fe * (float)(0.69314718055994530942 - 2839.0 / 4096.0) + lm);
+}
+
 // Inverse-CDF search in integers.  A uniform is xi = k 2^-24 with k the top
 // 24 bits of its word plus one, and xi <= cdf[j] holds exactly when
 // k <= floor(cdf[j] 2^24) = kcdf[j]; the smallest such j is the sample.  The
@@ -698,7 +726,7 @@ struct Lane {
         const uint4 wf = rs.block(P.rk);
         ++nsteps;
         if (GEN) ++c_steps;
-        tau = -gd_logf(uniform(wf.x));
+        tau = -log_uniform((wf.x >> 8) + 1u);
         tg = uniform(wf.y);
         if (GEN) wz = wf.z;
     }
@@ -712,16 +740,13 @@ struct Lane {
     // a flight crosses at most ncx + ncy + ncz cells; leaving the grid leaves
     // the box, from the last position inside.
     __device__ __forceinline__ void walk(const McParams& P, float b) {
-        float tx = (float)3.0e38, ty = tx, tz = tx;
-        if (dx > 0.0f) tx = (lm_plane(P, 0, cx + 1, P.ncx) - px) * idx;
-        else if (dx < 0.0f) tx = (lm_plane(P, 0, cx, P.ncx) - px) * idx;
-        if (dy > 0.0f) ty = (lm_plane(P, 1, cy + 1, P.ncy) - py) * idy;
-        else if (dy < 0.0f) ty = (lm_plane(P, 1, cy, P.ncy) - py) * idy;
-        if (dz > 0.0f) tz = (lm_plane(P, 2, cz + 1, P.ncz) - pz) * idz;
-        else if (dz < 0.0f) tz = (lm_plane(P, 2, cz, P.ncz) - pz) * idz;
-        if (dx != 0.0f && !(tx > 0.0f)) tx = 0.0f;       // already on the plane
-        if (dy != 0.0f && !(ty > 0.0f)) ty = 0.0f;
-        if (dz != 0.0f && !(tz > 0.0f)) tz = 0.0f;
+        // distance to the cell's exit plane of an axis (0 when already on it)
+        auto exit_at = [&](int ax, int c, int n, float d, float p, float id) {
+            const float l = (lm_plane(P, ax, d > 0.0f ? c + 1 : c, n) - p) * id;
+            return d != 0.0f ? (l > 0.0f ? l : 0.0f) : (float)3.0e38;
+        };
+        const float tx = exit_at(0, cx, P.ncx, dx, px, idx), ty = exit_at(1, cy, P.ncy, dy, py, idy),
+                    tz = exit_at(2, cz, P.ncz, dz, pz, idz);
         const float t = fminf(tx, fminf(ty, tz));
         const float bt = b * t;
         if (tau < bt) {
@@ -1027,6 +1052,10 @@ constexpr int POOL_DEFAULT = 80;               // photons per warp: the most tha
 // Idle lanes at which the warp hands over and refills: 5, 6, 8 and 12 were
 // within 2 %, 4 was 3 % slower (a hand-over costs about half a flight).
 constexpr int REFILL_IDLE = 8;
+// With local majorants a third of the flights stop in every cell, so a refill at 8
+// would come after each: 2e7 histories of the 2 mm torso take 14.17 ms at 8, 13.93
+// at 14, 13.67 at 18, 13.57 from 20 to 24 and 14.17 at 30.
+constexpr int REFILL_IDLE_LM = 22;
 // a slot's flags beside its job
 constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_VIRTUAL = 0x10000000u,
                    JF_JOB = 0x0fffffffu;
@@ -1147,34 +1176,6 @@ __device__ __forceinline__ uint4 flight_block(uint32_t blk, const FlightKeys& k,
     return make_uint4(c0, c1, c2, c3);
 }
 
-// n / d for the logarithm's arguments (n = m - 1, d = m + 1, m in
-// [sqrt(1/2), sqrt(2))): the quotient from an approximate reciprocal and
-// Markstein's residual correction (P. Markstein, IBM J. Res. Dev. 34, 1990).
-// Equal to the correctly rounded quotient for every m of a 24-bit uniform (all
-// 2^24 compared), without the general division's range test and branch.
-__device__ __forceinline__ float log_quotient(float n, float d) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
-    const float q = __fmul_rn(n, y);
-    return __fmaf_rn(__fmaf_rn(-d, q, n), y, q);
-}
-
-// gd_logf(k 2^-24) for an integer 1 <= k <= 2^24: the same series on the same
-// m and e, which one addition separates (it carries into the exponent exactly
-// when the mantissa exceeds sqrt(2)'s).
-__device__ __forceinline__ float log_uniform(uint32_t k) {
-    constexpr uint32_t CARRY = 0x00800000u - 0x003504f4u;
-    const uint32_t t = __float_as_uint((float)k) + CARRY;
-    const float fe = __uint_as_float(0x4b000000u | (t >> 23)) - 8388759.0f;     // (t >> 23) - 127 - 24
-    const float m = __uint_as_float((t & 0x007fffffu) + (0x3f800000u - CARRY));
-    const float s = log_quotient(m - 1.0f, m + 1.0f);
-    const float s2 = s * s;
-    const float poly = (float)(1.0 / 3.0) + s2 * ((float)(1.0 / 5.0) + s2 * ((float)(1.0 / 7.0)
-                     + s2 * ((float)(1.0 / 9.0) + s2 * (float)(1.0 / 11.0))));
-    const float lm = 2.0f * s + (2.0f * s) * (s2 * poly);
-    return fe * (float)(2839.0 / 4096.0) + (fe * (float)(0.69314718055994530942 - 2839.0 / 4096.0) + lm);
-}
-
 // 0x4b000000 + floor(y - 1/2) for y = (x - lo) / vox >= 0: adding 2^23 - 1/2
 // with rounding down leaves the floor in the low bits (the sum is formed
 // exactly before it is rounded, and floorf(y - 0.5f) is the same floor: y -
@@ -1255,7 +1256,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
             for (;;) {
                 const unsigned act = __ballot_sync(FULL, code == F_ON);
                 int n_act = __popc(act);
-                if (n_act <= 32 - REFILL_IDLE) {
+                if (n_act <= 32 - (LM ? REFILL_IDLE_LM : REFILL_IDLE)) {
                     // hand over the photons whose flight stopped, refill the lanes
                     const unsigned mG = __ballot_sync(FULL, code == F_GATHER), mE = __ballot_sync(FULL, code >= F_ESC);
                     if (code > F_ON) {
