@@ -345,6 +345,33 @@ __device__ __forceinline__ void polar(Stream& rs, const RoundKeys& rk, bool ray,
     }
 }
 
+// The eight corners of a trilinear cell: weight times density, and material.
+__device__ __forceinline__ void corners(const McParams& P, float px, float py, float pz, float (&a)[8], int (&mc)[8]) {
+    const float fx = (px - P.lo[0]) * P.ivox[0] - 0.5f;
+    const float fy = (py - P.lo[1]) * P.ivox[1] - 0.5f;
+    const float fz = (pz - P.lo[2]) * P.ivox[2] - 0.5f;
+    const int gx = (int)floorf(fx), gy = (int)floorf(fy), gz = (int)floorf(fz);
+    const float tx = fx - (float)gx, ty = fy - (float)gy, tz = fz - (float)gz;
+    // inside the box f lies in [-1/2, n - 1/2], so g in [-1, n - 1]: the
+    // lower corner clamps only from below, the upper only from above
+    const int x0 = max(gx, 0), x1 = min(gx + 1, P.nx - 1);
+    const int y0 = max(gy, 0), y1 = min(gy + 1, P.ny - 1);
+    const int z0 = max(gz, 0), z1 = min(gz + 1, P.nz - 1);
+    const float wx0 = 1.0f - tx, wy0 = 1.0f - ty, wz0 = 1.0f - tz;
+    const float wxy[4] = {wx0 * wy0, tx * wy0, wx0 * ty, tx * ty};
+    const int bx[2] = {brick_x(x0), brick_x(x1)};
+    const int by[2] = {brick_y(y0, P.bsy), brick_y(y1, P.bsy)};
+    const int bz[2] = {brick_z(z0, P.bsz), brick_z(z1, P.bsz)};
+    const int rows[4] = {by[0] + bz[0], by[1] + bz[0], by[0] + bz[1], by[1] + bz[1]};
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int v = rows[c >> 1] + bx[c & 1];
+        const uint2 vx = __ldg(P.vox + v);
+        a[c] = (wxy[c & 3] * ((c >> 2) ? tz : wz0)) * __uint_as_float(vx.x);
+        mc[c] = (int)vx.y;
+    }
+}
+
 enum : uint32_t { OUT_PRIMARY = 0, OUT_SCATTER = 1, OUT_PHOTO = 2, OUT_CUTOFF = 3, OUT_MISS = 4, OUT_STEP_LIMIT = 5 };
 
 // Lane states.  A lane whose history needs an interaction, a tally or a new
@@ -802,31 +829,9 @@ struct Lane {
             real_collision(P, t, a0 * cf(1, m0), a0 * cf(2, m0), cnt);
             return;
         }
-        const float fx = (px - P.lo[0]) * P.ivox[0] - 0.5f;
-        const float fy = (py - P.lo[1]) * P.ivox[1] - 0.5f;
-        const float fz = (pz - P.lo[2]) * P.ivox[2] - 0.5f;
-        const int gx = (int)floorf(fx), gy = (int)floorf(fy), gz = (int)floorf(fz);
-        const float tx = fx - (float)gx, ty = fy - (float)gy, tz = fz - (float)gz;
-        // inside the box f lies in [-1/2, n - 1/2], so g in [-1, n - 1]: the
-        // lower corner clamps only from below, the upper only from above
-        const int x0 = max(gx, 0), x1 = min(gx + 1, P.nx - 1);
-        const int y0 = max(gy, 0), y1 = min(gy + 1, P.ny - 1);
-        const int z0 = max(gz, 0), z1 = min(gz + 1, P.nz - 1);
-        const float wx0 = 1.0f - tx, wy0 = 1.0f - ty, wz0 = 1.0f - tz;
-        const float wxy[4] = {wx0 * wy0, tx * wy0, wx0 * ty, tx * ty};
-        const int bx[2] = {brick_x(x0), brick_x(x1)};
-        const int by[2] = {brick_y(y0, P.bsy), brick_y(y1, P.bsy)};
-        const int bz[2] = {brick_z(z0, P.bsz), brick_z(z1, P.bsz)};
-        const int rows[4] = {by[0] + bz[0], by[1] + bz[0], by[0] + bz[1], by[1] + bz[1]};
         float a[8];
         int mc[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int v = rows[c >> 1] + bx[c & 1];
-            const uint2 vx = __ldg(P.vox + v);
-            a[c] = (wxy[c & 3] * ((c >> 2) ? tz : wz0)) * __uint_as_float(vx.x);
-            mc[c] = (int)vx.y;
-        }
+        corners(P, px, py, pz, a, mc);
         float muT = a[0] * total(mc[0]);
 #pragma unroll
         for (int c = 1; c < 8; ++c) muT = muT + a[c] * total(mc[c]);
@@ -1057,8 +1062,7 @@ constexpr int REFILL_IDLE = 8;
 // at 14, 13.67 at 18, 13.57 from 20 to 24 and 14.17 at 30.
 constexpr int REFILL_IDLE_LM = 22;
 // a slot's flags beside its job
-constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_VIRTUAL = 0x10000000u,
-                   JF_JOB = 0x0fffffffu;
+constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_JOB = 0x1fffffffu;
 
 template <int NM, bool GEN, bool LM>
 struct Slots {
@@ -1327,8 +1331,19 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                         // what decides a tentative collision is loaded first ...
                         float v[NM];
                         uint2 vx = make_uint2(0u, 0u);
-                        const bool nearest = GEN && P.nearest_voxel;
-                        if (nearest) {
+                        const bool nearest = GEN && P.nearest_voxel, open = GEN && P.cells == P.open_cell;
+                        float mu = 0.0f;
+                        if (open && !nearest) {
+                            // no cell test: the mixture itself, here where nearly all are virtual
+                            if (inside) {
+                                float a[8];
+                                int mc[8];
+                                corners(P, qx, qy, qz, a, mc);
+                                mu = a[0] * __uint_as_float(S.word(slot, 4, mc[0]));
+#pragma unroll
+                                for (int c = 1; c < 8; ++c) mu = mu + a[c] * __uint_as_float(S.word(slot, 4, mc[c]));
+                            }
+                        } else if (nearest) {
                             const int gx = min(max((int)floorf((qx - P.lo[0]) * P.ivox[0]), 0), P.nx - 1);
                             const int gy = min(max((int)floorf((qy - P.lo[1]) * P.ivox[1]), 0), P.ny - 1);
                             const int gv = min(max((int)floorf((qz - P.lo[2]) * P.ivox[2]), 0), P.nz - 1);
@@ -1350,7 +1365,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                         wy = w.y;
                         if (GEN) wz = w.z;
                         const bool skip = t > (nearest ? __uint_as_float(vx.x) * __uint_as_float(S.word(slot, 4, (int)vx.y))
-                                                       : bound_of<NM>(v, cf));
+                                                       : open ? mu : bound_of<NM>(v, cf));
                         L.tg = t;
                         if (inside) { L.px = qx; L.py = qy; L.pz = qz; }
                         code = skip ? F_ON : F_GATHER;
@@ -1438,24 +1453,22 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
             }
             tally(GDRR_ST_VIRTUAL, L.state == S_FLY);
             tally(GDRR_ST_PHOTO, ev.has(GDRR_ST_PHOTO));
-            // the interaction waits for its own full warp; so do the few virtual
-            // collisions, for that service's next-flight words (not LM, where
-            // most are virtual: they draw their next flight here)
-            const bool hit = L.state == S_RAY || L.state == S_COMP, wait = hit || (!LM && L.state == S_FLY);
-            const unsigned mI = __ballot_sync(FULL, wait);
-            if (wait) {
-                S.word(slot, 2, 3) = jf | (L.state == S_RAY ? JF_RAYLEIGH : 0u) | (hit ? 0u : JF_VIRTUAL);
+            // the interaction waits for its own full warp; a virtual collision draws
+            // its next flight here (through the interactions' list, where that is a
+            // full warp's, 2 mm torsos took 1 % longer with cells of 4 mm, 4 % with 8
+            // and 25 % with 128)
+            const bool hit = L.state == S_RAY || L.state == S_COMP;
+            const unsigned mI = __ballot_sync(FULL, hit);
+            if (hit) {
+                S.word(slot, 2, 3) = jf | (L.state == S_RAY ? JF_RAYLEIGH : 0u);
                 if (GEN) S.word(slot, S.Q_GEN, 2) = (uint32_t)L.m_ray;
                 qI[nI + __popc(mI & below)] = (uint8_t)slot;
-                if (!hit) L.state = S_COMP;       // it does not fly on from here
             }
             nI += __popc(mI);
             add(A_GATHER, (unsigned)n);
         } else if (which == S_COMP) {
-            const bool real = slot >= 0 && !(jf & JF_VIRTUAL);
-            jf &= ~(JF_VIRTUAL | JF_RAYLEIGH);
-            if (slot >= 0 && !real) L.state = S_FLY;
-            if (real) {
+            jf &= ~JF_RAYLEIGH;
+            if (slot >= 0) {
                 const uint32_t b0 = L.rs.blk;
                 L.need_e = false;
                 L.interact(P, ev);
@@ -1557,7 +1570,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
     if (!LM && lane == 0) {
         const unsigned long long inl = acc[GDRR_ST_STEPS] - acc[A_GATHER] - acc[A_ESC];
         acc[GDRR_ST_VIRTUAL] += inl;
-        if (!(GEN && P.nearest_voxel)) acc[GDRR_ST_CELL_SKIPS] += inl;
+        if (!(GEN && (P.nearest_voxel || P.cells == P.open_cell))) acc[GDRR_ST_CELL_SKIPS] += inl;
     }
     __syncwarp();
     if (lane < GDRR_NSTATS && acc[lane]) atomicAdd(&cnt[lane], acc[lane]);
@@ -1635,6 +1648,9 @@ cudaError_t launch_records_t(const McParams& p, int block, int per_sm_max, int n
     return cudaGetLastError();
 }
 
+// no cell test: none is wanted, or an axis has corners that corner_bits cannot count
+inline bool without_cells(const McParams& p) { return !p.cells || std::max(p.nx, std::max(p.ny, p.nz)) >= 1 << 22; }
+
 template <int NM, bool GEN, bool LM>
 cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm, cudaStream_t s) {
     const size_t bytes = warp_smem_bytes<NM, GEN, LM>(n_pool) * (WARP_BLOCK / 32);
@@ -1654,9 +1670,7 @@ cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm
     const int n_use = (int)std::min<uint64_t>((uint64_t)n_pool, share);
     const unsigned chunk = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)p.chunk, share / 4 + 1));
     McParams q = p;
-    // no cell test (or an axis whose corners corner_bits cannot count): one cell
-    // whose bound nothing exceeds
-    if (!q.cells || (!LM && std::max(q.nx, std::max(q.ny, q.nz)) >= 1 << 22)) {
+    if (!LM && without_cells(p)) {
         q.cells = q.open_cell;
         q.cshift = 30;
         q.csx = q.csy = 0;
@@ -1686,7 +1700,10 @@ cudaError_t launch_nm(const McParams& p, bool records, int block, int n_pool, in
 cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
                       cudaStream_t s) {
     if (p.lm && !p.cells) return cudaErrorInvalidValue;   // the local majorants are the cell bounds
-    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0;
+    // flights without a cell test evaluate the mixture in place, which only the
+    // general form has the registers for: 1e8 histories of the 2 mm torso by way of
+    // the gather service took 209 ms (156 with one photon per lane), so 134
+    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 || (!records && !p.lm && without_cells(p));
     const int n_pool = photons > 0 ? 32 * photons : POOL_DEFAULT;
     if (p.lm) return gen ? launch_nm<true, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s)
                          : launch_nm<false, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s);
