@@ -1061,6 +1061,9 @@ constexpr int REFILL_IDLE = 8;
 // would come after each: 2e7 histories of the 2 mm torso take 14.17 ms at 8, 13.93
 // at 14, 13.67 at 18, 13.57 from 20 to 24 and 14.17 at 30.
 constexpr int REFILL_IDLE_LM = 22;
+// Local-majorant cells of at least 2^5 voxels an edge, where most flights end in
+// the cell they start in: the general form decides them where they are.
+constexpr int LM_INLINE_SHIFT = 5;
 // a slot's flags beside its job
 constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_JOB = 0x1fffffffu;
 
@@ -1256,7 +1259,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
             uint32_t blk = 0, limit = 0, wy = 0, wz = 0, gz = 0;
             FlightKeys key = {0, 0, 0, 0};
             int slot = 0, code = F_NONE;
-            unsigned flown = 0, crossed = 0;
+            unsigned flown = 0, crossed = 0, drawn = 0;
             for (;;) {
                 const unsigned act = __ballot_sync(FULL, code == F_ON);
                 int n_act = __popc(act);
@@ -1318,11 +1321,34 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                     nR = max(0, nR - __popc(~act));
                 }
                 flown += (unsigned)n_act;
+                bool again = false;
                 if (code == F_ON) {
                     if constexpr (LM) {
                         L.state = S_FLY;
                         L.walk(P, bound_of<NM>(P, L.cx + P.csx * (L.cy + P.csy * L.cz), cf));
                         code = L.state == S_FLY ? F_ON : (L.state == S_GATHER ? F_GATHER : F_ESC);
+                        if (GEN && P.cshift >= LM_INLINE_SHIFT && code == F_GATHER && !P.nearest_voxel) {
+                            // coarse cells: the mixture and a virtual collision's next
+                            // flight here (a history at max_steps ends in the service)
+                            float a[8];
+                            int mc[8];
+                            corners(P, L.px, L.py, L.pz, a, mc);
+                            float mu = a[0] * __uint_as_float(S.word(slot, 4, mc[0]));
+#pragma unroll
+                            for (int c = 1; c < 8; ++c) mu = mu + a[c] * __uint_as_float(S.word(slot, 4, mc[c]));
+                            const uint32_t b = S.word(slot, 3, 0);
+                            if (L.tg > mu && b < S.word(slot, 3, 1)) {
+                                const uint4 w = flight_block(
+                                    b, flight_keys(P.jobs[S.word(slot, 2, 3) & JF_JOB].angle_index, S.word(slot, 2, 2),
+                                                   S.word(slot, 3, 2), P.rk), P.rk);
+                                S.word(slot, 3, 0) = b + 1u;
+                                S.word(slot, S.Q_GEN, 0) = w.z;
+                                L.tau = -log_uniform((w.x >> 8) + 1u);
+                                L.tg = uniform(w.y);
+                                code = F_ON;
+                                again = true;
+                            }
+                        }
                     } else {
                         const float s = nl * inv;
                         const float qx = L.px + s * L.dx, qy = L.py + s * L.dy, qz = L.pz + s * L.dz;
@@ -1373,7 +1399,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                         if (cut) code = F_LIMIT;
                     }
                 }
-                if (LM) crossed += (unsigned)__popc(__ballot_sync(FULL, code == F_ON));
+                if (LM) crossed += (unsigned)__popc(__ballot_sync(FULL, code == F_ON && !again));
+                if (LM && GEN) drawn += (unsigned)__popc(__ballot_sync(FULL, again));
             }
             // park the photons still in flight
             __syncwarp();
@@ -1394,6 +1421,10 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
             }
             nR += __popc(fly);
             add(LM ? GDRR_ST_CELL_CROSSINGS : GDRR_ST_STEPS, LM ? crossed : flown);
+            if (LM && GEN) {
+                add(GDRR_ST_STEPS, drawn);
+                add(GDRR_ST_VIRTUAL, drawn);
+            }
             __syncwarp();
             continue;
         }
@@ -1703,7 +1734,8 @@ cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photo
     // flights without a cell test evaluate the mixture in place, which only the
     // general form has the registers for: 1e8 histories of the 2 mm torso by way of
     // the gather service took 209 ms (156 with one photon per lane), so 134
-    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 || (!records && !p.lm && without_cells(p));
+    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 ||
+                     (!records && (p.lm ? p.cshift >= LM_INLINE_SHIFT : without_cells(p)));
     const int n_pool = photons > 0 ? 32 * photons : POOL_DEFAULT;
     if (p.lm) return gen ? launch_nm<true, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s)
                          : launch_nm<false, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s);

@@ -90,3 +90,11 @@ def test_ragged_jobs_equal_single_calls(gd, odd):
         for a in range(4):
             p, s = gd.gdrr_mc_project(ctx, int(budgets[a]), 4, float(angles[a]), a)
             assert torch.equal(p, bp[a]) and torch.equal(s, bs[a])
+
+
+@pytest.mark.parametrize("shift", [4, 5, 6])
+@pytest.mark.parametrize("extra", [{}, {"rayleigh_form_factor": 1}, {"max_steps": 9}])
+def test_local_majorants_in_coarse_cells(gd, odd, shift, extra):
+    names = {"rayleigh_form_factor": "rayleigh_ff"}
+    oopts = {names.get(k, k): (True if k == "rayleigh_form_factor" else v) for k, v in extra.items()}
+    _check(gd, odd, 20_011, 9, oopts={"local_majorant": True, **oopts}, local_majorant=1, cell_shift=shift, **extra)
