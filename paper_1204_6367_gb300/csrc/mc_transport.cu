@@ -1031,11 +1031,12 @@ __global__ void __launch_bounds__(512, 2) mc_kernel(const McParams P) {
 // photon carries those words through its slot, and only a collision or a new
 // history, whose blocks move on, forms them anew.
 //
-// What bounds it: instruction issue (71 % of the slots, 25 of 32 lanes active
-// per instruction, 28 in flight) beside L1 wavefronts (66 %).  2 mm torso, 1e8
-// histories (58 free flights each): 87.8 ms with one photon per lane and a
-// separate source pass, 58.0 ms so; per history 863 warp instructions before,
-// about 500 now, 230 of them free flights, 50 hand-overs, 77 interactions.
+// What bounds it: instruction issue (67 to 71 % of the slots, 25 of 32 lanes active
+// per instruction, 28 in flight) beside L1 wavefronts (63 %).  2 mm torso, 1e8
+// histories (46 free flights each): 75.3 ms with one photon per lane and a
+// separate source pass, 50.3 ms so; per history 725 warp instructions before and
+// 470 now.  Of a warp's time 40 % are free flights, 12 % hand-overs, 12 % gathers,
+// 15 % interactions and 10 % tallies and starts.
 //
 // A slot is Q float4 words: {px py pz, and t = xi mumax at a tentative
 // collision or the next flight's -ln xi} {dx dy dz E} {mumax 1/mumax, or the
@@ -1062,7 +1063,9 @@ constexpr int REFILL_IDLE = 8;
 // at 14, 13.67 at 18, 13.57 from 20 to 24 and 14.17 at 30.
 constexpr int REFILL_IDLE_LM = 22;
 // Local-majorant cells of at least 2^5 voxels an edge, where most flights end in
-// the cell they start in: the general form decides them where they are.
+// the cell they start in: the general form decides them where they are (2e7
+// histories of the 2 mm torso: 17.9 ms by way of the gather service and 15.5 so
+// with 64 mm cells, 31.8 and 21.2 with 128 mm; with 32 mm 11.8 and 13.1).
 constexpr int LM_INLINE_SHIFT = 5;
 // a slot's flags beside its job
 constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_JOB = 0x1fffffffu;
