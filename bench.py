@@ -163,11 +163,10 @@ def kernel_traffic(cell_shift=None):
     return int(v["bytes_per_launch"]) if v else None
 
 
-# The instruction count per flight depends on batch_min (how often the warp
-# serves its waiting lanes) and is keyed to the block size as well; the
-# histories a lane claims at a time (hist_per_thread) leave it unchanged
-# (measured: 266.14 and 266.12 per flight at 1 and 8), so a line's third
-# field is informational.
+# A line of the instruction record names the block size and batch_min it was
+# taken with.  Both only shape runs with event records (which batch their
+# waiting lanes), so the transport's count is the same for every choice; the
+# histories a lane claims at a time (a line's third field) leave it unchanged too.
 ISSUE_CONFIG_KEYS = ("block_size", "batch_min")
 
 
