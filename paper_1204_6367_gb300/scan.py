@@ -58,6 +58,8 @@ def scan(ctx, n_views: int, components: str = "P", n_photons: int = 1_000_000, s
 def reconstruct(ctx, angles, signal, shape, voxel, floor_rel: float = 1e-6):
     """FDK volume [nz, ny, nx] FP32 (attenuation, 1/mm) of a scan's signals."""
     I0 = gdrr.gdrr_air_scan(ctx)
+    if tuple(signal.shape[-2:]) != tuple(I0.shape):      # the kernels only see how many values there are
+        raise ValueError(f"signal must hold views of {tuple(I0.shape)} pixels, got {tuple(signal.shape)}")
     g = gdrr.gdrr_line_integrals_views(signal, I0, floor_rel)
     p = ctx.prob
     geo = gdrr.fdk_geometry(p.sad, p.sdd, ctx.nu, ctx.nv, p.du, p.dv, shape, voxel)
