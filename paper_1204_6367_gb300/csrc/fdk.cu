@@ -315,8 +315,11 @@ __device__ __forceinline__ Significand significand(uint64_t bits) {
     return {__uint_as_float(0x3f800000u | ((uint32_t)(bits >> 29) & 0x007fffffu)), (int)((uint32_t)bits & 0x1fffffffu)};
 }
 
+// Near a ratio of one the quotient's own rounding is all that its logarithm
+// would show, so there the difference (exact) is divided instead.
 __device__ __noinline__ float line_integral_64(double s, double a, double floor_rel) {
-    return (float)(-log(fmax(s, floor_rel * a) / a));
+    const double v = fmax(s, floor_rel * a), x = v - a;
+    return (float)(fabs(x) <= 0.5 * a ? -log1p(x / a) : -log(v / a));
 }
 
 __device__ __forceinline__ float line_integral(double s, double a, double least, double floor_rel,
@@ -327,19 +330,19 @@ __device__ __forceinline__ float line_integral(double s, double a, double least,
     const int ev = (int)(vb >> 52), ea = (int)(ab >> 52);
     if ((unsigned)(ev - 1) >= 2046u || (unsigned)(ea - 1) >= 2046u || lb <= 0) return line_integral_64(s, a, floor_rel);
     const Significand mv = significand((uint64_t)vb);
-    // the power of two that brings the ratio to [sqrt(1/2), sqrt(2))
-    int e = ev - ea;
-    float k = 1.0f;
-    if (mv.h > 1.41421354f * ma.h) { k = 2.0f; e += 1; }
-    else if (1.41421354f * mv.h < ma.h) { k = 0.5f; e -= 1; }
-    const float ah = k * ma.h, vl = (float)mv.l * TWO_M52, al = (float)ma.l * TWO_M52 * k;
-    // near 1 the difference is small: its low part exactly, as two floats
-    const int dl = mv.l - ma.l;
+    // the power of two k that brings the ratio to [sqrt(1/2), sqrt(2)); the
+    // difference mv - k ma: that of the heads is exact (a ratio within 2), that of
+    // the low parts an integer below 2^31, whatever k, taken as two floats
+    int e = ev - ea, dl = mv.l - ma.l;
+    float k = 1.0f, unit = TWO_M52;
+    if (mv.h > 1.41421354f * ma.h) { k = 2.0f; e += 1; dl -= ma.l; }
+    else if (1.41421354f * mv.h < ma.h) { k = 0.5f; e -= 1; dl += mv.l; unit = 0.5f * TWO_M52; }
+    const float ah = k * ma.h;
     const float d1 = (float)dl, d2 = (float)(dl - (int)d1);
-    Pair d = two_sum(__fsub_rn(mv.h, ah), k == 1.0f ? d1 * TWO_M52 : __fsub_rn(vl, al));   // the first difference is exact
-    if (k == 1.0f) d.l = __fmaf_rn(d2, TWO_M52, d.l);
+    Pair d = two_sum(__fsub_rn(mv.h, ah), d1 * unit);
+    d = two_sum(d.h, __fmaf_rn(d2, unit, d.l));
     Pair w = two_sum(mv.h, ah);
-    w.l = __fadd_rn(w.l, __fadd_rn(vl, al));
+    w.l = __fadd_rn(w.l, __fadd_rn((float)mv.l * TWO_M52, (float)ma.l * (k * TWO_M52)));
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(w.h));
     const float th = __fmul_rn(d.h, y);
