@@ -283,15 +283,24 @@ __global__ void __launch_bounds__(BP_BX * BP_BY, 3) fdk_backproject_kernel(const
 // Line integrals -ln(max(s, floor a) / a), rounded to FP32 from the FP64
 // inputs.  GB300 runs FP64 at 1/64 of the FP32 rate and the FP64 logarithm
 // bound the kernel (5.2 ms for 70.8 M pixels against 0.13 ms of memory
-// traffic), 0.41 ms as below: the value is formed in pairs of floats from the integer bits of
+// traffic), 0.42 ms as below: the value is formed in pairs of floats from the integer bits of
 // the operands: with r = s / a brought to [sqrt(1/2), sqrt(2)) by a power of
 // two, ln r = 2 atanh(t), t = (ms - ma) / (ms + ma) (difference and sum of the
-// 53-bit significands, quotient with its remainder), atanh by its Taylor
-// series to t^15, whose first correction t^2 / 3 is also carried as a pair.
-// The result's relative error is below 2^-36; where that leaves the rounding
-// to FP32 open (one pixel in about 2000), and for operands that are not
-// positive normal numbers, the FP64 logarithm decides, so what is written is
-// the FP32 rounding of the logarithm, as before.
+// 53-bit significands, quotient with its remainder), atanh t = t (1 + c) by its
+// Taylor series to t^15, c = u (1/3 + u (1/5 + u q)), u = t^2, with q alone a
+// single float.
+//
+// Relative error of the pair, below 2^-39.5: |t| <= 0.1716, so u <= 0.0295 and
+// u q <= 0.0043; q and u q carry four roundings of 2^-24 (q's last step, its
+// constant, u's low part left out, the product), which u^2 <= 8.7e-4 scales to
+// 4.3 x 0.0043 x 8.7e-4 x 2^-24 < 2^-39.8.  The terms left out (t^16 / 17 and on:
+// 2^-44.7), and the roundings of the pairs' low parts (t, u, the outer steps, the
+// sums with e ln 2: at most 2^-43 each) come to less than 2^-41.  (The largest of
+// 1.8e7 values against a 113-bit logarithm: 2^-39.97, whether the reciprocal is
+// rounded or off by one ulp either way.)  Where an error of 2^-38 leaves the
+// rounding to FP32 open (one pixel in about 8000), and for operands that are not
+// positive normal numbers, the FP64 logarithm decides: what is written is the
+// FP32 rounding of the logarithm.
 constexpr int LI_VIEWS = 8;       // pixels of consecutive views per thread: the air pixel's part is formed once
 
 struct Pair {
@@ -301,6 +310,10 @@ struct Pair {
 __device__ __forceinline__ Pair two_sum(float a, float b) {
     const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
     return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ Pair fast_two_sum(float a, float b) {      // |a| >= |b|
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
 // the significand of a positive normal double as a pair in [1, 2): its first
@@ -345,35 +358,44 @@ __device__ __forceinline__ float line_integral(double s, double a, double least,
     w.l = __fadd_rn(w.l, __fadd_rn((float)mv.l * TWO_M52, (float)ma.l * (k * TWO_M52)));
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(w.h));
-    const float th = __fmul_rn(d.h, y);
-    const float tl = __fmul_rn(__fadd_rn(__fmaf_rn(-th, w.h, d.h), __fmaf_rn(-th, w.l, d.l)), y);
-    const float uh = __fmul_rn(th, th);
-    const float ul = __fmaf_rn(2.0f * th, tl, __fmaf_rn(th, th, -uh));
-    float p = (float)(1.0 / 15.0);
-    p = __fmaf_rn(p, uh, (float)(1.0 / 13.0));
-    p = __fmaf_rn(p, uh, (float)(1.0 / 11.0));
-    p = __fmaf_rn(p, uh, (float)(1.0 / 9.0));
-    p = __fmaf_rn(p, uh, (float)(1.0 / 7.0));
-    p = __fmaf_rn(p, uh, (float)(1.0 / 5.0));
+    Pair t;
+    t.h = __fmul_rn(d.h, y);
+    t.l = __fmul_rn(__fadd_rn(__fmaf_rn(-t.h, w.h, d.h), __fmaf_rn(-t.h, w.l, d.l)), y);
+    t = fast_two_sum(t.h, t.l);
+    const float uh = __fmul_rn(t.h, t.h);
+    const float ul = __fmaf_rn(2.0f * t.h, t.l, __fmaf_rn(t.h, t.h, -uh));
+    float q = (float)(1.0 / 15.0);
+    q = __fmaf_rn(q, uh, (float)(1.0 / 13.0));
+    q = __fmaf_rn(q, uh, (float)(1.0 / 11.0));
+    q = __fmaf_rn(q, uh, (float)(1.0 / 9.0));
+    q = __fmaf_rn(q, uh, (float)(1.0 / 7.0));
+    // c = u (1/3 + u (1/5 + u q)), the two outer steps in pairs
     constexpr float C3H = (float)(1.0 / 3.0), C3L = (float)(1.0 / 3.0 - (double)C3H);
-    const float ch = __fmul_rn(uh, C3H);
-    const float cl = __fadd_rn(__fmaf_rn(uh, C3H, -ch), __fmaf_rn(uh, C3L, __fmaf_rn(ul, C3H, __fmul_rn(uh, __fmul_rn(uh, p)))));
+    constexpr float C5H = (float)(1.0 / 5.0), C5L = (float)(1.0 / 5.0 - (double)C5H);
+    Pair p = fast_two_sum(C5H, __fmul_rn(uh, q));
+    p.l = __fadd_rn(p.l, C5L);
+    const float vh = __fmul_rn(uh, p.h);
+    const float vl = __fadd_rn(__fmaf_rn(uh, p.h, -vh), __fmaf_rn(uh, p.l, __fmul_rn(ul, p.h)));
+    p = fast_two_sum(C3H, vh);
+    p.l = __fadd_rn(p.l, __fadd_rn(vl, C3L));
+    const float ch = __fmul_rn(uh, p.h);
+    const float cl = __fadd_rn(__fmaf_rn(uh, p.h, -ch), __fmaf_rn(uh, p.l, __fmul_rn(ul, p.h)));
     // ln r = 2 (t + t c)
-    const float bh = __fmul_rn(th, ch);
-    const float bl = __fmaf_rn(th, ch, -bh);
-    Pair g = two_sum(th, bh);
-    g.l = __fadd_rn(g.l, __fadd_rn(__fadd_rn(tl, bl), __fmaf_rn(tl, ch, __fmul_rn(th, cl))));
+    const float bh = __fmul_rn(t.h, ch);
+    const float bl = __fadd_rn(__fmaf_rn(t.h, ch, -bh), __fmaf_rn(t.h, cl, __fmul_rn(t.l, ch)));
+    Pair g = fast_two_sum(t.h, bh);
+    g.l = __fadd_rn(g.l, __fadd_rn(t.l, bl));
     // + e ln 2: e times the 12-bit head is exact
     const float fe = (float)e;
     constexpr double LN2 = 0.69314718055994530942;
     constexpr float L1 = (float)(2839.0 / 4096.0), L2 = (float)(LN2 - 2839.0 / 4096.0);
     constexpr float L3 = (float)(LN2 - 2839.0 / 4096.0 - (double)L2);
     const float mh = __fmul_rn(fe, L2);
-    Pair q = two_sum(__fmul_rn(fe, L1), 2.0f * g.h);
-    const Pair m = two_sum(q.h, mh);
-    q.l = __fadd_rn(__fadd_rn(q.l, m.l), __fmaf_rn(2.0f, g.l, __fmaf_rn(fe, L3, __fmaf_rn(fe, L2, -mh))));
-    const Pair r = two_sum(m.h, q.l);
-    const float err = fabsf(r.h) * (float)(1.0 / 34359738368.0);             // 2^-35
+    const Pair f = two_sum(__fmul_rn(fe, L1), 2.0f * g.h);
+    const Pair m = two_sum(f.h, mh);
+    const float lo = __fadd_rn(__fadd_rn(f.l, m.l), __fmaf_rn(2.0f, g.l, __fmaf_rn(fe, L3, __fmaf_rn(fe, L2, -mh))));
+    const Pair r = fast_two_sum(m.h, lo);
+    const float err = fabsf(r.h) * (float)(1.0 / 274877906944.0);            // 2^-38
     if (__fadd_rn(r.h, __fadd_rn(r.l, err)) != r.h || __fadd_rn(r.h, __fsub_rn(r.l, err)) != r.h)
         return line_integral_64(s, a, floor_rel);
     return -r.h;

@@ -38,3 +38,12 @@ def test_signal_and_air_on_either_side_of_a_power_of_two(gd, gap, power):
     assert _ulps(gd, above, below).max() <= 0.5 + 2.0 ** -20
     swapped = power * (1.0 - gap * rng.uniform(0.01, 1.0, (9, 20_000)))
     assert _ulps(gd, swapped, above[0]).max() <= 0.5 + 2.0 ** -20
+
+
+@pytest.mark.parametrize("lo, hi", [(0.5, 0.7072), (0.7071, 0.9), (0.9, 1.1), (1.1, 1.4143), (1.4142, 2.0)])
+def test_ratios_of_every_size(gd, lo, hi):
+    rng = np.random.default_rng(int(1000 * lo))
+    air = np.exp(rng.uniform(-25.0, 3.0, 200_003))
+    sig = air[None] * rng.uniform(lo, hi, (10, 200_003))
+    sig = np.clip(sig, 0.5 * air, 2.0 * air)
+    assert _ulps(gd, sig, air).max() <= 0.5 + 2.0 ** -20
