@@ -33,7 +33,7 @@ SOURCES = {
     "fdk.cu": [],
     "probes.cu": [],
 }
-HEADERS = [os.path.join(INCLUDE, "gdrr.h"), os.path.join(CSRC, "gdrr_internal.cuh"), os.path.join(CSRC, "cnn_epi.cuh")]
+HEADERS = [os.path.join(INCLUDE, "gdrr.h")] + [os.path.join(CSRC, h) for h in ("gdrr_internal.cuh", "cnn_epi.cuh", "fdk_rows.h")]
 
 
 def nvcc() -> str:

@@ -18,6 +18,7 @@
 // per-view geometry (depth, u, weight) is computed once per column.
 #include <cmath>
 
+#include "fdk_rows.h"
 #include "gdrr_internal.cuh"
 
 namespace gdrr {
@@ -205,16 +206,18 @@ __global__ void __launch_bounds__(BP_BX * BP_BY, 3) fdk_backproject_kernel(const
 #pragma unroll
     for (int h = 0; h < BP_ZT / 2; ++h) {
         accp[h] = 0ull;
-        zp[h] = pack2(p.z0 + (float)(iz0 + 2 * h) * p.dz, p.z0 + (float)(iz0 + 2 * h + 1) * p.dz);
+        zp[h] = pack2(bp_height(p.z0, iz0 + 2 * h, p.dz), bp_height(p.z0, iz0 + 2 * h + 1, p.dz));
     }
     const size_t view = (size_t)p.nu * p.nv;
-    const float z_lo = p.z0 + (float)iz0 * p.dz, z_hi = p.z0 + (float)(iz0 + BP_ZT - 1) * p.dz;
+    const float z_lo = bp_height(p.z0, iz0, p.dz), z_hi = bp_height(p.z0, iz0 + BP_ZT - 1, p.dz);
     for (int i = 0; i < p.n_ang; ++i) {
         const float cph = p.cs[i].x, sph = p.cs[i].y;
         const float depth = p.sad + x * cph + y * sph;
-        float inv;                                                // Newton's step on an approximate reciprocal
+        // the rounded reciprocal: the approximate one (within 1 ulp) and Newton's step,
+        // equal to 1 / depth for every significand (all 2^23 compared)
+        float inv;
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(depth));
-        inv = inv + inv * (1.0f - depth * inv);
+        inv = fmaf(inv, fmaf(-depth, inv, 1.0f), inv);
         const float fu = p.sad * (x * sph - y * cph) * inv * p.inv_tau_u + p.hu;
         const float fiu = floorf(fu);
         if (fiu < -1.0f || fiu > (float)(p.nu - 1)) continue;   // the column misses the detector
@@ -225,15 +228,15 @@ __global__ void __launch_bounds__(BP_BX * BP_BY, 3) fdk_backproject_kernel(const
         const float sv = m * p.inv_tau_v;                           // dv-index per mm of z
         const float* img = q + (size_t)(p.first_view + i) * view;
         const float wu0 = 1.0f - wu;
-        const float v_lo = z_lo * sv + p.hv, v_hi = z_hi * sv + p.hv;
+        const float v_lo = bp_row(z_lo, sv, p.hv), v_hi = bp_row(z_hi, sv, p.hv);
         if (v_hi <= -1.0f || v_lo >= (float)p.nv) continue;        // its voxels miss the detector
-        if (p.unchecked && iu >= 0 && iu < p.nu - 1 && v_lo >= 0.0f && v_hi < (float)(p.nv - 1)) {
+        if (p.unchecked && iu >= 0 && iu < p.nu - 1 && bp_rows_inside(v_lo, v_hi, p.nv)) {
             // 0x4b000000 + iv is the bit pattern of 2^23 + iv
             const uint32_t nu = (uint32_t)p.nu, first = (uint32_t)iu - 0x4b000000u * nu;
             const uint64_t svp = twice(sv), wup = twice(wu), wu0p = twice(wu0), w2p = twice(w2);
 #pragma unroll
             for (int h = 0; h < BP_ZT / 2; ++h) {                     // two voxels as packed pairs
-                const uint64_t fv = fma2(zp[h], svp, twice(p.hv));
+                const uint64_t fv = fma2(zp[h], svp, twice(p.hv));   // bp_row of both
                 const uint64_t t = add2_down(fv, twice(8388608.0f));   // 2^23 + floor(fv)
                 const uint64_t wv = fma2(add2(t, twice(-8388608.0f)), twice(-1.0f), fv);
                 float2 v[4];
@@ -257,9 +260,8 @@ __global__ void __launch_bounds__(BP_BX * BP_BY, 3) fdk_backproject_kernel(const
         }
 #pragma unroll
         for (int k = 0; k < BP_ZT; ++k) {
-            const float z = p.z0 + (float)(iz0 + k) * p.dz;
             // clamped two samples beyond the edges (those taps read zero)
-            const float fv = fminf(fmaxf(z * sv + p.hv, -2.0f), (float)p.nv + 1.0f);
+            const float fv = fminf(fmaxf(bp_row(bp_height(p.z0, iz0 + k, p.dz), sv, p.hv), -2.0f), (float)p.nv + 1.0f);
             const float fiv = floorf(fv);
             const int iv = (int)fiv;
             const float wv = fv - fiv;
