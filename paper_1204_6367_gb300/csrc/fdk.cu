@@ -173,6 +173,7 @@ struct BpParams {
     int unchecked;           // 1: a view's rows and samples can be counted by the unchecked taps
     float2 cs[BP_MAX_ANGLES];   // (cos phi, sin phi) of each view
     int first_view;          // index of cs[0] in the filtered stack
+    int first_group;         // group of BP_ZT slices of the launch's first block
 };
 
 __device__ __forceinline__ float tap(const float* __restrict__ img, int nu, int nv, int iu, int iv) {
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(BP_BX * BP_BY, 3) fdk_backproject_kernel(const
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ix = blockIdx.x * BP_BX + (warp % (BP_BX / BP_WX)) * BP_WX + lane % BP_WX;
     const int iy = blockIdx.y * BP_BY + (warp / (BP_BX / BP_WX)) * (32 / BP_WX) + lane / BP_WX;
-    const int iz0 = blockIdx.z * BP_ZT;
+    const int iz0 = (p.first_group + (int)blockIdx.z) * BP_ZT;
     if (ix >= p.nx || iy >= p.ny) return;
     const float x = p.x0 + (float)ix * p.dx;
     const float y = p.y0 + (float)iy * p.dy;
@@ -496,8 +497,8 @@ extern "C" GDRR_API int gdrr_fdk_backproject(const gdrr_fdk_geometry* g, int32_t
     p.d_beta = (float)d_beta;
     p.unchecked = g->nv < (1 << 22) && (int64_t)g->nu * g->nv < ((int64_t)1 << 31) ? 1 : 0;
     const int block = gdrr::BP_BX * gdrr::BP_BY;
-    const dim3 grid((unsigned)((g->nx + gdrr::BP_BX - 1) / gdrr::BP_BX), (unsigned)((g->ny + gdrr::BP_BY - 1) / gdrr::BP_BY),
-                    (unsigned)((g->nz + gdrr::BP_ZT - 1) / gdrr::BP_ZT));
+    // (a launch has at most 65535 blocks in z: taller volumes take several)
+    const int groups = (g->nz - 1) / gdrr::BP_ZT + 1;
     if (n_proj == 0 && !accumulate) {
         if (cudaMemsetAsync(volume_dev, 0, sizeof(float) * (size_t)g->nx * g->ny * g->nz, s) != cudaSuccess)
             return GDRR_ERR_CUDA;
@@ -510,8 +511,13 @@ extern "C" GDRR_API int gdrr_fdk_backproject(const gdrr_fdk_geometry* g, int32_t
         p.accumulate = (first > 0 || accumulate) ? 1 : 0;
         for (int i = 0; i < n; ++i)
             p.cs[i] = make_float2((float)std::cos(angles_rad[first + i]), (float)std::sin(angles_rad[first + i]));
-        gdrr::fdk_backproject_kernel<<<grid, block, 0, s>>>(p, filtered_dev, volume_dev);
-        if (cudaGetLastError() != cudaSuccess) return GDRR_ERR_CUDA;
+        for (p.first_group = 0; p.first_group < groups; p.first_group += 65535) {
+            const dim3 grid((unsigned)((g->nx + gdrr::BP_BX - 1) / gdrr::BP_BX),
+                            (unsigned)((g->ny + gdrr::BP_BY - 1) / gdrr::BP_BY),
+                            (unsigned)std::min(65535, groups - p.first_group));
+            gdrr::fdk_backproject_kernel<<<grid, block, 0, s>>>(p, filtered_dev, volume_dev);
+            if (cudaGetLastError() != cudaSuccess) return GDRR_ERR_CUDA;
+        }
     }
     return GDRR_OK;
 }
