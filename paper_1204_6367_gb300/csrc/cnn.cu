@@ -345,6 +345,8 @@ __global__ void pool_kernel(const View X, int C, int B, int H, int W, bf16* __re
 // Pixels per block of the activation backward: the block holds pt x Co
 // values, at most 4096 for wide layers.
 inline int act_tile(int co) { return co >= 256 ? 16 : (co >= 128 ? 32 : 64); }
+constexpr int MAX_BASE = 64, MAX_CO = 8 * MAX_BASE;   // channels of the first layer, of any layer
+inline size_t act_back_smem(int co) { return (size_t)act_tile(co) * (co + 1) * 4 + (size_t)co * (act_tile(co) + 8) * 2; }
 
 // dZ = dY * (Y > 0) (or dY when relu == 0) for a block of pt pixels (a
 // multiple of 16, at most 64) and all Co channels: BF16 NHWC dz16[p][c] (the
@@ -1051,10 +1053,9 @@ cudaError_t conv_backward(gdrr_cnn* n, SumJobs& sums, const Conv& L, int B, cons
         // written by head_grad_kernel
     } else if (L.implicit_dw) {
         const int tiles = std::max(1, std::min(ACT_PIX / pt, 4096 / (pt * L.co)));
-        const size_t smem = (size_t)tiles * pt * (L.co + 4) * 4;
+        const size_t smem = (size_t)tiles * pt * (L.co + 4) * 4;       // 33 KB at most (512 channels)
         auto act = dy.mode == GRAD_PLACE ? act_back4_kernel<GRAD_PLACE>
                    : dy.mode == GRAD_POOL ? act_back4_kernel<GRAD_POOL> : act_back4_kernel<GRAD_PLAIN>;
-        CK(cudaFuncSetAttribute(act, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         act<<<(n_blk + tiles - 1) / tiles, 256, smem, st>>>(dy, Y, L.H, L.W, P, L.co, L.relu, pt, tiles, n->dz16,
                                                             L.db_part);
     } else {
@@ -1067,8 +1068,8 @@ cudaError_t conv_backward(gdrr_cnn* n, SumJobs& sums, const Conv& L, int B, cons
                 pool_back_kernel<<<nblk(P * L.co / 4), TB, 0, st>>>(dy.g, dy.ld, dy.off, dy.dp, B, L.co, L.H, L.W, dy.buf);
             CK(cudaGetLastError());
         }
-        const size_t smem = (size_t)pt * (L.co + 1) * 4 + (size_t)L.co * (pt + 8) * 2;
-        CK(cudaFuncSetAttribute(act_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const size_t smem = act_back_smem(L.co);
+        CK(allow_smem(act_back_kernel, act_back_smem(MAX_CO)));
         act_back_kernel<<<n_blk, TB, smem, st>>>(g, Y, L.H, L.W, P, L.co, L.relu, pt, n->dz16, n->dz_cp, Pp,
                                                  L.db_part);
     }
@@ -1104,7 +1105,7 @@ extern "C" {
 GDRR_API int gdrr_cnn_create(int32_t max_batch, int32_t height, int32_t width, int32_t base_channels, uint64_t seed,
                              void* cuda_stream, gdrr_cnn** out) {
     if (!out || max_batch <= 0 || height <= 0 || width <= 0 || height % 8 || width % 8 || base_channels <= 0 ||
-        base_channels > 64 || base_channels % 8)
+        base_channels > MAX_BASE || base_channels % 8)
         return GDRR_ERR_INVALID_ARG;
     gdrr_cnn* n = new (std::nothrow) gdrr_cnn();
     if (!n) return GDRR_ERR_OOM;
@@ -1261,9 +1262,7 @@ GDRR_API int gdrr_cnn_forward(gdrr_cnn* n, int32_t batch, const float* in_dev, f
     const float* P = n->params;
     do {
         // encoder: e1 -> cat1[2c..3c), e2 -> cat2[4c..6c), e3 -> cat3[8c..12c), e4 -> cat3[0..8c) upsampled
-        if ((e = cudaFuncSetAttribute(first_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)first_layer_smem(c))))
-            break;
+        if ((e = allow_smem(first_layer_kernel, first_layer_smem(MAX_BASE)))) break;
         first_layer_kernel<<<(unsigned)((s1 / 4 + 32 * FIRST_WARPS - 1) / (32 * FIRST_WARPS)), 32 * FIRST_WARPS,
                              first_layer_smem(c), st>>>(
             in_dev, B, H, W, L[0].w16, L[0].K9p, P + L[0].b_off, c, n->x16, n->cat1 + 2 * c, 3 * c, n->p1);

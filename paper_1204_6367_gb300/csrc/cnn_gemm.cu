@@ -1503,7 +1503,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_tap_kernel(const __grid_
 // batch 16 on 96 x 128 pixels: 96 -> 32 channels 217 us -> 45, 192 -> 64 at half
 // the grid 125 -> 42, 384 -> 128 at a quarter 74 -> 36 (partial sums included).
 constexpr int WG_PIX = 64, WG_SLABS = 12;
-constexpr uint32_t WG_SLAB = WG_PIX * CONV_BK * 2;
+constexpr uint32_t WG_SLAB = WG_PIX * CONV_BK * 2, WG_RING = 216u * 1024u;
 
 // 64-byte-swizzled MN-major operand: atoms of 32 channels x 8 pixels; the next
 // 32 channels a slab further, the next 8 pixels 512 bytes further.
@@ -1757,8 +1757,7 @@ cudaError_t launch_conv_t(const ConvMaps& m, ConvGeo g, int M, int N, const Conv
     g.stages = conv_stages(g.Wb, BN, MT);
     if (g.stages < 2) return cudaErrorInvalidValue;
     const size_t smem = (size_t)g.stages * (g.a_bytes + 3u * BN * CONV_BK * 2) + CONV_OUT + 1024;
-    cudaError_t e = cudaFuncSetAttribute(conv_implicit_kernel<BN, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(conv_implicit_kernel<BN, MT>, CONV_RING + CONV_OUT + 1024);
     if (e != cudaSuccess) return e;
     const int64_t n_tiles = (int64_t)(M / (GEMM_BM * MT)) * ((N + BN - 1) / BN);
     const int grid = (int)std::min<int64_t>(n_tiles, n_sm);
@@ -1788,8 +1787,7 @@ cudaError_t launch_tma_t(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B
     const int per = (k_slices + splits - 1) / splits;
     splits = (k_slices + per - 1) / per;
     const size_t smem = (size_t)STAGES * (GEMM_BM + BN) * GEMM_BK * 2 + 1024;
-    cudaError_t e = cudaFuncSetAttribute(gemm_tma_kernel<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(gemm_tma_kernel<BN, STAGES>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)(((M + GEMM_BM - 1) / GEMM_BM) * ((N + BN - 1) / BN)), 1, splits);
     gemm_tma_kernel<BN, STAGES><<<grid, TMA_THREADS, smem, s>>>(mA, mB, C, ldc, M, N, K, per * GEMM_BK,
@@ -1808,8 +1806,7 @@ cudaError_t launch_persistent_t(const __nv_bfloat16* A, int lda, const __nv_bflo
     const int per = (k_slices + splits - 1) / splits;
     splits = (k_slices + per - 1) / per;
     const size_t smem = (size_t)STAGES * (GEMM_BM + BN) * GEMM_BK * 2 + 1024;
-    cudaError_t e = cudaFuncSetAttribute(gemm_persistent_kernel<BN, STAGES>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(gemm_persistent_kernel<BN, STAGES>, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, n_sm = 1;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1841,7 +1838,7 @@ cudaError_t launch_pair(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B,
             return cudaErrorInvalidValue;
     }
     const size_t smem = (size_t)PAIR_STAGES * 2 * PAIR_HALF + CONV_OUT + 1024;
-    cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(gemm_pair_kernel, smem);
     if (e != cudaSuccess) return e;
     // as many pairs as are resident at once (an odd SM of a cluster group stays idle)
     static std::atomic<int> resident[64];
@@ -2049,7 +2046,7 @@ cudaError_t launch_conv_tap(const ConvArgs& a, const __nv_bfloat16* w, int ldw, 
     }
     const size_t smem = (size_t)g.stages * stage + CONV_OUT + 1024;
     auto launch = [&](auto kernel) {
-        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t r = allow_smem(kernel, CONV_RING + CONV_OUT + 1024);
         if (r != cudaSuccess) return r;
         kernel<<<std::min(g.n_tiles, n_sm), PERSIST_THREADS, smem, s>>>(m, g, a.N, half ? epi.bias : nullptr, epi.relu, err);
         return cudaGetLastError();
@@ -2143,11 +2140,11 @@ cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int ks, int C, int ldx, in
     g.groups = (g.slabs + g.group - 1) / g.group;
     g.a_slabs = (g.group + 3) / 4 * 4;
     const uint32_t stage = (uint32_t)(g.a_slabs + nb / 32) * WG_SLAB;
-    g.stages = (int)std::min<uint32_t>(CONV_MAX_STAGES, 216u * 1024u / stage);
+    g.stages = (int)std::min<uint32_t>(CONV_MAX_STAGES, WG_RING / stage);
     const size_t smem = (size_t)g.stages * stage + 1024;
     const dim3 grid((unsigned)splits, (unsigned)(ks * g.groups * (N / nb)));
     auto launch = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kernel, WG_RING + 1024);
         if (e != cudaSuccess) return e;
         kernel<<<grid, PERSIST_THREADS, smem, s>>>(mX, mZ, g, part, N, err);
         return cudaGetLastError();

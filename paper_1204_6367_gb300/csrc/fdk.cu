@@ -460,7 +460,8 @@ extern "C" GDRR_API int gdrr_fdk_filter(const gdrr_fdk_geometry* g, int32_t n_pr
     p.scale = (float)(0.5 / (g->du_mm * mag));
     const gdrr::FilterShape f = gdrr::filter_shape(g->nu);
     const size_t smem = gdrr::filter_smem(f);
-    if (cudaFuncSetAttribute(gdrr::fdk_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    // (the widest row's shape needs the most)
+    if (gdrr::allow_smem(gdrr::fdk_filter_kernel, gdrr::filter_smem(gdrr::filter_shape(gdrr::FILTER_MAX_NU))) != cudaSuccess)
         return GDRR_ERR_CUDA;
     const int64_t n_rows = (int64_t)g->nv * n_proj;
     gdrr::fdk_filter_kernel<<<(unsigned)((n_rows + f.rows - 1) / f.rows), gdrr::FILTER_BLOCK, smem,

@@ -181,6 +181,15 @@ struct RtParams {
 // blocks (of `block` threads) per SM.
 cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
                       cudaStream_t s);
+// A kernel's limit of dynamic shared memory is one setting of the process, and a
+// launch above it fails: it is set to the most that any launch of the kernel
+// takes, whatever the launch at hand needs, so that a thread cannot lower it
+// between another thread's call and its launch.
+template <class K>
+inline cudaError_t allow_smem(K kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Packed FP32 pairs: each half is its own IEEE-rounded FMA.
 __device__ __forceinline__ uint64_t twice(float v) {
     uint64_t r;

@@ -356,7 +356,7 @@ cudaError_t launch_denoise_fused(const double* s_hat, double* s_out, int nu, int
     const void* kernel = ppt <= 1 ? (const void*)denoise_fused_kernel<1>
                        : ppt <= 2 ? (const void*)denoise_fused_kernel<2> : (const void*)denoise_fused_kernel<FUSED_MAX_PPT>;
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(kernel, 2 * (size_t)FUSED_MAX_PPT * 1024 * sizeof(double));
         if (e != cudaSuccess) return e;
     }
     void* args[] = {(void*)&s_hat, (void*)&s_out, (void*)&nu, (void*)&nv, (void*)&tile_w, (void*)&tile_h,

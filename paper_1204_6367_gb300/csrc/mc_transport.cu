@@ -1055,6 +1055,7 @@ constexpr int WARP_BLOCK = 128;                // threads; the warps of a block 
 // (64 registers, spills in the flight loop) were 1 and 8 % slower.
 constexpr int WARP_MIN_BLOCKS = 6, WARP_MIN_BLOCKS_GEN = 5;
 constexpr int POOL_DEFAULT = 80;               // photons per warp: the most that 24 warps' shared memory holds
+constexpr int POOL_MAX = 96;                   // the largest pool that an option asks for
 // Idle lanes at which the warp hands over and refills: 5, 6, 8 and 12 were
 // within 2 %, 4 was 3 % slower (a hand-over costs about half a flight).
 constexpr int REFILL_IDLE = 8;
@@ -1670,8 +1671,7 @@ template <int NM, bool GEN, bool LM>
 cudaError_t launch_records_t(const McParams& p, int block, int per_sm_max, int n_sm, cudaStream_t s) {
     const size_t bytes = smem_bytes<NM>(block);
     cudaError_t e = cudaSuccess;
-    if (bytes > 47 * 1024)
-        e = cudaFuncSetAttribute(mc_kernel<NM, GEN, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (smem_bytes<NM>(512) > 47 * 1024) e = allow_smem(mc_kernel<NM, GEN, LM>, smem_bytes<NM>(512));
     int per_sm = per_sm_max;
     if (e == cudaSuccess && per_sm <= 0)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mc_kernel<NM, GEN, LM>, block, bytes);
@@ -1688,8 +1688,7 @@ inline bool without_cells(const McParams& p) { return !p.cells || std::max(p.nx,
 template <int NM, bool GEN, bool LM>
 cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm, cudaStream_t s) {
     const size_t bytes = warp_smem_bytes<NM, GEN, LM>(n_pool) * (WARP_BLOCK / 32);
-    cudaError_t e = cudaFuncSetAttribute(mc_warp_kernel<NM, GEN, LM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bytes);
+    cudaError_t e = allow_smem(mc_warp_kernel<NM, GEN, LM>, warp_smem_bytes<NM, GEN, LM>(POOL_MAX) * (WARP_BLOCK / 32));
     int per_sm = 0;
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mc_warp_kernel<NM, GEN, LM>, WARP_BLOCK, bytes);
