@@ -903,7 +903,7 @@ struct gdrr_cnn {
     float *g_d3 = nullptr, *g_cat3 = nullptr, *g_e4 = nullptr, *g_p3 = nullptr, *g_e3 = nullptr, *g_p2 = nullptr;
     float *g_e2 = nullptr, *g_p1 = nullptr, *g_e1 = nullptr;
     // workspaces
-    bf16* cols = nullptr;      // column matrix, either layout
+    bf16* cols = nullptr;      // column matrix, either layout; the first layer's tap rows
     float* gemm = nullptr;     // column-path GEMM output
     float* partials = nullptr; // per-split partial products of a column-form weight gradient
     bf16* dz16 = nullptr;      // dZ, NHWC
@@ -1036,6 +1036,10 @@ cudaError_t wgrad_columns(gdrr_cnn* n, const Conv& L, int B, const View& X) {
     return cudaSuccess;
 }
 
+// Whether the loss, the output layer's backward and the last 3 x 3 layer's dZ are
+// one kernel: where that layer's weight gradient does not need dZ channel-major.
+bool head_fused(const gdrr_cnn* n) { return n->conv[6].implicit_dw && act_tile(n->c) == 64; }
+
 // Backward of one 3 x 3 convolution L on its grid: dy (gradient of the layer
 // output), Y (view of its BF16 output, for the ReLU mask), X (its plain NHWC
 // input, ci channels).  Writes the parameter gradients, those that sums of parts
@@ -1135,13 +1139,29 @@ GDRR_API int gdrr_cnn_create(int32_t max_batch, int32_t height, int32_t width, i
     }
     n->n_params = off;
     const int64_t B = max_batch, HW = (int64_t)H * W;
-    int64_t max_cols = 0, max_gemm = 0, max_dz = 0, max_part = 0;
-    for (const Conv& L : n->conv) {
+    // the forms of each layer's products, which the grid and the channels decide
+    // (not the batch), and the workspaces that those forms use
+    int64_t cols = 0, gemm = 0, dz = 0, dz_cp = 0, parts = 0;
+    for (Conv& L : n->conv) {
         const int64_t P = B * L.H * L.W, Pp = pad64(P);
-        max_cols = std::max({max_cols, Pp * L.K9p, P * L.K9dp});
-        max_gemm = std::max({max_gemm, P * L.ci, (int64_t)L.co * L.K9p, P * L.co});
-        max_dz = std::max({max_dz, P * L.co, (int64_t)L.co * Pp});
-        max_part = std::max(max_part, (int64_t)wgrad_splits(P) * L.co * L.K9p);
+        const bool first = &L == &n->conv.front(), last = L.ks == 1;
+        if (last) continue;
+        // (the two-channel input's: rows of 18 tap values in place of the tensor)
+        L.implicit_dw = first ? L.co % 32 == 0 : conv_wgrad_ok(L.ci, L.co, L.H, L.W);
+        dz = std::max(dz, P * L.co);
+        if (first && L.implicit_dw) cols = std::max(cols, P * 32);
+        if (!first && !conv_implicit_ok(L.ci, L.H, L.W) && !conv_tap_ok(L.ci, L.co)) {     // forward by columns
+            cols = std::max(cols, P * L.K9p);
+            gemm = std::max(gemm, P * L.co);
+        }
+        if (!first && !conv_implicit_ok(L.co, L.H, L.W) && !conv_tap_ok(L.co, L.ci))        // data gradient
+            cols = std::max(cols, P * L.K9dp);
+        if (!L.implicit_dw) {                                                               // weight gradient
+            cols = std::max(cols, Pp * L.K9p);
+            gemm = std::max(gemm, (int64_t)L.co * L.K9p);
+            dz_cp = std::max(dz_cp, (int64_t)L.co * Pp);
+            if (wgrad_splits(P) > 1) parts = std::max(parts, (int64_t)wgrad_splits(P) * L.co * L.K9p);
+        }
     }
     cudaError_t e = cudaSuccess;
     do {
@@ -1153,8 +1173,6 @@ GDRR_API int gdrr_cnn_create(int32_t max_batch, int32_t height, int32_t width, i
             const int64_t P = B * L.H * L.W;
             const bool first = &L == &n->conv.front(), last = L.ks == 1;
             const bool fwd = !last && conv_implicit_ok(L.ci, L.H, L.W), back = conv_implicit_ok(L.co, L.H, L.W);
-            // (the two-channel input's: rows of 18 tap values in place of the tensor)
-            L.implicit_dw = first ? L.co % 32 == 0 : !last && conv_wgrad_ok(L.ci, L.co, L.H, L.W);
             const int64_t k16 = (int64_t)L.co * L.K9p, kf16 = (int64_t)L.ci * L.K9dp, k3 = (int64_t)L.co * L.K9;
             if (fwd ? dalloc(n, &L.w3, k3) : (dalloc(n, &L.w16, k16) || cudaMemset(L.w16, 0, k16 * sizeof(bf16)))) bad = true;
             if (!first && !last &&
@@ -1171,17 +1189,20 @@ GDRR_API int gdrr_cnn_create(int32_t max_batch, int32_t height, int32_t width, i
             (e = dalloc(n, &n->p2, 2 * c * s3)) || (e = dalloc(n, &n->cat3, 12 * c * s3)) ||
             (e = dalloc(n, &n->p3, 4 * c * s4)) || (e = dalloc(n, &n->d1, c * s1)) || (e = dalloc(n, &n->out, s1)))
             break;
-        if ((e = dalloc(n, &n->g_out, s1)) || (e = dalloc(n, &n->g_d1, c * s1)) ||
-            (e = dalloc(n, &n->g_cat1, 3 * c * s1)) || (e = dalloc(n, &n->g_d2, 2 * c * s2)) ||
-            (e = dalloc(n, &n->g_cat2, 6 * c * s2)) || (e = dalloc(n, &n->g_d3, 4 * c * s3)) ||
-            (e = dalloc(n, &n->g_cat3, 12 * c * s3)) || (e = dalloc(n, &n->g_e4, 8 * c * s4)) ||
-            (e = dalloc(n, &n->g_p3, 4 * c * s4)) || (e = dalloc(n, &n->g_e3, 4 * c * s3)) ||
-            (e = dalloc(n, &n->g_p2, 2 * c * s3)) || (e = dalloc(n, &n->g_e2, 2 * c * s2)) ||
-            (e = dalloc(n, &n->g_p1, c * s2)) || (e = dalloc(n, &n->g_e1, c * s1)))
+        if ((e = dalloc(n, &n->g_cat1, 3 * c * s1)) || (e = dalloc(n, &n->g_cat2, 6 * c * s2)) ||
+            (e = dalloc(n, &n->g_cat3, 12 * c * s3)) || (e = dalloc(n, &n->g_p3, 4 * c * s4)) ||
+            (e = dalloc(n, &n->g_p2, 2 * c * s3)) || (e = dalloc(n, &n->g_p1, c * s2)))
             break;
-        if ((e = dalloc(n, &n->cols, max_cols)) || (e = dalloc(n, &n->gemm, max_gemm)) ||
-            (e = dalloc(n, &n->dz16, max_dz)) || (e = dalloc(n, &n->dz_cp, max_dz)) ||
-            (e = dalloc(n, &n->partials, max_part)) || (e = dalloc(n, &n->dloss, 1)) || (e = dalloc(n, &n->err, 1)))
+        // gradients that only a column form's passes write out
+        auto column = [&](int i) { return n->conv[i].implicit_dw ? 0 : 1; };
+        if ((e = dalloc(n, &n->g_out, head_fused(n) ? 0 : s1)) || (e = dalloc(n, &n->g_d1, head_fused(n) ? 0 : c * s1)) ||
+            (e = dalloc(n, &n->g_d2, 2 * c * s2 * column(5))) || (e = dalloc(n, &n->g_d3, 4 * c * s3 * column(4))) ||
+            (e = dalloc(n, &n->g_e4, 8 * c * s4 * column(3))) || (e = dalloc(n, &n->g_e3, 4 * c * s3 * column(2))) ||
+            (e = dalloc(n, &n->g_e2, 2 * c * s2 * column(1))) || (e = dalloc(n, &n->g_e1, c * s1 * column(0))))
+            break;
+        if ((e = dalloc(n, &n->cols, cols)) || (e = dalloc(n, &n->gemm, gemm)) || (e = dalloc(n, &n->dz16, dz)) ||
+            (e = dalloc(n, &n->dz_cp, dz_cp)) || (e = dalloc(n, &n->partials, parts)) || (e = dalloc(n, &n->dloss, 1)) ||
+            (e = dalloc(n, &n->err, 1)))
             break;
         // He-normal initial weights, zero biases
         std::vector<float> h(off, 0.0f);
@@ -1311,9 +1332,8 @@ GDRR_API int gdrr_cnn_backward(gdrr_cnn* n, const float* target_dev, double* los
         if ((e = cudaMemsetAsync(n->dloss, 0, sizeof(double), st))) break;
         SumJobs sums;
         sums.n = sums.blocks = 0;
-        // loss and the 1 x 1 output layer; the last 3 x 3 layer's dZ with them where
-        // its weight gradient does not need it channel-major
-        const bool fused_head = L[6].implicit_dw && act_tile(c) == 64;
+        // loss and the 1 x 1 output layer
+        const bool fused_head = head_fused(n);
         {
             const int nb = (int)((s1 + 255) / 256);
             float* pw = L[7].db_part;
