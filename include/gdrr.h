@@ -410,11 +410,12 @@ GDRR_API int gdrr_fdk_backproject(const gdrr_fdk_geometry* geometry, int32_t n_p
 GDRR_API int gdrr_probe_l2_gather(int64_t working_set_bytes, double* gbs_out, void* cuda_stream);
 GDRR_API int gdrr_probe_fp32(double* tflops_out, void* cuda_stream);
 
-/* Check of the bounded device-side wait (not part of the method): one CTA
- * waits, with a wait bounded by %globaltimer as the denoiser's are, for a flag
- * that nothing sets.  The wait gives up after limit_ns nanoseconds (1 ..
- * 2e9) and the call returns GDRR_ERR_TIMEOUT; GDRR_OK would mean the flag was
- * seen.  Allocates 16 bytes, runs on cuda_stream, synchronises. */
+/* Check of the denoiser's bounded wait (not part of the method): one tile of
+ * the one-launch denoiser runs without its neighbour and waits for pixels that
+ * nothing publishes.  The wait gives up after limit_ns nanoseconds (1 .. 2e9),
+ * the tile leaves its output unwritten and the call returns GDRR_ERR_TIMEOUT;
+ * GDRR_OK would mean that it went on.  Allocates 6 KB, runs on cuda_stream,
+ * synchronises. */
 GDRR_API int gdrr_probe_bounded_wait(uint64_t limit_ns, void* cuda_stream);
 
 /* Autotuner: time gdrr_mc_project of n_probe histories at angle_rad for each

@@ -120,38 +120,10 @@ struct McParams {
     int* status;                   // NULL, or where a bounded loop that gave up records it
 };
 
-// Bounded waits on flags that another CTA publishes (release store, acquire
-// load, both at GPU scope).  Every spin ends after limit_ns nanoseconds of
-// %globaltimer, so a flag that is never set costs a bounded delay and a
-// recorded timeout, not a hung GPU.
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
-}
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Waits until flags[j] >= want for the neighbour bands j = b - 1 and b + 1
-// that exist (0 <= j < G); false once limit_ns has passed.
-__device__ __forceinline__ bool wait_band_neighbours(const unsigned* flags, int b, int G, unsigned want,
-                                                     unsigned long long limit_ns) {
-    const unsigned long long t0 = globaltimer_ns();
-    for (int j = b - 1; j <= b + 1; j += 2) {
-        if (j < 0 || j >= G) continue;
-        while (ld_acquire_u32(flags + j) < want) {
-            if (globaltimer_ns() - t0 > limit_ns) return false;
-        }
-    }
-    return true;
 }
 
 // Material slots of the transport kernel (and of a macro-cell record) for
@@ -255,13 +227,19 @@ cudaError_t launch_noise(const double* ph, const double* p, const double* sh, co
 cudaError_t launch_denoise(const double* s_hat, double* s, int nu, int nv, double count_scale, double beta,
                            const double* scal_dev, double omega, int iters, double* scratch, cudaStream_t stream);
 size_t denoise_scratch_doubles(int nu, int nv);
-// Eq. 5 denoiser in one cooperative launch (images that fit its row bands):
+// Eq. 5 denoiser in one cooperative launch (images that fit a tile per SM):
 // scratch of denoise_fused_scratch_bytes; a wait that gives up sets *status.
 bool denoise_fused_fits(int nu, int nv);
 size_t denoise_fused_scratch_bytes(int nu, int nv);
 cudaError_t launch_denoise_fused(const double* s_hat, double* s_out, int nu, int nv, double count_scale,
                                  double beta, const double* scal_dev, double omega, int iters, void* scratch,
                                  int* status, cudaStream_t stream);
+// One tile of that kernel beside a tile that is not launched: it gives up after
+// limit_ns, sets *status and leaves out (DENOISE_PROBE_PIXELS doubles) as it was.
+// words: DENOISE_PROBE_WORDS bytes, zeroed.
+constexpr int DENOISE_PROBE_PIXELS = 128, DENOISE_PROBE_WORDS = 2 * DENOISE_PROBE_PIXELS * 16;
+cudaError_t launch_denoise_lone_tile(const double* in, double* out, void* words, unsigned long long limit_ns, int* status,
+                                     cudaStream_t stream);
 // gdrr_project's Step 3 scalars from the coarse scatter tally and the counters.
 cudaError_t launch_project_scalars(const int64_t* coarse, int n, const unsigned long long* stats,
                                    double tally_to_signal, double inv_n_photons, double beta, double smoothing_px,

@@ -2,7 +2,7 @@
 //  * tally -> signal per source photon (Section 2.6 normalisation);
 //  * exact integer binning to the coarse scatter grid, bilinear upsampling;
 //  * Step 3, Section 2.5: the Eq. 5 relaxation iteration of the Poisson
-//    denoiser (Eq. 2-4), in one cooperative launch whose row bands exchange
+//    denoiser (Eq. 2-4), in one cooperative launch whose tiles exchange
 //    iterates with their neighbours, or one launch per iteration with
 //    ping-pong buffers (images too large for the one-launch form, and the
 //    allocation-free entry point);
@@ -208,7 +208,7 @@ template <int PPT>
 __global__ void __launch_bounds__(1024) denoise_fused_kernel(
     const double* __restrict__ s_hat, double* __restrict__ s_out, int nu, int nv, int tile_w, int tile_h, int tiles_x,
     double count_scale_h, double beta_h, const double* __restrict__ scal, double omega, int iters, ulonglong2* words,
-    int* status) {
+    unsigned long long wait_ns, int* status) {
     extern __shared__ double img[];                  // [2][tile_h tile_w]
     const int x0 = (blockIdx.x % tiles_x) * tile_w, y0 = (blockIdx.x / tiles_x) * tile_h;
     const int w = min(tile_w, nu - x0), h = min(tile_h, nv - y0), npx = w * h;
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(1024) denoise_fused_kernel(
                         if ((want & 8u) && poll(me - nu, (unsigned)k + 1u, nb[3])) want &= ~8u;
                         if ((tries & 63u) == 63u) {
                             if (t0 == 0) t0 = globaltimer_ns();
-                            if (globaltimer_ns() - t0 > WAIT_NS) {
+                            if (globaltimer_ns() - t0 > wait_ns) {
                                 atomicOr(status, 1);
                                 fail = 1;
                                 break;
@@ -351,6 +351,7 @@ cudaError_t launch_denoise_fused(const double* s_hat, double* s_out, int nu, int
     cudaError_t e = cudaMemsetAsync(words, 0, denoise_fused_scratch_bytes(nu, nv), stream);   // no iterate's number
     if (e != cudaSuccess) return e;
     int tile_w = f.tile_w, tile_h = f.tile_h, tiles_x = f.tiles_x;
+    unsigned long long wait_ns = WAIT_NS;
     const size_t smem = 2 * (size_t)tile_w * tile_h * sizeof(double);
     const int ppt = (tile_w * tile_h + f.block - 1) / f.block;
     const void* kernel = ppt <= 1 ? (const void*)denoise_fused_kernel<1>
@@ -361,9 +362,19 @@ cudaError_t launch_denoise_fused(const double* s_hat, double* s_out, int nu, int
     }
     void* args[] = {(void*)&s_hat, (void*)&s_out, (void*)&nu, (void*)&nv, (void*)&tile_w, (void*)&tile_h,
                     (void*)&tiles_x, (void*)&count_scale, (void*)&beta, (void*)&scal_dev, (void*)&omega, (void*)&iters,
-                    (void*)&words, (void*)&status};
+                    (void*)&words, (void*)&wait_ns, (void*)&status};
     return cudaLaunchCooperativeKernel(kernel, dim3(f.grid), dim3(f.block), args, smem,
                                        stream);
+}
+
+cudaError_t launch_denoise_lone_tile(const double* in, double* out, void* words, unsigned long long limit_ns, int* status,
+                                     cudaStream_t stream) {
+    constexpr int TW = 32, TH = 2, TILES = 2, ITERS = 2;
+    static_assert(TW * TH * TILES == DENOISE_PROBE_PIXELS, "the probe's image");
+    denoise_fused_kernel<1><<<1, TW * TH, 2 * TW * TH * sizeof(double), stream>>>(
+        in, out, TW * TILES, TH, TW, TH, TILES, 1.0, 1.0, nullptr, 0.8, ITERS, static_cast<ulonglong2*>(words), limit_ns,
+        status);
+    return cudaGetLastError();
 }
 
 namespace {

@@ -8,8 +8,8 @@
 //    flops per FMA.
 // Both kernels keep their results live (a checksum store) so nothing is
 // optimised away; both run a fixed amount of work per thread.
-// A third probe checks the bounded wait that CTA-to-CTA exchanges use: a
-// wait on a flag that nothing sets must give up after its limit and report
+// A third probe checks the bounded wait of the denoiser's tiles: a tile whose
+// neighbour is not there must give up after its limit and report
 // GDRR_ERR_TIMEOUT.
 #include "gdrr_internal.cuh"
 
@@ -46,30 +46,31 @@ __global__ void __launch_bounds__(PROBE_BLOCK) fp32_fma_kernel(float seed, int i
     if (s == 12345.678f) sink[0] = s;
 }
 
-// One CTA waiting, with the bounded wait of the CTA-to-CTA exchanges, for a
-// neighbour flag that nothing sets: the wait must give up and record it.
-__global__ void wait_probe_kernel(const unsigned* flags, unsigned long long limit_ns, int* status) {
-    if (threadIdx.x == 0 && !wait_band_neighbours(flags, 0, 2, 1u, limit_ns)) atomicOr(status, 1);
-}
-
 }  // namespace
 }  // namespace gdrr
 
 extern "C" GDRR_API int gdrr_probe_bounded_wait(uint64_t limit_ns, void* cuda_stream) {
     if (limit_ns == 0 || limit_ns > 2000000000ull) return GDRR_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    unsigned* buf = nullptr;
+    // status, then input and output pixels, then the words that nothing publishes
+    constexpr size_t PIXELS = gdrr::DENOISE_PROBE_PIXELS * sizeof(double);
+    uint8_t* buf = nullptr;
     int status = 0;
-    if (cudaMalloc((void**)&buf, 4 * sizeof(unsigned)) != cudaSuccess) return GDRR_ERR_OOM;
-    cudaError_t e = cudaMemsetAsync(buf, 0, 4 * sizeof(unsigned), s);
-    if (e == cudaSuccess) {
-        gdrr::wait_probe_kernel<<<1, 32, 0, s>>>(buf, (unsigned long long)limit_ns, reinterpret_cast<int*>(buf + 2));
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, buf + 2, sizeof(int), cudaMemcpyDeviceToHost, s);
+    uint64_t out[gdrr::DENOISE_PROBE_PIXELS];
+    if (cudaMalloc((void**)&buf, 16 + 2 * PIXELS + gdrr::DENOISE_PROBE_WORDS) != cudaSuccess) return GDRR_ERR_OOM;
+    uint8_t* const pixels = buf + 16;
+    cudaError_t e = cudaMemsetAsync(buf, 0, 16 + 2 * PIXELS + gdrr::DENOISE_PROBE_WORDS, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(pixels + PIXELS, 0xff, PIXELS, s);
+    if (e == cudaSuccess)
+        e = gdrr::launch_denoise_lone_tile(reinterpret_cast<const double*>(pixels), reinterpret_cast<double*>(pixels + PIXELS),
+                                           pixels + 2 * PIXELS, (unsigned long long)limit_ns, reinterpret_cast<int*>(buf), s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, buf, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, pixels + PIXELS, PIXELS, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(buf);
     if (e != cudaSuccess) return GDRR_ERR_CUDA;
+    for (uint64_t v : out)
+        if (v != ~0ull) return GDRR_OK;          // the tile went on
     return status ? GDRR_ERR_TIMEOUT : GDRR_OK;
 }
 

@@ -560,7 +560,7 @@ def gdrr_probe_l2_gather(working_set_bytes: int = 32 << 20, stream=None) -> floa
 
 
 def gdrr_probe_bounded_wait(limit_ns: int, stream=None) -> int:
-    """Return code of a bounded device wait on a flag nothing sets (-7: timed out)."""
+    """Return code of a denoiser tile that waits for a neighbour that is not there (-7: timed out)."""
     h, _ = _stream_handle(stream)
     return lib().gdrr_probe_bounded_wait(int(limit_ns), h)
 
