@@ -659,6 +659,11 @@ GDRR_API int gdrr_cnn_adam_step(gdrr_cnn* net, float lr, float beta1, float beta
 GDRR_API int gdrr_stream_words(uint64_t seed, uint32_t angle_index, uint64_t hid0, int32_t n_hist,
                                int32_t n_blocks, uint32_t* out_dev, void* cuda_stream);
 
+/* Parity hook: ln(k 2^-24) for the integers k = k0 .. k0 + n - 1 within 1 ..
+ * 2^24, exactly as the transport's free flights form it.  out_dev: device
+ * float[n].  Runs on cuda_stream. */
+GDRR_API int gdrr_flight_logs(int32_t k0, int32_t n, float* out_dev, void* cuda_stream);
+
 #ifdef __cplusplus
 }
 #endif

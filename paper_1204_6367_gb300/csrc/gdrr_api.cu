@@ -1460,4 +1460,9 @@ GDRR_API int gdrr_stream_words(uint64_t seed, uint32_t angle_index, uint64_t hid
     return cuda_err(launch_stream_words(seed, angle_index, hid0, n_hist, n_blocks, out_dev, (cudaStream_t)cuda_stream));
 }
 
+GDRR_API int gdrr_flight_logs(int32_t k0, int32_t n, float* out_dev, void* cuda_stream) {
+    if (n < 0 || k0 < 1 || (int64_t)k0 + n - 1 > (1 << 24) || (n > 0 && !out_dev)) return GDRR_ERR_INVALID_ARG;
+    return cuda_err(launch_flight_logs((uint32_t)k0, n, out_dev, (cudaStream_t)cuda_stream));
+}
+
 }  // extern "C"

@@ -215,6 +215,7 @@ cudaError_t launch_air(const RtParams& p, double* out, cudaStream_t s);
 cudaError_t launch_gather_probe(const McParams& p, uint64_t n_cells, int grid, unsigned int* sink, cudaStream_t s);
 cudaError_t launch_stream_words(uint64_t seed, uint32_t angle_index, uint64_t hid0, int n_hist,
                                 int n_blocks, uint32_t* out, cudaStream_t s);
+cudaError_t launch_flight_logs(uint32_t k0, int n, float* out, cudaStream_t s);
 
 cudaError_t launch_finalize(const int64_t* t, int64_t n, double scale, double* out, int* bad, cudaStream_t s);
 cudaError_t launch_bin(const int64_t* t, int nu, int nv, int f, int64_t* out, cudaStream_t s);

@@ -1662,6 +1662,11 @@ __global__ void stream_words_kernel(const RoundKeys rk, uint32_t angle_index, ui
     }
 }
 
+__global__ void flight_logs_kernel(uint32_t k0, int n, float* out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = log_uniform(k0 + (uint32_t)i);
+}
+
 template <int NM>
 constexpr size_t smem_bytes(int block) { return (size_t)3 * NM * block * sizeof(float); }
 
@@ -1755,6 +1760,12 @@ cudaError_t launch_stream_words(uint64_t seed, uint32_t angle_index, uint64_t hi
     if (n_hist <= 0) return cudaSuccess;
     stream_words_kernel<<<(n_hist + 127) / 128, 128, 0, s>>>(round_keys(seed), angle_index, hid0, n_hist, n_blocks,
                                                              out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_flight_logs(uint32_t k0, int n, float* out, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    flight_logs_kernel<<<(n + 255) / 256, 256, 0, s>>>(k0, n, out);
     return cudaGetLastError();
 }
 

@@ -146,6 +146,7 @@ def lib():
             "gdrr_noise_calibrate": [vp, vp, vp, vp, vp, i64, u64, dbl, dbl, vp],
             "gdrr_fit_zeta": [vp, vp, i32, u64, vp, vp],
             "gdrr_stream_words": [u64, u32, u64, i32, i32, vp, vp],
+            "gdrr_flight_logs": [i32, i32, vp, vp],
             "gdrr_gather_roofline": [vp, u64, vp],
             "gdrr_scan_create": [vp, i32, vp, vp, u64, vp, vp, vp, i32, vp],
             "gdrr_scan_launch": [vp],
@@ -541,6 +542,15 @@ def gdrr_stream_words(seed: int, angle_index: int, hid0: int, n_hist: int, n_blo
     h, _ = _stream_handle(stream)
     _check("gdrr_stream_words", lib().gdrr_stream_words(int(seed), int(angle_index), int(hid0), int(n_hist),
                                                         int(n_blocks), _dev_ptr(out, torch.int32, None, "out"), h))
+    return out
+
+
+def gdrr_flight_logs(k0: int, n: int, stream=None):
+    """ln(k 2^-24) FP32 for k = k0 .. k0 + n - 1, as the free flights form it."""
+    import torch
+    out = torch.empty(n, dtype=torch.float32, device="cuda")
+    h, _ = _stream_handle(stream)
+    _check("gdrr_flight_logs", lib().gdrr_flight_logs(int(k0), int(n), _dev_ptr(out, torch.float32, None, "out"), h))
     return out
 
 
