@@ -30,7 +30,8 @@ constexpr int RT_BX = 16, RT_BY = 8;      // pixels of a block of the tri-linear
 // samples before them are of one material, and only a sample that mixes
 // materials, or meets another one, takes the per-material sums apart.  Each
 // material's terms are added in the order of the plain loop over samples,
-// corners and materials, so the result is the same to the bit.  2 mm torso, 512
+// corners and materials, one rounded product and one rounded addition each on
+// either path (never contracted to an FMA), so the result is the same to the bit.  2 mm torso, 512
 // x 384 pixels: 0.99 ms with every corner tested against every material and
 // warps of 32 x 1 pixels, 0.53 ms so.  WIDE: an axis has 2^22 voxels or more,
 // beyond the floor by addition.
@@ -137,19 +138,19 @@ __global__ void __launch_bounds__(RT_BX * RT_BY) rt_kernel(const RtParams P, int
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const uint2 vx = __ldg(P.vox + v0 + (c & 1 ? sx : 0) + (c & 2 ? sy : 0) + (c & 4 ? sz : 0));
-                a[c] = (wxy[c & 3] * (c & 4 ? w1[2] : u1[2])) * __uint_as_float(vx.x);
+                a[c] = __fmul_rn(__fmul_rn(wxy[c & 3], c & 4 ? w1[2] : u1[2]), __uint_as_float(vx.x));
                 mc[c] = (int)vx.y;
                 mixed |= vx.y ^ (unsigned)cur;
             }
             if (mixed == 0u) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c) e += a[c];
+                for (int c = 0; c < 8; ++c) e = __fadd_rn(e, a[c]);
             } else {
 #pragma unroll
                 for (int m = 0; m < NM; ++m) {
                     float l = cur == m ? e : ell[m];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) l += mc[c] == m ? a[c] : 0.0f;
+                    for (int c = 0; c < 8; ++c) l = __fadd_rn(l, mc[c] == m ? a[c] : 0.0f);
                     ell[m] = l;
                 }
                 cur = mc[7];
