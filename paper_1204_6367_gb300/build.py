@@ -33,7 +33,8 @@ SOURCES = {
     "fdk.cu": [],
     "probes.cu": [],
 }
-HEADERS = [os.path.join(INCLUDE, "gdrr.h")] + [os.path.join(CSRC, h) for h in ("gdrr_internal.cuh", "cnn_epi.cuh", "fdk_rows.h")]
+HEADERS = [os.path.join(INCLUDE, "gdrr.h")] + [os.path.join(CSRC, h) for h in (
+    "gdrr_internal.cuh", "cnn_epi.cuh", "fdk_rows.h", "transport_rules.h")]
 
 
 def nvcc() -> str:

@@ -117,6 +117,7 @@ struct McParams {
     // majorant; the cells' planes need the voxel edges
     int lm;
     float vox_mm[3];
+    int in_place;                  // general form: tentative collisions are decided in the flight
     int* status;                   // NULL, or where a bounded loop that gave up records it
 };
 

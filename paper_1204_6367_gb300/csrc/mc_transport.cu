@@ -69,6 +69,7 @@
 #include <algorithm>
 
 #include "gdrr_internal.cuh"
+#include "transport_rules.h"
 
 namespace gdrr {
 namespace {
@@ -1063,11 +1064,6 @@ constexpr int REFILL_IDLE = 8;
 // would come after each: 2e7 histories of the 2 mm torso take 14.17 ms at 8, 13.93
 // at 14, 13.67 at 18, 13.57 from 20 to 24 and 14.17 at 30.
 constexpr int REFILL_IDLE_LM = 22;
-// Local-majorant cells of at least 2^5 voxels an edge, where most flights end in
-// the cell they start in: the general form decides them where they are (2e7
-// histories of the 2 mm torso: 17.9 ms by way of the gather service and 15.5 so
-// with 64 mm cells, 31.8 and 21.2 with 128 mm; with 32 mm 11.8 and 13.1).
-constexpr int LM_INLINE_SHIFT = 5;
 // a slot's flags beside its job
 constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_JOB = 0x1fffffffu;
 
@@ -1331,7 +1327,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_M
                         L.state = S_FLY;
                         L.walk(P, bound_of<NM>(P, L.cx + P.csx * (L.cy + P.csy * L.cz), cf));
                         code = L.state == S_FLY ? F_ON : (L.state == S_GATHER ? F_GATHER : F_ESC);
-                        if (GEN && P.cshift >= LM_INLINE_SHIFT && code == F_GATHER && !P.nearest_voxel) {
+                        if (GEN && P.in_place && code == F_GATHER && !P.nearest_voxel) {
                             // coarse cells: the mixture and a virtual collision's next
                             // flight here (a history at max_steps ends in the service)
                             float a[8];
@@ -1690,6 +1686,10 @@ cudaError_t launch_records_t(const McParams& p, int block, int per_sm_max, int n
 // no cell test: none is wanted, or an axis has corners that corner_bits cannot count
 inline bool without_cells(const McParams& p) { return !p.cells || std::max(p.nx, std::max(p.ny, p.nz)) >= 1 << 22; }
 
+inline bool in_place(const McParams& p) {
+    return p.lm ? lm_in_place(cell_edge(p.vox_mm, p.cshift)) : without_cells(p);
+}
+
 template <int NM, bool GEN, bool LM>
 cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm, cudaStream_t s) {
     const size_t bytes = warp_smem_bytes<NM, GEN, LM>(n_pool) * (WARP_BLOCK / 32);
@@ -1708,6 +1708,7 @@ cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm
     const int n_use = (int)std::min<uint64_t>((uint64_t)n_pool, share);
     const unsigned chunk = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)p.chunk, share / 4 + 1));
     McParams q = p;
+    q.in_place = in_place(p);
     if (!LM && without_cells(p)) {
         q.cells = q.open_cell;
         q.cshift = 30;
@@ -1741,8 +1742,7 @@ cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photo
     // flights without a cell test evaluate the mixture in place, which only the
     // general form has the registers for: 1e8 histories of the 2 mm torso by way of
     // the gather service took 209 ms (156 with one photon per lane), so 134
-    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 ||
-                     (!records && (p.lm ? p.cshift >= LM_INLINE_SHIFT : without_cells(p)));
+    const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 || (!records && in_place(p));
     const int n_pool = photons > 0 ? 32 * photons : POOL_DEFAULT;
     if (p.lm) return gen ? launch_nm<true, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s)
                          : launch_nm<false, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s);
