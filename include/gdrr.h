@@ -183,10 +183,10 @@ typedef struct {
                                   corner gathers, interactions, tallies and new
                                   histories each run on full warps.  Tallies, counters
                                   and records are the same for every choice; -1: the
-                                  pool that runs fastest, 80 photons per warp, which
-                                  local_majorant always takes (on the 2 mm torso 64, 72,
-                                  80 and 88 ran at 19.1, 18.2, 17.9 and 18.7 ms per 3e7
-                                  histories) [-1]                                     */
+                                  pool that runs fastest, 56 to 84 photons per warp by
+                                  the run's form, which local_majorant always takes (on
+                                  the 2 mm torso 64, 72, 80 and 88 ran at 19.1, 18.2,
+                                  17.9 and 18.7 ms per 3e7 histories) [-1]            */
     int32_t local_majorant;    /* 1: delta tracking with local majorants, an option
                                   beside the paper's global Woodcock majorant: the
                                   macro-cell bounds (cell_shift, which must not be -1)

@@ -1050,13 +1050,7 @@ __global__ void __launch_bounds__(512, 2) mc_kernel(const McParams P) {
 // max_steps costs no counter of its own.  The totals of free flights, and of
 // the virtual collisions the cells decided, follow from warp-wide counts of
 // lanes per iteration.
-constexpr int WARP_BLOCK = 128;                // threads; the warps of a block share nothing but counters
-// Resident blocks the registers are held down for: 24 warps per SM (80
-// registers), 20 for the general form.  On the 2 mm torso 28 warps (72) and 32
-// (64 registers, spills in the flight loop) were 1 and 8 % slower.
-constexpr int WARP_MIN_BLOCKS = 6, WARP_MIN_BLOCKS_GEN = 5;
-constexpr int POOL_DEFAULT = 80;               // photons per warp: the most that 24 warps' shared memory holds
-constexpr int POOL_MAX = 96;                   // the largest pool that an option asks for
+constexpr int WARP_BLOCK = 32 * POOL_WARPS;   // threads; the warps of a block share nothing but counters
 // Idle lanes at which the warp hands over and refills: 5, 6, 8 and 12 were
 // within 2 %, 4 was 3 % slower (a hand-over costs about half a flight).
 constexpr int REFILL_IDLE = 8;
@@ -1071,6 +1065,7 @@ template <int NM, bool GEN, bool LM>
 struct Slots {
     static constexpr int CF = NM < 4 ? 1 : NM / 4;              // float4 words of the total coefficients
     static constexpr int Q_LM = 4 + CF, Q_GEN = Q_LM + (LM ? 1 : 0), Q = Q_GEN + (GEN ? 1 : 0);
+    static_assert(Q == slot_words(NM, GEN, LM), "the rules' size of a slot");
     float4* s;
     __device__ __forceinline__ float4& at(int slot, int q) const { return s[slot * Q + q]; }
     __device__ __forceinline__ uint32_t& word(int slot, int q, int w) const {
@@ -1104,11 +1099,7 @@ enum : int { F_NONE = 0, F_ON = 1, F_GATHER = 2, F_ESC = 3, F_LIMIT = 4 };
 // a warp's counts: the statistics, then the flights that stopped at a
 // tentative collision and outside the box
 enum : int { A_GATHER = GDRR_NSTATS, A_ESC, A_N };
-
-template <int NM, bool GEN, bool LM>
-__host__ __device__ constexpr size_t warp_smem_bytes(int n) {
-    return (size_t)n * Slots<NM, GEN, LM>::Q * 16 + (size_t)2 * NM * 32 * 4 + (size_t)4 * n + (A_N + 3) / 2 * 16;
-}
+static_assert(A_N == POOL_COUNTS, "the rules' size of a warp's counts");
 
 // One row of the energy-major coefficient table [energy][kind][NM].
 template <int NM>
@@ -1210,15 +1201,15 @@ __device__ __forceinline__ float bound_of(const McParams& P, int cell, const flo
 
 
 template <int NM, bool GEN, bool LM>
-__global__ void __launch_bounds__(WARP_BLOCK, GEN ? WARP_MIN_BLOCKS_GEN : WARP_MIN_BLOCKS) mc_warp_kernel(const McParams P, int n_pool, int n_use, unsigned chunk,
-                                                            uint32_t cell0) {
+__global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_kernel(
+    const McParams P, int n_pool, int n_use, unsigned chunk, uint32_t cell0) {
     extern __shared__ __align__(16) unsigned char warp_smem[];
     __shared__ unsigned long long cnt[GDRR_NSTATS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     for (int i = threadIdx.x; i < GDRR_NSTATS; i += WARP_BLOCK) cnt[i] = 0ull;
     __syncthreads();
-    unsigned char* base = warp_smem + (size_t)warp * warp_smem_bytes<NM, GEN, LM>(n_pool);
+    unsigned char* base = warp_smem + (size_t)warp * pool_bytes(n_pool, NM, GEN, LM);
     Slots<NM, GEN, LM> S;
     S.s = reinterpret_cast<float4*>(base);
     float* coef = reinterpret_cast<float*>(base + (size_t)n_pool * S.Q * 16) + lane;       // [2 NM][32], this lane's column
@@ -1692,14 +1683,15 @@ inline bool in_place(const McParams& p) {
 
 template <int NM, bool GEN, bool LM>
 cudaError_t launch_warp_t(const McParams& p, int n_pool, int warps_max, int n_sm, cudaStream_t s) {
-    const size_t bytes = warp_smem_bytes<NM, GEN, LM>(n_pool) * (WARP_BLOCK / 32);
-    cudaError_t e = allow_smem(mc_warp_kernel<NM, GEN, LM>, warp_smem_bytes<NM, GEN, LM>(POOL_MAX) * (WARP_BLOCK / 32));
+    if (n_pool <= 0) n_pool = default_pool(NM, GEN, LM);
+    const size_t bytes = pool_bytes(n_pool, NM, GEN, LM) * POOL_WARPS;
+    cudaError_t e = allow_smem(mc_warp_kernel<NM, GEN, LM>, pool_bytes(POOL_MAX, NM, GEN, LM) * POOL_WARPS);
     int per_sm = 0;
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mc_warp_kernel<NM, GEN, LM>, WARP_BLOCK, bytes);
     if (e != cudaSuccess) return e;
     if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-    constexpr int WPB = WARP_BLOCK / 32;
+    constexpr int WPB = POOL_WARPS;
     if (warps_max > 0) per_sm = std::max(1, std::min(per_sm, (warps_max + WPB - 1) / WPB));
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * n_sm, (int64_t)((p.total + WPB - 1) / WPB)));
     const int64_t warps = grid * WPB;
@@ -1743,7 +1735,7 @@ cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photo
     // general form has the registers for: 1e8 histories of the 2 mm torso by way of
     // the gather service took 209 ms (156 with one photon per lane), so 134
     const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 || (!records && in_place(p));
-    const int n_pool = photons > 0 ? 32 * photons : POOL_DEFAULT;
+    const int n_pool = photons > 0 ? 32 * photons : 0;
     if (p.lm) return gen ? launch_nm<true, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s)
                          : launch_nm<false, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s);
     return gen ? launch_nm<true, false>(p, records, block, n_pool, blocks_per_sm, n_sm, s)

@@ -19,7 +19,7 @@ def _evaluate(tmp_path, expressions):
     src.write_text('#include <cstdio>\n#include "transport_rules.h"\nusing namespace gdrr;\n'
                    "static float edge(float x, float y, float z, int s) { const float v[3] = {x, y, z}; "
                    "return cell_edge(v, s); }\nint main() {\n" + lines + "\n}\n")
-    subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, "-I", os.path.join(ROOT, "include"), str(src), "-o", str(exe)], check=True)
     return [float(v) for v in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()]
 
 
@@ -33,3 +33,17 @@ def test_local_majorants_in_place_by_the_cells_edge(tmp_path):
     assert got == [float(mm >= 64.0) for _, _, mm in CELLS]
     # the smallest edge counts
     assert _evaluate(tmp_path, ["edge(2.0f, 3.0f, 1.0f, 5)", "edge(4.0f, 2.0f, 8.0f, 3)"]) == [32.0, 16.0]
+
+
+@pytest.mark.parametrize("nm", [2, 4, 8])
+@pytest.mark.parametrize("gen", [0, 1])
+@pytest.mark.parametrize("lm", [0, 1])
+def test_default_pools_leave_the_sm_its_l1(tmp_path, nm, gen, lm):
+    n, held, aligned = _evaluate(tmp_path, [f"default_pool({nm}, {gen}, {lm})",
+                                            f"shared_of_blocks(default_pool({nm}, {gen}, {lm}), {nm}, {gen}, {lm})",
+                                            f"pool_bytes(default_pool({nm}, {gen}, {lm}), {nm}, {gen}, {lm}) % 16"])
+    # 256 KB of L1 and shared memory per SM, 60 KB of it L1; a pool is more than a
+    # warp, its slots count in bytes, and the next warp's slots stay aligned
+    assert held <= 196 * 1024 and 32 < n <= 84 and aligned == 0
+    if (nm, gen, lm) == (4, 0, 0):
+        assert n == 80
