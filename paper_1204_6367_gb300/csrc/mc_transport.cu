@@ -1182,6 +1182,16 @@ __device__ __forceinline__ uint4 flight_block(uint32_t blk, const FlightKeys& k,
 // copy of cell 0 in the table.
 __device__ __forceinline__ uint32_t corner_bits(float y) { return __float_as_uint(__fadd_rd(y, 8388607.5f)); }
 
+// The macro cell of a point inside the box: that of its lower trilinear corner,
+// as gather() computes it (cell0: the number that corner_bits' offset makes of
+// cell 0).
+__device__ __forceinline__ int cell_at(const McParams& P, float x, float y, float z, uint32_t cell0) {
+    const uint32_t ux = corner_bits((x - P.lo[0]) * P.ivox[0]) >> P.cshift;
+    const uint32_t uy = corner_bits((y - P.lo[1]) * P.ivox[1]) >> P.cshift;
+    const uint32_t uz = corner_bits((z - P.lo[2]) * P.ivox[2]) >> P.cshift;
+    return (int)(ux + P.csx * (uy + P.csy * uz) - cell0);
+}
+
 // The macro-cell bound (Lane::cell_bound) from the cell's densities.
 template <int NM>
 __device__ __forceinline__ float bound_of(const float (&v)[NM], const float (&cf)[NM]) {
@@ -1250,7 +1260,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
             uint32_t blk = 0, limit = 0, wy = 0, wz = 0, gz = 0;
             FlightKeys key = {0, 0, 0, 0};
             int slot = 0, code = F_NONE;
-            unsigned flown = 0, crossed = 0, drawn = 0;
+            unsigned flown = 0, crossed = 0, drawn = 0, celled = 0;
             for (;;) {
                 const unsigned act = __ballot_sync(FULL, code == F_ON);
                 int n_act = __popc(act);
@@ -1312,7 +1322,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
                     nR = max(0, nR - __popc(~act));
                 }
                 flown += (unsigned)n_act;
-                bool again = false;
+                bool again = false, over = false;
                 if (code == F_ON) {
                     if constexpr (LM) {
                         L.state = S_FLY;
@@ -1348,10 +1358,12 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
                         // what decides a tentative collision is loaded first ...
                         float v[NM];
                         uint2 vx = make_uint2(0u, 0u);
-                        const bool nearest = GEN && P.nearest_voxel, open = GEN && P.cells == P.open_cell;
+                        const bool nearest = GEN && P.nearest_voxel, here = GEN && P.in_place;
                         float mu = 0.0f;
-                        if (open && !nearest) {
-                            // no cell test: the mixture itself, here where nearly all are virtual
+                        if (here && !nearest) {
+                            // no cells, or cells so coarse that few collisions are virtual by their
+                            // bound: the mixture itself, here where nearly all are virtual, and the
+                            // bound (never below it) for the count of those it decides
                             if (inside) {
                                 float a[8];
                                 int mc[8];
@@ -1359,6 +1371,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
                                 mu = a[0] * __uint_as_float(S.word(slot, 4, mc[0]));
 #pragma unroll
                                 for (int c = 1; c < 8; ++c) mu = mu + a[c] * __uint_as_float(S.word(slot, 4, mc[c]));
+                                if (P.cells != P.open_cell)
+                                    over = t > bound_of<NM>(P, cell_at(P, qx, qy, qz, cell0), cf);
                             }
                         } else if (nearest) {
                             const int gx = min(max((int)floorf((qx - P.lo[0]) * P.ivox[0]), 0), P.nx - 1);
@@ -1366,11 +1380,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
                             const int gv = min(max((int)floorf((qz - P.lo[2]) * P.ivox[2]), 0), P.nz - 1);
                             vx = __ldg(P.vox + brick_x(gx) + brick_y(gy, P.bsy) + brick_z(gv, P.bsz));
                         } else {
-                            // the lower trilinear corner, as gather() computes it, locates the macro cell
-                            const uint32_t ux = corner_bits((qx - P.lo[0]) * P.ivox[0]) >> P.cshift;
-                            const uint32_t uy = corner_bits((qy - P.lo[1]) * P.ivox[1]) >> P.cshift;
-                            const uint32_t uz = corner_bits((qz - P.lo[2]) * P.ivox[2]) >> P.cshift;
-                            const int cell = (int)(ux + P.csx * (uy + P.csy * uz) - cell0);
+                            const int cell = cell_at(P, qx, qy, qz, cell0);
                             coef_row<NM>(P.cells + (ptrdiff_t)(inside ? cell : 0) * NM, v);
                         }
                         // ... and the next flight's words formed while it comes
@@ -1382,7 +1392,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
                         wy = w.y;
                         if (GEN) wz = w.z;
                         const bool skip = t > (nearest ? __uint_as_float(vx.x) * __uint_as_float(S.word(slot, 4, (int)vx.y))
-                                                       : open ? mu : bound_of<NM>(v, cf));
+                                                       : here ? mu : bound_of<NM>(v, cf));
                         L.tg = t;
                         if (inside) { L.px = qx; L.py = qy; L.pz = qz; }
                         code = skip ? F_ON : F_GATHER;
@@ -1392,6 +1402,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
                 }
                 if (LM) crossed += (unsigned)__popc(__ballot_sync(FULL, code == F_ON && !again));
                 if (LM && GEN) drawn += (unsigned)__popc(__ballot_sync(FULL, again));
+                if (!LM && GEN && P.in_place) celled += (unsigned)__popc(__ballot_sync(FULL, code == F_ON && over));
             }
             // park the photons still in flight
             __syncwarp();
@@ -1412,6 +1423,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
             }
             nR += __popc(fly);
             add(LM ? GDRR_ST_CELL_CROSSINGS : GDRR_ST_STEPS, LM ? crossed : flown);
+            if (!LM && GEN) add(GDRR_ST_CELL_SKIPS, celled);
             if (LM && GEN) {
                 add(GDRR_ST_STEPS, drawn);
                 add(GDRR_ST_VIRTUAL, drawn);
@@ -1592,7 +1604,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, pool_blocks(NM, GEN, LM)) mc_warp_
     if (!LM && lane == 0) {
         const unsigned long long inl = acc[GDRR_ST_STEPS] - acc[A_GATHER] - acc[A_ESC];
         acc[GDRR_ST_VIRTUAL] += inl;
-        if (!(GEN && (P.nearest_voxel || P.cells == P.open_cell))) acc[GDRR_ST_CELL_SKIPS] += inl;
+        if (!(GEN && (P.nearest_voxel || P.in_place))) acc[GDRR_ST_CELL_SKIPS] += inl;
     }
     __syncwarp();
     if (lane < GDRR_NSTATS && acc[lane]) atomicAdd(&cnt[lane], acc[lane]);
@@ -1678,7 +1690,8 @@ cudaError_t launch_records_t(const McParams& p, int block, int per_sm_max, int n
 inline bool without_cells(const McParams& p) { return !p.cells || std::max(p.nx, std::max(p.ny, p.nz)) >= 1 << 22; }
 
 inline bool in_place(const McParams& p) {
-    return p.lm ? lm_in_place(cell_edge(p.vox_mm, p.cshift)) : without_cells(p);
+    return p.lm ? lm_in_place(cell_edge(p.vox_mm, p.cshift))
+                : without_cells(p) || coarse_in_place(cell_edge(p.vox_mm, p.cshift));
 }
 
 template <int NM, bool GEN, bool LM>
@@ -1731,9 +1744,9 @@ cudaError_t launch_nm(const McParams& p, bool records, int block, int n_pool, in
 cudaError_t launch_mc(const McParams& p, int block, int blocks_per_sm, int photons, bool records, int n_sm,
                       cudaStream_t s) {
     if (p.lm && !p.cells) return cudaErrorInvalidValue;   // the local majorants are the cell bounds
-    // flights without a cell test evaluate the mixture in place, which only the
-    // general form has the registers for: 1e8 histories of the 2 mm torso by way of
-    // the gather service took 209 ms (156 with one photon per lane), so 134
+    // the mixture in the flight or walk is the general form's alone, which has the
+    // registers for it: 1e8 histories of the 2 mm torso without a cell test took
+    // 209 ms by way of the gather service (156 with one photon per lane), so 134
     const bool gen = p.nearest_voxel != 0 || p.scatter_filter != 0 || p.ray_ff != 0 || (!records && in_place(p));
     const int n_pool = photons > 0 ? 32 * photons : 0;
     if (p.lm) return gen ? launch_nm<true, true>(p, records, block, n_pool, blocks_per_sm, n_sm, s)

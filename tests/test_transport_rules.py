@@ -35,6 +35,12 @@ def test_local_majorants_in_place_by_the_cells_edge(tmp_path):
     assert _evaluate(tmp_path, ["edge(2.0f, 3.0f, 1.0f, 5)", "edge(4.0f, 2.0f, 8.0f, 3)"]) == [32.0, 16.0]
 
 
+def test_coarse_cells_in_place_by_their_edge(tmp_path):
+    cells = CELLS + [(3.0, 5, 96.0), (5.0, 5, 160.0), (3.0, 6, 192.0), (16.0, 4, 256.0), (4.0, 1, 8.0)]
+    got = _evaluate(tmp_path, [f"coarse_in_place(edge({v}f, {v}f, {v}f, {s}))" for v, s, _ in cells])
+    assert got == [float(mm >= 128.0) for _, _, mm in cells]
+
+
 @pytest.mark.parametrize("nm", [2, 4, 8])
 @pytest.mark.parametrize("gen", [0, 1])
 @pytest.mark.parametrize("lm", [0, 1])
