@@ -34,7 +34,7 @@ SOURCES = {
     "probes.cu": [],
 }
 HEADERS = [os.path.join(INCLUDE, "gdrr.h")] + [os.path.join(CSRC, h) for h in (
-    "gdrr_internal.cuh", "cnn_epi.cuh", "fdk_rows.h", "transport_rules.h")]
+    "gdrr_internal.cuh", "cnn_epi.cuh", "fdk_filter.h", "fdk_rows.h", "transport_rules.h")]
 
 
 def nvcc() -> str:

@@ -16,16 +16,17 @@
 // memory with register tiles; the backprojection gathers 4 detector samples per voxel
 // and view from L1 / L2 and keeps a few voxels of a column in registers, so the
 // per-view geometry (depth, u, weight) is computed once per column.
+#include <algorithm>
 #include <cmath>
+#include <functional>
 
+#include "fdk_filter.h"
 #include "fdk_rows.h"
 #include "gdrr_internal.cuh"
 
 namespace gdrr {
 namespace {
 
-constexpr int FILTER_BLOCK = 256;
-constexpr int FILTER_MAX_NU = 4096;
 constexpr int BP_MAX_ANGLES = 128;     // views per backprojection launch (kernel parameters)
 constexpr int BP_ZT = 4;               // voxels of a column per thread
 constexpr int BP_BX = 32, BP_BY = 8;   // voxels of a block in x and y, by warps of 8 x 4
@@ -52,33 +53,9 @@ struct FilterParams {
 // at 128 per SM and cycle) and the rows' weighting before it: 0.88 ms.  One row
 // per block and 4 outputs per thread took 2.6 ms at the full shared-memory
 // rate; 8 rows per thread (2 blocks per SM) 0.95 ms, 2 rows 0.85 ms.
-constexpr int FO = 8, FR = 4, FL = 16;
-constexpr int FILTER_TASKS = FILTER_BLOCK;      // thread tasks a block aims at
+constexpr int FL = 16;                          // loads of a lane under way at a time
 
-struct FilterShape {
-    int nb;          // sources of a parity, rounded up to a multiple of FO
-    int oct;         // output groups of FO per parity
-    int stride;      // samples of a row and parity in shared memory
-    int tab;         // padded coefficients per parity
-    int rows;        // rows per block, a multiple of FR
-};
-
-__host__ __device__ inline int filter_pad(int i) { return i + i / FO; }
-
-inline FilterShape filter_shape(int nu) {
-    FilterShape f;
-    f.nb = ((nu + 1) / 2 + FO - 1) / FO * FO;
-    f.oct = f.nb / FO;
-    f.stride = f.nb + 4;
-    f.tab = (filter_pad(2 * f.nb + FO) + 3) / 4 * 4;
-    const int groups = FILTER_TASKS / (2 * f.oct);
-    f.rows = FR * (groups < 1 ? 1 : groups);
-    return f;
-}
-
-inline size_t filter_smem(const FilterShape& f) { return sizeof(float) * ((size_t)2 * f.rows * f.stride + 2 * f.tab); }
-
-__global__ void __launch_bounds__(FILTER_BLOCK, 3) fdk_filter_kernel(const FilterParams p, const FilterShape f,
+__global__ void __launch_bounds__(FILTER_BLOCK, FILTER_BLOCKS_PER_SM) fdk_filter_kernel(const FilterParams p, const FilterShape f,
                                                                     int64_t n_rows, const float* __restrict__ g,
                                                                     float* __restrict__ out) {
     extern __shared__ __align__(16) float sm[];
@@ -112,8 +89,10 @@ __global__ void __launch_bounds__(FILTER_BLOCK, 3) fdk_filter_kernel(const Filte
         }
     }
     __syncthreads();
-    const int tasks = (f.rows / FR) * 2 * f.oct;
-    for (int task = threadIdx.x; task < tasks; task += FILTER_BLOCK) {
+    // this block's part of the rows' tasks
+    const int per_part = (filter_tasks(f) + f.parts - 1) / f.parts, first = blockIdx.y * per_part;
+    const int tasks = min(filter_tasks(f), first + per_part);
+    for (int task = first + threadIdx.x; task < tasks; task += FILTER_BLOCK) {
         const int o = task % f.oct, par = (task / f.oct) & 1, rg = task / (2 * f.oct);
         const uint64_t* q2 = reinterpret_cast<const uint64_t*>(q);            // one sample of two rows
         const uint64_t* own = q2 + (size_t)(par * (f.rows / 2) + rg * (FR / 2)) * f.stride + o * FO;
@@ -458,14 +437,18 @@ extern "C" GDRR_API int gdrr_fdk_filter(const gdrr_fdk_geometry* g, int32_t n_pr
     p.mag_dv = (float)(g->dv_mm * mag);
     p.sad = (float)g->sad_mm;
     p.scale = (float)(0.5 / (g->du_mm * mag));
-    const gdrr::FilterShape f = gdrr::filter_shape(g->nu);
-    const size_t smem = gdrr::filter_smem(f);
-    // (the widest row's shape needs the most)
-    if (gdrr::allow_smem(gdrr::fdk_filter_kernel, gdrr::filter_smem(gdrr::filter_shape(gdrr::FILTER_MAX_NU))) != cudaSuccess)
+    const int64_t n_rows = (int64_t)g->nv * n_proj, n = n_rows * g->nu;
+    const bool apart = std::less_equal<const float*>()(proj_dev + n, filtered_dev) ||
+                       std::less_equal<const float*>()(filtered_dev + n, proj_dev);
+    int dev = 0, n_sm = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return GDRR_ERR_CUDA;
-    const int64_t n_rows = (int64_t)g->nv * n_proj;
-    gdrr::fdk_filter_kernel<<<(unsigned)((n_rows + f.rows - 1) / f.rows), gdrr::FILTER_BLOCK, smem,
-                              (cudaStream_t)cuda_stream>>>(p, f, n_rows, proj_dev, filtered_dev);
+    const gdrr::FilterShape f = gdrr::filter_shape(g->nu, n_rows, n_sm, apart);
+    if (gdrr::allow_smem(gdrr::fdk_filter_kernel, gdrr::filter_smem_most()) != cudaSuccess) return GDRR_ERR_CUDA;
+    const dim3 grid((unsigned)((n_rows + f.rows - 1) / f.rows), (unsigned)f.parts);
+    gdrr::fdk_filter_kernel<<<grid, gdrr::FILTER_BLOCK, gdrr::filter_smem(f), (cudaStream_t)cuda_stream>>>(
+        p, f, n_rows, proj_dev, filtered_dev);
     return cudaGetLastError() == cudaSuccess ? GDRR_OK : GDRR_ERR_CUDA;
 }
 
