@@ -1,12 +1,14 @@
 // BF16 GEMM on the 5th-generation tensor cores (tcgen05) of sm_103a, for the
-// convolutions of the learned scatter estimator.  Three GEMM forms: the one
+// convolutions of the learned scatter estimator.  Four GEMM forms: the one
 // below, whose threads stage the tiles (outputs narrower than 32 columns, or
 // no tensor-map encoder); a TMA-fed, multi-stage, warp-specialised form with
-// one tile per CTA for 64 < N < 256; and its persistent form with two TMEM
-// accumulators for N >= 256 and for 32 <= N <= 64.  All read operand rows in
-// 16-byte pieces: A and B start on 16-byte boundaries.  A fourth kernel, the
-// implicit-GEMM convolution, takes its A tiles straight from an NHWC
-// activation tensor by 4-D TMA copies (further below).
+// one tile per CTA for 64 < N < 256; its persistent form with two TMEM
+// accumulators for 32 <= N <= 64; and pairs of CTAs on 256 x 256 tiles for N >=
+// 256 (the persistent form where the pairs' TMA stores do not apply).  All read
+// operand rows in 16-byte pieces: A and B start on 16-byte boundaries.  Three
+// more kernels take their tiles straight from NHWC tensors by 4-D TMA copies: the
+// implicit convolution, its tap-ordered form for any grid, and the implicit
+// weight gradient (further below).
 //
 //   C[M x N] (FP32)  =  A[M x K] . B[N x K]^T      (A, B BF16, rows K-contiguous)
 //
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_bf16_kernel(const __nv_bflo
 }
 
 // ---------------------------------------------------------------------------
-// The TMA-fed, pipelined form for outputs at least 128 columns wide.
+// The TMA-fed, pipelined form for outputs of 65 to 255 columns.
 //
 // Operand tiles (128 x 64 of A, BN x 64 of B) arrive by TMA
 // (cp.async.bulk.tensor) in the tensor core's 128-byte-swizzled K-major layout
@@ -1019,7 +1021,8 @@ __global__ void __launch_bounds__(PERSIST_THREADS) conv_implicit_kernel(
 // both CTAs' copies, its commits reach both CTAs' "empty" and accumulator barriers,
 // and both epilogues release an accumulator to it.
 //
-// Bound: the tensor cores (8192^3 at 0.94 of the measured cuBLAS rate).  One CTA a
+// Bound: the tensor cores (8192^3: the kernel alone at 0.95 of the measured cuBLAS
+// rate, 1.94 PFLOP/s, a call with its allocation and status at 0.82 to 0.9).  One CTA a
 // tile of 128 x 256, whose instruction takes 175 clocks where the peak's rate is
 // 128, and lanes that store their rows: 8192^3 in 0.69 ms, 0.60 so; a call at 8192
 // x 8192 x 512 156 us -> 126, x 64, where the epilogue bound it, 140 -> 86.
@@ -1721,9 +1724,12 @@ int conv_stages(int Wb, int BN, int mt) {
 // passes of n_sm tiles, each its stages' longer one of copies (39 bytes per SM
 // and cycle) and MMAs (60 + 0.45 N cycles), but no less than its epilogue (900
 // cycles per 32 columns and subtile), which adds to it where a second set of
-// accumulators does not fit to hide it.  The four rates reproduce the measured
-// times of every layer of the estimator at batches 16 and 64 for one to four
-// subtiles to 15 %.
+// accumulators does not fit to hide it.  For the three large layers of the
+// estimator (d1, d2, d3 at batches 16 and 64, one to four subtiles) the estimates
+// lie within 23 % of the measured times; the two small ones (e2, e3) take 6 to 9 us
+// more than theirs, whatever the count.  The chosen count is the fastest in five of
+// the ten cases, within 0.7 us of it in two and 2 to 4.5 us (8 to 13 %) behind it in
+// e2, e3 and d2 at 64.
 int conv_subtiles(int M, int H, int Wb, int tiles_n, int BN, int n_kb, int n_sm) {
     int best = 1;
     double least = 0.0;
@@ -2063,11 +2069,12 @@ cudaError_t launch_conv_tap(const ConvArgs& a, const __nv_bfloat16* w, int ldw, 
 // of waves x the longest of a stage's copies (38 bytes a clock and SM), its MMAs
 // (60 + 0.45 NB clocks each) and its issue (600 clocks).  The pixel ranges are
 // given (they fix the order of the sums), so a narrow layer fills the chip by
-// smaller blocks.
+// smaller blocks.  At batches 16 and 64 of the estimator's six layers the choice is
+// within 4 % of the fastest of the plans with 1 to 12 slabs and 32 to 128 channels.
 struct WgradSplit {
     int group, nb;
 };
-static WgradSplit wgrad_plan(int ks, int C, int N, int splits, int per_split) {
+static WgradSplit wgrad_plan(int ks, int C, int N, int splits, int per_split, int n_sm) {
     const int slabs = ks * C / CONV_BK;
     WgradSplit best{1, 32};
     double least = 1e300;
@@ -2076,7 +2083,7 @@ static WgradSplit wgrad_plan(int ks, int C, int N, int splits, int per_split) {
         for (int gs = 1; gs <= std::min(WG_SLABS, slabs); ++gs) {
             const int64_t blocks = (int64_t)splits * ks * ((slabs + gs - 1) / gs) * (N / nb);
             const double copies = (gs + nb / 32) * WG_SLAB / 38.0, mma = 4.0 * ((gs + 3) / 4) * (60.0 + 0.45 * nb);
-            const double t = (double)((blocks + 151) / 152) * (3000.0 + per_split * std::max({copies, mma, 600.0}));
+            const double t = (double)((blocks + n_sm - 1) / n_sm) * (3000.0 + per_split * std::max({copies, mma, 600.0}));
             if (t < least) {
                 least = t;
                 best = {gs, nb};
@@ -2101,7 +2108,11 @@ cudaError_t launch_conv_wgrad(const __nv_bfloat16* x, int ks, int C, int ldx, in
     g.tiles = (int)((P + WG_PIX - 1) / WG_PIX);
     g.per_split = (g.tiles + std::max(1, std::min(splits, g.tiles)) - 1) / std::max(1, std::min(splits, g.tiles));
     *used = splits = (g.tiles + g.per_split - 1) / g.per_split;
-    const WgradSplit plan = wgrad_plan(ks, C, N, splits, g.per_split);
+    int dev = 0, n_sm = 1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const WgradSplit plan = wgrad_plan(ks, C, N, splits, g.per_split, n_sm);
     const int nb = plan.nb;
     // a copy: as many pixels as divide both a row and a stage, and whole rows
     // where a stage is whole rows of one image
@@ -2177,8 +2188,8 @@ cudaError_t launch_gemm_bf16(const void* A, int lda, const void* B, int ldb, flo
         *splits_used = (k_slices + per - 1) / per;
     }
     if (N < 32) return launch_gemm_t<32>(a, lda, b, ldb, C, ldc, M, N, K, splits, partial_stride, err, s);
-    // measured at 8192^3 (fraction of the BF16 peak): pairs of CTAs on 256 x 256
-    // 0.94; one CTA a tile, persistent and 256 wide with two TMEM accumulators
+    // kernels measured at 8192^3 (fraction of the BF16 peak): pairs of CTAs on 256 x
+    // 256 0.95; one CTA a tile, persistent and 256 wide with two TMEM accumulators
     // 0.78, which takes what the pairs' TMA stores cannot (rows of C that are not
     // multiples of 16 bytes, splits that add up in place) and a single row of
     // tiles; per-tile CTAs, two per SM, 256 x 2 stages 0.74 and 128 x 3 0.67.
