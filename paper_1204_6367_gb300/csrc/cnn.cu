@@ -26,11 +26,13 @@
 //   forward   Y[P x Co]   = cols(x)[P x 9Ci] . W[Co x 9Ci]^T
 //   data grad dX[P x Ci]  = cols(dZ)[P x 9Co] . Wf[Ci x 9Co]^T   (Wf: taps flipped)
 //   weight    dW[Co x 9Ci] = dZ^T[Co x P] . cols(x)[P x 9Ci]
-// The forward and data-gradient products run as implicit GEMMs
-// (launch_conv_implicit: the tensor-core kernel loads each tap's shifted input
-// tile by TMA, no column matrix) where the layer's grid tiles into 128-pixel
-// rows; otherwise, and for the weight gradient (whose K runs over pixels),
-// a column matrix is built and multiplied by launch_gemm_bf16.
+// The tensor-core kernels copy each tap's shifted pixels by TMA, so that no column
+// matrix is written, where the channel counts are multiples of 32: forward and
+// data gradient by launch_conv_implicit on grids that tile into 128-pixel rows and
+// by launch_conv_tap on any other, the weight gradient (whose K runs over pixels)
+// by launch_conv_wgrad where 16 pixels fit a row.  Otherwise a column matrix is
+// built and multiplied by launch_gemm_bf16.  The first layer has a kernel of its
+// own (first_layer_kernel).
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>

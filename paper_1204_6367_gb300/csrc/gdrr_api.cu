@@ -543,7 +543,8 @@ void set_defaults(gdrr_mc_options* o) {
 // L2); the results do not depend on the choice.  With local majorants the
 // cells are the flights' majorant and every cell a flight passes costs a
 // crossing: about 32 mm by default (on the 2 mm torso, 8, 16, 32 and 64 mm
-// cells gave 92.2, 71.8, 70.3 and 87.5 ms per 1e8 histories).
+// cells take 70.7, 54.5, 54.9 and 71.1 ms per 1e8 histories; the draws depend
+// on the size, so the default stays).
 int default_cell_shift(const gdrr_ctx* c, bool local_majorant) {
     const double v = std::min(c->vox[0], std::min(c->vox[1], c->vox[2]));
     const int s = (int)std::lround(std::log2((local_majorant ? 32.0 : 4.0) / v));
@@ -1245,7 +1246,7 @@ static int denoise_scratch(gdrr_ctx* ctx, int nu, int nv) {
 
 // Step 3's iteration with the scalars on the host (scal_dev NULL) or on the
 // device (scal_dev[0] count scale, [1] beta): one cooperative launch when the
-// image fits its bands, else one launch per iteration.
+// image fits a tile per SM, else one launch per iteration.
 static int denoise_on_ctx(gdrr_ctx* ctx, const double* S_hat_dev, double* S_dev, int nu, int nv, double count_scale,
                           double beta, const double* scal_dev, double omega, int iters, bool* fused) {
     int rc = denoise_scratch(ctx, nu, nv);

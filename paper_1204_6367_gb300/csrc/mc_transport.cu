@@ -1055,8 +1055,8 @@ constexpr int WARP_BLOCK = 32 * POOL_WARPS;   // threads; the warps of a block s
 // within 2 %, 4 was 3 % slower (a hand-over costs about half a flight).
 constexpr int REFILL_IDLE = 8;
 // With local majorants a third of the flights stop in every cell, so a refill at 8
-// would come after each: 2e7 histories of the 2 mm torso take 14.17 ms at 8, 13.93
-// at 14, 13.67 at 18, 13.57 from 20 to 24 and 14.17 at 30.
+// would come after each: 2e7 histories of the 2 mm torso take 12.9 ms at 8, 12.7 at
+// 14, 12.5 at 18, 12.4 from 20 to 24, 12.6 at 26 and 13.5 at 30.
 constexpr int REFILL_IDLE_LM = 22;
 // a slot's flags beside its job
 constexpr uint32_t JF_SCATTERED = 0x80000000u, JF_DEAD = 0x40000000u, JF_RAYLEIGH = 0x20000000u, JF_JOB = 0x1fffffffu;
